@@ -94,6 +94,7 @@ int run_layer(dsvt_ctx* ctx, const float* x, int32_t n, const int32_t* table, in
     a.rowoff = rowoff_scratch;
   }
   if (tc) return dsvt_launch_layer_tc(ctx, a);
+  if (dsvt_layer_f32_supported(a)) return dsvt_launch_layer_f32(ctx, a);
   return dsvt_launch_layer_fma(ctx, a);
 }
 

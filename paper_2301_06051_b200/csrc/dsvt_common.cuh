@@ -114,6 +114,9 @@ struct dsvt_fused_args {
   int32_t attention_only;  // 1: y = attention output (no residual, LN, MLP)
 };
 int dsvt_launch_layer_fma(dsvt_ctx* ctx, const dsvt_fused_args& a);
+// fp32 weights, C in {64, 128, 192}, hidden in {0, C, 2C} (layer_f32.cu); everything else is layer_fma.cu's.
+bool dsvt_layer_f32_supported(const dsvt_fused_args& a);
+int dsvt_launch_layer_f32(dsvt_ctx* ctx, const dsvt_fused_args& a);
 // tcgen05 path: bfloat16 weights, C in {64, 128, 192}, head dim in {16, 24, 32}, set size <= 96.
 bool dsvt_layer_tc_supported(const dsvt_fused_args& a);
 int dsvt_launch_layer_tc(dsvt_ctx* ctx, const dsvt_fused_args& a);
@@ -122,9 +125,10 @@ int dsvt_launch_layer_tc(dsvt_ctx* ctx, const dsvt_fused_args& a);
 // DSVT_MAX_CHAIN_LAYERS layers; every voxel a later layer reads must be written by the layer before it.
 bool dsvt_layer_tc_chainable(const dsvt_fused_args& a, const dsvt_fused_args& b);
 int dsvt_launch_layers_tc(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_layers);
-// CUtensorMap (128 bytes, 64-byte aligned) of a row-major bf16 matrix [rows][cols]: boxes of 64 columns x box_rows
-// rows, 128-byte swizzle; encoded once per matrix and context.  Returns false if the driver cannot encode it.
-bool dsvt_cached_weight_map(dsvt_ctx* ctx, void* tensor_map, const void* w, int rows, int cols, int box_rows);
+// CUtensorMap (128 bytes, 64-byte aligned) of a row-major bf16 (fp32) matrix [rows][cols]: boxes of 64 (32) columns x
+// box_rows rows, 128-byte swizzle; encoded once per matrix and context.  Returns false if the driver cannot encode it.
+bool dsvt_cached_weight_map(dsvt_ctx* ctx, void* tensor_map, const void* w, int rows, int cols, int box_rows,
+                            bool fp32 = false);
 
 // Attention-style pooling with the projections on tcgen05 (pool_tc.cu): bfloat16 weights, C / head dim as for the
 // layer kernel, a power-of-two number of slots per region (at most 32).  The region bookkeeping (cell map, region

@@ -1,0 +1,43 @@
+"""The fp32 layer kernel through the C ABI against the CPU oracle, at the sizes where its tiling changes.  Needs a B200."""
+import numpy as np
+import pytest
+import torch
+
+import dsvt_inputs as di
+from gpu_helpers import check_close, dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,grid,window,tau,C,heads,hidden,option", [
+    (1, 24, 12, 36, 128, 8, 0, ""),           # one voxel: one row, blocks without work
+    (9, 12, 12, 36, 192, 8, 192, "pe"),       # one set of nine rows: 8-row groups of a thread tile
+    (144, 12, 12, 36, 192, 8, 384, ""),       # one full window: four sets of 36 rows, one per tile
+    (560, 24, 12, 64, 192, 8, 384, "rpb"),    # fewer rows than blocks x set size; sets of up to 64 rows, a tile's most
+    (3000, 60, 30, 96, 128, 4, 256, ""),      # tiles of up to 96 rows, head dim 32
+    (9000, 100, 12, 36, 64, 4, 128, "pe"),    # several tiles per block
+    (20000, 150, 12, 36, 128, 8, 128, "rpb"),
+])
+def test_layer_fp32_matches_oracle(oracle, n, grid, window, tau, C, heads, hidden, option):
+    from paper_2301_06051_b200 import api
+
+    case = di.random_case(n + C, n, (grid, grid, 1), (window, window, 1), tau, C, heads, hidden, layernorm=hidden > 0)
+    layer = case["blocks"][0][0]
+    rng = np.random.default_rng(n)
+    pe = rng.standard_normal((n, C)).astype(np.float32) if option == "pe" else None
+    if option == "rpb":
+        layer["rpb"] = rng.standard_normal((heads, (2 * window - 1) ** 2)).astype(np.float32)
+        layer["rpb_extent"] = (window, window, 1)
+    ctx = api.Context(n, (-(-grid // window)) ** 2, C)
+    coords, x = dev(case["coords"]), dev(case["feats"])
+    table = ctx.partition(coords, 1, case["grid"], case["window"], tau, 0)
+    w = api.device_weights(layer, api.FP32, ctx.device)
+    y = torch.empty_like(x)
+    ctx.layer(x, table, w, y, pe=None if pe is None else dev(pe), coords=coords)
+    assert ctx.status_sync() == 0
+    p = oracle.partition(case["coords"], 1, case["grid"], case["window"], tau, 0)
+    want = oracle.layer(case["feats"], p.set_table, layer, pe=pe, coords=case["coords"])
+    check_close(y.cpu().numpy(), want, "fp32", "n=%d C=%d" % (n, C))
+    z = x.clone()  # in place: a tile's rows are its own
+    ctx.layer(z, table, w, z, pe=None if pe is None else dev(pe), coords=coords)
+    assert ctx.status_sync() == 0 and torch.equal(y, z)
