@@ -21,10 +21,12 @@
 // operand (if its rows are ready by then), so that its first projections overlap the current tile's tail.
 //
 // The projections of a layer are chunks of at most 192 output columns (K, V, Q, O, MLP-1 in pieces of
-// 128 or 64 hidden columns, MLP-2), accumulated in three TMEM regions (map at compute_role) so the
+// 128 or 64 hidden columns, MLP-2), accumulated in TMEM (map at Tm) so the
 // tensor pipe works on one chunk while the compute warps drain another.  The fp32 residual stream never
 // leaves the chip inside a layer: x is staged in shared memory for the first residual, and
-// x1 + b_2 = LN1(x + attention) + b_2 is parked in TMEM, where MLP-2 accumulates on top of it.
+// x1 + b_2 = LN1(x + attention) + b_2 is parked in TMEM, where MLP-2 accumulates on top of it.  x1 and the MLP hidden
+// are A operands in TMEM, the hidden one piece at a time: MLP-2 of a piece runs under the GELU of the next, and the
+// tensor pipe reads half the shared memory it would need for both operands.
 //
 // Every operand tile in shared memory uses the K-major 128-byte-swizzled layout that tcgen05.mma and
 // TMA share: 64 bf16 columns per 128-byte row, 8-row groups of 1024 bytes, 16-byte chunk index XORed
@@ -59,10 +61,19 @@ constexpr int kStages = 3;             // weight ring depth
 constexpr int kStampPolls = 1 << 18;  // polls of a row's stamp, about a microsecond each
 constexpr int kMaxLayers = DSVT_MAX_CHAIN_LAYERS;  // layers one launch can chain
 
+// TMEM map (512 columns): K, then Q accumulate at 0, V at C; R = the last C columns: output projection, x1 + b_2 parked,
+// MLP-2 on top of it; x1 as a bf16 A operand at 0; an MLP-1 accumulator piece (128 columns); an MLP hidden piece as a
+// bf16 A operand (64).  The next tile's K starts once x1 and the last MLP-1 piece are dead, its V (which overlaps the
+// hidden piece and, for C = 192, R) once R has been read.
+template <int C>
+struct Tm {
+  static constexpr uint32_t k = 0, v = C, x1 = 0, acc = C / 2, h = C / 2 + 128, r = kTmemCols - C;
+  static_assert(2 * C <= kTmemCols && h + 64 <= r, "TMEM");
+};
+
 struct TcGeom {
   int hidden, heads, tau;
-  int nkb_h;    // hidden / 64: K blocks of the MLP-2 contraction
-  int NF;       // MLP-1 chunk width (128 or 64)
+  int NF;       // MLP piece: hidden columns (128 or 64)
   int n_f1;     // hidden / NF
   int mode;     // 0: attention only, 1: attention + residual + LN1, 2: full layer
   uint32_t off_a, off_kv, off_stage, off_par;  // byte offsets from the 1024-aligned base
@@ -95,9 +106,11 @@ struct TcArgs {
 };
 
 struct Misc {  // small shared state beside the big regions
-  // weight ring; accumulator regions 0 / 1 / 2 (see the TMEM map at compute_role); operand hand-offs
+  // weight ring; accumulators K / Q / MLP-1, V, R (see Tm); operand hand-offs
   unsigned long long full[kStages], empty[kStages], acc_full[3], acc_free[3];
-  unsigned long long a_ready;   // compute warps -> MMA: attention output / x1 / MLP hidden is in place
+  unsigned long long o_full;           // output projection done
+  unsigned long long h_ready, h_free;  // MLP hidden piece in TMEM: written / read by MLP-2
+  unsigned long long a_ready;   // compute warps -> MMA: attention output / x1 is in place
   unsigned long long x_ready;   // compute warps -> MMA: the gathered rows of a tile are in the A operand
   unsigned long long rl_ready[2];   // loader warp -> compute: row-list buffer b describes its next tile
   unsigned long long dep_ready[2];  // loader warp -> compute: the rows listed in buffer b carry the previous layer's stamp
@@ -344,7 +357,7 @@ struct RoleCtx {
   uint32_t sbase;     // 1024-aligned shared-memory base as a shared-space address
   uint32_t tmem;      // TMEM base address of the CTA's allocation
   // copies of the kernel parameters the two single-thread roles use (registers instead of parameter-space loads)
-  int mode, n_f1, NF, nkb_h, tau, n_layers;
+  int mode, n_f1, NF, tau, n_layers;
   int pe;  // the value projection comes first and the A operand is rewritten (x + pe) before the key and query ones
   uint32_t off_a, off_kv, off_stage;
 };
@@ -356,6 +369,15 @@ __device__ __forceinline__ int ld_acquire_gpu(const int32_t* p) {
 }
 __device__ __forceinline__ void st_relaxed_gpu(int32_t* p, int v) {
   asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// Order of the MLP pieces: M1(0), M1(1), M2(0), M1(2), M2(1), ..., M1(n-1), M2(n-2), M2(n-1), so that the next
+// piece's first product runs while the compute warps apply GELU to the current one.  q in [0, 2n): piece and kind.
+__device__ __forceinline__ bool mlp_step(int q, int n, int& piece) {  // true: M1
+  if (q == 0) { piece = 0; return true; }
+  if (q == 2 * n - 1) { piece = n - 1; return false; }
+  piece = (q & 1) ? (q + 1) >> 1 : (q >> 1) - 1;
+  return (q & 1) != 0;
 }
 
 // The scheduler and the MMA issuer are separate (not inlined) functions so that their polling loops get
@@ -376,7 +398,7 @@ __device__ __noinline__ void producer_role(const TcArgs& a, const RoleCtx rc) {
   volatile int* abort_flag = &mi->abort_flag;
   int32_t* status = a.status;
   const bool mlp = rc.mode == 2;
-  const int n_chunks = 4 + (mlp ? rc.n_f1 + 1 : 0);
+  const int n_chunks = 4 + (mlp ? 2 * rc.n_f1 : 0);
   const int L = rc.n_layers;
   const int Rv = kTM - rc.tau + 1;
   // the chain's tile counts
@@ -458,19 +480,22 @@ __device__ __noinline__ void producer_role(const TcArgs& a, const RoleCtx rc) {
     const TcLayer& ly = a.layer[wl[wread & 1]];
     for (int c = 0; c < n_chunks; ++c) {
       const CUtensorMap* map;
-      int row0, nkb;
+      int row0 = 0, col0 = 0, nkb = NKB;
       uint32_t bytes = STAGE_BYTES;
       if (c < 3) {  // K, V, Q; with a positional term V, K, Q
-        map = &ly.qkv; nkb = NKB;
+        map = &ly.qkv;
         row0 = (rc.pe ? (c == 0 ? 2 : c == 1 ? 1 : 0) : (c == 0 ? 1 : c == 1 ? 2 : 0)) * C;
+      } else if (c == 3) {
+        map = &ly.o;
+      } else {
+        int piece;
+        if (mlp_step(c - 4, rc.n_f1, piece)) { map = &ly.w1; row0 = piece * rc.NF; bytes = (uint32_t)rc.NF * 128u; }
+        else { map = &ly.w2; col0 = piece * rc.NF; nkb = rc.NF / 64; }
       }
-      else if (c == 3) { map = &ly.o; row0 = 0; nkb = NKB; }
-      else if (c < 4 + rc.n_f1) { map = &ly.w1; row0 = (c - 4) * rc.NF; nkb = NKB; bytes = (uint32_t)rc.NF * 128u; }
-      else { map = &ly.w2; row0 = 0; nkb = rc.nkb_h; }
       for (int kb = 0; kb < nkb; ++kb) {
         if (!mbar_wait(&mi->empty[stage], phase ^ 1u, abort_flag)) goto producer_done;
         mbar_expect_tx(&mi->full[stage], bytes);
-        tma_load_2d(st_base + stage * STAGE_BYTES, map, kb * 64, row0, &mi->full[stage]);
+        tma_load_2d(st_base + stage * STAGE_BYTES, map, col0 + kb * 64, row0, &mi->full[stage]);
         ++issued[stage];
         if (++stage == kStages) { stage = 0; phase ^= 1u; }
       }
@@ -495,63 +520,85 @@ producer_done:
 template <int C>
 __device__ __noinline__ void mma_role(const RoleCtx rc) {
   constexpr int NKB = C / 64;        // K blocks of a C-deep contraction
-  constexpr uint32_t COL_B = C;      // second accumulator buffer
   constexpr uint32_t STAGE_BYTES = C * 128;
-  const uint32_t sbase = rc.sbase, tmem = rc.tmem;
+  const uint32_t tmem = rc.tmem;
   Misc* mi = &s_mi;
-  const uint32_t a_base = sbase + rc.off_a, kv_base = sbase + rc.off_kv, st_base = sbase + rc.off_stage;
+  const uint32_t a_base = rc.sbase + rc.off_a, st_base = rc.sbase + rc.off_stage;
   volatile int* abort_flag = &mi->abort_flag;
   const bool mlp = rc.mode == 2;
-  const int n_chunks = 4 + (mlp ? rc.n_f1 + 1 : 0);
+  const int c_v = rc.pe ? 0 : 1;  // the V chunk
   int stage = 0, slot = 0;
-  uint32_t phase = 0, a_phase = 0, x_phase = 0, sphase = 0;
-  uint32_t uses[3] = {0u, 0u, 0u};  // how often each accumulator region has been used
-  for (;;) {
+  uint32_t phase = 0, a_phase = 0, x_phase = 0, sphase = 0, tile = 0;
+  uint32_t uses = 0, m2 = 0;  // of the K / Q / MLP-1 accumulator; MLP-2 pieces
+  // n_kb K blocks of 64 from the weight ring; issue(kb, k4, B descriptor) issues one MMA
+  auto blocks = [&](int n_kb, auto issue) -> bool {
+    for (int kb = 0; kb < n_kb; ++kb) {
+      if (!mbar_wait(&mi->full[stage], phase, abort_flag)) return false;
+      tc_fence_after();
+      const uint32_t sb = st_base + stage * STAGE_BYTES;
+#pragma unroll
+      for (int k4 = 0; k4 < 4; ++k4) issue(kb, k4, umma_desc(sb + k4 * 32));
+      umma_commit(&mi->empty[stage]);  // frees the weight stage once these MMAs have read it
+      if (++stage == kStages) { stage = 0; phase ^= 1u; }
+    }
+    return true;
+  };
+  for (;; ++tile) {
     if (!mbar_wait(&mi->sched_full[slot], sphase, abort_flag)) break;
     const int ns = mi->tile[slot][1];
     mbar_arrive(&mi->sched_empty[slot]);
     if (++slot == 2) { slot = 0; sphase ^= 1u; }
     if (ns < 0) break;
-    for (int c = 0; c < n_chunks; ++c) {
-      // a fresh A operand: X (chunks 0-2), attention output (3), x1 (4..), MLP hidden (last)
+    // ---- K, V, Q, then the output projection ----
+    for (int c = 0; c < 4; ++c) {
       if (c == 0 || (c == 1 && rc.pe)) {  // (with a positional term the operand is rewritten after the V chunk)
         if (!mbar_wait(&mi->x_ready, x_phase, abort_flag)) goto mma_done;
         x_phase ^= 1u;
-      } else if (c == 3 || c == 4 || c == 4 + rc.n_f1) {
+      } else if (c == 3) {
         if (!mbar_wait(&mi->a_ready, a_phase, abort_flag)) goto mma_done;
         a_phase ^= 1u;
       }
-      // accumulator placement: K -> region 0, V -> 1, Q -> 0, O -> 0, MLP-1 piece i -> i & 1, MLP-2 -> 2
-      // (on top of the parked x1 + b_2)
-      uint32_t bar, col, n;
-      const int c_v = rc.pe ? 0 : 1;  // the V chunk
-      if (c < 4) { bar = (c == c_v) ? 1u : 0u; col = (c == c_v) ? COL_B : 0u; n = C; }
-      else if (c < 4 + rc.n_f1) { bar = (uint32_t)(c - 4) & 1u; col = bar * COL_B; n = (uint32_t)rc.NF; }
-      else { bar = 2u; col = kTmemCols - C; n = C; }
       if (c == c_v) {
-        // region 1 may overlap region 2: the previous tile's MLP-2 result must have been read
-        if (!mbar_wait(&mi->acc_free[2], (uses[2] & 1u) ^ 1u, abort_flag)) goto mma_done;
+        // the columns may overlap R and the MLP hidden: the previous tile's result must have been read
+        if (!mbar_wait(&mi->acc_free[2], (tile & 1u) ^ 1u, abort_flag)) goto mma_done;
+        if (!mbar_wait(&mi->acc_free[1], (tile & 1u) ^ 1u, abort_flag)) goto mma_done;
+      } else if (c < 3) {
+        if (!mbar_wait(&mi->acc_free[0], (uses & 1u) ^ 1u, abort_flag)) goto mma_done;
+        ++uses;
       }
-      if (bar != 2u && !mbar_wait(&mi->acc_free[bar], (uses[bar] & 1u) ^ 1u, abort_flag)) goto mma_done;
-      ++uses[bar];
       tc_fence_after();
-      const bool last = mlp && c == 4 + rc.n_f1;
-      const uint32_t abase = last ? kv_base : a_base;
-      const int nkb = last ? rc.nkb_h : NKB;
-      const uint32_t idesc = umma_idesc((int)n);
-      const uint32_t d_tmem = tmem + col;
-      for (int kb = 0; kb < nkb; ++kb) {
-        if (!mbar_wait(&mi->full[stage], phase, abort_flag)) goto mma_done;
-        tc_fence_after();
-        const uint32_t sa = abase + kb * (kTM * 128), sb = st_base + stage * STAGE_BYTES;
-#pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4)
-          umma_bf16(d_tmem, umma_desc(sa + k4 * 32), umma_desc(sb + k4 * 32), idesc, (last || (kb | k4) != 0) ? 1u : 0u);
-        umma_commit(&mi->empty[stage]);  // frees the weight stage once these MMAs have read it
-        if (++stage == kStages) { stage = 0; phase ^= 1u; }
-      }
-      umma_commit(&mi->acc_full[bar]);
+      const uint32_t d = tmem + (c == 3 ? Tm<C>::r : c == c_v ? Tm<C>::v : Tm<C>::k);
+      if (!blocks(NKB, [&](int kb, int k4, uint64_t b) {
+            umma_bf16(d, umma_desc(a_base + kb * (kTM * 128) + k4 * 32), b, umma_idesc(C), (kb | k4) != 0 ? 1u : 0u);
+          })) goto mma_done;
+      umma_commit(c == 3 ? &mi->o_full : &mi->acc_full[c == c_v ? 1 : 0]);
     }
+    if (!mlp) continue;
+    // ---- MLP, piece by piece, on top of the residual parked in R ----
+    if (!mbar_wait(&mi->a_ready, a_phase, abort_flag)) goto mma_done;
+    a_phase ^= 1u;
+    for (int c = 0; c < 2 * rc.n_f1; ++c) {
+      int piece;
+      if (mlp_step(c, rc.n_f1, piece)) {
+        if (!mbar_wait(&mi->acc_free[0], (uses & 1u) ^ 1u, abort_flag)) goto mma_done;
+        ++uses;
+        tc_fence_after();
+        const uint32_t idesc = umma_idesc(rc.NF);
+        if (!blocks(NKB, [&](int kb, int k4, uint64_t b) {  // (16 bf16 operand columns are 8 TMEM columns)
+              umma_bf16_ts(tmem + Tm<C>::acc, tmem + Tm<C>::x1 + kb * 32 + k4 * 8, b, idesc, (kb | k4) != 0 ? 1u : 0u);
+            })) goto mma_done;
+        umma_commit(&mi->acc_full[0]);
+      } else {
+        if (!mbar_wait(&mi->h_ready, m2 & 1u, abort_flag)) goto mma_done;
+        ++m2;
+        tc_fence_after();
+        if (!blocks(rc.NF / 64, [&](int kb, int k4, uint64_t b) {
+              umma_bf16_ts(tmem + Tm<C>::r, tmem + Tm<C>::h + kb * 32 + k4 * 8, b, umma_idesc(C), 1u);
+            })) goto mma_done;
+        umma_commit(&mi->h_free);
+      }
+    }
+    umma_commit(&mi->acc_full[2]);
   }
 mma_done:
   if (*abort_flag) {
@@ -762,9 +809,9 @@ __device__ __noinline__ void phase_gather(int b, int rows) {
 //   dst_off   byte offset of the destination operand tile from the shared-memory base
 //   c8_0      16-byte chunk index of the chunk's first column in the destination rows
 //   need      number of leading tile rows whose results are needed (warps wholly past it only release)
-// GELU = true applies gelu first (MLP-1); BIAS = false skips the bias (the key projection: a key bias adds
+// BIAS = false skips the bias (the key projection: a key bias adds
 // the same amount q . b_k to every score of a query, which the softmax cancels).
-template <int QC, bool GELU, bool BIAS>
+template <int QC, bool BIAS>
 __device__ __noinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_off, uint32_t dst_off, int c8_0, int need) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
@@ -793,13 +840,46 @@ __device__ __noinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_off
       v[2] = __fadd2_rn(v[2], make_float2(b1.x, b1.y));
       v[3] = __fadd2_rn(v[3], make_float2(b1.z, b1.w));
     }
-    if (GELU) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) v[e] = gelu_fast2(v[e]);
-    }
     *reinterpret_cast<uint4*>(dst + swz(row, c8 + q)) =
         make_uint4(pack_bf16(v[0].x, v[0].y), pack_bf16(v[1].x, v[1].y), pack_bf16(v[2].x, v[2].y), pack_bf16(v[3].x, v[3].y));
   }
+}
+
+// MLP-1 piece: HC = NF / 4 hidden columns per thread, H = gelu(x1 W_1^T + b_1) into TMEM as the A operand of MLP-2.
+//   bias_off  float offset of the piece's bias in the parameter block
+//   h_phase   parity of h_free that says that the MLP-2 of the piece before has read its hidden columns
+template <int C, int HC>
+__device__ __noinline__ void phase_mlp1(int bias_off, uint32_t h_phase) {
+  const int warp = threadIdx.x >> 5, hq = warp >> 2;
+  const uint32_t lane_base = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16);
+  if (32 * (warp & 3) >= s_mi.rows) {  // a warp without rows keeps step with the others
+    tc_fence_before();
+    mbar_arrive(&s_mi.acc_free[0]);
+    mbar_wait(&s_mi.h_free, h_phase, &s_mi.abort_flag);
+    mbar_arrive(&s_mi.h_ready);
+    return;
+  }
+  const float* bias = reinterpret_cast<const float*>(s_mi.sm + s_mi.off_par) + bias_off + hq * HC;
+  float rr[HC];
+  tmem_ld_row(lane_base + Tm<C>::acc + hq * HC, rr);
+  tmem_wait_ld();
+  tc_fence_before();
+  mbar_arrive(&s_mi.acc_free[0]);  // the next piece may be accumulated
+  uint32_t p[HC / 2];
+#pragma unroll
+  for (int q = 0; q < HC / 4; ++q) {
+    const float4 b4 = *reinterpret_cast<const float4*>(bias + 4 * q);
+    const float2 g0 = gelu_fast2(__fadd2_rn(make_float2(rr[4 * q], rr[4 * q + 1]), make_float2(b4.x, b4.y)));
+    const float2 g1 = gelu_fast2(__fadd2_rn(make_float2(rr[4 * q + 2], rr[4 * q + 3]), make_float2(b4.z, b4.w)));
+    p[2 * q] = pack_bf16(g0.x, g0.y);
+    p[2 * q + 1] = pack_bf16(g1.x, g1.y);
+  }
+  mbar_wait(&s_mi.h_free, h_phase, &s_mi.abort_flag);  // (a wait that gives up raises the abort flag)
+  tc_fence_after();
+  tmem_st_row_u32(lane_base + Tm<C>::h + hq * (HC / 2), p);
+  tmem_wait_st();
+  tc_fence_before();
+  mbar_arrive(&s_mi.h_ready);
 }
 
 // x rows (fp32) for the first residual: asynchronous 16-byte copies global -> shared staging.
@@ -886,14 +966,13 @@ __device__ __forceinline__ void layer_norm_rows(float (&t)[QC], float sum, const
 }
 
 // Output-projection epilogue: t = Z + b_o (+ staged x); LayerNorm 1; then either the fp32 rows go to the
-// staging area (mode 0 / 1: final result of the call) or x1 goes to the A operand (bf16) and x1 + b_2 to
-// TMEM region 2 (fp32), where the MLP-2 MMAs accumulate on top of it.  The accumulator is region 0.
+// staging area (mode 0 / 1: final result of the call) or, in TMEM, x1 to the A operand (bf16) and x1 + b_2 back to
+// R (fp32), where the MLP-2 MMAs accumulate on top of it.
 template <int C, int QC>
 __device__ __noinline__ void phase_epi_o() {
-  constexpr uint32_t COL_PARK = kTmemCols - C;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
-  const uint32_t taddr = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + hq * QC;
+  const uint32_t lane_base = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16), taddr = lane_base + Tm<C>::r + hq * QC;
   const float* par = reinterpret_cast<const float*>(s_mi.sm + s_mi.off_par);
   unsigned char* stage = s_mi.sm + s_mi.off_kv;
   const int mode = s_mi.mode;
@@ -903,7 +982,7 @@ __device__ __noinline__ void phase_epi_o() {
   tmem_ld_row(taddr, t);
   tmem_wait_ld();
   tc_fence_before();
-  mbar_arrive(&s_mi.acc_free[0]);
+  if (mode != 2) mbar_arrive(&s_mi.acc_free[2]);  // (R is not used any more)
 #pragma unroll
   for (int q = 0; q < QC / 4; ++q) {
     float4 x4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -928,12 +1007,13 @@ __device__ __noinline__ void phase_epi_o() {
           make_float4(t[4 * i4], t[4 * i4 + 1], t[4 * i4 + 2], t[4 * i4 + 3]);
     return;
   }
-  unsigned char* a_tile = s_mi.sm + s_mi.off_a;
 #pragma unroll
-  for (int q = 0; q < QC / 8; ++q)
-    *reinterpret_cast<uint4*>(a_tile + swz(row, ((hq * QC) >> 3) + q)) =
-        make_uint4(pack_bf16(t[8 * q], t[8 * q + 1]), pack_bf16(t[8 * q + 2], t[8 * q + 3]),
-                   pack_bf16(t[8 * q + 4], t[8 * q + 5]), pack_bf16(t[8 * q + 6], t[8 * q + 7]));
+  for (int c = 0; c < QC / 16; ++c) {
+    uint32_t p[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) p[i] = pack_bf16(t[16 * c + 2 * i], t[16 * c + 2 * i + 1]);
+    tmem_st8_u32(lane_base + Tm<C>::x1 + hq * (QC / 2) + 8 * c, p);
+  }
 #pragma unroll
   for (int q = 0; q < QC / 4; ++q) {
     const float4 b4 = *reinterpret_cast<const float4*>(par + ParOff<C>::b_2 + hq * QC + 4 * q);
@@ -942,20 +1022,18 @@ __device__ __noinline__ void phase_epi_o() {
     t[4 * q + 2] += b4.z;
     t[4 * q + 3] += b4.w;
   }
-  tmem_st_row(taddr + COL_PARK, t);
+  tmem_st_row(taddr, t);
   tmem_wait_st();
   tc_fence_before();
 }
 
-// MLP-2 epilogue: region 2 holds x1 + b_2 + M; LayerNorm 2; fp32 rows to the staging area (the MLP-2 MMAs
-// have read H: its region takes the output rows).  The exchange slots are the first eight bytes of each
+// MLP-2 epilogue: R holds x1 + b_2 + M; LayerNorm 2; fp32 rows to the staging area.  The exchange slots are the first eight bytes of each
 // thread's own output chunk, which is therefore stored last, after one more meeting of the row's threads.
 template <int C, int QC>
 __device__ __noinline__ void phase_epi_f2() {
-  constexpr uint32_t COL_PARK = kTmemCols - C;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
-  const uint32_t taddr = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + COL_PARK + hq * QC;
+  const uint32_t taddr = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + Tm<C>::r + hq * QC;
   const float* par = reinterpret_cast<const float*>(s_mi.sm + s_mi.off_par);
   unsigned char* stage = s_mi.sm + s_mi.off_kv;
   float t[QC];
@@ -1024,18 +1102,13 @@ __device__ __forceinline__ bool compute_all(bool pred) {
   return r != 0;
 }
 
-// TMEM map (512 columns): region 0 = [0, C): K, Q, O and the even MLP-1 pieces; region 1 = [C, 2C): V and
-// the odd MLP-1 pieces; region 2 = [512 - C, 512): x1 + b_2 parked by the output-projection epilogue, then
-// the MLP-2 accumulator.  Each region has its own full / free barrier pair.  For C = 192 regions 1 and 2
-// overlap, which is why the MMA issuer waits for region 2 before it starts the next tile's V.
 template <int C, int D, int NT, int VAR>
 __device__ __forceinline__ void compute_role(const TcArgs& a) {
   constexpr bool RPB = VAR == 1, PE = VAR == 2;
   constexpr int NKB = C / 64;        // K blocks of a C-deep contraction
   constexpr int QC = C / 4;          // epilogue columns per thread for a C-wide chunk (four threads per row)
-  constexpr uint32_t COL_B = C;      // accumulator region 1
   volatile int* abort_flag = &s_mi.abort_flag;
-  uint32_t uses[3] = {0u, 0u, 0u};
+  uint32_t uses[3] = {0u, 0u, 0u}, pieces = 0u;
   int slot = 0;
   uint32_t sphase = 0;
   bool ok = true;
@@ -1107,21 +1180,21 @@ __device__ __forceinline__ void compute_role(const TcArgs& a) {
       // the keys and the queries (the V chunk's accumulator being complete, nothing reads the operand any more)
       acc_wait(1u);
       if (new_params) wait_layer_params();
-      phase_epi_bf16<QC, false, true>(COL_B, 1, ParOff<C>::b_v, s_mi.off_kv + NKB * kTM * 128, 0, rows + 16);
+      phase_epi_bf16<QC, true>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + NKB * kTM * 128, 0, rows + 16);
       phase_gather<C, false, true>(k & 1, rows);
       fence_proxy_async();
       mbar_arrive(&s_mi.x_ready);
       acc_wait(0u);
-      phase_epi_bf16<QC, false, false>(0u, 0, 0, s_mi.off_kv, 0, rows + 16);
+      phase_epi_bf16<QC, false>(Tm<C>::k, 0, 0, s_mi.off_kv, 0, rows + 16);
     } else {
       acc_wait(0u);
-      phase_epi_bf16<QC, false, false>(0u, 0, 0, s_mi.off_kv, 0, rows + 16);
+      phase_epi_bf16<QC, false>(Tm<C>::k, 0, 0, s_mi.off_kv, 0, rows + 16);
       acc_wait(1u);
       if (new_params) wait_layer_params();  // (the key epilogue adds no bias: it needs none of the vectors)
-      phase_epi_bf16<QC, false, true>(COL_B, 1, ParOff<C>::b_v, s_mi.off_kv + NKB * kTM * 128, 0, rows + 16);
+      phase_epi_bf16<QC, true>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + NKB * kTM * 128, 0, rows + 16);
     }
     acc_wait(0u);
-    phase_epi_bf16<QC, false, true>(0u, 0, ParOff<C>::b_q, s_mi.off_a, 0, rows);
+    phase_epi_bf16<QC, true>(Tm<C>::k, 0, ParOff<C>::b_q, s_mi.off_a, 0, rows);
     compute_sync();
     // ---- attention inside each set ----
     attend_blocked<C, D, NT, RPB>();
@@ -1133,27 +1206,22 @@ __device__ __forceinline__ void compute_role(const TcArgs& a) {
       phase_stage_x<C>();
       compute_sync();
     }
-    // ---- chunk 3: output projection epilogue: Z + b_o (+ x, LayerNorm) ----
-    acc_wait(0u);
+    // ---- output projection epilogue: Z + b_o (+ x, LayerNorm) ----
+    ok = mbar_wait(&s_mi.o_full, (uint32_t)k & 1u, abort_flag) && ok;
+    tc_fence_after();
     phase_epi_o<C, QC>();
     if (mode != 2) {  // final result of this layer
       gather_next(k);  // the output projection was the last chunk to read the A operand
     } else {
-      fence_proxy_async();
       mbar_arrive(&s_mi.a_ready);  // x1 (bf16) is the A operand of MLP-1
-      // ---- MLP-1 pieces: H = gelu(x1 W_1^T + b_1) as the A operand of MLP-2 ----
+      // ---- MLP-1 pieces ----
       const int n_f1 = s_mi.n_f1, NF = s_mi.NF;
-      for (int c = 0; c < n_f1; ++c) {
-        const int bar = c & 1;
-        acc_wait((uint32_t)bar);
-        if (NF == 128)
-          phase_epi_bf16<32, true, true>(bar * COL_B, bar, ParOff<C>::b_1 + c * NF, s_mi.off_kv, (c * NF) >> 3, rows);
-        else
-          phase_epi_bf16<16, true, true>(bar * COL_B, bar, ParOff<C>::b_1 + c * NF, s_mi.off_kv, (c * NF) >> 3, rows);
+      for (int c = 0; c < n_f1; ++c, ++pieces) {
+        acc_wait(0u);
+        if (NF == 128) phase_mlp1<C, 32>(ParOff<C>::b_1 + c * NF, (pieces & 1u) ^ 1u);
+        else phase_mlp1<C, 16>(ParOff<C>::b_1 + c * NF, (pieces & 1u) ^ 1u);
       }
-      fence_proxy_async();
-      mbar_arrive(&s_mi.a_ready);  // H is in place
-      gather_next(k);  // the last MLP-1 piece has been drained: nothing reads the A operand any more
+      gather_next(k);  // (the operand has been free since the output projection)
       // ---- MLP-2 epilogue: y = LN2(x1 + M) ----
       acc_wait(2u);
       phase_epi_f2<C, QC>();
@@ -1220,6 +1288,9 @@ __global__ void __launch_bounds__(kThreads, 1) layer_tc_kernel(const __grid_cons
       mbar_init(&mi->dep_ready[i], kLoadThreads);
       mbar_init(&mi->stored[i], kComputeThreads);
     }
+    mbar_init(&mi->o_full, 1);
+    mbar_init(&mi->h_ready, kComputeThreads);
+    mbar_init(&mi->h_free, 1);
     mbar_init(&mi->a_ready, kComputeThreads);
     mbar_init(&mi->x_ready, kComputeThreads);
     mbar_init(&mi->drain, 1);
@@ -1246,7 +1317,7 @@ __global__ void __launch_bounds__(kThreads, 1) layer_tc_kernel(const __grid_cons
   RoleCtx rc;
   rc.sbase = raw + pad;
   rc.tmem = mi->tmem_base;
-  rc.mode = g.mode; rc.n_f1 = g.n_f1; rc.NF = g.NF; rc.nkb_h = g.nkb_h; rc.tau = g.tau; rc.n_layers = a.n_layers;
+  rc.mode = g.mode; rc.n_f1 = g.n_f1; rc.NF = g.NF; rc.tau = g.tau; rc.n_layers = a.n_layers;
   rc.off_a = g.off_a; rc.off_kv = g.off_kv; rc.off_stage = g.off_stage;
   rc.pe = VAR == 2;
 
@@ -1441,7 +1512,6 @@ int dsvt_launch_layers_tc(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_la
   g.heads = p.heads;
   g.tau = p.set_size;
   g.mode = a0.attention_only ? 0 : (g.hidden > 0 ? 2 : 1);
-  g.nkb_h = g.hidden / 64;
   g.NF = (g.hidden % 128 == 0 && C >= 128) ? 128 : 64;
   g.n_f1 = g.hidden / g.NF;
   g.rb_len = g.rb_sx = g.rb_sy = g.rb_centre = 0;
