@@ -137,7 +137,7 @@ struct Misc {  // small shared state beside the big regions
   int n, tau, heads, mode, NF, n_f1, ln1, ln2;
   float eps;
   // the tile the compute warps are working on, and which row-list buffer describes it
-  int s_lo, nsets, base, rows, buf, layer;
+  int rows, buf;
   int next_rows[2];        // rows of the tile listed in buffer b (< 0: there is no such tile), valid after rl_ready[b]
   const float* next_x[2];  // where that tile's input rows are read from
   int st_rows[2], st_stamp[2];  // for the stamp warp: rows of the stored tile in buffer b, the stamp they get (0: none)
@@ -195,7 +195,7 @@ __device__ __forceinline__ float rpb_term(const float* __restrict__ tab, int lin
 // NTB = key blocks of 8 a row block can need: ceil((2 tau + 14) / 8), at most the 16 of a whole tile.
 // ---------------------------------------------------------------------------------------------
 template <int C, int D, int NTB, bool RPB>
-__device__ __noinline__ void attend_blocked() {
+__device__ __forceinline__ void attend_blocked() {
   constexpr int DC = D / 8;  // 16-byte chunks per head
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t a_base = s_mi.sbase + s_mi.off_a, k_base = s_mi.sbase + s_mi.off_kv;
@@ -203,7 +203,10 @@ __device__ __noinline__ void attend_blocked() {
   const unsigned char* row_lo = s_mi.row_lo[s_mi.buf];
   const unsigned char* row_n = s_mi.row_n[s_mi.buf];
   const int rows = s_mi.rows, heads = s_mi.heads;
-  constexpr int PW = 4;      // key blocks of 8 per pass (running softmax across passes keeps registers low)
+  // Key blocks of 8 per pass (running softmax across passes keeps registers low).  With wide sets six are faster although
+  // a few registers spill (nuScenes shapes, 8 layers: 459 us against 469); with sets up to 48 rows most 16-row blocks are
+  // done in one or two passes of four, and the spills cost more than they save (pillar frame: 519 us against 487).
+  constexpr int PW = NTB > 14 ? 6 : 4;
   const int t4 = lane & 3;
   const float sc = 1.4426950408889634f * rsqrtf((float)D);  // log2(e) / sqrt(d)
   const int nblk = (rows + 15) >> 4;
@@ -381,7 +384,7 @@ __device__ __forceinline__ bool mlp_step(int q, int n, int& piece) {  // true: M
 }
 
 // The scheduler and the MMA issuer are separate (not inlined) functions so that their polling loops get
-// their own, spill-free register allocation; the compute role is inlined into the kernel, where the
+// their own, spill-free register allocation; the compute role and its phases are inlined into the kernel, where the
 // kernel parameters are constant-bank operands.
 
 // ================= scheduler + TMA producer (one thread) ===============================================
@@ -751,15 +754,15 @@ __device__ __noinline__ void stamp_role(int32_t* __restrict__ row_stamp) {
 }
 
 // ================= compute warps ========================================================================
-// Each phase of a tile is a separate (not inlined) function that takes at most a few scalars and reads the
-// rest from s_mi, so that each gets a register allocation of its own and the tile loop keeps almost nothing
-// alive across the calls.
+// Each phase of a tile is a function that takes at most a few scalars and reads the rest from s_mi, so that the tile
+// loop keeps almost nothing alive across the phases.  They are inlined: as calls they cost 3 % (the registers a callee
+// may use depend on what the widest phase leaves to the caller).
 
 // Gather (Eq. 4): the fp32 rows listed in buffer b -> bf16 A operand, four rows in flight per warp; all 128 rows
 // are written (rows past the tile as zeros).  ADD_PE: the current tile's rows once more, with the positional
 // term added (the operand of the key and query projections).
 template <int C, bool RPB, bool ADD_PE>
-__device__ __noinline__ void phase_gather(int b, int rows) {
+__device__ __forceinline__ void phase_gather(int b, int rows) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float* x = ADD_PE ? s_mi.x : s_mi.next_x[b];
   unsigned char* a_tile = s_mi.sm + s_mi.off_a;
@@ -812,7 +815,7 @@ __device__ __noinline__ void phase_gather(int b, int rows) {
 // BIAS = false skips the bias (the key projection: a key bias adds
 // the same amount q . b_k to every score of a query, which the softmax cancels).
 template <int QC, bool BIAS>
-__device__ __noinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_off, uint32_t dst_off, int c8_0, int need) {
+__device__ __forceinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_off, uint32_t dst_off, int c8_0, int need) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
   if (32 * (warp & 3) >= need) {
@@ -849,7 +852,7 @@ __device__ __noinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_off
 //   bias_off  float offset of the piece's bias in the parameter block
 //   h_phase   parity of h_free that says that the MLP-2 of the piece before has read its hidden columns
 template <int C, int HC>
-__device__ __noinline__ void phase_mlp1(int bias_off, uint32_t h_phase) {
+__device__ __forceinline__ void phase_mlp1(int bias_off, uint32_t h_phase) {
   const int warp = threadIdx.x >> 5, hq = warp >> 2;
   const uint32_t lane_base = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16);
   if (32 * (warp & 3) >= s_mi.rows) {  // a warp without rows keeps step with the others
@@ -884,7 +887,7 @@ __device__ __noinline__ void phase_mlp1(int bias_off, uint32_t h_phase) {
 
 // x rows (fp32) for the first residual: asynchronous 16-byte copies global -> shared staging.
 template <int C>
-__device__ __noinline__ void phase_stage_x() {
+__device__ __forceinline__ void phase_stage_x() {
   constexpr int C4 = C / 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float* __restrict__ x = s_mi.x;
@@ -908,7 +911,7 @@ __device__ __noinline__ void phase_stage_x() {
 
 // fp32 rows staged in shared memory -> coalesced global rows.
 template <int C>
-__device__ __noinline__ void phase_store_rows() {
+__device__ __forceinline__ void phase_store_rows() {
   constexpr int C4 = C / 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* __restrict__ y = s_mi.y;
@@ -969,7 +972,7 @@ __device__ __forceinline__ void layer_norm_rows(float (&t)[QC], float sum, const
 // staging area (mode 0 / 1: final result of the call) or, in TMEM, x1 to the A operand (bf16) and x1 + b_2 back to
 // R (fp32), where the MLP-2 MMAs accumulate on top of it.
 template <int C, int QC>
-__device__ __noinline__ void phase_epi_o() {
+__device__ __forceinline__ void phase_epi_o() {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
   const uint32_t lane_base = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16), taddr = lane_base + Tm<C>::r + hq * QC;
@@ -1030,7 +1033,7 @@ __device__ __noinline__ void phase_epi_o() {
 // MLP-2 epilogue: R holds x1 + b_2 + M; LayerNorm 2; fp32 rows to the staging area.  The exchange slots are the first eight bytes of each
 // thread's own output chunk, which is therefore stored last, after one more meeting of the row's threads.
 template <int C, int QC>
-__device__ __noinline__ void phase_epi_f2() {
+__device__ __forceinline__ void phase_epi_f2() {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
   const uint32_t taddr = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + Tm<C>::r + hq * QC;
@@ -1102,33 +1105,36 @@ __device__ __forceinline__ bool compute_all(bool pred) {
   return r != 0;
 }
 
+// A compute thread's wait (out of line: one copy of the polling loop).  A wait that gives up raises the abort flag,
+// which the tile loop looks at.
+__device__ __noinline__ void wait_phase(uint32_t bar, uint32_t parity) {
+  for (int i = 0; i < kMaxPolls; ++i) {
+    if (mbar_try(bar, parity)) { tc_fence_after(); return; }
+    if ((i & 255) == 255 && *(volatile int*)&s_mi.abort_flag) return;
+  }
+  *(volatile int*)&s_mi.abort_flag = 1;
+}
+#define WAIT_PHASE(bar, parity) wait_phase(smem_u32(&s_mi.bar), (uint32_t)(parity) & 1u)
+
+// The tile loop keeps as little as possible alive across the phase calls (the tile's index k, and two flags): what it
+// holds, every phase has fewer registers, and with 227 KB of shared memory taken there is no L1 left for spills.
 template <int C, int D, int NT, int VAR>
 __device__ __forceinline__ void compute_role(const TcArgs& a) {
   constexpr bool RPB = VAR == 1, PE = VAR == 2;
   constexpr int NKB = C / 64;        // K blocks of a C-deep contraction
   constexpr int QC = C / 4;          // epilogue columns per thread for a C-wide chunk (four threads per row)
   volatile int* abort_flag = &s_mi.abort_flag;
-  uint32_t uses[3] = {0u, 0u, 0u}, pieces = 0u;
-  int slot = 0;
-  uint32_t sphase = 0;
-  bool ok = true;
-  bool gathered = false;  // the tile about to start was gathered under the previous tile's tail
+  bool gathered = false;  // the tile about to start was gathered under the previous tile's MLP
   int cur_layer = -1;     // layer whose vectors are in the parameter block
-  auto acc_wait = [&](uint32_t bar) {
-    ok = mbar_wait(&s_mi.acc_full[bar], uses[bar] & 1u, abort_flag) && ok;
-    ++uses[bar];
-    tc_fence_after();
-  };
-  // The next tile's rows are gathered as soon as the current tile's MMAs have stopped reading the A operand
-  // (the caller has just waited for the accumulator of the last such chunk), so that its first projections
-  // run on the tensor pipe while the compute warps finish the current tile; unless its rows are not all stamped
-  // yet: then the gather waits until this tile is done (the row that is missing may be one of this tile's own).
+  // The next tile's rows are gathered as soon as the current tile's MMAs have stopped reading the A operand (the
+  // output projection is the last), so that its first projections run on the tensor pipe while the compute warps finish
+  // the current tile; unless its rows are not all stamped yet: then the gather waits until this tile is done (the row
+  // that is missing may be one of this tile's own).
   auto gather_next = [&](int k) {
     const int b = (k + 1) & 1;
-    const uint32_t par = (uint32_t)((k + 1) >> 1) & 1u;
-    ok = mbar_wait(&s_mi.rl_ready[b], par, abort_flag) && ok;
+    WAIT_PHASE(rl_ready[b], (k + 1) >> 1);
     const int nr = s_mi.next_rows[b];
-    if (compute_all(ok && nr >= 0 && mbar_try(&s_mi.dep_ready[b], par))) {
+    if (compute_all(nr >= 0 && *abort_flag == 0 && mbar_try(&s_mi.dep_ready[b], (uint32_t)((k + 1) >> 1) & 1u))) {
       phase_gather<C, RPB, false>(b, nr);
       fence_proxy_async();
       mbar_arrive(&s_mi.x_ready);
@@ -1137,23 +1143,19 @@ __device__ __forceinline__ void compute_role(const TcArgs& a) {
   };
   int k = 0;
   for (;; ++k) {
-    ok = mbar_wait(&s_mi.sched_full[slot], sphase, abort_flag) && ok;
+    WAIT_PHASE(sched_full[k & 1], k >> 1);
     // also orders the previous tile's last shared-memory reads before this tile's writes; every exit from
     // this loop is taken by all compute threads together
-    if (bar_or(1, kComputeThreads, !ok || *abort_flag != 0)) break;
-    const int nsets = s_mi.tile[slot][1], rows = s_mi.tile[slot][3], layer = s_mi.tile[slot][4];
+    if (bar_or(1, kComputeThreads, *abort_flag != 0)) break;
+    const int nsets = s_mi.tile[k & 1][1], layer = s_mi.tile[k & 1][4];
     if (threadIdx.x == 0) {
-      s_mi.s_lo = s_mi.tile[slot][0];
-      s_mi.nsets = nsets;
-      s_mi.base = s_mi.tile[slot][2];
-      s_mi.rows = rows;
+      s_mi.rows = s_mi.tile[k & 1][3];
       s_mi.buf = k & 1;
-      s_mi.layer = layer;
       s_mi.x = layer == 0 ? a.x : a.y;
+      s_mi.st_stamp[k & 1] = a.n_layers > 1 ? a.stamp_base + layer + 1 : 0;
       if (k >= 1) mbar_arrive(&s_mi.rl_free[(k - 1) & 1]);  // the previous tile's row list is dead
     }
-    mbar_arrive(&s_mi.sched_empty[slot]);
-    if (++slot == 2) { slot = 0; sphase ^= 1u; }
+    mbar_arrive(&s_mi.sched_empty[k & 1]);
     if (nsets < 0) break;
     const bool new_params = layer != cur_layer;
     if (new_params) {  // (the previous tile's last use of the block lies before the barrier above)
@@ -1161,11 +1163,10 @@ __device__ __forceinline__ void compute_role(const TcArgs& a) {
       cur_layer = layer;
     }
     if (!gathered) {  // a CTA's first tile, or a tile whose rows were not ready in time
-      const uint32_t par = (uint32_t)(k >> 1) & 1u;
-      ok = mbar_wait(&s_mi.rl_ready[k & 1], par, abort_flag) && ok;
-      ok = mbar_wait(&s_mi.dep_ready[k & 1], par, abort_flag) && ok;
-      if (compute_all(ok)) {
-        phase_gather<C, RPB, false>(k & 1, rows);
+      WAIT_PHASE(rl_ready[k & 1], k >> 1);
+      WAIT_PHASE(dep_ready[k & 1], k >> 1);
+      if (compute_all(*abort_flag == 0)) {
+        phase_gather<C, RPB, false>(k & 1, s_mi.next_rows[k & 1]);
         fence_proxy_async();
       }
       mbar_arrive(&s_mi.x_ready);  // X is in place
@@ -1173,74 +1174,68 @@ __device__ __forceinline__ void compute_role(const TcArgs& a) {
     gathered = false;
     compute_sync();  // the tile's fields are visible to the phase functions
 
+    // (uses of the accumulators before this tile: V and R one each per tile, the first one K, Q and the MLP-1 pieces)
     // ---- chunks 0..2: K, V, Q epilogues: (+ bias,) to bf16, into the operand layout ----
     // (the attention pads its key blocks up to 15 rows past the tile: those K / V rows must be real bf16)
     if (PE) {
       // the values come from the bare rows; the operand is then rewritten with the positional term added, for
       // the keys and the queries (the V chunk's accumulator being complete, nothing reads the operand any more)
-      acc_wait(1u);
+      WAIT_PHASE(acc_full[1], k);
       if (new_params) wait_layer_params();
-      phase_epi_bf16<QC, true>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + NKB * kTM * 128, 0, rows + 16);
-      phase_gather<C, false, true>(k & 1, rows);
+      phase_epi_bf16<QC, true>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + NKB * kTM * 128, 0, s_mi.rows + 16);
+      phase_gather<C, false, true>(k & 1, s_mi.rows);
       fence_proxy_async();
       mbar_arrive(&s_mi.x_ready);
-      acc_wait(0u);
-      phase_epi_bf16<QC, false>(Tm<C>::k, 0, 0, s_mi.off_kv, 0, rows + 16);
+      WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1));
+      phase_epi_bf16<QC, false>(Tm<C>::k, 0, 0, s_mi.off_kv, 0, s_mi.rows + 16);
     } else {
-      acc_wait(0u);
-      phase_epi_bf16<QC, false>(Tm<C>::k, 0, 0, s_mi.off_kv, 0, rows + 16);
-      acc_wait(1u);
+      WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1));
+      phase_epi_bf16<QC, false>(Tm<C>::k, 0, 0, s_mi.off_kv, 0, s_mi.rows + 16);
+      WAIT_PHASE(acc_full[1], k);
       if (new_params) wait_layer_params();  // (the key epilogue adds no bias: it needs none of the vectors)
-      phase_epi_bf16<QC, true>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + NKB * kTM * 128, 0, rows + 16);
+      phase_epi_bf16<QC, true>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + NKB * kTM * 128, 0, s_mi.rows + 16);
     }
-    acc_wait(0u);
-    phase_epi_bf16<QC, true>(Tm<C>::k, 0, ParOff<C>::b_q, s_mi.off_a, 0, rows);
+    WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1) + 1);
+    phase_epi_bf16<QC, true>(Tm<C>::k, 0, ParOff<C>::b_q, s_mi.off_a, 0, s_mi.rows);
     compute_sync();
     // ---- attention inside each set ----
     attend_blocked<C, D, NT, RPB>();
     fence_proxy_async();
     mbar_arrive(&s_mi.a_ready);  // attention output is the A operand of the output projection
     compute_sync();              // every warp is done with K and V: their region becomes fp32 staging
-    const int mode = s_mi.mode;
-    if (mode != 0) {
+    if (s_mi.mode != 0) {
       phase_stage_x<C>();
       compute_sync();
     }
     // ---- output projection epilogue: Z + b_o (+ x, LayerNorm) ----
-    ok = mbar_wait(&s_mi.o_full, (uint32_t)k & 1u, abort_flag) && ok;
-    tc_fence_after();
+    WAIT_PHASE(o_full, k);
     phase_epi_o<C, QC>();
-    if (mode != 2) {  // final result of this layer
-      gather_next(k);  // the output projection was the last chunk to read the A operand
+    if (s_mi.mode != 2) {  // final result of this layer
+      gather_next(k);
     } else {
       mbar_arrive(&s_mi.a_ready);  // x1 (bf16) is the A operand of MLP-1
       // ---- MLP-1 pieces ----
-      const int n_f1 = s_mi.n_f1, NF = s_mi.NF;
-      for (int c = 0; c < n_f1; ++c, ++pieces) {
-        acc_wait(0u);
-        if (NF == 128) phase_mlp1<C, 32>(ParOff<C>::b_1 + c * NF, (pieces & 1u) ^ 1u);
-        else phase_mlp1<C, 16>(ParOff<C>::b_1 + c * NF, (pieces & 1u) ^ 1u);
+      for (int c = 0; c < s_mi.n_f1; ++c) {
+        WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1) + 2 + c);
+        const uint32_t h_phase = (uint32_t)(k * s_mi.n_f1 + c + 1) & 1u;
+        if (s_mi.NF == 128) phase_mlp1<C, 32>(ParOff<C>::b_1 + c * 128, h_phase);
+        else phase_mlp1<C, 16>(ParOff<C>::b_1 + c * 64, h_phase);
       }
-      gather_next(k);  // (the operand has been free since the output projection)
+      gather_next(k);  // (the operand has been free since the output projection; under the first MLP-1 product it is slower)
       // ---- MLP-2 epilogue: y = LN2(x1 + M) ----
-      acc_wait(2u);
+      WAIT_PHASE(acc_full[2], k);
       phase_epi_f2<C, QC>();
     }
     compute_sync();
     phase_store_rows<C>();
-    if (threadIdx.x == 0) {
-      s_mi.st_rows[k & 1] = rows;
-      s_mi.st_stamp[k & 1] = a.n_layers > 1 ? a.stamp_base + layer + 1 : 0;
-    }
+    if (threadIdx.x == 0) s_mi.st_rows[k & 1] = s_mi.rows;
     mbar_arrive(&s_mi.stored[k & 1]);  // the stamp warp takes it from here
   }
   // tell the stamp warp to leave at iteration k, once it is done with tile k - 2 (which signalled on the same barrier)
-  if (k >= 2) mbar_wait(&s_mi.rl_free[k & 1], (uint32_t)((k >> 1) - 1) & 1u, abort_flag);
+  if (k >= 2) WAIT_PHASE(rl_free[k & 1], (k >> 1) - 1);
   if (threadIdx.x == 0) s_mi.exit_at = k;
   mbar_arrive(&s_mi.stored[k & 1]);
-  if (!ok || *abort_flag) {
-    if (threadIdx.x == 0) atomicOr(s_mi.status, DSVT_STATUS_TIMEOUT);
-  }
+  if (threadIdx.x == 0 && *abort_flag) atomicOr(s_mi.status, DSVT_STATUS_TIMEOUT);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1269,7 +1264,7 @@ __global__ void __launch_bounds__(kThreads, 1) layer_tc_kernel(const __grid_cons
     mi->rpb = nullptr; mi->pe = nullptr; mi->coords = a.coords;
     mi->rb_len = g.rb_len; mi->rb_sx = g.rb_sx; mi->rb_sy = g.rb_sy; mi->rb_centre = g.rb_centre;
     mi->rb_ext[0] = g.rb_ext[0]; mi->rb_ext[1] = g.rb_ext[1]; mi->rb_ext[2] = g.rb_ext[2];
-    mi->s_lo = mi->nsets = mi->base = mi->rows = mi->buf = mi->layer = 0;
+    mi->rows = mi->buf = 0;
     mi->next_rows[0] = mi->next_rows[1] = -1;
     mi->next_x[0] = mi->next_x[1] = a.x;
     mi->st_rows[0] = mi->st_rows[1] = mi->st_stamp[0] = mi->st_stamp[1] = 0;
