@@ -157,6 +157,28 @@ struct Misc {  // small shared state beside the big regions
 };
 __shared__ Misc s_mi;
 
+// Accesses to the big regions by shared-space address (through a generic pointer they would be generic accesses).
+// Volatile, so that they stay in program order and none is hoisted into registers ahead of its use.
+__device__ __forceinline__ float4 lds4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ float2 lds2(uint32_t a) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts4(uint32_t a, float4 v) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w));
+}
+__device__ __forceinline__ void sts4(uint32_t a, uint4 v) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
+}
+__device__ __forceinline__ void sts2(uint32_t a, float2 v) {
+  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y));
+}
+
 __device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kComputeThreads) : "memory"); }
 
 // gelu(t) = t Phi(t) with Phi(t) = 1 - h for t >= 0 and h for t < 0, h = erfc(|t| / sqrt 2) / 2; hence
@@ -343,14 +365,11 @@ __device__ __forceinline__ void attend_blocked() {
   }
 }
 
-// fp32 row staging in the K/V region: row r, 16-byte chunk c4 of C/4, rotated by the row so that both
+// fp32 row staging in the K/V region: row r, 16-byte chunk c4 of C/4, XORed with the row so that both
 // the warp-per-row pattern (global side) and the thread-per-row pattern (TMEM side) are conflict-free.
 template <int C>
 __device__ __forceinline__ uint32_t stage_off(int r, int c4) {
-  constexpr int NCH = C / 4;
-  int idx = c4 + (r % NCH);
-  if (idx >= NCH) idx -= NCH;
-  return (uint32_t)(r * (C * 4) + (idx << 4));
+  return (uint32_t)(r * (C * 4) + ((c4 ^ (r & 7)) << 4));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -765,7 +784,7 @@ template <int C, bool RPB, bool ADD_PE>
 __device__ __forceinline__ void phase_gather(int b, int rows) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float* x = ADD_PE ? s_mi.x : s_mi.next_x[b];
-  unsigned char* a_tile = s_mi.sm + s_mi.off_a;
+  const uint32_t a_tile = s_mi.sbase + s_mi.off_a;
   const int* rowvox = s_mi.rowvox[b];
   for (int r0 = warp; r0 < kTM; r0 += 4 * kComputeWarps) {
     float4 f[4][2];
@@ -797,9 +816,9 @@ __device__ __forceinline__ void phase_gather(int b, int rows) {
     if (lane < (C >> 3)) {
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        *reinterpret_cast<uint4*>(a_tile + swz(r0 + kComputeWarps * u, lane)) =
-            make_uint4(pack_bf16(f[u][0].x, f[u][0].y), pack_bf16(f[u][0].z, f[u][0].w),
-                       pack_bf16(f[u][1].x, f[u][1].y), pack_bf16(f[u][1].z, f[u][1].w));
+        sts4(a_tile + swz(r0 + kComputeWarps * u, lane),
+             make_uint4(pack_bf16(f[u][0].x, f[u][0].y), pack_bf16(f[u][0].z, f[u][0].w),
+                        pack_bf16(f[u][1].x, f[u][1].y), pack_bf16(f[u][1].z, f[u][1].w)));
     }
   }
 }
@@ -824,8 +843,8 @@ __device__ __forceinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_
     return;
   }
   const uint32_t taddr = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + tcol + hq * QC;
-  const float* bias = reinterpret_cast<const float*>(s_mi.sm + s_mi.off_par) + bias_off + hq * QC;
-  unsigned char* dst = s_mi.sm + dst_off;
+  const uint32_t bias = s_mi.sbase + s_mi.off_par + 4u * (uint32_t)(bias_off + hq * QC);
+  const uint32_t dst = s_mi.sbase + dst_off;
   const int c8 = c8_0 + ((hq * QC) >> 3);
   float rr[QC];
   tmem_ld_row(taddr, rr);
@@ -837,14 +856,14 @@ __device__ __forceinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_
     float2 v[4] = {make_float2(rr[8 * q], rr[8 * q + 1]), make_float2(rr[8 * q + 2], rr[8 * q + 3]),
                    make_float2(rr[8 * q + 4], rr[8 * q + 5]), make_float2(rr[8 * q + 6], rr[8 * q + 7])};
     if (BIAS) {
-      const float4 b0 = *reinterpret_cast<const float4*>(bias + 8 * q), b1 = *reinterpret_cast<const float4*>(bias + 8 * q + 4);
+      const float4 b0 = lds4(bias + 32 * q), b1 = lds4(bias + 32 * q + 16);
       v[0] = __fadd2_rn(v[0], make_float2(b0.x, b0.y));
       v[1] = __fadd2_rn(v[1], make_float2(b0.z, b0.w));
       v[2] = __fadd2_rn(v[2], make_float2(b1.x, b1.y));
       v[3] = __fadd2_rn(v[3], make_float2(b1.z, b1.w));
     }
-    *reinterpret_cast<uint4*>(dst + swz(row, c8 + q)) =
-        make_uint4(pack_bf16(v[0].x, v[0].y), pack_bf16(v[1].x, v[1].y), pack_bf16(v[2].x, v[2].y), pack_bf16(v[3].x, v[3].y));
+    sts4(dst + swz(row, c8 + q),
+         make_uint4(pack_bf16(v[0].x, v[0].y), pack_bf16(v[1].x, v[1].y), pack_bf16(v[2].x, v[2].y), pack_bf16(v[3].x, v[3].y)));
   }
 }
 
@@ -862,7 +881,7 @@ __device__ __forceinline__ void phase_mlp1(int bias_off, uint32_t h_phase) {
     mbar_arrive(&s_mi.h_ready);
     return;
   }
-  const float* bias = reinterpret_cast<const float*>(s_mi.sm + s_mi.off_par) + bias_off + hq * HC;
+  const uint32_t bias = s_mi.sbase + s_mi.off_par + 4u * (uint32_t)(bias_off + hq * HC);
   float rr[HC];
   tmem_ld_row(lane_base + Tm<C>::acc + hq * HC, rr);
   tmem_wait_ld();
@@ -871,7 +890,7 @@ __device__ __forceinline__ void phase_mlp1(int bias_off, uint32_t h_phase) {
   uint32_t p[HC / 2];
 #pragma unroll
   for (int q = 0; q < HC / 4; ++q) {
-    const float4 b4 = *reinterpret_cast<const float4*>(bias + 4 * q);
+    const float4 b4 = lds4(bias + 16 * q);
     const float2 g0 = gelu_fast2(__fadd2_rn(make_float2(rr[4 * q], rr[4 * q + 1]), make_float2(b4.x, b4.y)));
     const float2 g1 = gelu_fast2(__fadd2_rn(make_float2(rr[4 * q + 2], rr[4 * q + 3]), make_float2(b4.z, b4.w)));
     p[2 * q] = pack_bf16(g0.x, g0.y);
@@ -891,8 +910,7 @@ __device__ __forceinline__ void phase_stage_x() {
   constexpr int C4 = C / 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float* __restrict__ x = s_mi.x;
-  unsigned char* stage = s_mi.sm + s_mi.off_kv;
-  const uint32_t stage_saddr = s_mi.sbase + s_mi.off_kv;
+  const uint32_t stage = s_mi.sbase + s_mi.off_kv;
   const int rows = s_mi.rows;
   const int* rowvox = s_mi.rowvox[s_mi.buf];
   for (int r = warp; r < rows; r += kComputeWarps) {
@@ -900,10 +918,10 @@ __device__ __forceinline__ void phase_stage_x() {
     for (int c4 = lane; c4 < C4; c4 += 32) {
       const uint32_t off = stage_off<C>(r, c4);
       if (v >= 0)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage_saddr + off),
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage + off),
                      "l"(reinterpret_cast<const float4*>(x + (size_t)v * C) + c4) : "memory");
       else
-        *reinterpret_cast<float4*>(stage + off) = make_float4(0.f, 0.f, 0.f, 0.f);
+        sts4(stage + off, make_float4(0.f, 0.f, 0.f, 0.f));
     }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
@@ -915,14 +933,14 @@ __device__ __forceinline__ void phase_store_rows() {
   constexpr int C4 = C / 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* __restrict__ y = s_mi.y;
-  const unsigned char* stage = s_mi.sm + s_mi.off_kv;
+  const uint32_t stage = s_mi.sbase + s_mi.off_kv;
   const int rows = s_mi.rows;
   const int* rowvox = s_mi.rowvox[s_mi.buf];
   for (int r = warp; r < rows; r += kComputeWarps) {
     const int v = rowvox[r];
     if (v < 0) continue;
     for (int c4 = lane; c4 < C4; c4 += 32)
-      reinterpret_cast<float4*>(y + (size_t)v * C)[c4] = *reinterpret_cast<const float4*>(stage + stage_off<C>(r, c4));
+      reinterpret_cast<float4*>(y + (size_t)v * C)[c4] = lds4(stage + stage_off<C>(r, c4));
   }
 }
 
@@ -944,23 +962,22 @@ __device__ __forceinline__ void quarter_sync() {
   asm volatile("bar.sync %0, 128;" ::"r"(2 + ((threadIdx.x >> 5) & 3)) : "memory");
 }
 template <int C, int QC, class Slot>
-__device__ __forceinline__ void layer_norm_rows(float (&t)[QC], float sum, const float* gain, const float* shift, float eps,
+__device__ __forceinline__ void layer_norm_rows(float (&t)[QC], float sum, uint32_t gain, uint32_t shift, float eps,
                                                 int hq, Slot slot) {
   const float mq = sum * (1.0f / (float)QC);
   float m2 = 0.f;
 #pragma unroll
   for (int i = 0; i < QC; ++i) { const float d = t[i] - mq; m2 = fmaf(d, d, m2); }
-  *slot(hq) = make_float2(mq, m2);
+  sts2(slot(hq), make_float2(mq, m2));
   quarter_sync();
-  const float2 s0 = *slot(0), s1 = *slot(1), s2 = *slot(2), s3 = *slot(3);
+  const float2 s0 = lds2(slot(0)), s1 = lds2(slot(1)), s2 = lds2(slot(2)), s3 = lds2(slot(3));
   const float mean = 0.25f * ((s0.x + s1.x) + (s2.x + s3.x));
   const float d0 = s0.x - mean, d1 = s1.x - mean, d2 = s2.x - mean, d3 = s3.x - mean;
   const float ssq = ((s0.y + s1.y) + (s2.y + s3.y)) + (float)QC * ((d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3));
   const float inv = rsqrtf(ssq * (1.0f / (float)C) + eps);
 #pragma unroll
   for (int i4 = 0; i4 < QC / 4; ++i4) {
-    const float4 g4 = *reinterpret_cast<const float4*>(gain + hq * QC + 4 * i4);
-    const float4 b4 = *reinterpret_cast<const float4*>(shift + hq * QC + 4 * i4);
+    const float4 g4 = lds4(gain + 4u * (uint32_t)(hq * QC + 4 * i4)), b4 = lds4(shift + 4u * (uint32_t)(hq * QC + 4 * i4));
     t[4 * i4] = (t[4 * i4] - mean) * inv * g4.x + b4.x;
     t[4 * i4 + 1] = (t[4 * i4 + 1] - mean) * inv * g4.y + b4.y;
     t[4 * i4 + 2] = (t[4 * i4 + 2] - mean) * inv * g4.z + b4.z;
@@ -976,8 +993,7 @@ __device__ __forceinline__ void phase_epi_o() {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
   const uint32_t lane_base = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16), taddr = lane_base + Tm<C>::r + hq * QC;
-  const float* par = reinterpret_cast<const float*>(s_mi.sm + s_mi.off_par);
-  unsigned char* stage = s_mi.sm + s_mi.off_kv;
+  const uint32_t par = s_mi.sbase + s_mi.off_par, stage = s_mi.sbase + s_mi.off_kv;
   const int mode = s_mi.mode;
   const bool add_x = mode != 0 && row < s_mi.rows;
   float t[QC];
@@ -989,8 +1005,8 @@ __device__ __forceinline__ void phase_epi_o() {
 #pragma unroll
   for (int q = 0; q < QC / 4; ++q) {
     float4 x4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (add_x) x4 = *reinterpret_cast<const float4*>(stage + stage_off<C>(row, hq * (QC / 4) + q));
-    const float4 b4 = *reinterpret_cast<const float4*>(par + ParOff<C>::b_o + hq * QC + 4 * q);
+    if (add_x) x4 = lds4(stage + stage_off<C>(row, hq * (QC / 4) + q));
+    const float4 b4 = lds4(par + 4u * (uint32_t)(ParOff<C>::b_o + hq * QC + 4 * q));
     t[4 * q] += x4.x + b4.x;
     t[4 * q + 1] += x4.y + b4.y;
     t[4 * q + 2] += x4.z + b4.z;
@@ -999,15 +1015,14 @@ __device__ __forceinline__ void phase_epi_o() {
   }
   if (mode != 0 && s_mi.ln1) {
     // exchange slots: the first eight bytes of each thread's own (already consumed) x staging chunk
-    auto slot = [&](int quarter) { return reinterpret_cast<float2*>(stage + stage_off<C>(row, quarter * (QC / 4))); };
-    layer_norm_rows<C, QC>(t, sum, par + ParOff<C>::ln1_g, par + ParOff<C>::ln1_b, s_mi.eps, hq, slot);
+    auto slot = [&](int quarter) { return stage + stage_off<C>(row, quarter * (QC / 4)); };
+    layer_norm_rows<C, QC>(t, sum, par + 4 * ParOff<C>::ln1_g, par + 4 * ParOff<C>::ln1_b, s_mi.eps, hq, slot);
   }
   if (mode != 2) {
     compute_sync();  // the x staging (and the exchange slots in it) is dead once every thread has its t
 #pragma unroll
     for (int i4 = 0; i4 < QC / 4; ++i4)
-      *reinterpret_cast<float4*>(stage + stage_off<C>(row, hq * (QC / 4) + i4)) =
-          make_float4(t[4 * i4], t[4 * i4 + 1], t[4 * i4 + 2], t[4 * i4 + 3]);
+      sts4(stage + stage_off<C>(row, hq * (QC / 4) + i4), make_float4(t[4 * i4], t[4 * i4 + 1], t[4 * i4 + 2], t[4 * i4 + 3]));
     return;
   }
 #pragma unroll
@@ -1019,7 +1034,7 @@ __device__ __forceinline__ void phase_epi_o() {
   }
 #pragma unroll
   for (int q = 0; q < QC / 4; ++q) {
-    const float4 b4 = *reinterpret_cast<const float4*>(par + ParOff<C>::b_2 + hq * QC + 4 * q);
+    const float4 b4 = lds4(par + 4u * (uint32_t)(ParOff<C>::b_2 + hq * QC + 4 * q));
     t[4 * q] += b4.x;
     t[4 * q + 1] += b4.y;
     t[4 * q + 2] += b4.z;
@@ -1037,8 +1052,7 @@ __device__ __forceinline__ void phase_epi_f2() {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
   const uint32_t taddr = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + Tm<C>::r + hq * QC;
-  const float* par = reinterpret_cast<const float*>(s_mi.sm + s_mi.off_par);
-  unsigned char* stage = s_mi.sm + s_mi.off_kv;
+  const uint32_t par = s_mi.sbase + s_mi.off_par, stage = s_mi.sbase + s_mi.off_kv;
   float t[QC];
   tmem_ld_row(taddr, t);
   tmem_wait_ld();
@@ -1049,15 +1063,14 @@ __device__ __forceinline__ void phase_epi_f2() {
     float sum = 0.f;
 #pragma unroll
     for (int q = 0; q < QC / 4; ++q) sum += (t[4 * q] + t[4 * q + 1]) + (t[4 * q + 2] + t[4 * q + 3]);
-    auto slot = [&](int quarter) { return reinterpret_cast<float2*>(stage + stage_off<C>(row, quarter * (QC / 4))); };
-    layer_norm_rows<C, QC>(t, sum, par + ParOff<C>::ln2_g, par + ParOff<C>::ln2_b, s_mi.eps, hq, slot);
+    auto slot = [&](int quarter) { return stage + stage_off<C>(row, quarter * (QC / 4)); };
+    layer_norm_rows<C, QC>(t, sum, par + 4 * ParOff<C>::ln2_g, par + 4 * ParOff<C>::ln2_b, s_mi.eps, hq, slot);
   }
 #pragma unroll
   for (int i4 = 1; i4 < QC / 4; ++i4)
-    *reinterpret_cast<float4*>(stage + stage_off<C>(row, hq * (QC / 4) + i4)) =
-        make_float4(t[4 * i4], t[4 * i4 + 1], t[4 * i4 + 2], t[4 * i4 + 3]);
+    sts4(stage + stage_off<C>(row, hq * (QC / 4) + i4), make_float4(t[4 * i4], t[4 * i4 + 1], t[4 * i4 + 2], t[4 * i4 + 3]));
   if (ln) quarter_sync();  // the row's other threads have read this thread's slot
-  *reinterpret_cast<float4*>(stage + stage_off<C>(row, hq * (QC / 4))) = make_float4(t[0], t[1], t[2], t[3]);
+  sts4(stage + stage_off<C>(row, hq * (QC / 4)), make_float4(t[0], t[1], t[2], t[3]));
 }
 
 // The layer's biases and LayerNorm vectors into the parameter block (absent vectors as zeros), and its scalars.
