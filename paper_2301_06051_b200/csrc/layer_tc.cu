@@ -175,6 +175,9 @@ __device__ __forceinline__ void sts4(uint32_t a, float4 v) {
 __device__ __forceinline__ void sts4(uint32_t a, uint4 v) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
 }
+__device__ __forceinline__ void sts2(uint32_t a, uint2 v) {
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y));
+}
 __device__ __forceinline__ void sts2(uint32_t a, float2 v) {
   asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y));
 }
@@ -777,48 +780,57 @@ __device__ __noinline__ void stamp_role(int32_t* __restrict__ row_stamp) {
 // loop keeps almost nothing alive across the phases.  They are inlined: as calls they cost 3 % (the registers a callee
 // may use depend on what the widest phase leaves to the caller).
 
-// Gather (Eq. 4): the fp32 rows listed in buffer b -> bf16 A operand, four rows in flight per warp; all 128 rows
-// are written (rows past the tile as zeros).  ADD_PE: the current tile's rows once more, with the positional
-// term added (the operand of the key and query projections).
+// Gather (Eq. 4): the fp32 rows listed in buffer b -> bf16 A operand; all 128 rows are written (rows past the tile as
+// zeros).  A unit of one or two rows is a whole number of coalesced 16-byte warp loads; all of a warp's eight rows are
+// in flight at once (C = 192: 12 loads per lane; with two rounds of four rows and a quarter of the lanes idle the gather
+// cost one L2 round trip more).  ADD_PE: the current tile's rows once more, with the positional term added (the operand
+// of the key and query projections).
 template <int C, bool RPB, bool ADD_PE>
 __device__ __forceinline__ void phase_gather(int b, int rows) {
+  constexpr int C4 = C / 4, RU = C4 % 32 == 0 ? 1 : 2, IU = RU * C4 / 32;  // chunks per row; rows, loads per unit
+  constexpr int kFly = ADD_PE ? (RU == 2 ? 2 : 4) : 8 / RU;                // units in flight
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float* x = ADD_PE ? s_mi.x : s_mi.next_x[b];
   const uint32_t a_tile = s_mi.sbase + s_mi.off_a;
   const int* rowvox = s_mi.rowvox[b];
-  for (int r0 = warp; r0 < kTM; r0 += 4 * kComputeWarps) {
-    float4 f[4][2];
+  for (int r0 = RU * warp; r0 < kTM; r0 += kFly * RU * kComputeWarps) {
+    float4 f[kFly][IU];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int r = r0 + kComputeWarps * u;
-      const int v = r < rows ? rowvox[r] : -1;
-      f[u][0] = f[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (v >= 0 && lane < (C >> 3)) {
-        const float4* src = reinterpret_cast<const float4*>(x + (size_t)v * C) + 2 * lane;
-        f[u][0] = __ldcg(src);  // (L2: the rows of a later layer were written during this launch, by any SM)
-        f[u][1] = __ldcg(src + 1);
-        if (ADD_PE) {
-          const float4* pp = reinterpret_cast<const float4*>(s_mi.pe + (size_t)v * C) + 2 * lane;
-          const float4 p0 = __ldg(pp), p1 = __ldg(pp + 1);
-          f[u][0].x += p0.x; f[u][0].y += p0.y; f[u][0].z += p0.z; f[u][0].w += p0.w;
-          f[u][1].x += p1.x; f[u][1].y += p1.y; f[u][1].z += p1.z; f[u][1].w += p1.w;
-        }
-      }
-      if (RPB && !ADD_PE && lane == 31) {  // (lane 31 carries no feature columns: C / 8 <= 24)
-        int lin = 0;
+    for (int u = 0; u < kFly; ++u) {
+#pragma unroll
+      for (int i = 0; i < IU; ++i) {
+        const int e = lane + 32 * i, r = r0 + u * RU * kComputeWarps + e / C4, c4 = e % C4;
+        const int v = r < rows ? rowvox[r] : -1;
+        f[u][i] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (v >= 0) {
-          const int4 c = __ldg(s_mi.coords + v);
-          lin = c.y * s_mi.rb_sx + c.z * s_mi.rb_sy + c.w;
+          // (L2: the rows of a later layer were written during this launch, by any SM)
+          f[u][i] = __ldcg(reinterpret_cast<const float4*>(x + (size_t)v * C) + c4);
+          if (ADD_PE) {
+            const float4 p = __ldg(reinterpret_cast<const float4*>(s_mi.pe + (size_t)v * C) + c4);
+            f[u][i].x += p.x; f[u][i].y += p.y; f[u][i].z += p.z; f[u][i].w += p.w;
+          }
         }
-        s_mi.rowlin[r] = (short)lin;
       }
     }
-    if (lane < (C >> 3)) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        sts4(a_tile + swz(r0 + kComputeWarps * u, lane),
-             make_uint4(pack_bf16(f[u][0].x, f[u][0].y), pack_bf16(f[u][0].z, f[u][0].w),
-                        pack_bf16(f[u][1].x, f[u][1].y), pack_bf16(f[u][1].z, f[u][1].w)));
+    for (int u = 0; u < kFly; ++u) {
+#pragma unroll
+      for (int i = 0; i < IU; ++i) {
+        const int e = lane + 32 * i, r = r0 + u * RU * kComputeWarps + e / C4, c4 = e % C4;
+        sts2(a_tile + swz(r, c4 >> 1) + 8 * (c4 & 1),
+             make_uint2(pack_bf16(f[u][i].x, f[u][i].y), pack_bf16(f[u][i].z, f[u][i].w)));
+      }
+    }
+  }
+  if (RPB && !ADD_PE) {
+    for (int r = threadIdx.x; r < kTM; r += kComputeThreads) {
+      const int v = r < rows ? rowvox[r] : -1;
+      int lin = 0;
+      if (v >= 0) {
+        const int4 c = __ldg(s_mi.coords + v);
+        lin = c.y * s_mi.rb_sx + c.z * s_mi.rb_sy + c.w;
+      }
+      s_mi.rowlin[r] = (short)lin;
     }
   }
 }
