@@ -28,11 +28,17 @@
 // are A operands in TMEM, the hidden one piece at a time: MLP-2 of a piece runs under the GELU of the next, and the
 // tensor pipe reads half the shared memory it would need for both operands.
 //
-// Every operand tile in shared memory uses the K-major 128-byte-swizzled layout that tcgen05.mma and
-// TMA share: 64 bf16 columns per 128-byte row, 8-row groups of 1024 bytes, 16-byte chunk index XORed
-// with (row & 7).  Q, K, V and the attention output live in that same layout, so the attention phase
-// (mma.sync m16n8k16 with ldmatrix) reads it without bank conflicts and writes its result straight
-// into the A operand of the output projection.
+// Attention runs on the tensor cores too: per head, S = Q K^T over the whole tile (128 x 128) in TMEM, softmax with a
+// row per thread, P back to TMEM as a bf16 A operand, O = P V.  Sets are kept apart inside the product: spare K
+// columns carry a code of the row's set (see write_codes), which adds exactly zero to a score inside a set and -2^100
+// to one across sets.  The products beyond a set cost the tensor pipe 3 k cycles per tile; in exchange the softmax has
+// no shuffles, no per-element mask and 16 independent elements per step.
+//
+// Operand layouts in shared memory: the gathered rows and the weights use the K-major 128-byte-swizzled layout
+// (64 bf16 columns per 128-byte row, 8-row groups of 1024 bytes, 16-byte chunk index XORed with (row & 7)).  Q, K, V
+// and the attention output are unswizzled and chunk-major, [8-column chunk][128 rows][16 bytes]: a row per thread
+// writes it without bank conflicts, heads of 24 columns start on a chunk, and V needs no transposition (it is read
+// N-major).
 //
 // Every wait (on an mbarrier, on a row stamp) is bounded; a wait that gives up raises DSVT_STATUS_TIMEOUT and
 // all roles leave their loops.
@@ -59,9 +65,12 @@ constexpr int kStampWarp = kLoadWarp0 + kLoadWarps;  // writes the completion st
 constexpr int kThreads = kComputeThreads + 64 + kLoadThreads + 32;
 constexpr int kStages = 3;             // weight ring depth
 constexpr int kStampPolls = 1 << 18;  // polls of a row's stamp, about a microsecond each
+constexpr int kMaxIdle = 1 << 24;     // rounds of looks at the attention's barriers that find nothing to do
+constexpr uint32_t kChunkBytes = kTM * 16;  // an 8-column chunk of an unswizzled operand
 constexpr int kMaxLayers = DSVT_MAX_CHAIN_LAYERS;  // layers one launch can chain
 
-// TMEM map (512 columns): K, then Q accumulate at 0, V at C; R = the last C columns: output projection, x1 + b_2 parked,
+// TMEM map (512 columns): K, then Q accumulate at 0, V at C; in the attention every group of four warps has 128 columns
+// for S, P and O; then R = the last C columns: output projection, x1 + b_2 parked,
 // MLP-2 on top of it; x1 as a bf16 A operand at 0; an MLP-1 accumulator piece (128 columns); an MLP hidden piece as a
 // bf16 A operand (64).  The next tile's K starts once x1 and the last MLP-1 piece are dead, its V (which overlaps the
 // hidden piece and, for C = 192, R) once R has been read.
@@ -76,7 +85,7 @@ struct TcGeom {
   int NF;       // MLP piece: hidden columns (128 or 64)
   int n_f1;     // hidden / NF
   int mode;     // 0: attention only, 1: attention + residual + LN1, 2: full layer
-  uint32_t off_a, off_kv, off_stage, off_par;  // byte offsets from the 1024-aligned base
+  uint32_t off_a, off_kv, off_code, off_stage;  // byte offsets in the dynamic shared memory
   // relative position bias (rb_len == 0: none): entries per head, strides of the x and y offsets in the table,
   // index of the zero offset, extent of the table
   int rb_len, rb_sx, rb_sy, rb_centre, rb_ext[3];
@@ -105,12 +114,26 @@ struct TcArgs {
   TcLayer layer[kMaxLayers];
 };
 
-struct Misc {  // small shared state beside the big regions
+// Vectors of the layer that stay in shared memory (float offsets; for b_o, b_1 and b_2 see LateOff).
+template <int C>
+struct ParOff {
+  static constexpr int b_q = 0, b_v = C, ln1_g = 2 * C, ln1_b = 3 * C, ln2_g = 4 * C, ln2_b = 5 * C;  // no key bias
+  static constexpr int vectors = 6;
+};
+// b_o, b_2 and b_1 lie where the set codes are during the attention, from the end of the attention to the last MLP-1
+// piece (float offsets; copied with the x rows).
+template <int C>
+struct LateOff { static constexpr int b_o = 0, b_2 = C, b_1 = 2 * C; };
+
+// Small shared state beside the big regions.  It fills whole kilobytes, so that the dynamic shared memory behind it
+// starts on a 1024-byte boundary (with C = 192 there is no byte to spare for padding).
+struct alignas(1024) Misc {
   // weight ring; accumulators K / Q / MLP-1, V, R (see Tm); operand hand-offs
   unsigned long long full[kStages], empty[kStages], acc_full[3], acc_free[3];
   unsigned long long o_full;           // output projection done
+  unsigned long long s_full[4], p_ready[4], ov_full[4], o_read[4];  // attention, one set per group of four warps
   unsigned long long h_ready, h_free;  // MLP hidden piece in TMEM: written / read by MLP-2
-  unsigned long long a_ready;   // compute warps -> MMA: attention output / x1 is in place
+  unsigned long long a_ready;   // compute warps -> MMA: Q / attention output / x1 is in place
   unsigned long long x_ready;   // compute warps -> MMA: the gathered rows of a tile are in the A operand
   unsigned long long rl_ready[2];   // loader warp -> compute: row-list buffer b describes its next tile
   unsigned long long dep_ready[2];  // loader warp -> compute: the rows listed in buffer b carry the previous layer's stamp
@@ -121,9 +144,9 @@ struct Misc {  // small shared state beside the big regions
   uint32_t tmem_base;
   int abort_flag;
   int exit_at;   // tile iteration at which the compute warps left their loop (-1: still running; read by the stamp warp)
-  int tile[2][6];  // ring of tiles: first set, number of sets (< 0: no more tiles), first row, rows, layer
-  // the scheduler's view of the chain: tiles before the end of each layer, sets per layer, plan or not
-  int tile_end[kMaxLayers], lay_S[kMaxLayers];
+  int tile[2][5];  // ring of tiles: first set, number of sets (< 0: no more tiles), first row, rows, layer
+  // the scheduler's view of the chain: tiles before the end of each layer, plan or not
+  int tile_end[kMaxLayers];
   unsigned char lay_plan[kMaxLayers];
   // launch constants, written once before the roles start: the phase functions read them from here
   // instead of taking them as arguments, so that nothing has to stay in registers across their calls
@@ -131,11 +154,11 @@ struct Misc {  // small shared state beside the big regions
   const float* pe;  // the layer's positional term (kernels with one)
   float* y;
   int32_t* status;
-  unsigned char* sm;   // 1024-aligned base of the dynamic shared memory (generic address)
-  uint32_t sbase;      // the same as a shared-space address
-  uint32_t off_a, off_kv, off_par;
+  uint32_t sbase;      // base of the dynamic shared memory as a shared-space address
+  uint32_t off_a, off_kv, off_code;
   int n, tau, heads, mode, NF, n_f1, ln1, ln2;
   float eps;
+  const float *b_o, *b_1, *b_2;  // see LateOff (16-byte aligned, or NULL)
   // the tile the compute warps are working on, and which row-list buffer describes it
   int rows, buf;
   int next_rows[2];        // rows of the tile listed in buffer b (< 0: there is no such tile), valid after rl_ready[b]
@@ -145,6 +168,7 @@ struct Misc {  // small shared state beside the big regions
   // the compute warps gather tile k + 1 as soon as tile k's MMAs no longer read the A operand
   int rowvox[2][kTM];              // tile row -> voxel (-1: none)
   unsigned char row_lo[2][kTM], row_n[2][kTM];  // per tile row: first row and row count of its set
+  uint32_t starts[2][4];           // bit r: row r is the first of its set
   // relative position bias.  The table index is linear in the coordinate offset, so one integer per row,
   // x * rb_sx + y * rb_sy + z, serves every (query, key) pair: index = lin[query] - lin[key] + rb_centre.  Offsets
   // inside a covered set are at most (table length - 1) / 2 < 2^15 in magnitude (tables of up to 65,535 entries
@@ -154,7 +178,9 @@ struct Misc {  // small shared state beside the big regions
   const int4* coords;
   int rb_len, rb_sx, rb_sy, rb_centre, rb_ext[3];
   short rowlin[kTM];
+  alignas(16) float par[6 * 192];
 };
+static_assert(sizeof(Misc) == 7 * 1024, "shared memory");
 __shared__ Misc s_mi;
 
 // Accesses to the big regions by shared-space address (through a generic pointer they would be generic accesses).
@@ -209,162 +235,165 @@ __device__ __forceinline__ float rpb_term(const float* __restrict__ tab, int lin
   return __ldg(tab + min((unsigned)idx, (unsigned)(s_mi.rb_len - 1))) * root;  // (a negative index clamps too)
 }
 
+// A compute thread's wait (out of line: one copy of the polling loop).  A wait that gives up raises the abort flag,
+// which the tile loop looks at.
+__device__ __noinline__ void wait_phase(uint32_t bar, uint32_t parity) {
+  for (int i = 0; i < kMaxPolls; ++i) {
+    if (mbar_try(bar, parity)) { tc_fence_after(); return; }
+    if ((i & 255) == 255 && *(volatile int*)&s_mi.abort_flag) return;
+  }
+  *(volatile int*)&s_mi.abort_flag = 1;
+}
+#define WAIT_PHASE(bar, parity) wait_phase(smem_u32(&s_mi.bar), (uint32_t)(parity) & 1u)
+
 // ---------------------------------------------------------------------------------------------
-// Attention of one tile with mma.sync, blocked by 16 consecutive tile rows rather than by set: one warp per (row
-// block, head).  The keys of a block are the rows of every set that the block touches; a score is
-// kept only where query and key belong to the same set (row_lo / row_n give each row's set range).
-// The arithmetic per query row is exactly the per-set softmax attention, but sparse regions with
-// many tiny sets cost one item per 16 rows instead of one per set, and the running softmax over passes of four key
-// blocks keeps the registers low for sets of any size (a version with one item per set and all of a set's scores in
-// registers spilled for set sizes near 96 and was a quarter slower there).
-// NTB = key blocks of 8 a row block can need: ceil((2 tau + 14) / 8), at most the 16 of a whole tile.
+// Attention
 // ---------------------------------------------------------------------------------------------
-template <int C, int D, int NTB, bool RPB>
-__device__ __forceinline__ void attend_blocked() {
-  constexpr int DC = D / 8;  // 16-byte chunks per head
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t a_base = s_mi.sbase + s_mi.off_a, k_base = s_mi.sbase + s_mi.off_kv;
-  const uint32_t v_base = k_base + (C / 64) * (kTM * 128);
+// Set codes: sets of a tile are numbered 0, 1, 2, ... modulo kCodes.  A query row carries 2^100 at its set's place and
+// zeros elsewhere, a key row 0 at its set's place and -1 elsewhere, so that their product is exactly 0 inside a set and
+// -2^100 across sets of different numbers; key rows past the tile hold -1 throughout.  A warp whose keys span more than
+// kCodes sets masks by comparing instead (softmax_rows).  Head dim 24 leaves 8 of the 32 columns of its two K steps to
+// the code, the other head dims take a K step of 16 for it.
+template <int D>
+constexpr int kCodes = D == 24 ? 8 : 16;
+
+template <int D>
+__device__ __forceinline__ void write_codes(int b, int rows) {
+  const int row = threadIdx.x;
+  if (row >= kTM) return;
+  const int w = row >> 5, lane = row & 31;
+  int ord = __popc(s_mi.starts[b][w] & (0xffffffffu >> (31 - lane)));
+  for (int j = 0; j < w; ++j) ord += __popc(s_mi.starts[b][j]);
+  const int code = row < rows ? ord & (kCodes<D> - 1) : -1;
+  const uint32_t base = s_mi.sbase + s_mi.off_code + row * 16;
+#pragma unroll
+  for (int c = 0; c < kCodes<D> / 8; ++c) {
+    uint32_t q[4], k[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int e = code - 8 * c - 2 * i;  // 0: the low element of the pair, 1: the high one
+      const bool low = code >= 0 && e == 0, high = code >= 0 && e == 1;
+      q[i] = low ? 0x00007180u : high ? 0x71800000u : 0u;
+      k[i] = low ? 0xbf800000u : high ? 0x0000bf80u : 0xbf80bf80u;
+    }
+    sts4(base + c * kChunkBytes, make_uint4(q[0], q[1], q[2], q[3]));
+    sts4(base + (kCodes<D> / 8 + c) * kChunkBytes, make_uint4(k[0], k[1], k[2], k[3]));
+  }
+}
+
+// The keys of a warp's 32 rows: blocks of 16 tile rows [kb0, kb1), and whether the codes keep their sets apart.
+struct KeyRange { int kb0, kb1; bool coded; };
+template <int D>
+__device__ __forceinline__ KeyRange key_range(int r0, int rows) {
   const unsigned char* row_lo = s_mi.row_lo[s_mi.buf];
-  const unsigned char* row_n = s_mi.row_n[s_mi.buf];
-  const int rows = s_mi.rows, heads = s_mi.heads;
-  // Key blocks of 8 per pass (running softmax across passes keeps registers low).  With wide sets six are faster although
-  // a few registers spill (nuScenes shapes, 8 layers: 459 us against 469); with sets up to 48 rows most 16-row blocks are
-  // done in one or two passes of four, and the spills cost more than they save (pillar frame: 519 us against 487).
-  constexpr int PW = NTB > 14 ? 6 : 4;
-  const int t4 = lane & 3;
+  const int rl = min(r0 + 31, rows - 1);
+  KeyRange k;
+  k.kb0 = row_lo[r0] >> 4;
+  k.kb1 = min((row_lo[rl] + s_mi.row_n[s_mi.buf][rl] + 15) >> 4, (rows + 15) >> 4);
+  const int from = 16 * k.kb0 + 1, to = min(16 * k.kb1, rows);  // set starts in here, and the set at the front
+  int sets = 1;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int lo = min(max(from - 32 * j, 0), 32), hi = min(max(to - 32 * j, 0), 32);
+    if (hi > lo) sets += __popc(s_mi.starts[s_mi.buf][j] & (0xffffffffu >> (32 - hi)) & (0xffffffffu << lo));
+  }
+  k.coded = sets <= kCodes<D>;
+  return k;
+}
+
+// Softmax of one head for the 32 rows of a warp, a row per thread: S (fp32, TMEM columns [t_s, t_s + 128)) -> P (bf16
+// pairs, columns [t_s, t_s + 64), zeros outside the warp's key blocks).  Returns the row's sum.  P overwrites S: block
+// b's 8 columns lie in S blocks up to b, which have been read by then.
+// [lo, lo + n): the rows of this row's set, by which keys are masked where the codes do not do it (!coded).
+template <int D, bool RPB>
+__device__ __forceinline__ float softmax_rows(uint32_t t_s, const KeyRange& k, int n_blocks, int row, int lo, int n, int h) {
   const float sc = 1.4426950408889634f * rsqrtf((float)D);  // log2(e) / sqrt(d)
-  const int nblk = (rows + 15) >> 4;
-  for (int item = warp; item < nblk * heads; item += kComputeWarps) {
-    const int blk = item / heads, h = item - blk * heads;
-    const int c0 = h * DC;
-    const int q0 = 16 * blk;
-    const int k_lo = row_lo[q0];
-    const int r_last = min(q0 + 15, rows - 1);
-    const int ntu = min((row_lo[r_last] + row_n[r_last] - k_lo + 7) >> 3, NTB);
-    const int ra = q0 + (lane >> 2), rb = ra + 8;
-    // each thread's two query rows: first key and number of keys of their sets, relative to k_lo
-    // (rows past the tile get zero keys)
-    const unsigned loA = ra < rows ? (unsigned)(row_lo[ra] - k_lo) : 0u;
-    const unsigned nA = ra < rows ? (unsigned)row_n[ra] : 0u;
-    const unsigned loB = rb < rows ? (unsigned)(row_lo[rb] - k_lo) : 0u;
-    const unsigned nB = rb < rows ? (unsigned)row_n[rb] : 0u;
-    const float root = sqrtf((float)D);
-    const float* tab = RPB ? s_mi.rpb + (size_t)h * s_mi.rb_len : nullptr;
-    const int linA = RPB ? s_mi.rowlin[min(ra, kTM - 1)] : 0, linB = RPB ? s_mi.rowlin[min(rb, kTM - 1)] : 0;
-    uint32_t qa[4], qb[4];
-    {
-      const int row = q0 + (lane & 15);  // <= 127
-      ldsm_x4(a_base + swz(row, c0 + (lane >> 4)), qa);
-      if (D > 16) ldsm_x4(a_base + swz(row, c0 + 2 + ((D == 32) ? (lane >> 4) : 0)), qb);
+  auto mask = [&](float (&s)[16], int b) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if ((unsigned)(16 * b + i - lo) >= (unsigned)n) s[i] = -INFINITY;
+  };
+  float mx = -INFINITY;
+#pragma unroll 1
+  for (int b = k.kb0; b < k.kb1; ++b) {
+    float s[16];
+    tmem_ld16_at<0>(t_s + 16 * b, s);
+    tmem_wait_ld();
+    if (RPB) {
+      const float* tab = s_mi.rpb + (size_t)h * s_mi.rb_len;
+      const float root = sqrtf((float)D);
+      const int lin = s_mi.rowlin[row];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) s[i] += rpb_term(tab, lin, s_mi.rowlin[16 * b + i], root);
+      tmem_st16_at<0>(t_s + 16 * b, s);
     }
-    // Row addresses advance by one 1024-byte group per key block of 8 (the swizzle depends on row & 7 only).
-    // Reads may run up to two groups past row 127: they land in the neighbouring operand block or, for the last
-    // 64 value columns, in the weight ring, and meet zero probabilities.  Those bytes are this tile's own K / V
-    // values or this layer's weights: a non-finite value among them (0 x Inf) could only come from a non-finite
-    // weight or feature, and every output row of a layer depends on every weight of the layer, so such a layer has
-    // no finite output row to spoil.
-    uint32_t k_addr = k_base + swz(k_lo + (lane & 7), c0 + min(lane >> 3, DC - 1));
-    uint32_t v_addr[DC];
+    if (!k.coded) mask(s, b);
+    float m0 = fmaxf(s[0], s[1]), m1 = fmaxf(s[2], s[3]);
 #pragma unroll
-    for (int dn = 0; dn < DC; ++dn) v_addr[dn] = v_base + swz(k_lo + (lane & 15), c0 + dn);
-    float o[DC][4];
+    for (int i = 4; i < 16; i += 4) { m0 = fmaxf(m0, fmaxf(s[i], s[i + 1])); m1 = fmaxf(m1, fmaxf(s[i + 2], s[i + 3])); }
+    mx = fmaxf(mx, fmaxf(m0, m1));
+  }
+  if (RPB) tmem_wait_st();
+  const float off = mx == -INFINITY ? 0.f : -mx * sc;  // (rows past the tile may have no key)
+  const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+  for (int b = 0; b < k.kb0; ++b) tmem_st8_u32(t_s + 8 * b, zero);
+  float2 sum = make_float2(0.f, 0.f);
+#pragma unroll 1
+  for (int b = k.kb0; b < k.kb1; ++b) {
+    float s[16];
+    tmem_ld16_at<0>(t_s + 16 * b, s);
+    tmem_wait_ld();
+    if (!k.coded) mask(s, b);
+    uint32_t p[8];
 #pragma unroll
-    for (int dn = 0; dn < DC; ++dn) o[dn][0] = o[dn][1] = o[dn][2] = o[dn][3] = 0.f;
-    float mA = -INFINITY, mB = -INFINITY, l0 = 0.f, l1 = 0.f;  // running row maxima and sums
-    for (int j0 = 0; j0 < ntu; j0 += PW) {
-      float s[PW][4];
-      float mx0 = mA, mx1 = mB;
-#pragma unroll
-      for (int jj = 0; jj < PW; ++jj) {
-        if (j0 + jj < ntu) {
-          s[jj][0] = s[jj][1] = s[jj][2] = s[jj][3] = 0.f;
-          uint32_t kf[4];
-          ldsm_x4(k_addr + 1024u * jj, kf);
-          mma_16816(s[jj], qa, kf[0], kf[1]);
-          if (D == 24) mma_1688(s[jj], qb[0], qb[1], kf[2]);
-          if (D == 32) mma_16816(s[jj], qb, kf[2], kf[3]);
-          const unsigned key = (unsigned)(8 * (j0 + jj) + 2 * t4);
-          if (RPB) {
-            const int kr = k_lo + (int)key;  // (rows past the tile are masked below: any entry will do)
-            const int lk0 = s_mi.rowlin[min(kr, kTM - 1)], lk1 = s_mi.rowlin[min(kr + 1, kTM - 1)];
-            s[jj][0] += rpb_term(tab, linA, lk0, root);
-            s[jj][1] += rpb_term(tab, linA, lk1, root);
-            s[jj][2] += rpb_term(tab, linB, lk0, root);
-            s[jj][3] += rpb_term(tab, linB, lk1, root);
-          }
-          if (key - loA >= nA) s[jj][0] = -INFINITY;  // unsigned: also true for key < lo
-          if (key + 1u - loA >= nA) s[jj][1] = -INFINITY;
-          if (key - loB >= nB) s[jj][2] = -INFINITY;
-          if (key + 1u - loB >= nB) s[jj][3] = -INFINITY;
-          mx0 = fmaxf(mx0, fmaxf(s[jj][0], s[jj][1]));
-          mx1 = fmaxf(mx1, fmaxf(s[jj][2], s[jj][3]));
-        }
-      }
-      k_addr += 1024u * PW;
-      mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
-      mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
-      mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
-      mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
-      // rows without any key so far (rows past the tile) keep finite arithmetic
-      const float off0 = (mx0 == -INFINITY) ? 0.f : -mx0 * sc, off1 = (mx1 == -INFINITY) ? 0.f : -mx1 * sc;
-      if (j0 > 0) {  // rescale what the earlier passes accumulated to the new maxima
-        const float al0 = (mA == -INFINITY) ? 0.f : ex2_approx(fmaf(mA, sc, off0));
-        const float al1 = (mB == -INFINITY) ? 0.f : ex2_approx(fmaf(mB, sc, off1));
-        l0 *= al0;
-        l1 *= al1;
-#pragma unroll
-        for (int dn = 0; dn < DC; ++dn) { o[dn][0] *= al0; o[dn][1] *= al0; o[dn][2] *= al1; o[dn][3] *= al1; }
-      }
-      mA = mx0;
-      mB = mx1;
-#pragma unroll
-      for (int kk = 0; kk < PW / 2; ++kk) {
-        if (j0 + 2 * kk < ntu) {
-          const bool two = j0 + 2 * kk + 1 < ntu;
-          float e[8];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            e[u] = ex2_approx(fmaf(s[2 * kk][u], sc, u < 2 ? off0 : off1));
-            e[4 + u] = two ? ex2_approx(fmaf(s[2 * kk + 1][u], sc, u < 2 ? off0 : off1)) : 0.f;
-          }
-          l0 += (e[0] + e[1]) + (e[4] + e[5]);
-          l1 += (e[2] + e[3]) + (e[6] + e[7]);
-          uint32_t pa[4];
-          pa[0] = pack_bf16(e[0], e[1]);
-          pa[1] = pack_bf16(e[2], e[3]);
-          pa[2] = pack_bf16(e[4], e[5]);
-          pa[3] = pack_bf16(e[6], e[7]);
-#pragma unroll
-          for (int dn = 0; dn < DC; ++dn) {
-            uint32_t vf[2];
-            ldsm_x2_trans(v_addr[dn] + 2048u * kk, vf);
-            mma_16816(o[dn], pa, vf[0], vf[1]);
-          }
-        }
-      }
-#pragma unroll
-      for (int dn = 0; dn < DC; ++dn) v_addr[dn] += 1024u * PW;
+    for (int i = 0; i < 8; ++i) {
+      const float2 u = __ffma2_rn(make_float2(s[2 * i], s[2 * i + 1]), make_float2(sc, sc), make_float2(off, off));
+      const float2 e = make_float2(ex2_approx(u.x), ex2_approx(u.y));
+      sum = __fadd2_rn(sum, e);
+      p[i] = pack_bf16(e.x, e.y);
     }
-    // the per-thread partial sums of a row live in the four threads of its quad
-    l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
-    l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
-    l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
-    l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
-    const float i0 = __fdividef(1.0f, l0), i1 = __fdividef(1.0f, l1);
-    // the query rows of this block and head are dead now: their slots take the attention output
-    if (ra < rows) {
+    tmem_st8_u32(t_s + 8 * b, p);
+  }
+  for (int b = k.kb1; b < n_blocks; ++b) tmem_st8_u32(t_s + 8 * b, zero);
+  tmem_wait_st();
+  return sum.x + sum.y;
+}
+
+// Attention of tile k: warps 4 q + (0..3) take heads q, q + 4, ... ; their S, then P, then O live in TMEM columns
+// [128 q, 128 q + 128).  The output of a head replaces its (dead) query columns.
+template <int C, int D, bool RPB>
+__device__ __forceinline__ void attend(int k) {
+  constexpr int DC = D / 8;  // 16-byte chunks per head
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp >> 2;
+  const int rows = s_mi.rows, row = 32 * (warp & 3) + lane;
+  const bool on = 32 * (warp & 3) < rows;  // (the whole warp)
+  const uint32_t t_s = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + 128 * q;
+  KeyRange kr = {0, 0, true};
+  if (on) kr = key_range<D>(32 * (warp & 3), rows);
+  const int lo = s_mi.row_lo[s_mi.buf][row], n = s_mi.row_n[s_mi.buf][row];
+#pragma unroll 1
+  for (int h = q; h < s_mi.heads; h += 4) {
+    const uint32_t par = (uint32_t)(k * (s_mi.heads >> 2) + (h >> 2)) & 1u;  // (heads so far of this group)
+    wait_phase(smem_u32(&s_mi.s_full[0]) + 8 * q, par);
+    float l = 1.f;
+    if (on) l = softmax_rows<D, RPB>(t_s, kr, (rows + 15) >> 4, row, lo, n, h);
+    tc_fence_before();
+    mbar_arrive(&s_mi.p_ready[q]);
+    wait_phase(smem_u32(&s_mi.ov_full[0]) + 8 * q, par);
+    if (on) {
+      float o[D];
+      tmem_ld_row(t_s + 64, o);
+      tmem_wait_ld();
+      const float inv = __fdividef(1.0f, l);
+      const uint32_t out = s_mi.sbase + s_mi.off_a + h * DC * kChunkBytes + row * 16;
 #pragma unroll
-      for (int dn = 0; dn < DC; ++dn)
-        asm volatile("st.shared.b32 [%0], %1;" ::"r"(a_base + swz(ra, c0 + dn) + 4 * t4),
-                     "r"(pack_bf16(o[dn][0] * i0, o[dn][1] * i0)) : "memory");
+      for (int c = 0; c < DC; ++c)
+        sts4(out + c * kChunkBytes,
+             make_uint4(pack_bf16(o[8 * c] * inv, o[8 * c + 1] * inv), pack_bf16(o[8 * c + 2] * inv, o[8 * c + 3] * inv),
+                        pack_bf16(o[8 * c + 4] * inv, o[8 * c + 5] * inv), pack_bf16(o[8 * c + 6] * inv, o[8 * c + 7] * inv)));
     }
-    if (rb < rows) {
-#pragma unroll
-      for (int dn = 0; dn < DC; ++dn)
-        asm volatile("st.shared.b32 [%0], %1;" ::"r"(a_base + swz(rb, c0 + dn) + 4 * t4),
-                     "r"(pack_bf16(o[dn][2] * i1, o[dn][3] * i1)) : "memory");
-    }
+    tc_fence_before();
+    mbar_arrive(&s_mi.o_read[q]);
   }
 }
 
@@ -382,9 +411,9 @@ struct RoleCtx {
   uint32_t sbase;     // 1024-aligned shared-memory base as a shared-space address
   uint32_t tmem;      // TMEM base address of the CTA's allocation
   // copies of the kernel parameters the two single-thread roles use (registers instead of parameter-space loads)
-  int mode, n_f1, NF, tau, n_layers;
+  int mode, n_f1, NF, tau, n_layers, heads;
   int pe;  // the value projection comes first and the A operand is rewritten (x + pe) before the key and query ones
-  uint32_t off_a, off_kv, off_stage;
+  uint32_t off_a, off_kv, off_code, off_stage;
 };
 
 __device__ __forceinline__ int ld_acquire_gpu(const int32_t* p) {
@@ -432,7 +461,6 @@ __device__ __noinline__ void producer_role(const TcArgs& a, const RoleCtx rc) {
     const TcLayer& ly = a.layer[l];
     const int S = min(__ldg(ly.num_sets), ly.cap_sets);
     int T = __ldg(ly.rowoff + ly.cap_sets + 1);
-    mi->lay_S[l] = S;
     mi->lay_plan[l] = T < 0 ? 0 : (T & DSVT_PLAN_PACKED) ? 2 : 1;  // none / in table order / over a reordering
     if (T < 0) T = S > 0 ? (__ldg(ly.rowoff + S) + Rv - 1) / Rv : 0;
     else T = min(T & ~DSVT_PLAN_PACKED, S);
@@ -450,7 +478,7 @@ __device__ __noinline__ void producer_role(const TcArgs& a, const RoleCtx rc) {
       while (l + 1 < L && g >= mi->tile_end[l]) ++l;
       const int t = g - (l ? mi->tile_end[l - 1] : 0);
       const TcLayer& ly = a.layer[l];
-      const int S = mi->lay_S[l];
+      const int S = min(__ldg(ly.num_sets), ly.cap_sets);
       int f, e;
       if (mi->lay_plan[l]) {
         const int32_t* plan = ly.rowoff + ly.cap_sets + 1;
@@ -541,63 +569,146 @@ producer_done:
   }
 }
 
-// ================= MMA issuer (one thread) =============================================================
-template <int C>
-__device__ __noinline__ void mma_role(const RoleCtx rc) {
+// ================= MMA issuer (one warp) ===============================================================
+// The whole warp runs this code with warp-uniform values and one elected lane issues: operands then stay in uniform
+// registers.  Issued by a single thread from divergent code every MMA took 46 to 65 cycles of issue (measured: eight
+// N = 32 MMAs done after 788 cycles, against 249 this way), which is more than the tensor pipe needs for N <= 128 (N / 2
+// cycles).  Descriptors are kept as 32-bit low words (address and leading offset, to which byte offsets / 16 are added)
+// and constant high words.
+template <int C, int D>
+__device__ __forceinline__ void mma_role(const RoleCtx& rc) {
   constexpr int NKB = C / 64;        // K blocks of a C-deep contraction
-  constexpr uint32_t STAGE_BYTES = C * 128;
+  constexpr uint32_t STAGE16 = C * 128 / 16;
+  constexpr uint32_t kChunk16 = kChunkBytes / 16, kRows16 = kTM * 128 / 16;  // a chunk; a K block of the swizzled operand
+  constexpr uint32_t kHeadStep = (D / 8) * kChunk16;  // from a head's Q, K or V columns to the next head's
+  constexpr uint32_t SW = kDescHiSwizzled, KM = desc_hi_plain(128), NM = desc_hi_plain(kChunkBytes);
   const uint32_t tmem = rc.tmem;
   Misc* mi = &s_mi;
-  const uint32_t a_base = rc.sbase + rc.off_a, st_base = rc.sbase + rc.off_stage;
+  const uint32_t a_addr = rc.sbase + rc.off_a, k_addr = rc.sbase + rc.off_kv, v_addr = k_addr + (C / 8) * kChunkBytes;
+  const uint32_t q_code = rc.sbase + rc.off_code, k_code = q_code + kCodes<D> / 8 * kChunkBytes;
+  const uint32_t x_lo = desc_lo_swizzled(a_addr), w_lo = desc_lo_swizzled(rc.sbase + rc.off_stage);
+  const uint32_t q_lo = desc_lo_plain(a_addr, kChunkBytes), k_lo = desc_lo_plain(k_addr, kChunkBytes);
+  const uint32_t v_lo = desc_lo_plain(v_addr, 128);
   volatile int* abort_flag = &mi->abort_flag;
   const bool mlp = rc.mode == 2;
   const int c_v = rc.pe ? 0 : 1;  // the V chunk
   int stage = 0, slot = 0;
   uint32_t phase = 0, a_phase = 0, x_phase = 0, sphase = 0, tile = 0;
-  uint32_t uses = 0, m2 = 0;  // of the K / Q / MLP-1 accumulator; MLP-2 pieces
-  // n_kb K blocks of 64 from the weight ring; issue(kb, k4, B descriptor) issues one MMA
+  uint32_t uses = 0, m2 = 0, heads_done = 0;  // of the K / Q / MLP-1 accumulator; MLP-2 pieces; heads of a group
+  // n_kb K blocks of 64 from the weight ring; issue(kb, k4, low word of B) issues one MMA
   auto blocks = [&](int n_kb, auto issue) -> bool {
     for (int kb = 0; kb < n_kb; ++kb) {
       if (!mbar_wait(&mi->full[stage], phase, abort_flag)) return false;
       tc_fence_after();
-      const uint32_t sb = st_base + stage * STAGE_BYTES;
+      const uint32_t b = w_lo + stage * STAGE16;
+      if (elect_one()) {
 #pragma unroll
-      for (int k4 = 0; k4 < 4; ++k4) issue(kb, k4, umma_desc(sb + k4 * 32));
-      umma_commit(&mi->empty[stage]);  // frees the weight stage once these MMAs have read it
+        for (int k4 = 0; k4 < 4; ++k4) issue(kb, k4, b + 2 * k4);
+        umma_commit(&mi->empty[stage]);  // frees the weight stage once these MMAs have read it
+      }
+      __syncwarp();
       if (++stage == kStages) { stage = 0; phase ^= 1u; }
     }
     return true;
   };
+  auto commit = [&](unsigned long long* bar) {
+    if (elect_one()) umma_commit(bar);
+    __syncwarp();
+  };
   for (;; ++tile) {
     if (!mbar_wait(&mi->sched_full[slot], sphase, abort_flag)) break;
-    const int ns = mi->tile[slot][1];
-    mbar_arrive(&mi->sched_empty[slot]);
+    const int ns = __shfl_sync(0xffffffffu, mi->tile[slot][1], 0), rows = __shfl_sync(0xffffffffu, mi->tile[slot][3], 0);
+    if (elect_one()) mbar_arrive(&mi->sched_empty[slot]);
     if (++slot == 2) { slot = 0; sphase ^= 1u; }
     if (ns < 0) break;
-    // ---- K, V, Q, then the output projection ----
-    for (int c = 0; c < 4; ++c) {
+    // ---- K, V, Q ----
+    for (int c = 0; c < 3; ++c) {
       if (c == 0 || (c == 1 && rc.pe)) {  // (with a positional term the operand is rewritten after the V chunk)
         if (!mbar_wait(&mi->x_ready, x_phase, abort_flag)) goto mma_done;
         x_phase ^= 1u;
-      } else if (c == 3) {
-        if (!mbar_wait(&mi->a_ready, a_phase, abort_flag)) goto mma_done;
-        a_phase ^= 1u;
       }
       if (c == c_v) {
         // the columns may overlap R and the MLP hidden: the previous tile's result must have been read
         if (!mbar_wait(&mi->acc_free[2], (tile & 1u) ^ 1u, abort_flag)) goto mma_done;
         if (!mbar_wait(&mi->acc_free[1], (tile & 1u) ^ 1u, abort_flag)) goto mma_done;
-      } else if (c < 3) {
+      } else {
         if (!mbar_wait(&mi->acc_free[0], (uses & 1u) ^ 1u, abort_flag)) goto mma_done;
         ++uses;
       }
       tc_fence_after();
-      const uint32_t d = tmem + (c == 3 ? Tm<C>::r : c == c_v ? Tm<C>::v : Tm<C>::k);
-      if (!blocks(NKB, [&](int kb, int k4, uint64_t b) {
-            umma_bf16(d, umma_desc(a_base + kb * (kTM * 128) + k4 * 32), b, umma_idesc(C), (kb | k4) != 0 ? 1u : 0u);
+      const uint32_t d = tmem + (c == c_v ? Tm<C>::v : Tm<C>::k);
+      if (!blocks(NKB, [&](int kb, int k4, uint32_t b) {
+            umma_ss(d, x_lo + kb * kRows16 + 2 * k4, SW, b, SW, umma_idesc(C), (kb | k4) != 0 ? 1u : 0u);
           })) goto mma_done;
-      umma_commit(c == 3 ? &mi->o_full : &mi->acc_full[c == c_v ? 1 : 0]);
+      commit(&mi->acc_full[c == c_v ? 1 : 0]);
     }
+    // ---- attention: S = Q K^T, O = P V, four heads at a time ----
+    if (!mbar_wait(&mi->a_ready, a_phase, abort_flag)) goto mma_done;
+    a_phase ^= 1u;
+    tc_fence_after();
+    {
+      const int n_blocks = (rows + 15) >> 4;  // of 16 keys
+      const uint32_t id_s = umma_idesc(16 * n_blocks), id_o = umma_idesc(D == 24 ? 32 : D) | (1u << 16);  // V: N-major
+      const int rounds = rc.heads >> 2;
+      auto scores = [&](int q, int i) {
+        const uint32_t d = tmem + 128 * q, step = (uint32_t)(4 * i + q) * kHeadStep;
+        umma_ss(d, q_lo + step, KM, k_lo + step, KM, id_s, 0u);
+        if (D == 24) {  // the last 8 columns and the code: the leading offset leads from one to the other
+          const uint32_t qa = (a_addr >> 4) + 2 * kChunk16 + step, ka = (k_addr >> 4) + 2 * kChunk16 + step;
+          umma_ss(d, qa | ((q_code >> 4) - qa) << 16, KM, ka | ((k_code >> 4) - ka) << 16, KM, id_s, 1u);
+        } else {
+          if (D == 32) umma_ss(d, q_lo + step + 2 * kChunk16, KM, k_lo + step + 2 * kChunk16, KM, id_s, 1u);
+          umma_ss(d, desc_lo_plain(q_code, kChunkBytes), KM, desc_lo_plain(k_code, kChunkBytes), KM, id_s, 1u);
+        }
+        umma_commit(&mi->s_full[q]);
+      };
+      if (elect_one()) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) scores(q, 0);
+      }
+      __syncwarp();
+      // the four groups advance on their own: step 2 i of a group waits for P of its head i, step 2 i + 1 for O having
+      // been read (not needed after the last head: a_ready follows it)
+      int left = 4 * (2 * rounds - 1);
+      uint32_t step = 0;  // 8 bits per group
+      for (int idle = 0; left > 0; ++idle) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int st = (int)(step >> (8 * q)) & 255, i = st >> 1;
+          if (st >= 2 * rounds - 1) continue;
+          if (!__all_sync(0xffffffffu, mbar_test((st & 1) ? &mi->o_read[q] : &mi->p_ready[q], (heads_done + (uint32_t)i) & 1u)))
+            continue;
+          tc_fence_after();
+          if (elect_one()) {
+            if (st & 1) {
+              scores(q, i + 1);
+            } else {
+              const uint32_t v = v_lo + (uint32_t)(4 * i + q) * kHeadStep;
+#pragma unroll
+              for (int s = 0; s < 8; ++s)  // (16 keys: 8 columns of P, 256 bytes of each chunk of V)
+                if (s < n_blocks)
+                  umma_ts(tmem + 128 * q + 64, tmem + 128 * q + 8 * s, v + 16 * s, NM, id_o, s != 0 ? 1u : 0u);
+              umma_commit(&mi->ov_full[q]);
+            }
+          }
+          __syncwarp();
+          step += 1u << (8 * q);
+          --left;
+          idle = 0;
+        }
+        if ((idle & 255) == 255 && *abort_flag) goto mma_done;
+        if (idle > kMaxIdle) { *abort_flag = 1; goto mma_done; }
+      }
+      heads_done += (uint32_t)rounds;
+    }
+    // ---- output projection ----
+    if (!mbar_wait(&mi->a_ready, a_phase, abort_flag)) goto mma_done;
+    a_phase ^= 1u;
+    tc_fence_after();
+    if (!blocks(NKB, [&](int kb, int k4, uint32_t b) {
+          umma_ss(tmem + Tm<C>::r, q_lo + (8 * kb + 2 * k4) * kChunk16, KM, b, SW, umma_idesc(C), (kb | k4) != 0 ? 1u : 0u);
+        })) goto mma_done;
+    commit(&mi->o_full);
     if (!mlp) continue;
     // ---- MLP, piece by piece, on top of the residual parked in R ----
     if (!mbar_wait(&mi->a_ready, a_phase, abort_flag)) goto mma_done;
@@ -609,26 +720,26 @@ __device__ __noinline__ void mma_role(const RoleCtx rc) {
         ++uses;
         tc_fence_after();
         const uint32_t idesc = umma_idesc(rc.NF);
-        if (!blocks(NKB, [&](int kb, int k4, uint64_t b) {  // (16 bf16 operand columns are 8 TMEM columns)
-              umma_bf16_ts(tmem + Tm<C>::acc, tmem + Tm<C>::x1 + kb * 32 + k4 * 8, b, idesc, (kb | k4) != 0 ? 1u : 0u);
+        if (!blocks(NKB, [&](int kb, int k4, uint32_t b) {  // (16 bf16 operand columns are 8 TMEM columns)
+              umma_ts(tmem + Tm<C>::acc, tmem + Tm<C>::x1 + kb * 32 + k4 * 8, b, SW, idesc, (kb | k4) != 0 ? 1u : 0u);
             })) goto mma_done;
-        umma_commit(&mi->acc_full[0]);
+        commit(&mi->acc_full[0]);
       } else {
         if (!mbar_wait(&mi->h_ready, m2 & 1u, abort_flag)) goto mma_done;
         ++m2;
         tc_fence_after();
-        if (!blocks(rc.NF / 64, [&](int kb, int k4, uint64_t b) {
-              umma_bf16_ts(tmem + Tm<C>::r, tmem + Tm<C>::h + kb * 32 + k4 * 8, b, umma_idesc(C), 1u);
+        if (!blocks(rc.NF / 64, [&](int kb, int k4, uint32_t b) {
+              umma_ts(tmem + Tm<C>::r, tmem + Tm<C>::h + kb * 32 + k4 * 8, b, SW, umma_idesc(C), 1u);
             })) goto mma_done;
-        umma_commit(&mi->h_free);
+        commit(&mi->h_free);
       }
     }
-    umma_commit(&mi->acc_full[2]);
+    commit(&mi->acc_full[2]);
   }
 mma_done:
   if (*abort_flag) {
     // leaving early: the MMAs already issued must have completed before the TMEM columns are returned
-    umma_commit(&mi->drain);
+    commit(&mi->drain);
     for (int it = 0; it < kMaxPolls && !mbar_try(&mi->drain, 0u); ++it) {}
   }
 }
@@ -731,13 +842,20 @@ __device__ __noinline__ void loader_role(const TcArgs& a) {
                            packed ? ly.rowoff + 2 * (size_t)ly.cap_sets + 3 : nullptr, ly.cap_sets, b, lt, s_lo, nsets, base);
       if (lt == 0) s_mi.next_x[b] = lay == 0 ? a.x : a.y;
     }
+    if (nsets >= 0) {
+      loader_sync();  // the row list is complete
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t m = __ballot_sync(0xffffffffu, s_mi.row_lo[b][32 * j + lane] == 32 * j + lane);
+        if (lane == 0) s_mi.starts[b][j] = m;
+      }
+    }
     if (lt == 0) s_mi.next_rows[b] = nsets < 0 ? -1 : rows;
     mbar_arrive(&s_mi.rl_ready[b]);
     if (nsets < 0) break;
     // a tile of a later layer reads rows the previous layer wrote, possibly on other SMs: each row must carry that
     // layer's stamp (written after the row's store) before the tile is gathered
     if (lay > 0) {
-      loader_sync();  // the row list is complete
       const int want = a.stamp_base + lay;
       for (int r = lt; r < rows && ok; r += kLoadThreads) {
         const int v = s_mi.rowvox[b][r];
@@ -785,7 +903,7 @@ __device__ __noinline__ void stamp_role(int32_t* __restrict__ row_stamp) {
 // in flight at once (C = 192: 12 loads per lane; with two rounds of four rows and a quarter of the lanes idle the gather
 // cost one L2 round trip more).  ADD_PE: the current tile's rows once more, with the positional term added (the operand
 // of the key and query projections).
-template <int C, bool RPB, bool ADD_PE>
+template <int C, int D, bool RPB, bool ADD_PE>
 __device__ __forceinline__ void phase_gather(int b, int rows) {
   constexpr int C4 = C / 4, RU = C4 % 32 == 0 ? 1 : 2, IU = RU * C4 / 32;  // chunks per row; rows, loads per unit
   constexpr int kFly = ADD_PE ? (RU == 2 ? 2 : 4) : 8 / RU;                // units in flight
@@ -793,6 +911,7 @@ __device__ __forceinline__ void phase_gather(int b, int rows) {
   const float* x = ADD_PE ? s_mi.x : s_mi.next_x[b];
   const uint32_t a_tile = s_mi.sbase + s_mi.off_a;
   const int* rowvox = s_mi.rowvox[b];
+  if (!ADD_PE) write_codes<D>(b, rows);  // (the previous tile's attention is over)
   for (int r0 = RU * warp; r0 < kTM; r0 += kFly * RU * kComputeWarps) {
     float4 f[kFly][IU];
 #pragma unroll
@@ -835,29 +954,27 @@ __device__ __forceinline__ void phase_gather(int b, int rows) {
   }
 }
 
-// Epilogue of a projection chunk: QC accumulator columns per thread + bias -> bf16 into an operand tile.
-// Four threads per tile row: warp w owns TMEM lanes 32 (w % 4) .. + 31 and column quarter w / 4.
+// Epilogue of a K, V or Q chunk: QC accumulator columns per thread + bias -> bf16 into an unswizzled operand tile.
+// Four threads per tile row: warp w owns TMEM lanes 32 (w % 4) .. + 31 and column quarter w / 4.  Warps without rows
+// only release the accumulator.
 //   tcol      first TMEM column of the chunk's accumulator
 //   bar       accumulator barrier pair to release
 //   bias_off  float offset of the chunk's bias in the parameter block
-//   dst_off   byte offset of the destination operand tile from the shared-memory base
-//   c8_0      16-byte chunk index of the chunk's first column in the destination rows
-//   need      number of leading tile rows whose results are needed (warps wholly past it only release)
+//   dst_off   byte offset of the destination operand from the shared-memory base
 // BIAS = false skips the bias (the key projection: a key bias adds
 // the same amount q . b_k to every score of a query, which the softmax cancels).
 template <int QC, bool BIAS>
-__device__ __forceinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_off, uint32_t dst_off, int c8_0, int need) {
+__device__ __forceinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_off, uint32_t dst_off) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
-  if (32 * (warp & 3) >= need) {
+  if (32 * (warp & 3) >= s_mi.rows) {
     tc_fence_before();
     mbar_arrive(&s_mi.acc_free[bar]);
     return;
   }
   const uint32_t taddr = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + tcol + hq * QC;
-  const uint32_t bias = s_mi.sbase + s_mi.off_par + 4u * (uint32_t)(bias_off + hq * QC);
-  const uint32_t dst = s_mi.sbase + dst_off;
-  const int c8 = c8_0 + ((hq * QC) >> 3);
+  const uint32_t bias = smem_u32(s_mi.par) + 4u * (uint32_t)(bias_off + hq * QC);
+  const uint32_t dst = s_mi.sbase + dst_off + (uint32_t)(hq * (QC / 8)) * kChunkBytes + row * 16;
   float rr[QC];
   tmem_ld_row(taddr, rr);
   tmem_wait_ld();
@@ -874,13 +991,13 @@ __device__ __forceinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_
       v[2] = __fadd2_rn(v[2], make_float2(b1.x, b1.y));
       v[3] = __fadd2_rn(v[3], make_float2(b1.z, b1.w));
     }
-    sts4(dst + swz(row, c8 + q),
+    sts4(dst + q * kChunkBytes,
          make_uint4(pack_bf16(v[0].x, v[0].y), pack_bf16(v[1].x, v[1].y), pack_bf16(v[2].x, v[2].y), pack_bf16(v[3].x, v[3].y)));
   }
 }
 
 // MLP-1 piece: HC = NF / 4 hidden columns per thread, H = gelu(x1 W_1^T + b_1) into TMEM as the A operand of MLP-2.
-//   bias_off  float offset of the piece's bias in the parameter block
+//   bias_off  float offset of the piece's bias among the late vectors
 //   h_phase   parity of h_free that says that the MLP-2 of the piece before has read its hidden columns
 template <int C, int HC>
 __device__ __forceinline__ void phase_mlp1(int bias_off, uint32_t h_phase) {
@@ -893,7 +1010,7 @@ __device__ __forceinline__ void phase_mlp1(int bias_off, uint32_t h_phase) {
     mbar_arrive(&s_mi.h_ready);
     return;
   }
-  const uint32_t bias = s_mi.sbase + s_mi.off_par + 4u * (uint32_t)(bias_off + hq * HC);
+  const uint32_t bias = s_mi.sbase + s_mi.off_code + 4u * (uint32_t)(bias_off + hq * HC);
   float rr[HC];
   tmem_ld_row(lane_base + Tm<C>::acc + hq * HC, rr);
   tmem_wait_ld();
@@ -916,6 +1033,17 @@ __device__ __forceinline__ void phase_mlp1(int bias_off, uint32_t h_phase) {
   mbar_arrive(&s_mi.h_ready);
 }
 
+template <int C>
+__device__ __forceinline__ void stage_late_vectors() {
+  const int i = 4 * threadIdx.x;
+  if (i >= 2 * C + s_mi.NF * s_mi.n_f1) return;
+  const float* v = i < C ? s_mi.b_o : i < 2 * C ? s_mi.b_2 : s_mi.b_1;
+  const int j = i < C ? i : i < 2 * C ? i - C : i - 2 * C;
+  const uint32_t dst = s_mi.sbase + s_mi.off_code + 4u * (uint32_t)i;
+  if (v) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(v + j) : "memory");
+  else sts4(dst, make_float4(0.f, 0.f, 0.f, 0.f));
+}
+
 // x rows (fp32) for the first residual: asynchronous 16-byte copies global -> shared staging.
 template <int C>
 __device__ __forceinline__ void phase_stage_x() {
@@ -936,6 +1064,7 @@ __device__ __forceinline__ void phase_stage_x() {
         sts4(stage + off, make_float4(0.f, 0.f, 0.f, 0.f));
     }
   }
+  stage_late_vectors<C>();
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
@@ -955,14 +1084,6 @@ __device__ __forceinline__ void phase_store_rows() {
       reinterpret_cast<float4*>(y + (size_t)v * C)[c4] = lds4(stage + stage_off<C>(r, c4));
   }
 }
-
-// Per-layer vectors staged in shared memory (float offsets into the parameter block).
-template <int C>
-struct ParOff {
-  static constexpr int b_q = 0, b_v = C, b_o = 2 * C, b_2 = 3 * C, ln1_g = 4 * C, ln1_b = 5 * C, ln2_g = 6 * C,
-                       ln2_b = 7 * C, b_1 = 8 * C;  // b_1 has `hidden` entries and comes last; no key bias
-  static constexpr int vectors = 8;
-};
 
 // LayerNorm over the row that four threads share: t holds this thread's QC values, sum their sum.  Each
 // thread reduces its own quarter to (mean, sum of squared deviations), the four pairs are exchanged once
@@ -1005,8 +1126,9 @@ __device__ __forceinline__ void phase_epi_o() {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
   const uint32_t lane_base = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16), taddr = lane_base + Tm<C>::r + hq * QC;
-  const uint32_t par = s_mi.sbase + s_mi.off_par, stage = s_mi.sbase + s_mi.off_kv;
+  const uint32_t par = smem_u32(s_mi.par), stage = s_mi.sbase + s_mi.off_kv;
   const int mode = s_mi.mode;
+  const uint32_t late = s_mi.sbase + s_mi.off_code;
   const bool add_x = mode != 0 && row < s_mi.rows;
   float t[QC];
   float sum = 0.f;
@@ -1018,7 +1140,7 @@ __device__ __forceinline__ void phase_epi_o() {
   for (int q = 0; q < QC / 4; ++q) {
     float4 x4 = make_float4(0.f, 0.f, 0.f, 0.f);
     if (add_x) x4 = lds4(stage + stage_off<C>(row, hq * (QC / 4) + q));
-    const float4 b4 = lds4(par + 4u * (uint32_t)(ParOff<C>::b_o + hq * QC + 4 * q));
+    const float4 b4 = lds4(late + 4u * (uint32_t)(LateOff<C>::b_o + hq * QC + 4 * q));
     t[4 * q] += x4.x + b4.x;
     t[4 * q + 1] += x4.y + b4.y;
     t[4 * q + 2] += x4.z + b4.z;
@@ -1046,7 +1168,7 @@ __device__ __forceinline__ void phase_epi_o() {
   }
 #pragma unroll
   for (int q = 0; q < QC / 4; ++q) {
-    const float4 b4 = lds4(par + 4u * (uint32_t)(ParOff<C>::b_2 + hq * QC + 4 * q));
+    const float4 b4 = lds4(late + 4u * (uint32_t)(LateOff<C>::b_2 + hq * QC + 4 * q));
     t[4 * q] += b4.x;
     t[4 * q + 1] += b4.y;
     t[4 * q + 2] += b4.z;
@@ -1064,7 +1186,7 @@ __device__ __forceinline__ void phase_epi_f2() {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
   const uint32_t taddr = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + Tm<C>::r + hq * QC;
-  const uint32_t par = s_mi.sbase + s_mi.off_par, stage = s_mi.sbase + s_mi.off_kv;
+  const uint32_t par = smem_u32(s_mi.par), stage = s_mi.sbase + s_mi.off_kv;
   float t[QC];
   tmem_ld_row(taddr, t);
   tmem_wait_ld();
@@ -1085,27 +1207,25 @@ __device__ __forceinline__ void phase_epi_f2() {
   sts4(stage + stage_off<C>(row, hq * (QC / 4)), make_float4(t[0], t[1], t[2], t[3]));
 }
 
-// The layer's biases and LayerNorm vectors into the parameter block (absent vectors as zeros), and its scalars.
-// Order of ParOff: b_q, b_v, b_o, b_2, ln1_g, ln1_b, ln2_g, ln2_b, then b_1 (the key bias is not needed).
+// The layer's vectors of the parameter block (absent ones as zeros; order of ParOff: b_q, b_v, ln1_g, ln1_b, ln2_g,
+// ln2_b; the key bias is not needed), its scalars and the pointers to the other vectors.
 template <int C>
-__device__ __forceinline__ void load_layer_params(const TcLayer& ly, int hidden) {
-  float* par = reinterpret_cast<float*>(s_mi.sm + s_mi.off_par);
-  const uint32_t par_saddr = s_mi.sbase + s_mi.off_par;
-  const int n_par = ParOff<C>::vectors * C + hidden;
+__device__ __forceinline__ void load_layer_params(const TcLayer& ly) {
+  const uint32_t par = smem_u32(s_mi.par);
   // asynchronous 4-byte copies, all in flight at once: the first reader is the V epilogue, which waits for them
   // (wait_layer_params) after the K epilogue
-  for (int i = threadIdx.x; i < n_par; i += kComputeThreads) {
+  for (int i = threadIdx.x; i < ParOff<C>::vectors * C; i += kComputeThreads) {
     const int which = i / C;
-    const float* v = which == 0 ? ly.b_qkv : which == 1 ? (ly.b_qkv ? ly.b_qkv + 2 * C : nullptr) : which == 2 ? ly.b_o
-                   : which == 3 ? ly.b_2 : which == 4 ? ly.ln1_g : which == 5 ? ly.ln1_b : which == 6 ? ly.ln2_g
-                   : which == 7 ? ly.ln2_b : (ly.b_1 ? ly.b_1 - ParOff<C>::b_1 + which * C : nullptr);
-    if (v) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(par_saddr + 4u * (uint32_t)i), "l"(v + i % C) : "memory");
-    else par[i] = 0.f;
+    const float* v = which == 0 ? ly.b_qkv : which == 1 ? (ly.b_qkv ? ly.b_qkv + 2 * C : nullptr) : which == 2 ? ly.ln1_g
+                   : which == 3 ? ly.ln1_b : which == 4 ? ly.ln2_g : ly.ln2_b;
+    if (v) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(par + 4u * (uint32_t)i), "l"(v + i % C) : "memory");
+    else s_mi.par[i] = 0.f;
   }
   if (threadIdx.x == 0) {
     s_mi.ln1 = ly.ln1_g != nullptr;
     s_mi.ln2 = ly.ln2_g != nullptr;
     s_mi.eps = ly.eps;
+    s_mi.b_o = ly.b_o; s_mi.b_1 = ly.b_1; s_mi.b_2 = ly.b_2;
     s_mi.rpb = ly.rpb;
     s_mi.pe = ly.pe;
   }
@@ -1130,23 +1250,11 @@ __device__ __forceinline__ bool compute_all(bool pred) {
   return r != 0;
 }
 
-// A compute thread's wait (out of line: one copy of the polling loop).  A wait that gives up raises the abort flag,
-// which the tile loop looks at.
-__device__ __noinline__ void wait_phase(uint32_t bar, uint32_t parity) {
-  for (int i = 0; i < kMaxPolls; ++i) {
-    if (mbar_try(bar, parity)) { tc_fence_after(); return; }
-    if ((i & 255) == 255 && *(volatile int*)&s_mi.abort_flag) return;
-  }
-  *(volatile int*)&s_mi.abort_flag = 1;
-}
-#define WAIT_PHASE(bar, parity) wait_phase(smem_u32(&s_mi.bar), (uint32_t)(parity) & 1u)
-
 // The tile loop keeps as little as possible alive across the phase calls (the tile's index k, and two flags): what it
 // holds, every phase has fewer registers, and with 227 KB of shared memory taken there is no L1 left for spills.
-template <int C, int D, int NT, int VAR>
+template <int C, int D, int VAR>
 __device__ __forceinline__ void compute_role(const TcArgs& a) {
   constexpr bool RPB = VAR == 1, PE = VAR == 2;
-  constexpr int NKB = C / 64;        // K blocks of a C-deep contraction
   constexpr int QC = C / 4;          // epilogue columns per thread for a C-wide chunk (four threads per row)
   volatile int* abort_flag = &s_mi.abort_flag;
   bool gathered = false;  // the tile about to start was gathered under the previous tile's MLP
@@ -1160,7 +1268,7 @@ __device__ __forceinline__ void compute_role(const TcArgs& a) {
     WAIT_PHASE(rl_ready[b], (k + 1) >> 1);
     const int nr = s_mi.next_rows[b];
     if (compute_all(nr >= 0 && *abort_flag == 0 && mbar_try(&s_mi.dep_ready[b], (uint32_t)((k + 1) >> 1) & 1u))) {
-      phase_gather<C, RPB, false>(b, nr);
+      phase_gather<C, D, RPB, false>(b, nr);
       fence_proxy_async();
       mbar_arrive(&s_mi.x_ready);
       gathered = true;
@@ -1184,14 +1292,14 @@ __device__ __forceinline__ void compute_role(const TcArgs& a) {
     if (nsets < 0) break;
     const bool new_params = layer != cur_layer;
     if (new_params) {  // (the previous tile's last use of the block lies before the barrier above)
-      load_layer_params<C>(a.layer[layer], a.g.hidden);
+      load_layer_params<C>(a.layer[layer]);
       cur_layer = layer;
     }
     if (!gathered) {  // a CTA's first tile, or a tile whose rows were not ready in time
       WAIT_PHASE(rl_ready[k & 1], k >> 1);
       WAIT_PHASE(dep_ready[k & 1], k >> 1);
       if (compute_all(*abort_flag == 0)) {
-        phase_gather<C, RPB, false>(k & 1, s_mi.next_rows[k & 1]);
+        phase_gather<C, D, RPB, false>(k & 1, s_mi.next_rows[k & 1]);
         fence_proxy_async();
       }
       mbar_arrive(&s_mi.x_ready);  // X is in place
@@ -1201,37 +1309,40 @@ __device__ __forceinline__ void compute_role(const TcArgs& a) {
 
     // (uses of the accumulators before this tile: V and R one each per tile, the first one K, Q and the MLP-1 pieces)
     // ---- chunks 0..2: K, V, Q epilogues: (+ bias,) to bf16, into the operand layout ----
-    // (the attention pads its key blocks up to 15 rows past the tile: those K / V rows must be real bf16)
     if (PE) {
       // the values come from the bare rows; the operand is then rewritten with the positional term added, for
       // the keys and the queries (the V chunk's accumulator being complete, nothing reads the operand any more)
       WAIT_PHASE(acc_full[1], k);
       if (new_params) wait_layer_params();
-      phase_epi_bf16<QC, true>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + NKB * kTM * 128, 0, s_mi.rows + 16);
-      phase_gather<C, false, true>(k & 1, s_mi.rows);
+      phase_epi_bf16<QC, true>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + (C / 8) * kChunkBytes);
+      phase_gather<C, D, false, true>(k & 1, s_mi.rows);
       fence_proxy_async();
       mbar_arrive(&s_mi.x_ready);
       WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1));
-      phase_epi_bf16<QC, false>(Tm<C>::k, 0, 0, s_mi.off_kv, 0, s_mi.rows + 16);
+      phase_epi_bf16<QC, false>(Tm<C>::k, 0, 0, s_mi.off_kv);
     } else {
       WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1));
-      phase_epi_bf16<QC, false>(Tm<C>::k, 0, 0, s_mi.off_kv, 0, s_mi.rows + 16);
+      phase_epi_bf16<QC, false>(Tm<C>::k, 0, 0, s_mi.off_kv);
       WAIT_PHASE(acc_full[1], k);
       if (new_params) wait_layer_params();  // (the key epilogue adds no bias: it needs none of the vectors)
-      phase_epi_bf16<QC, true>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + NKB * kTM * 128, 0, s_mi.rows + 16);
+      phase_epi_bf16<QC, true>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + (C / 8) * kChunkBytes);
     }
     WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1) + 1);
-    phase_epi_bf16<QC, true>(Tm<C>::k, 0, ParOff<C>::b_q, s_mi.off_a, 0, s_mi.rows);
-    compute_sync();
+    phase_epi_bf16<QC, true>(Tm<C>::k, 0, ParOff<C>::b_q, s_mi.off_a);
+    fence_proxy_async();
+    mbar_arrive(&s_mi.a_ready);  // Q, K and V are in place
     // ---- attention inside each set ----
-    attend_blocked<C, D, NT, RPB>();
+    attend<C, D, RPB>(k);
     fence_proxy_async();
     mbar_arrive(&s_mi.a_ready);  // attention output is the A operand of the output projection
     compute_sync();              // every warp is done with K and V: their region becomes fp32 staging
     if (s_mi.mode != 0) {
       phase_stage_x<C>();
-      compute_sync();
+    } else {
+      stage_late_vectors<C>();
+      asm volatile("cp.async.wait_all;" ::: "memory");
     }
+    compute_sync();
     // ---- output projection epilogue: Z + b_o (+ x, LayerNorm) ----
     WAIT_PHASE(o_full, k);
     phase_epi_o<C, QC>();
@@ -1243,8 +1354,8 @@ __device__ __forceinline__ void compute_role(const TcArgs& a) {
       for (int c = 0; c < s_mi.n_f1; ++c) {
         WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1) + 2 + c);
         const uint32_t h_phase = (uint32_t)(k * s_mi.n_f1 + c + 1) & 1u;
-        if (s_mi.NF == 128) phase_mlp1<C, 32>(ParOff<C>::b_1 + c * 128, h_phase);
-        else phase_mlp1<C, 16>(ParOff<C>::b_1 + c * 64, h_phase);
+        if (s_mi.NF == 128) phase_mlp1<C, 32>(LateOff<C>::b_1 + c * 128, h_phase);
+        else phase_mlp1<C, 16>(LateOff<C>::b_1 + c * 64, h_phase);
       }
       gather_next(k);  // (the operand has been free since the output projection; under the first MLP-1 product it is slower)
       // ---- MLP-2 epilogue: y = LN2(x1 + M) ----
@@ -1267,25 +1378,24 @@ __device__ __forceinline__ void compute_role(const TcArgs& a) {
 // The kernel
 // ---------------------------------------------------------------------------------------------
 // VAR: 0 plain, 1 relative position bias on the logits, 2 additive positional term on the query / key inputs
-template <int C, int D, int NT, int VAR>
+template <int C, int D, int VAR>
 __global__ void __launch_bounds__(kThreads, 1) layer_tc_kernel(const __grid_constant__ TcArgs a) {
   constexpr bool RPB = VAR == 1;
   extern __shared__ unsigned char smem_raw[];
-  const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t pad = (1024u - (raw & 1023u)) & 1023u;
-  unsigned char* sm = smem_raw + pad;
+  unsigned char* sm = smem_raw;  // 1024-aligned: the static block before it fills whole kilobytes
   Misc* mi = &s_mi;
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (warp-uniform)
   const TcGeom& g = a.g;
   if (tid == 0) {  // launch constants for the phase functions
-    mi->abort_flag = 0;
+    mi->abort_flag = (smem_u32(smem_raw) & 1023u) != 0;  // (never: checked because the layouts rest on it)
     mi->exit_at = -1;
     mi->x = a.x; mi->y = a.y; mi->status = a.status;
-    mi->sm = sm; mi->sbase = raw + pad;
-    mi->off_a = g.off_a; mi->off_kv = g.off_kv; mi->off_par = g.off_par;
+    mi->sbase = smem_u32(sm);
+    mi->off_a = g.off_a; mi->off_kv = g.off_kv; mi->off_code = g.off_code;
     mi->n = a.n; mi->tau = g.tau; mi->heads = g.heads; mi->mode = g.mode; mi->NF = g.NF; mi->n_f1 = g.n_f1;
     mi->ln1 = mi->ln2 = 0;
     mi->eps = 0.f;
+    mi->b_o = mi->b_1 = mi->b_2 = nullptr;
     mi->rpb = nullptr; mi->pe = nullptr; mi->coords = a.coords;
     mi->rb_len = g.rb_len; mi->rb_sx = g.rb_sx; mi->rb_sy = g.rb_sy; mi->rb_centre = g.rb_centre;
     mi->rb_ext[0] = g.rb_ext[0]; mi->rb_ext[1] = g.rb_ext[1]; mi->rb_ext[2] = g.rb_ext[2];
@@ -1308,6 +1418,12 @@ __global__ void __launch_bounds__(kThreads, 1) layer_tc_kernel(const __grid_cons
       mbar_init(&mi->dep_ready[i], kLoadThreads);
       mbar_init(&mi->stored[i], kComputeThreads);
     }
+    for (int i = 0; i < 4; ++i) {
+      mbar_init(&mi->s_full[i], 1);
+      mbar_init(&mi->p_ready[i], kComputeThreads / 4);
+      mbar_init(&mi->ov_full[i], 1);
+      mbar_init(&mi->o_read[i], kComputeThreads / 4);
+    }
     mbar_init(&mi->o_full, 1);
     mbar_init(&mi->h_ready, kComputeThreads);
     mbar_init(&mi->h_free, 1);
@@ -1321,10 +1437,9 @@ __global__ void __launch_bounds__(kThreads, 1) layer_tc_kernel(const __grid_cons
                  "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  // rows of K / V past the end of a tile are read (and masked) by the attention: never let them hold
-  // uninitialised bit patterns
-  // (the weight ring behind it as well: key blocks that run past row 127 read a little of it)
-  for (uint32_t i = tid; i < ((uint32_t)kTM * 2 * C * 2 + kStages * (uint32_t)C * 128u) / 16; i += kThreads)
+  // keys past a tile's rows meet zero probabilities: never let K, V or the chunks behind V hold uninitialised bit
+  // patterns there (0 x NaN)
+  for (uint32_t i = tid; i < (g.off_stage - g.off_kv + kStages * (uint32_t)C * 128u) / 16; i += kThreads)
     reinterpret_cast<uint4*>(sm + g.off_kv)[i] = make_uint4(0u, 0u, 0u, 0u);
   fence_proxy_async();  // the TMA writes that follow must not be overtaken by these generic stores
   // everything above touched only this CTA's own state; from here on the kernel reads what earlier kernels in the
@@ -1335,24 +1450,24 @@ __global__ void __launch_bounds__(kThreads, 1) layer_tc_kernel(const __grid_cons
   __syncthreads();
   tc_fence_after();
   RoleCtx rc;
-  rc.sbase = raw + pad;
-  rc.tmem = mi->tmem_base;
-  rc.mode = g.mode; rc.n_f1 = g.n_f1; rc.NF = g.NF; rc.tau = g.tau; rc.n_layers = a.n_layers;
-  rc.off_a = g.off_a; rc.off_kv = g.off_kv; rc.off_stage = g.off_stage;
+  rc.sbase = smem_u32(sm);
+  rc.tmem = __shfl_sync(0xffffffffu, mi->tmem_base, 0);
+  rc.mode = g.mode; rc.n_f1 = g.n_f1; rc.NF = g.NF; rc.tau = g.tau; rc.n_layers = a.n_layers; rc.heads = g.heads;
+  rc.off_a = g.off_a; rc.off_kv = g.off_kv; rc.off_code = g.off_code; rc.off_stage = g.off_stage;
   rc.pe = VAR == 2;
 
   if (warp == kTmaWarp) {
     if ((tid & 31) == 0) producer_role<C>(a, rc);
     __syncwarp();
   } else if (warp == kMmaWarp) {
-    if ((tid & 31) == 0) mma_role<C>(rc);
+    mma_role<C, D>(rc);
     __syncwarp();
   } else if (warp == kStampWarp) {
     stamp_role(a.row_stamp);
   } else if (warp >= kLoadWarp0) {
     loader_role<C, RPB>(a);
   } else {
-    compute_role<C, D, NT, VAR>(a);
+    compute_role<C, D, VAR>(a);
   }
   // ---- teardown: everyone meets here, then the allocating warp returns the TMEM columns ----
   tc_fence_before();
@@ -1438,10 +1553,10 @@ bool cached_weight_map(dsvt_ctx* ctx, CUtensorMap* out, const void* w, int rows,
   return true;
 }
 
-template <int C, int D, int NT, int VAR>
+template <int C, int D, int VAR>
 int launch_tc_one(dsvt_ctx* ctx, const TcArgs& a, int grid, size_t smem, int inst) {
   if (!(ctx->maps->attr_done & (1u << inst))) {  // once per instantiation and context (the attribute is per device)
-    cudaError_t e = cudaFuncSetAttribute(layer_tc_kernel<C, D, NT, VAR>,
+    cudaError_t e = cudaFuncSetAttribute(layer_tc_kernel<C, D, VAR>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) { ctx->last_cuda_error = (int)e; return DSVT_ERR_CUDA; }
     ctx->maps->attr_done |= 1u << inst;
@@ -1454,7 +1569,7 @@ int launch_tc_one(dsvt_ctx* ctx, const TcArgs& a, int grid, size_t smem, int ins
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at; cfg.numAttrs = 1;
-  cudaError_t le = cudaLaunchKernelEx(&cfg, layer_tc_kernel<C, D, NT, VAR>, a);
+  cudaError_t le = cudaLaunchKernelEx(&cfg, layer_tc_kernel<C, D, VAR>, a);
   if (le != cudaSuccess) { ctx->last_cuda_error = (int)le; cudaGetLastError(); return DSVT_ERR_CUDA; }
   DSVT_LAUNCHED(ctx);
   return DSVT_OK;
@@ -1462,24 +1577,15 @@ int launch_tc_one(dsvt_ctx* ctx, const TcArgs& a, int grid, size_t smem, int ins
 
 // The position bias and the positional term are compile-time variants: a layer without them runs a kernel that
 // holds none of their code.
-template <int C, int D, int NT>
+template <int C, int D>
 int launch_tc(dsvt_ctx* ctx, const TcArgs& a, int grid, size_t smem, int inst) {
-  if (a.g.rb_len != 0) return launch_tc_one<C, D, NT, 1>(ctx, a, grid, smem, 2 * inst + 1);
+  if (a.g.rb_len != 0) return launch_tc_one<C, D, 1>(ctx, a, grid, smem, 3 * inst + 1);
   if (a.layer[0].pe) {
-    // (the variant with a positional term is built for the paper's shape only: C = 192, set size up to 48)
-    if constexpr (C == 192 && NT <= 14) return launch_tc_one<C, D, NT, 2>(ctx, a, grid, smem, 24 + inst);
+    // (the variant with a positional term is built for the paper's shape only: C = 192)
+    if constexpr (C == 192) return launch_tc_one<C, D, 2>(ctx, a, grid, smem, 3 * inst + 2);
     return DSVT_ERR_UNSUPPORTED;
   }
-  return launch_tc_one<C, D, NT, 0>(ctx, a, grid, smem, 2 * inst);
-}
-
-template <int C, int D>
-int launch_tc_nt(dsvt_ctx* ctx, const TcArgs& a, int grid, size_t smem, int inst) {
-  // NT = key blocks of 8 a 16-row block can need: the rows of every set it touches, ceil((2 tau + 14) / 8), at most
-  // the 16 blocks of a whole tile
-  if (a.g.tau <= 36) return launch_tc<C, D, 11>(ctx, a, grid, smem, 3 * inst);
-  if (a.g.tau <= 48) return launch_tc<C, D, 14>(ctx, a, grid, smem, 3 * inst + 1);
-  return launch_tc<C, D, 16>(ctx, a, grid, smem, 3 * inst + 2);
+  return launch_tc_one<C, D, 0>(ctx, a, grid, smem, 3 * inst);
 }
 
 int tc_hidden(const dsvt_fused_args& a) { return a.attention_only ? 0 : a.p.hidden; }
@@ -1544,13 +1650,13 @@ int dsvt_launch_layers_tc(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_la
     g.rb_centre = (L - 1) * g.rb_sx + (W - 1) * g.rb_sy + (H - 1);
     g.rb_ext[0] = L; g.rb_ext[1] = W; g.rb_ext[2] = H;
   }
-  const uint32_t a_bytes = kTM * C * 2;
+  const int d = C / p.heads;
   g.off_a = 0;
-  g.off_kv = a_bytes;
-  g.off_stage = g.off_kv + (uint32_t)kTM * 2 * C * 2;  // K + V (bf16) = fp32 staging = MLP hidden (<= 2C) bytes
-  g.off_par = g.off_stage + kStages * (uint32_t)C * 128u;
-  const size_t smem = (size_t)g.off_par + (size_t)(8 * C + g.hidden) * sizeof(float) + 1024;
-  if (smem + sizeof(Misc) + 16 > 227 * 1024) return DSVT_ERR_UNSUPPORTED;  // s_mi is static shared memory
+  g.off_kv = (uint32_t)kTM * C * 2;
+  g.off_code = g.off_kv + (uint32_t)kTM * 2 * C * 2;  // K + V (bf16) = fp32 staging bytes
+  g.off_stage = g.off_code + 2 * (d == 24 ? 1 : 2) * kChunkBytes;
+  const size_t smem = (size_t)g.off_stage + kStages * (size_t)C * 128;
+  if (smem + sizeof(Misc) > 227 * 1024) return DSVT_ERR_UNSUPPORTED;  // s_mi is static shared memory
   int64_t grid = 1;
   for (int l = 0; l < n_layers; ++l) {
     const dsvt_fused_args& a = layers[l];
@@ -1587,11 +1693,10 @@ int dsvt_launch_layers_tc(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_la
   if (grid > ctx->sm_count) grid = ctx->sm_count;
   if (ctx->layer_ctas > 0 && grid > ctx->layer_ctas) grid = ctx->layer_ctas;
   if (grid < 1) grid = 1;
-  const int d = C / p.heads;
-  if (C == 192) return launch_tc_nt<192, 24>(ctx, ta, (int)grid, smem, 0);
-  if (C == 128 && d == 16) return launch_tc_nt<128, 16>(ctx, ta, (int)grid, smem, 1);
-  if (C == 128) return launch_tc_nt<128, 32>(ctx, ta, (int)grid, smem, 2);
-  return launch_tc_nt<64, 16>(ctx, ta, (int)grid, smem, 3);
+  if (C == 192) return launch_tc<192, 24>(ctx, ta, (int)grid, smem, 0);
+  if (C == 128 && d == 16) return launch_tc<128, 16>(ctx, ta, (int)grid, smem, 1);
+  if (C == 128) return launch_tc<128, 32>(ctx, ta, (int)grid, smem, 2);
+  return launch_tc<64, 16>(ctx, ta, (int)grid, smem, 3);
 }
 
 int dsvt_launch_layer_tc(dsvt_ctx* ctx, const dsvt_fused_args& a) { return dsvt_launch_layers_tc(ctx, &a, 1); }
