@@ -86,44 +86,47 @@ done:
   }
 }
 
-// ================= MMA issuer (one thread) ==============================================================
+// ================= MMA issuer (one warp) ================================================================
 // Chunks of a tile: Q (A = P, region 0), K (A = X~, region 1), V (A = X~, region 0 once the scores have read Q),
-// O (A = attention output in P's place, region 1 once the scores have read K).
+// O (A = attention output in P's place, region 1 once the scores have read K).  Warp-uniform code, an elected lane
+// issues (from one divergent thread an MMA took 46 cycles and more to issue).
 template <int C>
-__device__ __noinline__ void pool_mma(uint32_t x_base, uint32_t p_base, uint32_t st_base, uint32_t tmem, int my_tiles) {
+__device__ __forceinline__ void pool_mma(uint32_t x_base, uint32_t p_base, uint32_t st_base, uint32_t tmem, int my_tiles) {
   constexpr int NKB = C / 64;
-  constexpr uint32_t STAGE_BYTES = C * 128;
+  constexpr uint32_t STAGE16 = C * 128 / 16, kRows16 = kTM * 128 / 16, SW = kDescHiSwizzled;
   volatile int* abort_flag = &s_pm.abort_flag;
-  const uint32_t idesc = umma_idesc(C);
+  const uint32_t x_lo = desc_lo_swizzled(x_base), p_lo = desc_lo_swizzled(p_base), w_lo = desc_lo_swizzled(st_base);
   int stage = 0;
-  uint32_t phase = 0;
-  uint32_t uses[2] = {0u, 0u};
+  uint32_t phase = 0, uses = 0;  // uses of either accumulator: two per tile
   for (int t = 0; t < my_tiles; ++t) {
     for (int c = 0; c < 4; ++c) {
       const uint32_t bar = (c == 0 || c == 2) ? 0u : 1u;
       if (c == 0 && !mbar_wait(&s_pm.ab_ready, (uint32_t)t & 1u, abort_flag)) goto done;
       if (c == 3 && !mbar_wait(&s_pm.ao_ready, (uint32_t)t & 1u, abort_flag)) goto done;
-      if (!mbar_wait(&s_pm.acc_free[bar], (uses[bar] & 1u) ^ 1u, abort_flag)) goto done;
-      ++uses[bar];
+      uses = 2u * (uint32_t)t + (uint32_t)(c >> 1);
+      if (!mbar_wait(&s_pm.acc_free[bar], (uses & 1u) ^ 1u, abort_flag)) goto done;
       tc_fence_after();
-      const uint32_t abase = (c == 0 || c == 3) ? p_base : x_base;
-      const uint32_t d_tmem = tmem + bar * C;
+      const uint32_t a_lo = (c == 0 || c == 3) ? p_lo : x_lo, d_tmem = tmem + bar * C;
       for (int kb = 0; kb < NKB; ++kb) {
         if (!mbar_wait(&s_pm.full[stage], phase, abort_flag)) goto done;
         tc_fence_after();
-        const uint32_t sa = abase + kb * (kTM * 128), sb = st_base + stage * STAGE_BYTES;
+        if (elect_one()) {
 #pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4)
-          umma_bf16(d_tmem, umma_desc(sa + k4 * 32), umma_desc(sb + k4 * 32), idesc, (kb | k4) != 0 ? 1u : 0u);
-        umma_commit(&s_pm.empty[stage]);
+          for (int k4 = 0; k4 < 4; ++k4)
+            umma_ss(d_tmem, a_lo + kb * kRows16 + 2 * k4, SW, w_lo + stage * STAGE16 + 2 * k4, SW, umma_idesc(C),
+                    (kb | k4) != 0 ? 1u : 0u);
+          umma_commit(&s_pm.empty[stage]);
+          if (kb == NKB - 1) umma_commit(&s_pm.acc_full[bar]);
+        }
+        __syncwarp();
         if (++stage == kStages) { stage = 0; phase ^= 1u; }
       }
-      umma_commit(&s_pm.acc_full[bar]);
     }
   }
 done:
   if (*abort_flag) {  // the MMAs already issued must have completed before the TMEM columns are returned
-    umma_commit(&s_pm.drain);
+    if (elect_one()) umma_commit(&s_pm.drain);
+    __syncwarp();
     for (int it = 0; it < kMaxPolls && !mbar_try(&s_pm.drain, 0u); ++it) {}
   }
 }
@@ -144,7 +147,7 @@ struct PoolTcArgs {
 // Work item = (region, 16-byte channel chunk): the chunk of every slot row of the region (all loads of a thread's
 // items in flight together), the channel-wise maximum, X~ rows and P rows as bf16.
 template <int C, int NS>
-__device__ __forceinline__ void pool_gather_ns(const PoolTcArgs& a, unsigned char* xs, unsigned char* ps, int nr) {
+__device__ __forceinline__ void pool_gather_ns(const PoolTcArgs& a, uint32_t xs, uint32_t ps, int nr) {
   constexpr int C4 = C / 4, TR = kTM / NS, ITEMS = TR * C4;
   constexpr int PER = (ITEMS + kComputeThreads - 1) / kComputeThreads;  // items per thread
   constexpr int GROUP = NS <= 4 ? NS : 4;                               // slot rows loaded together
@@ -182,7 +185,7 @@ __device__ __forceinline__ void pool_gather_ns(const PoolTcArgs& a, unsigned cha
           const float4 e = __ldg(reinterpret_cast<const float4*>(a.slot_pe + (size_t)s * C) + c4);
           g.x += e.x; g.y += e.y; g.z += e.z; g.w += e.w;
         }
-        *reinterpret_cast<uint2*>(xs + swz(r, c4 >> 1) + (c4 & 1) * 8) = make_uint2(pack_bf16(g.x, g.y), pack_bf16(g.z, g.w));
+        sts2(xs + swz(r, c4 >> 1) + (c4 & 1) * 8, make_uint2(pack_bf16(g.x, g.y), pack_bf16(g.z, g.w)));
       }
     }
   }
@@ -194,12 +197,12 @@ __device__ __forceinline__ void pool_gather_ns(const PoolTcArgs& a, unsigned cha
     const uint2 p2 = make_uint2(pack_bf16(m4.x, m4.y), pack_bf16(m4.z, m4.w));
 #pragma unroll
     for (int s = 0; s < NS; ++s)  // the region's maximum, once per slot row
-      *reinterpret_cast<uint2*>(ps + swz(ri * NS + s, c4 >> 1) + (c4 & 1) * 8) = p2;
+      sts2(ps + swz(ri * NS + s, c4 >> 1) + (c4 & 1) * 8, p2);
   }
 }
 
 template <int C>
-__device__ __forceinline__ void pool_gather(const PoolTcArgs& a, unsigned char* xs, unsigned char* ps, int nr, int ns) {
+__device__ __forceinline__ void pool_gather(const PoolTcArgs& a, uint32_t xs, uint32_t ps, int nr, int ns) {
   switch (ns) {
     case 1: pool_gather_ns<C, 1>(a, xs, ps, nr); break;
     case 2: pool_gather_ns<C, 2>(a, xs, ps, nr); break;
@@ -223,11 +226,11 @@ __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const __grid_const
   const uint32_t pad = (1024u - (raw & 1023u)) & 1023u;
   unsigned char* sm = pool_tc_smem + pad;
   const uint32_t sbase = raw + pad;
-  unsigned char* xs = sm;                       // X~ (bf16 operand); later the fp32 output staging
-  unsigned char* ps = sm + TILE_BYTES;          // P (bf16 operand); later the attention output
+  // X~ (bf16 operand), later the fp32 output staging; P (bf16 operand), later the attention output
   const uint32_t st_base = sbase + 2 * TILE_BYTES;
+  const uint32_t xs_s = sbase, ps_s = sbase + TILE_BYTES, par_s = st_base + kStages * C * 128;
   float* par = reinterpret_cast<float*>(sm + 2 * TILE_BYTES + kStages * C * 128);  // b_q, b_k, b_v, b_o
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int ns = a.nslots, TR = kTM / ns;
   volatile int* abort_flag = &s_pm.abort_flag;
   if (tid == 0) {
@@ -265,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const __grid_const
     if (lane == 0) pool_producer<C>(maps, st_base, my_tiles);
     __syncwarp();
   } else if (warp == kMmaWarp) {
-    if (lane == 0) pool_mma<C>(sbase, sbase + TILE_BYTES, st_base, tmem, my_tiles);
+    pool_mma<C>(sbase, sbase + TILE_BYTES, st_base, __shfl_sync(0xffffffffu, tmem, 0), my_tiles);
     __syncwarp();
   } else {
     const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
@@ -298,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const __grid_const
       compute_sync();
       v_next = row_voxel(key_next);
       key_next = row_key(tl + 2);
-      pool_gather<C>(a, xs, ps, nr, ns);
+      pool_gather<C>(a, xs_s, ps_s, nr, ns);
       fence_proxy_async();
       mbar_arrive(&s_pm.ab_ready);
       // ---- scores: q . k per head of this quarter, softmax over the region's slots (neighbouring lanes) ----
@@ -321,7 +324,7 @@ __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const __grid_const
 #pragma unroll
         for (int c = 0; c < D; c += 4) {
           const int cc = hq * QC + j * D + c;
-          const float4 bq = *reinterpret_cast<const float4*>(par + cc), bk = *reinterpret_cast<const float4*>(par + C + cc);
+          const float4 bq = lds4(par_s + 4u * (uint32_t)cc), bk = lds4(par_s + 4u * (uint32_t)(C + cc));
           acc = fmaf(qr[j * D + c] + bq.x, k[c] + bk.x, acc);
           acc = fmaf(qr[j * D + c + 1] + bq.y, k[c + 1] + bk.y, acc);
           acc = fmaf(qr[j * D + c + 2] + bq.z, k[c + 2] + bk.z, acc);
@@ -346,22 +349,48 @@ __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const __grid_const
         tc_fence_before();
         mbar_arrive(&s_pm.acc_free[0]);
 #pragma unroll
-        for (int c4 = 0; c4 < QC; c4 += 4) {
-          const float4 bv = *reinterpret_cast<const float4*>(par + 2 * C + hq * QC + c4);
-          const float b4[4] = {bv.x, bv.y, bv.z, bv.w};
+        for (int c = 0; c < QC; ++c) v[c] *= p[c / D];
+        // Only one row of a region is needed.  Two halvings: lanes whose bit 0 (then bit 1) of the slot differs exchange
+        // half (then a quarter) of the columns, and each goes on with the sum of the part it keeps; further slots are
+        // summed over those columns by whole exchanges.  QC (3/4 of QC) shuffles for 4 (2) slots, 2 QC for a butterfly.
+        int c0 = 0;  // first column this lane keeps
+        if (ns >= 2) {
+          const bool up = lane & 1;
+          c0 = up ? QC / 2 : 0;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int cc = c4 + e;
-            float t2 = p[cc / D] * v[cc];
-            for (int o = ns >> 1; o > 0; o >>= 1) t2 += __shfl_xor_sync(0xffffffffu, t2, o);
-            v[cc] = live ? t2 + b4[e] : 0.f;  // the probabilities sum to one: + b_v once
+          for (int c = 0; c < QC / 2; ++c) {
+            const float got = __shfl_xor_sync(0xffffffffu, up ? v[c] : v[c + QC / 2], 1);
+            v[c] = (up ? v[c + QC / 2] : v[c]) + got;
           }
         }
+        if (ns >= 4) {
+          const bool up = lane & 2;
+          c0 += up ? QC / 4 : 0;
 #pragma unroll
-        for (int q8 = 0; q8 < QC / 8; ++q8)
-          *reinterpret_cast<uint4*>(ps + swz(row, ((hq * QC) >> 3) + q8)) =
-              make_uint4(pack_bf16(v[8 * q8], v[8 * q8 + 1]), pack_bf16(v[8 * q8 + 2], v[8 * q8 + 3]),
-                         pack_bf16(v[8 * q8 + 4], v[8 * q8 + 5]), pack_bf16(v[8 * q8 + 6], v[8 * q8 + 7]));
+          for (int c = 0; c < QC / 4; ++c) {
+            const float got = __shfl_xor_sync(0xffffffffu, up ? v[c] : v[c + QC / 4], 2);
+            v[c] = (up ? v[c + QC / 4] : v[c]) + got;
+          }
+          for (int o = 4; o < ns; o <<= 1) {
+#pragma unroll
+            for (int c = 0; c < QC / 4; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+          }
+        }
+        // the region's result goes to its slot-0 row (the probabilities sum to one: + b_v once), from the lanes that hold
+        // its parts: 4 columns at a time
+        const int keep = ns >= 4 ? QC / 4 : ns == 2 ? QC / 2 : QC, r0 = row - s_of;
+        if (s_of < 4) {
+#pragma unroll
+          for (int c4 = 0; c4 < QC; c4 += 4) {
+            if (c4 < keep) {
+              const int cc = hq * QC + c0 + c4;
+              const float4 bv = lds4(par_s + 4u * (uint32_t)(2 * C + cc));
+              const uint2 o2 = live ? make_uint2(pack_bf16(v[c4] + bv.x, v[c4 + 1] + bv.y), pack_bf16(v[c4 + 2] + bv.z, v[c4 + 3] + bv.w))
+                                    : make_uint2(0u, 0u);
+              sts2(ps_s + swz(r0, cc >> 3) + 2u * (uint32_t)(cc & 4), o2);
+            }
+          }
+        }
       }
       fence_proxy_async();
       mbar_arrive(&s_pm.ao_ready);
@@ -376,17 +405,16 @@ __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const __grid_const
         if (live && s_of == 0) {  // (X~ is dead: the value projection has been read)
 #pragma unroll
           for (int q4 = 0; q4 < QC / 4; ++q4) {
-            const float4 bo = *reinterpret_cast<const float4*>(par + 3 * C + hq * QC + 4 * q4);
-            *reinterpret_cast<float4*>(xs + out_off<C>(ri, hq * (QC / 4) + q4)) =
-                make_float4(o[4 * q4] + bo.x, o[4 * q4 + 1] + bo.y, o[4 * q4 + 2] + bo.z, o[4 * q4 + 3] + bo.w);
+            const float4 bo = lds4(par_s + 4u * (uint32_t)(3 * C + hq * QC + 4 * q4));
+            sts4(xs_s + out_off<C>(ri, hq * (QC / 4) + q4),
+                 make_float4(o[4 * q4] + bo.x, o[4 * q4 + 1] + bo.y, o[4 * q4 + 2] + bo.z, o[4 * q4 + 3] + bo.w));
           }
         }
       }
       compute_sync();
       for (int r = warp; r < nr; r += kComputeWarps)
         for (int c4 = lane; c4 < C / 4; c4 += 32)
-          reinterpret_cast<float4*>(a.out_feats + (size_t)(r_lo + r) * C)[c4] =
-              *reinterpret_cast<const float4*>(xs + out_off<C>(r, c4));
+          reinterpret_cast<float4*>(a.out_feats + (size_t)(r_lo + r) * C)[c4] = lds4(xs_s + out_off<C>(r, c4));
     }
     if (!ok || *abort_flag) {
       if (tid == 0) atomicOr(a.status, DSVT_STATUS_TIMEOUT);
