@@ -219,18 +219,28 @@ __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(const uint3
 }
 
 // ---- per-window scans (Eq. 2) ------------------------------------------------------------------
+// Where the sort keys of the tile plan lie in a row-offset buffer (one per set, until the plan's order takes their place).
+__device__ __forceinline__ int32_t* plan_keys(int32_t* rowoff, int32_t cap_sets) { return rowoff + 2 * (size_t)cap_sets + 3; }
+
 // Single block.  win_start = exclusive scan of N_w; win_setoff = exclusive scan of S_w = ceil(N_w / tau).
+// rowoff0 / rowoff1 (or NULL): the sets' row offsets, from the values the scan has in registers; set j of a window of N
+// voxels in S sets starts at rank floor(j N / S) (proof of Theorem A.2), and beside those of the first buffer the rows
+// of the window's largest set (plan_keys).  ITEMS: windows per thread and round (two while that covers all windows in
+// one round, so that the block's threads share the work; they are consecutive, so the loads of a thread are too).
+template <int ITEMS>
 __device__ __forceinline__ void window_scan_body(const int32_t* __restrict__ win_count, int32_t num_windows,
                                                  int32_t tau, int32_t* win_start, int32_t* win_setoff, int32_t cap_sets,
-                                                 int32_t* num_sets0, int32_t* num_sets1, int32_t* status) {
+                                                 int32_t* num_sets0, int32_t* num_sets1, int32_t* status,
+                                                 int32_t* rowoff0 = nullptr, int32_t* rowoff1 = nullptr,
+                                                 int32_t* count_out = nullptr) {
   __shared__ int warp_tot[33];
   int carry_n = 0, carry_s = 0;
-  for (int base = 0; base < num_windows; base += kScanTile) {
-    int cn[kScanItems], cs[kScanItems];
+  for (int base = 0; base < num_windows; base += kScanThreads * ITEMS) {
+    int cn[ITEMS], cs[ITEMS];
     int sn = 0, ss = 0;
-    const int i0 = base + threadIdx.x * kScanItems;
+    const int i0 = base + threadIdx.x * ITEMS;
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
+    for (int k = 0; k < ITEMS; ++k) {
       const int N = (i0 + k < num_windows) ? win_count[i0 + k] : 0;
       cn[k] = N;
       cs[k] = N / tau + ((N % tau) > 0 ? 1 : 0);  // Eq. 2
@@ -241,10 +251,23 @@ __device__ __forceinline__ void window_scan_body(const int32_t* __restrict__ win
     int pn = carry_n + block_excl_scan(sn, warp_tot, &tn);
     int ps = carry_s + block_excl_scan(ss, warp_tot, &ts);
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
+    for (int k = 0; k < ITEMS; ++k) {
       if (i0 + k < num_windows) {
         win_start[i0 + k] = pn;
         win_setoff[i0 + k] = ps;
+        if (count_out) count_out[i0 + k] = cn[k];
+        if (rowoff0 || rowoff1) {
+          const int N = cn[k], S = cs[k];
+          const bool small = (int64_t)N * S < (1ll << 31);
+          int32_t* first = rowoff0 ? rowoff0 : rowoff1;
+          const int key = S > 0 ? (N + S - 1) / S : 0;
+          for (int j = 0; j < S && ps + j < cap_sets; ++j) {
+            const int v = pn + (small ? (int)((unsigned)(j * N) / (unsigned)S) : (int)(((int64_t)j * N) / S));
+            if (rowoff0) rowoff0[ps + j] = v;
+            if (rowoff1) rowoff1[ps + j] = v;
+            plan_keys(first, cap_sets)[ps + j] = key;
+          }
+        }
       }
       pn += cn[k];
       ps += cs[k];
@@ -269,7 +292,7 @@ __global__ void __launch_bounds__(kScanThreads) window_scan_kernel(const int32_t
                                                                    int32_t* win_start, int32_t* win_setoff,
                                                                    int32_t cap_sets, int32_t* num_sets,
                                                                    int32_t* status) {
-  window_scan_body(win_count, num_windows, tau, win_start, win_setoff, cap_sets, num_sets, nullptr, status);
+  window_scan_body<kScanItems>(win_count, num_windows, tau, win_start, win_setoff, cap_sets, num_sets, nullptr, status);
 }
 
 // ---- set table fill (Eq. 3, Eq. 4's rank -> voxel id) -------------------------------------------
@@ -357,7 +380,8 @@ __host__ __device__ constexpr size_t plan_smem_bytes(int smax) {
 // Written behind the plan header: the sets in tile order (order[p]) and the rows before each position (prow[p]);
 // tile t covers positions [plan[1 + t], plan[2 + t]).  Returns the number of tiles, or 0 (nothing written) if some set
 // has no row or more than max_rows, or no candidate below `limit` tiles fits.
-struct PlanWindows {  // optional: the windows behind the sets (sets of a window are consecutive), or win_setoff = NULL
+struct PlanWindows {  // optional: the windows behind the sets (sets of a window are consecutive), or all NULL
+  const int32_t* keys;  // the rows of the largest set of each set's window; or, in the window arrays, what gives them
   const int32_t* win_setoff;
   const int32_t* win_count;
   int32_t num_windows;
@@ -371,14 +395,21 @@ __device__ int packed_plan_body(int32_t* rowoff, int32_t* rowoff_copy, int S, in
   unsigned char* ssz = reinterpret_cast<unsigned char*>(ro + (smax + 1));  // rows of srt[i]
   PackScratch* ps = reinterpret_cast<PackScratch*>(ssz + (((size_t)smax + 15) & ~(size_t)15));
   constexpr int kRowMask = 0xffffff;  // (at most smax * max_rows rows: 24 bits hold them)
-  for (int s = tid; s <= S; s += nthr) ro[s] = rowoff[s];
+  if (pw.keys && rowoff[S] <= kRowMask) {  // (see below)
+    for (int s = tid; s <= S; s += nthr) {
+      const int v = rowoff[s], key = s < S ? pw.keys[s] : 0;
+      ro[s] = v | (key >= 1 && key <= max_rows ? key << 24 : 0);
+    }
+  } else {
+    for (int s = tid; s <= S; s += nthr) ro[s] = rowoff[s];
+  }
   for (int b = tid; b < kPackBins; b += nthr) ps->hist[b] = 0;
   __syncthreads();
   // Sort key of a set: the rows of its window's largest set, so that the sets of a window (whose sizes differ by
   // at most one) stay neighbours in the sorted order and land in neighbouring tiles.  The same plan serves every
   // layer on these windows, so the voxels a tile reads were written by tiles a few numbers away in the layer
   // before, not by tiles anywhere in it.  Kept in the top byte of the set's row offset; 0 = the set's own rows.
-  if (pw.win_setoff && ro[S] <= kRowMask) {
+  if (!pw.keys && pw.win_setoff && ro[S] <= kRowMask) {
     for (int w = tid; w < pw.num_windows; w += nthr) {
       const int so = pw.win_setoff[w], cnt = pw.win_setoff[w + 1] - so;
       if (cnt <= 0 || so < 0) continue;
@@ -402,12 +433,9 @@ __device__ int packed_plan_body(int32_t* rowoff, int32_t* rowoff_copy, int S, in
   __syncthreads();
   const int per_warp = (S + nwarp - 1) / nwarp;
   const int w0 = min(warp * per_warp, S), w1 = min(w0 + per_warp, S);
-  for (int b0 = w0; b0 < w1; b0 += 32) {
-    const int s = b0 + lane;
-    const int c = s < w1 ? key_of(s) : 0;  // the bin
-    const unsigned same = __match_any_sync(0xffffffffu, c);
-    if (c && lane == __ffs(same) - 1) ps->whist[warp][c] = (unsigned short)(ps->whist[warp][c] + __popc(same));
-    __syncwarp();
+  for (int s = w0 + lane; s < w1; s += 32) {  // (two 16-bit counts to a word)
+    const int c = key_of(s);  // the bin
+    if (c) atomicAdd(reinterpret_cast<unsigned*>(&ps->whist[warp][c & ~1]), 1u << (16 * (c & 1)));
   }
   __syncthreads();
   if (tid >= 1 && tid <= max_rows) {  // bin tid: the warps' counts -> exclusive prefixes, and the bin's size
@@ -698,24 +726,15 @@ __global__ void __launch_bounds__(kScanThreads) bm_scan_kernel(const int32_t* __
                                                                int32_t* win_setoff, int32_t cap_sets,
                                                                int32_t* num_sets0, int32_t* num_sets1, BmJob job,
                                                                int32_t wpw, int32_t* rowoff0, int32_t* rowoff1,
-                                                               int32_t* status) {
+                                                               int32_t* count_out, int32_t* status) {
   pdl_enter();
   if (blockIdx.x == 0) {
-    window_scan_body(win_count, num_windows, tau, win_start, win_setoff, cap_sets, num_sets0, num_sets1, status);
+    if (num_windows <= 2 * kScanThreads)
+      window_scan_body<2>(win_count, num_windows, tau, win_start, win_setoff, cap_sets, num_sets0, num_sets1, status, rowoff0, rowoff1, count_out);
+    else
+      window_scan_body<kScanItems>(win_count, num_windows, tau, win_start, win_setoff, cap_sets, num_sets0, num_sets1, status, rowoff0, rowoff1, count_out);
     if (!rowoff0 && !rowoff1) return;
     __syncthreads();  // the scans are visible to the whole block
-    // row offsets: set j of a window of N voxels in S sets starts at rank floor(j N / S) (proof of Theorem A.2);
-    // they depend on the windows only, so both axes get the same ones
-    for (int w = threadIdx.x; w < num_windows; w += kScanThreads) {
-      const int N = win_count[w];
-      if (N == 0) continue;
-      const int so = win_setoff[w], S = win_setoff[w + 1] - so, start = win_start[w];
-      for (int j = 0; j < S && so + j < cap_sets; ++j) {
-        const int v = start + (int)(((int64_t)j * N) / S);
-        if (rowoff0) rowoff0[so + j] = v;
-        if (rowoff1) rowoff1[so + j] = v;
-      }
-    }
     if (threadIdx.x == 0) {
       const int S_all = min(win_setoff[num_windows], cap_sets);
       // (with more sets than the caller's capacity the last kept set ends where the first dropped one starts)
@@ -775,7 +794,7 @@ __global__ void __launch_bounds__(kScanThreads) bm_place_fill_kernel(int32_t n_m
   if (blockIdx.x == 0) {  // the plan (one for both axes: their row offsets are the same)
     int32_t* r0 = out.rowoff[0] ? out.rowoff[0] : out.rowoff[1];
     int32_t* r1 = out.rowoff[0] ? out.rowoff[1] : nullptr;
-    const PlanWindows pw{win_setoff, win_count, num_windows};
+    const PlanWindows pw{r0 ? plan_keys(r0, cap_sets) : nullptr, nullptr, nullptr, 0};
     if (r0) tile_plan_body(r0, r1, min(*num_sets, cap_sets), cap_sets, smax, 128, pw, plan_smem, warp_tot);
     return;
   }
@@ -801,7 +820,15 @@ __global__ void __launch_bounds__(kScanThreads) bm_place_fill_kernel(int32_t n_m
       const uint64_t N = (uint64_t)win_count[win];
       const int so = win_setoff[win];
       const uint64_t St = (uint64_t)(win_setoff[win + 1] - so) * (uint64_t)tau;
-      const uint64_t m_lo = ((uint64_t)r * St + N - 1) / N, m_hi = ((uint64_t)(r + 1) * St + N - 1) / N;
+      uint64_t m_lo, m_hi;
+      if ((uint64_t)(r + 1) * St + N <= 0xffffffffull) {  // (windows of up to some 60,000 voxels)
+        const uint32_t N32 = (uint32_t)N, a32 = (uint32_t)r * (uint32_t)St + N32 - 1;
+        m_lo = a32 / N32;
+        m_hi = (a32 + (uint32_t)St) / N32;
+      } else {
+        m_lo = ((uint64_t)r * St + N - 1) / N;
+        m_hi = ((uint64_t)(r + 1) * St + N - 1) / N;
+      }
       const int64_t room = ((int64_t)cap_sets - so) * tau;  // slots of this window that fit the caller's table
       int32_t* dst = out.table[a] + (size_t)so * tau;
       for (uint64_t m = m_lo; m < m_hi && (int64_t)m < room; ++m) dst[m] = i;
@@ -883,7 +910,7 @@ static int launch_tile_plans(dsvt_ctx* ctx, const int32_t* num_sets, int32_t cap
 }
 
 int dsvt_launch_tile_plan(dsvt_ctx* ctx, const int32_t* num_sets, int32_t cap_sets, int32_t* set_rowoff) {
-  return launch_tile_plans(ctx, num_sets, cap_sets, set_rowoff, nullptr, PlanWindows{nullptr, nullptr, 0});
+  return launch_tile_plans(ctx, num_sets, cap_sets, set_rowoff, nullptr, PlanWindows{nullptr, nullptr, nullptr, 0});
 }
 
 static int key_bits_for(uint64_t max_key) {
@@ -988,7 +1015,7 @@ int partition_sorted(dsvt_ctx* ctx, const PartCall& pc, const PartOut& o) {
     }
     if (o.set_rowoff && s_bound > 0) {
       int rc = launch_tile_plans(ctx, o.num_sets, cap_sets, o.set_rowoff, nullptr,
-                                 PlanWindows{ctx->win_setoff, ctx->win_count, nw});
+                                 PlanWindows{nullptr, ctx->win_setoff, ctx->win_count, nw});
       if (rc != DSVT_OK) return rc;
     }
     if (o.perm)
@@ -1035,10 +1062,13 @@ int partition_bitmap(dsvt_ctx* ctx, const PartCall& pc, int32_t wpw, int naxes, 
   if (rank_blocks > 2 * (int64_t)ctx->sm_count) rank_blocks = 2 * (int64_t)ctx->sm_count;
   int32_t* r0 = o[0].set_rowoff;
   int32_t* r1 = naxes > 1 ? o[1].set_rowoff : nullptr;
+  // the caller's window arrays, where there are any, are written in the first place
+  int32_t* win_start = pc.win_start ? pc.win_start : ctx->win_start;
+  int32_t* win_setoff = pc.win_setoff ? pc.win_setoff : ctx->win_setoff;
   DSVT_CUDA_TRY(ctx, launch_pdl(bm_scan_kernel, dim3((unsigned)(1 + rank_blocks)), dim3(kScanThreads), 0, st,
-                                (const int32_t*)counts, nw, pc.set_size, ctx->win_start, ctx->win_setoff, pc.cap_sets,
+                                (const int32_t*)counts, nw, pc.set_size, win_start, win_setoff, pc.cap_sets,
                                 o[0].num_sets, naxes > 1 ? o[1].num_sets : (int32_t*)nullptr, job, wpw, r0, r1,
-                                ctx->status));
+                                pc.win_count, ctx->status));
   DSVT_LAUNCHED(ctx);
   // plan capacity: no more sets than floor(n / tau) + non-empty windows
   const int64_t s_bound = sets_bound(pc);
@@ -1058,11 +1088,11 @@ int partition_bitmap(dsvt_ctx* ctx, const PartCall& pc, int32_t wpw, int naxes, 
   }
   const unsigned fill_blocks = (unsigned)dsvt_ceil_div(n, kScanThreads);
   DSVT_CUDA_TRY(ctx, launch_pdl(bm_place_fill_kernel, dim3(fill_blocks + 1), dim3(kScanThreads), smem, st, n, pc.n_dev, job, wpw,
-                                (const int32_t*)ctx->bm_dup, (const int32_t*)counts, (const int32_t*)ctx->win_start,
-                                (const int32_t*)ctx->win_setoff, pc.set_size, pc.cap_sets,
+                                (const int32_t*)ctx->bm_dup, (const int32_t*)counts, (const int32_t*)win_start,
+                                (const int32_t*)win_setoff, pc.set_size, pc.cap_sets,
                                 (const int32_t*)o[0].num_sets, fo, smax, nw));
   DSVT_LAUNCHED(ctx);
-  return copy_window_arrays(ctx, pc, counts);
+  return DSVT_OK;
 }
 
 }  // namespace
