@@ -1022,21 +1022,26 @@ __device__ __forceinline__ void stage_late_vectors() {
 // x rows (fp32) for the first residual: asynchronous 16-byte copies global -> shared staging.
 template <int C>
 __device__ __forceinline__ void phase_stage_x() {
-  constexpr int C4 = C / 4;
+  constexpr int C4 = C / 4, RU = C4 % 32 == 0 ? 1 : 2, IU = RU * C4 / 32;  // as in phase_gather
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float* __restrict__ x = s_mi.x;
   const uint32_t stage = s_mi.sbase + s_mi.off_kv;
   const int rows = s_mi.rows;
   const int* rowvox = s_mi.rowvox[s_mi.buf];
-  for (int r = warp; r < rows; r += kComputeWarps) {
-    const int v = rowvox[r];
-    for (int c4 = lane; c4 < C4; c4 += 32) {
-      const uint32_t off = stage_off<C>(r, c4);
-      if (v >= 0)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage + off),
-                     "l"(reinterpret_cast<const float4*>(x + (size_t)v * C) + c4) : "memory");
-      else
-        sts4(stage + off, make_float4(0.f, 0.f, 0.f, 0.f));
+#pragma unroll
+  for (int u = 0; u < kTM / (RU * kComputeWarps); ++u) {
+#pragma unroll
+    for (int i = 0; i < IU; ++i) {
+      const int e = lane + 32 * i, r = RU * (warp + u * kComputeWarps) + e / C4, c4 = e % C4;
+      if (r < rows) {
+        const int v = rowvox[r];
+        const uint32_t dst = stage + stage_off<C>(r, c4);
+        if (v >= 0)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
+                       "l"(reinterpret_cast<const float4*>(x + (size_t)v * C) + c4) : "memory");
+        else
+          sts4(dst, make_float4(0.f, 0.f, 0.f, 0.f));
+      }
     }
   }
   stage_late_vectors<C>();
@@ -1046,17 +1051,26 @@ __device__ __forceinline__ void phase_stage_x() {
 // fp32 rows staged in shared memory -> coalesced global rows.
 template <int C>
 __device__ __forceinline__ void phase_store_rows() {
-  constexpr int C4 = C / 4;
+  constexpr int C4 = C / 4, RU = C4 % 32 == 0 ? 1 : 2, IU = RU * C4 / 32;  // as in phase_gather
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* __restrict__ y = s_mi.y;
   const uint32_t stage = s_mi.sbase + s_mi.off_kv;
   const int rows = s_mi.rows;
   const int* rowvox = s_mi.rowvox[s_mi.buf];
-  for (int r = warp; r < rows; r += kComputeWarps) {
-    const int v = rowvox[r];
-    if (v < 0) continue;
-    for (int c4 = lane; c4 < C4; c4 += 32)
-      reinterpret_cast<float4*>(y + (size_t)v * C)[c4] = lds4(stage + stage_off<C>(r, c4));
+#pragma unroll
+  for (int u = 0; u < kTM / (RU * kComputeWarps); ++u) {
+    float4 f[IU];
+#pragma unroll
+    for (int i = 0; i < IU; ++i) {
+      const int e = lane + 32 * i, r = RU * (warp + u * kComputeWarps) + e / C4, c4 = e % C4;
+      f[i] = lds4(stage + stage_off<C>(r, c4));
+    }
+#pragma unroll
+    for (int i = 0; i < IU; ++i) {
+      const int e = lane + 32 * i, r = RU * (warp + u * kComputeWarps) + e / C4, c4 = e % C4;
+      const int v = r < rows ? rowvox[r] : -1;
+      if (v >= 0) reinterpret_cast<float4*>(y + (size_t)v * C)[c4] = f[i];
+    }
   }
 }
 
