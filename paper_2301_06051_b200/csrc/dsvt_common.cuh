@@ -96,6 +96,8 @@ static inline int64_t dsvt_ceil_div(int64_t a, int64_t b) { return (a + b - 1) /
 // ---- launchers implemented in the .cu files (all enqueue on ctx->stream) ----
 // Exclusive scan; out has count + 1 entries (out[count] = total).  in == out is allowed.
 int dsvt_launch_scan_i32(dsvt_ctx* ctx, const int32_t* in, int32_t* out, int64_t count, int32_t* total_out);
+// The same over the popcounts of bitmap words (16-byte aligned).
+int dsvt_launch_popc_scan(dsvt_ctx* ctx, const uint32_t* words, int32_t* out, int64_t count);
 int dsvt_launch_sort_pairs(dsvt_ctx* ctx, int32_t n, int key_bits, int* final_buf);
 int dsvt_launch_rowoff_from_table(dsvt_ctx* ctx, const int32_t* table, int32_t cap_sets, const int32_t* num_sets,
                                   int32_t set_size, int32_t* rowoff);

@@ -78,7 +78,38 @@ __global__ void __launch_bounds__(kScanThreads) scan_loop_kernel(const int32_t* 
   }
 }
 
+// Exclusive scan of the words' popcounts in one launch: a block sums the words before its own by reading them again,
+// which for the few blocks a bitmap takes (8192 words each) costs less than the two further launches of a scan with
+// block sums.  words is 16-byte aligned; out has count + 1 entries.
+__global__ void __launch_bounds__(kScanThreads) popc_scan_kernel(const uint32_t* __restrict__ words, int32_t* out, int64_t count) {
+  __shared__ int warp_tot[33];
+  pdl_enter();
+  const int64_t first = (int64_t)blockIdx.x * kScanTile;
+  int before = 0;
+  for (int64_t i = 4 * (int64_t)threadIdx.x; i < first; i += 4 * kScanThreads) {
+    const uint4 w = *reinterpret_cast<const uint4*>(words + i);
+    before += __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
+  }
+  int v[kScanItems], s = 0;
+  const int64_t i0 = first + (int64_t)threadIdx.x * kScanItems;
+#pragma unroll
+  for (int k = 0; k < kScanItems; ++k) {
+    v[k] = i0 + k < count ? __popc(words[i0 + k]) : 0;
+    s += v[k];
+  }
+  int carry, tot;
+  block_excl_scan(before, warp_tot, &carry);
+  int p = carry + block_excl_scan(s, warp_tot, &tot);
+#pragma unroll
+  for (int k = 0; k < kScanItems; ++k) {
+    if (i0 + k < count) out[i0 + k] = p;
+    p += v[k];
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[count] = carry + tot;
+}
+
 // Multi-block variant: (1) per-block local scan + block sums, (2) scan of block sums, (3) add.
+template <bool POPC>
 __global__ void __launch_bounds__(kScanThreads) scan_local_kernel(const int32_t* in, int32_t* out, int64_t count,
                                                                   int32_t* block_sums) {
   __shared__ int warp_tot[33];
@@ -88,7 +119,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_local_kernel(const int32_t*
   const int64_t i0 = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
-    v[k] = (i0 + k < count) ? in[i0 + k] : 0;
+    v[k] = (i0 + k < count) ? (POPC ? __popc((unsigned)in[i0 + k]) : in[i0 + k]) : 0;
     s += v[k];
   }
   int tot;
@@ -839,16 +870,12 @@ __global__ void __launch_bounds__(kScanThreads) bm_place_fill_kernel(int32_t n_m
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------------
-int dsvt_launch_scan_i32(dsvt_ctx* ctx, const int32_t* in, int32_t* out, int64_t count, int32_t* total_out) {
-  // (the scan kernels wait for their predecessor themselves: their launches may overlap its tail)
+namespace {
+template <bool POPC>
+int launch_scan_blocks(dsvt_ctx* ctx, const int32_t* in, int32_t* out, int64_t count, int32_t* total_out) {
   cudaStream_t st = ctx->stream;
-  if (count <= 8 * (int64_t)kScanTile) {
-    DSVT_CUDA_TRY(ctx, launch_pdl(scan_loop_kernel, dim3(1), dim3(kScanThreads), 0, st, in, out, count, total_out));
-    DSVT_LAUNCHED(ctx);
-    return DSVT_OK;
-  }
   const int64_t nblocks = dsvt_ceil_div(count, kScanTile);
-  DSVT_CUDA_TRY(ctx, launch_pdl(scan_local_kernel, dim3((unsigned)nblocks), dim3(kScanThreads), 0, st, in, out, count,
+  DSVT_CUDA_TRY(ctx, launch_pdl(scan_local_kernel<POPC>, dim3((unsigned)nblocks), dim3(kScanThreads), 0, st, in, out, count,
                                 ctx->scan_tmp));
   DSVT_LAUNCHED(ctx);
   DSVT_CUDA_TRY(ctx, launch_pdl(scan_loop_kernel, dim3(1), dim3(kScanThreads), 0, st, (const int32_t*)ctx->scan_tmp,
@@ -856,6 +883,26 @@ int dsvt_launch_scan_i32(dsvt_ctx* ctx, const int32_t* in, int32_t* out, int64_t
   DSVT_LAUNCHED(ctx);
   DSVT_CUDA_TRY(ctx, launch_pdl(scan_add_kernel, dim3((unsigned)nblocks), dim3(kScanThreads), 0, st, out, count,
                                 (const int32_t*)ctx->scan_tmp, nblocks, total_out));
+  DSVT_LAUNCHED(ctx);
+  return DSVT_OK;
+}
+}  // namespace
+
+int dsvt_launch_scan_i32(dsvt_ctx* ctx, const int32_t* in, int32_t* out, int64_t count, int32_t* total_out) {
+  // (the scan kernels wait for their predecessor themselves: their launches may overlap its tail)
+  if (count <= 8 * (int64_t)kScanTile) {
+    DSVT_CUDA_TRY(ctx, launch_pdl(scan_loop_kernel, dim3(1), dim3(kScanThreads), 0, ctx->stream, in, out, count, total_out));
+    DSVT_LAUNCHED(ctx);
+    return DSVT_OK;
+  }
+  return launch_scan_blocks<false>(ctx, in, out, count, total_out);
+}
+
+int dsvt_launch_popc_scan(dsvt_ctx* ctx, const uint32_t* words, int32_t* out, int64_t count) {
+  // up to 32 blocks (8 M bits) the re-reading is at most 1 MB per block, from L2
+  const int64_t nblocks = dsvt_ceil_div(count, kScanTile);
+  if (nblocks > 32) return launch_scan_blocks<true>(ctx, reinterpret_cast<const int32_t*>(words), out, count, nullptr);
+  DSVT_CUDA_TRY(ctx, launch_pdl(popc_scan_kernel, dim3((unsigned)nblocks), dim3(kScanThreads), 0, ctx->stream, words, out, count));
   DSVT_LAUNCHED(ctx);
   return DSVT_OK;
 }
