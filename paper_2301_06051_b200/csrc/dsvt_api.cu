@@ -34,6 +34,7 @@ void carve(dsvt_ctx* c, unsigned char* base, size_t* total) {
   c->vals[1] = k.take<int32_t>(nv);
   c->hist = k.take<int32_t>(hist);
   c->scan_tmp = k.take<int32_t>(longest_scan / 8192 + 2);
+  c->popc_sums = k.take<uint64_t>(nw / DSVT_POPC_TILE + 2);
   c->win_count = k.take<int32_t>(nw + 1);
   c->win_start = k.take<int32_t>(nw + 1);
   c->win_setoff = k.take<int32_t>(nw + 1);

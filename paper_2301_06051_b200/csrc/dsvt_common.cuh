@@ -27,6 +27,7 @@ struct dsvt_ctx {
   int32_t* vals[2];     // radix sort ping-pong voxel ids   [max_voxels]
   int32_t* hist;        // per-tile digit histograms        [256 * sort tiles + 1]
   int32_t* scan_tmp;    // block sums of the generic scan
+  uint64_t* popc_sums;
   int32_t* win_count;   // [max_windows + 1]  (pooling: region occupancy flags)
   int32_t* win_start;   // [max_windows + 1]  (pooling: region rank)
   int32_t* win_setoff;  // [max_windows + 1]
@@ -96,8 +97,21 @@ static inline int64_t dsvt_ceil_div(int64_t a, int64_t b) { return (a + b - 1) /
 // ---- launchers implemented in the .cu files (all enqueue on ctx->stream) ----
 // Exclusive scan; out has count + 1 entries (out[count] = total).  in == out is allowed.
 int dsvt_launch_scan_i32(dsvt_ctx* ctx, const int32_t* in, int32_t* out, int64_t count, int32_t* total_out);
-// The same over the popcounts of bitmap words (16-byte aligned).
-int dsvt_launch_popc_scan(dsvt_ctx* ctx, const uint32_t* words, int32_t* out, int64_t count);
+constexpr int DSVT_POPC_TILE = 1024;  // words per block of the bitmap scan
+// Exclusive scans over a bitmap's words (16-byte aligned): of their popcounts, and (out_fields != NULL) of how many of their fields of
+// `field` bits (a power of two) are not empty.  Outputs have count + 1 entries, count <= max_windows + 1.
+int dsvt_launch_popc_scan(dsvt_ctx* ctx, const uint32_t* words, int32_t field, int32_t* out_bits, int32_t* out_fields,
+                          int64_t count);
+// The lowest bit of every `field`-bit field of w that has a bit set.
+__device__ __forceinline__ uint32_t dsvt_field_bits(uint32_t w, int field) {
+  uint32_t keep = 0xffffffffu;
+  if (field >= 2) { w |= w >> 1; keep = 0x55555555u; }
+  if (field >= 4) { w |= w >> 2; keep = 0x11111111u; }
+  if (field >= 8) { w |= w >> 4; keep = 0x01010101u; }
+  if (field >= 16) { w |= w >> 8; keep = 0x00010001u; }
+  if (field >= 32) { w |= w >> 16; keep = 1u; }
+  return w & keep;
+}
 int dsvt_launch_sort_pairs(dsvt_ctx* ctx, int32_t n, int key_bits, int* final_buf);
 int dsvt_launch_rowoff_from_table(dsvt_ctx* ctx, const int32_t* table, int32_t cap_sets, const int32_t* num_sets,
                                   int32_t set_size, int32_t* rowoff);
@@ -133,12 +147,14 @@ bool dsvt_cached_weight_map(dsvt_ctx* ctx, void* tensor_map, const void* w, int 
                             bool fp32 = false);
 
 // Attention-style pooling with the projections on tcgen05 (pool_tc.cu): bfloat16 weights, C / head dim as for the
-// layer kernel, a power-of-two number of slots per region (at most 32).  The region bookkeeping (cell map, region
-// keys, output count) has been done by the caller.
+// layer kernel, a power-of-two number of slots per region (at most 32).  The region bookkeeping (row list or cell map
+// and region keys, output count) has been done by the caller.
 struct dsvt_pool_tc_call {
   const float* feats;
-  const int32_t* cell_map;
-  const int32_t* region_key;
+  const int4* rows;         // voxels in (region, slot) order (see pool_rows_kernel), and how many;
+  const int32_t* num_rows;
+  const int32_t* cell_map;  // or, where empty slots are rows too (rows == NULL): (region, slot) -> voxel,
+  const int32_t* region_key;  // and the regions in order
   const int32_t* num_out;
   int32_t cap_m, n;
   const void* W[4];  // W_q, W_k, W_v, W_o

@@ -17,31 +17,33 @@ constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 
 
-__device__ __forceinline__ int warp_incl_scan(int v) {
+template <typename T>
+__device__ __forceinline__ T warp_incl_scan(T v) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    int t = __shfl_up_sync(0xffffffffu, v, o);
+    T t = __shfl_up_sync(0xffffffffu, v, o);
     if (lane >= o) v += t;
   }
   return v;
 }
 
 // Exclusive scan of one value per thread over the whole block (blockDim.x <= 1024, multiple of 32).
-// warp_tot: shared int[33].  Returns the exclusive prefix; *total = block sum.
-__device__ __forceinline__ int block_excl_scan(int v, int* warp_tot, int* total) {
+// warp_tot: shared T[33].  Returns the exclusive prefix; *total = block sum.
+template <typename T>
+__device__ __forceinline__ T block_excl_scan(T v, T* warp_tot, T* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  const int incl = warp_incl_scan(v);
+  const T incl = warp_incl_scan(v);
   if (lane == 31) warp_tot[warp] = incl;
   __syncthreads();
   if (warp == 0) {
-    int t = lane < nwarp ? warp_tot[lane] : 0;
-    int ti = warp_incl_scan(t);
+    T t = lane < nwarp ? warp_tot[lane] : 0;
+    T ti = warp_incl_scan(t);
     warp_tot[lane] = ti - t;
     if (lane == 31) warp_tot[32] = ti;
   }
   __syncthreads();
-  const int r = warp_tot[warp] + incl - v;
+  const T r = warp_tot[warp] + incl - v;
   *total = warp_tot[32];
   __syncthreads();
   return r;
@@ -78,38 +80,59 @@ __global__ void __launch_bounds__(kScanThreads) scan_loop_kernel(const int32_t* 
   }
 }
 
-// Exclusive scan of the words' popcounts in one launch: a block sums the words before its own by reading them again,
-// which for the few blocks a bitmap takes (8192 words each) costs less than the two further launches of a scan with
-// block sums.  words is 16-byte aligned; out has count + 1 entries.
-__global__ void __launch_bounds__(kScanThreads) popc_scan_kernel(const uint32_t* __restrict__ words, int32_t* out, int64_t count) {
-  __shared__ int warp_tot[33];
+// Exclusive scans over a bitmap's words of their popcounts (low half of a packed sum) and of their non-empty fields of
+// `field` bits (high half).  Two launches: block sums, then every block adds the sums before its own and scans its words.
+// Small blocks: 219,000 words (7 M cells) make 214 of them; in blocks of 8192 words the two took 22 us.
+constexpr int kPopcThreads = 256, kPopcTile = 4 * kPopcThreads;
+static_assert(kPopcTile == DSVT_POPC_TILE, "size of the block sums");
+__device__ __forceinline__ uint64_t popc_pair(uint32_t w, int field) {
+  return (uint64_t)__popc(w) | ((uint64_t)__popc(dsvt_field_bits(w, field)) << 32);
+}
+__device__ __forceinline__ void popc_load(const uint32_t* words, int64_t i0, int64_t count, int field, uint64_t (&v)[4]) {
+  uint4 w = make_uint4(0u, 0u, 0u, 0u);
+  if (i0 + 4 <= count) w = *reinterpret_cast<const uint4*>(words + i0);
+  else if (i0 < count) {
+    w.x = words[i0];
+    if (i0 + 1 < count) w.y = words[i0 + 1];
+    if (i0 + 2 < count) w.z = words[i0 + 2];
+  }
+  v[0] = popc_pair(w.x, field); v[1] = popc_pair(w.y, field); v[2] = popc_pair(w.z, field); v[3] = popc_pair(w.w, field);
+}
+__global__ void __launch_bounds__(kPopcThreads) popc_sums_kernel(const uint32_t* __restrict__ words, int field, int64_t count,
+                                                                 uint64_t* __restrict__ sums) {
+  __shared__ uint64_t warp_tot[33];
   pdl_enter();
-  const int64_t first = (int64_t)blockIdx.x * kScanTile;
-  int before = 0;
-  for (int64_t i = 4 * (int64_t)threadIdx.x; i < first; i += 4 * kScanThreads) {
-    const uint4 w = *reinterpret_cast<const uint4*>(words + i);
-    before += __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
-  }
-  int v[kScanItems], s = 0;
-  const int64_t i0 = first + (int64_t)threadIdx.x * kScanItems;
-#pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    v[k] = i0 + k < count ? __popc(words[i0 + k]) : 0;
-    s += v[k];
-  }
-  int carry, tot;
+  uint64_t v[4], tot;
+  popc_load(words, (int64_t)blockIdx.x * kPopcTile + 4 * threadIdx.x, count, field, v);
+  block_excl_scan(v[0] + v[1] + v[2] + v[3], warp_tot, &tot);
+  if (threadIdx.x == 0) sums[blockIdx.x] = tot;
+}
+__global__ void __launch_bounds__(kPopcThreads) popc_scan_kernel(const uint32_t* __restrict__ words, int field,
+                                                                 const uint64_t* __restrict__ sums, int32_t* out_bits,
+                                                                 int32_t* out_fields, int64_t count) {
+  __shared__ uint64_t warp_tot[33];
+  pdl_enter();
+  uint64_t v[4], before = 0, carry, tot;
+  const int64_t i0 = (int64_t)blockIdx.x * kPopcTile + 4 * threadIdx.x;
+  popc_load(words, i0, count, field, v);
+  for (unsigned j = threadIdx.x; j < blockIdx.x; j += kPopcThreads) before += sums[j];
   block_excl_scan(before, warp_tot, &carry);
-  int p = carry + block_excl_scan(s, warp_tot, &tot);
+  uint64_t p = carry + block_excl_scan(v[0] + v[1] + v[2] + v[3], warp_tot, &tot);
 #pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    if (i0 + k < count) out[i0 + k] = p;
+  for (int k = 0; k < 4; ++k) {
+    if (i0 + k < count) {
+      out_bits[i0 + k] = (int32_t)(uint32_t)p;
+      if (out_fields) out_fields[i0 + k] = (int32_t)(p >> 32);
+    }
     p += v[k];
   }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[count] = carry + tot;
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+    out_bits[count] = (int32_t)(uint32_t)(carry + tot);
+    if (out_fields) out_fields[count] = (int32_t)((carry + tot) >> 32);
+  }
 }
 
 // Multi-block variant: (1) per-block local scan + block sums, (2) scan of block sums, (3) add.
-template <bool POPC>
 __global__ void __launch_bounds__(kScanThreads) scan_local_kernel(const int32_t* in, int32_t* out, int64_t count,
                                                                   int32_t* block_sums) {
   __shared__ int warp_tot[33];
@@ -119,7 +142,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_local_kernel(const int32_t*
   const int64_t i0 = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
-    v[k] = (i0 + k < count) ? (POPC ? __popc((unsigned)in[i0 + k]) : in[i0 + k]) : 0;
+    v[k] = (i0 + k < count) ? in[i0 + k] : 0;
     s += v[k];
   }
   int tot;
@@ -870,12 +893,16 @@ __global__ void __launch_bounds__(kScanThreads) bm_place_fill_kernel(int32_t n_m
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------------
-namespace {
-template <bool POPC>
-int launch_scan_blocks(dsvt_ctx* ctx, const int32_t* in, int32_t* out, int64_t count, int32_t* total_out) {
+int dsvt_launch_scan_i32(dsvt_ctx* ctx, const int32_t* in, int32_t* out, int64_t count, int32_t* total_out) {
+  // (the scan kernels wait for their predecessor themselves: their launches may overlap its tail)
   cudaStream_t st = ctx->stream;
+  if (count <= 8 * (int64_t)kScanTile) {
+    DSVT_CUDA_TRY(ctx, launch_pdl(scan_loop_kernel, dim3(1), dim3(kScanThreads), 0, st, in, out, count, total_out));
+    DSVT_LAUNCHED(ctx);
+    return DSVT_OK;
+  }
   const int64_t nblocks = dsvt_ceil_div(count, kScanTile);
-  DSVT_CUDA_TRY(ctx, launch_pdl(scan_local_kernel<POPC>, dim3((unsigned)nblocks), dim3(kScanThreads), 0, st, in, out, count,
+  DSVT_CUDA_TRY(ctx, launch_pdl(scan_local_kernel, dim3((unsigned)nblocks), dim3(kScanThreads), 0, st, in, out, count,
                                 ctx->scan_tmp));
   DSVT_LAUNCHED(ctx);
   DSVT_CUDA_TRY(ctx, launch_pdl(scan_loop_kernel, dim3(1), dim3(kScanThreads), 0, st, (const int32_t*)ctx->scan_tmp,
@@ -886,23 +913,18 @@ int launch_scan_blocks(dsvt_ctx* ctx, const int32_t* in, int32_t* out, int64_t c
   DSVT_LAUNCHED(ctx);
   return DSVT_OK;
 }
-}  // namespace
 
-int dsvt_launch_scan_i32(dsvt_ctx* ctx, const int32_t* in, int32_t* out, int64_t count, int32_t* total_out) {
-  // (the scan kernels wait for their predecessor themselves: their launches may overlap its tail)
-  if (count <= 8 * (int64_t)kScanTile) {
-    DSVT_CUDA_TRY(ctx, launch_pdl(scan_loop_kernel, dim3(1), dim3(kScanThreads), 0, ctx->stream, in, out, count, total_out));
+int dsvt_launch_popc_scan(dsvt_ctx* ctx, const uint32_t* words, int32_t field, int32_t* out_bits, int32_t* out_fields,
+                          int64_t count) {
+  const int64_t nblocks = dsvt_ceil_div(count, kPopcTile);
+  uint64_t* sums = ctx->popc_sums;
+  if (nblocks > 1) {  // (a single block reads no sums)
+    DSVT_CUDA_TRY(ctx, launch_pdl(popc_sums_kernel, dim3((unsigned)nblocks), dim3(kPopcThreads), 0, ctx->stream, words, field,
+                                  count, sums));
     DSVT_LAUNCHED(ctx);
-    return DSVT_OK;
   }
-  return launch_scan_blocks<false>(ctx, in, out, count, total_out);
-}
-
-int dsvt_launch_popc_scan(dsvt_ctx* ctx, const uint32_t* words, int32_t* out, int64_t count) {
-  // up to 32 blocks (8 M bits) the re-reading is at most 1 MB per block, from L2
-  const int64_t nblocks = dsvt_ceil_div(count, kScanTile);
-  if (nblocks > 32) return launch_scan_blocks<true>(ctx, reinterpret_cast<const int32_t*>(words), out, count, nullptr);
-  DSVT_CUDA_TRY(ctx, launch_pdl(popc_scan_kernel, dim3((unsigned)nblocks), dim3(kScanThreads), 0, ctx->stream, words, out, count));
+  DSVT_CUDA_TRY(ctx, launch_pdl(popc_scan_kernel, dim3((unsigned)nblocks), dim3(kPopcThreads), 0, ctx->stream, words, field,
+                                (const uint64_t*)sums, out_bits, out_fields, count));
   DSVT_LAUNCHED(ctx);
   return DSVT_OK;
 }

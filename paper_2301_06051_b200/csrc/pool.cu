@@ -1,5 +1,6 @@
-// Attention-style 3D pooling (Eq. 6, Eq. 7): dense cell map -> region ranks -> fused
-// pad / max-pool / cross-attention kernel.  The region bookkeeping is exact integer work; the
+// Attention-style 3D pooling (Eq. 6, Eq. 7): bitmap of occupied cells -> voxels in region order -> attention kernel on
+// tcgen05; or, where that kernel does not apply, dense cell map -> region ranks -> fused pad / max-pool /
+// cross-attention kernel.  The region bookkeeping is exact integer work; the
 // attention runs on the fp32 FMA pipes with float or bfloat16 weights.
 #include <cuda.h>
 
@@ -26,10 +27,12 @@ __device__ __forceinline__ int4 clamp_coord(int4 c, const PoolGeom& g, int32_t* 
   return c;
 }
 
-// Each voxel claims its cell of the dense (region, slot) map and marks its region as non-empty.
+// Each voxel claims its cell: its bit in the bitmap of cells (CELLS), or its entry of the dense (region, slot) map and
+// its region's bit in the bitmap of non-empty regions.
+template <bool CELLS>
 __global__ void pool_mark_kernel(const int4* __restrict__ coords, int32_t n_max, const int32_t* __restrict__ n_dev,
                                  PoolGeom g, int32_t* __restrict__ cell_map,
-                                 uint32_t* __restrict__ region_bits, uint32_t* __restrict__ vox_region,
+                                 uint32_t* __restrict__ bits, uint32_t* __restrict__ vox_bit,
                                  int32_t* __restrict__ slot_of, int32_t* __restrict__ status) {
   pdl_enter();  // (lets the scan's first kernel start under this one's tail)
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -39,10 +42,13 @@ __global__ void pool_mark_kernel(const int4* __restrict__ coords, int32_t n_max,
   const int X = c.y / g.l, Y = c.z / g.w, Z = c.w / g.h;
   const int slot = ((c.y - X * g.l) * g.w + (c.z - Y * g.w)) * g.h + (c.w - Z * g.h);
   const uint32_t region = (uint32_t)(((c.x * g.GX + X) * g.GY + Y) * g.GZ + Z);
-  const int old = atomicExch(&cell_map[(size_t)region * g.nslots + slot], i);
-  if (old != -1) atomicOr(status, DSVT_STATUS_DUPLICATE_CELL);
-  atomicOr(&region_bits[region >> 5], 1u << (region & 31));
-  vox_region[i] = region;
+  bool taken;
+  const uint32_t b = CELLS ? region * g.nslots + slot : region, one = 1u << (b & 31);
+  const uint32_t old = atomicOr(&bits[b >> 5], one);
+  if (CELLS) taken = old & one;
+  else taken = atomicExch(&cell_map[(size_t)region * g.nslots + slot], i) != -1;
+  if (taken) atomicOr(status, DSVT_STATUS_DUPLICATE_CELL);
+  vox_bit[i] = b;
   if (slot_of) slot_of[i] = slot;
 }
 
@@ -69,6 +75,39 @@ __global__ void pool_finish_kernel(int32_t n_max, const int32_t* __restrict__ n_
   if (r < cap_m) {  // every member of a region writes the same values
     region_key[r] = (int32_t)region;
     uint32_t t = region;
+    const int Z = t % g.GZ; t /= g.GZ;
+    const int Y = t % g.GY; t /= g.GY;
+    const int X = t % g.GX; t /= g.GX;
+    reinterpret_cast<int4*>(out_coords)[r] = make_int4((int)t, X, Y, Z);
+  }
+}
+
+// Voxels in (region, slot) order: row -> (voxel, the region's voxels | slot << 8 | first of its region << 16, region's
+// rank), from the popcounts of the bitmap of cells; a field of nslots bits is a region.
+__global__ void pool_rows_kernel(int32_t n_max, const int32_t* __restrict__ n_dev, PoolGeom g,
+                                 const uint32_t* __restrict__ vox_cell, const uint32_t* __restrict__ cell_bits,
+                                 const int32_t* __restrict__ cell_rank, const int32_t* __restrict__ region_rank,
+                                 int32_t num_words, int32_t cap_m, int32_t* __restrict__ out_coords, int4* __restrict__ rows,
+                                 int32_t* __restrict__ region_of, int32_t* __restrict__ num_out, int32_t* __restrict__ status) {
+  pdl_enter();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) {
+    const int m = region_rank[num_words];
+    if (m > cap_m) atomicOr(status, DSVT_STATUS_TABLE_OVERFLOW);
+    *num_out = min(m, cap_m);
+  }
+  const int n = n_dev ? min(max(*n_dev, 0), n_max) : n_max;
+  if (i >= n) return;
+  const uint32_t cell = vox_cell[i], w = cell_bits[cell >> 5], b = cell & 31, b0 = b & ~(uint32_t)(g.nslots - 1);
+  const uint32_t region_bits = (w >> b0) & (0xffffffffu >> (32 - g.nslots));
+  const uint32_t below = w & ((1u << b) - 1u);
+  const int slot = (int)(b - b0), row = cell_rank[cell >> 5] + __popc(below);
+  const int r = region_rank[cell >> 5] + __popc(dsvt_field_bits(w & ((1u << b0) - 1u), g.nslots));
+  const bool first = (below >> b0) == 0;
+  rows[row] = make_int4(i, __popc(region_bits) | (slot << 8) | ((int)first << 16), r, 0);
+  if (region_of) region_of[i] = r;
+  if (first && r < cap_m) {
+    uint32_t t = cell / (uint32_t)g.nslots;
     const int Z = t % g.GZ; t /= g.GZ;
     const int Y = t % g.GY; t /= g.GY;
     const int X = t % g.GX; t /= g.GX;
@@ -622,6 +661,35 @@ extern "C" int dsvt_pool_counted(dsvt_ctx* ctx, const int32_t* coords, const flo
     return DSVT_OK;
   }
   const size_t cells = (size_t)num_regions * (size_t)nslots;
+  const unsigned vb = (unsigned)dsvt_ceil_div(n, 256);
+  uint32_t* bits = reinterpret_cast<uint32_t*>(ctx->win_count);  // at most one word per region
+  const bool tc = precision == DSVT_BF16_FP32ACC && dsvt_pool_tc_supported(C, heads, (int)nslots);
+  dsvt_pool_tc_call c;
+  c.feats = feats; c.cell_map = nullptr; c.region_key = nullptr; c.rows = nullptr; c.num_rows = nullptr; c.num_out = num_out;
+  c.cap_m = cap_m; c.n = n;
+  c.W[0] = W_q; c.W[1] = W_k; c.W[2] = W_v; c.W[3] = W_o;
+  c.b_q = b_q; c.b_k = b_k; c.b_v = b_v; c.b_o = b_o; c.slot_pe = slot_pe;
+  c.out_feats = out_feats; c.C = C; c.heads = heads; c.nslots = (int32_t)nslots; c.mask_empty = mask_empty ? 1 : 0;
+  // bfloat16 weights, a power-of-two number of slots: the projections on tcgen05, over the voxels alone, unless empty
+  // slots are keys of their own (they take part and carry a slot term).  Over all slots as rows the three poolings of the
+  // voxel stages (120,000 voxels, 4 slots, 1.9 of them occupied in the first) took 234 us more, this kernel's other
+  // changes and the dense cell map's 28 MB of clearing included; full regions take (nslots - 1) / 128 more tiles.
+  if (tc && (mask_empty || !slot_pe)) {
+    const int64_t num_words = (int64_t)((cells + 31) / 32);
+    DSVT_CUDA_TRY(ctx, cudaMemsetAsync(bits, 0, sizeof(uint32_t) * (size_t)num_words, st));
+    pool_mark_kernel<true><<<vb, 256, 0, st>>>((const int4*)coords, n, n_dev, g, nullptr, bits, ctx->keys[0], slot_of, ctx->status);
+    DSVT_LAUNCHED(ctx);
+    int rc = dsvt_launch_popc_scan(ctx, bits, (int32_t)nslots, ctx->win_start, ctx->win_setoff, num_words);
+    if (rc != DSVT_OK) return rc;
+    int4* rows = reinterpret_cast<int4*>(ctx->rowoff_a);
+    DSVT_CUDA_TRY(ctx, launch_pdl(pool_rows_kernel, dim3(vb), dim3(256), 0, st, n, n_dev, g, (const uint32_t*)ctx->keys[0],
+                                  (const uint32_t*)bits, (const int32_t*)ctx->win_start, (const int32_t*)ctx->win_setoff,
+                                  (int32_t)num_words, cap_m, out_coords, rows, region_of, num_out, ctx->status));
+    DSVT_LAUNCHED(ctx);
+    if (cap_m == 0) return DSVT_OK;
+    c.rows = rows; c.num_rows = ctx->win_start + num_words;
+    return dsvt_launch_pool_tc(ctx, c);
+  }
   if (cells > ctx->cell_map_entries) {  // grow the dense cell map (the one allocation a call may make)
     DSVT_CUDA_TRY(ctx, cudaStreamSynchronize(st));
     if (ctx->cell_map) DSVT_CUDA_TRY(ctx, cudaFree(ctx->cell_map));
@@ -634,18 +702,14 @@ extern "C" int dsvt_pool_counted(dsvt_ctx* ctx, const int32_t* coords, const flo
   // Non-empty regions as a bitmap: a region's rank is the popcount before it.  (As one flag per region the three scan
   // launches over 1.75 M flags took 31 us of a 212 us call on 120,000 voxels.)
   const int64_t num_words = (num_regions + 31) / 32;
-  uint32_t* region_bits = reinterpret_cast<uint32_t*>(ctx->win_count);
-  DSVT_CUDA_TRY(ctx, cudaMemsetAsync(region_bits, 0, sizeof(uint32_t) * (size_t)num_words, st));
-  const unsigned vb = (unsigned)dsvt_ceil_div(n, 256);
-  pool_mark_kernel<<<vb, 256, 0, st>>>((const int4*)coords, n, n_dev, g, ctx->cell_map, region_bits, ctx->keys[0], slot_of,
-                                       ctx->status);
+  DSVT_CUDA_TRY(ctx, cudaMemsetAsync(bits, 0, sizeof(uint32_t) * (size_t)num_words, st));
+  pool_mark_kernel<false><<<vb, 256, 0, st>>>((const int4*)coords, n, n_dev, g, ctx->cell_map, bits, ctx->keys[0], slot_of, ctx->status);
   DSVT_LAUNCHED(ctx);
-  int rc = dsvt_launch_popc_scan(ctx, region_bits, ctx->win_start, num_words);
+  int rc = dsvt_launch_popc_scan(ctx, bits, 1, ctx->win_start, nullptr, num_words);
   if (rc != DSVT_OK) return rc;
   DSVT_CUDA_TRY(ctx, launch_pdl(pool_finish_kernel, dim3(vb), dim3(256), 0, st, n, n_dev, g, (const uint32_t*)ctx->keys[0],
-                                (const uint32_t*)region_bits, (const int32_t*)ctx->win_start, (int32_t)num_words, cap_m, out_coords,
-                                ctx->region_key,
-                                region_of, num_out, ctx->status));
+                                (const uint32_t*)bits, (const int32_t*)ctx->win_start, (int32_t)num_words, cap_m, out_coords,
+                                ctx->region_key, region_of, num_out, ctx->status));
   DSVT_LAUNCHED(ctx);
   if (cap_m == 0) return DSVT_OK;
 
@@ -655,14 +719,8 @@ extern "C" int dsvt_pool_counted(dsvt_ctx* ctx, const int32_t* coords, const flo
   a.W_q = W_q; a.W_k = W_k; a.W_v = W_v; a.W_o = W_o;
   a.b_q = b_q; a.b_k = b_k; a.b_v = b_v; a.b_o = b_o; a.slot_pe = slot_pe;
   a.out_feats = out_feats; a.C = C; a.heads = heads; a.nslots = (int32_t)nslots; a.mask_empty = mask_empty ? 1 : 0;
-  // bfloat16 weights, a power-of-two number of slots: the projections on tcgen05
-  if (precision == DSVT_BF16_FP32ACC && dsvt_pool_tc_supported(C, heads, (int)nslots)) {
-    dsvt_pool_tc_call c;
-    c.feats = feats; c.cell_map = ctx->cell_map; c.region_key = ctx->region_key; c.num_out = num_out;
-    c.cap_m = cap_m; c.n = n;
-    c.W[0] = W_q; c.W[1] = W_k; c.W[2] = W_v; c.W[3] = W_o;
-    c.b_q = b_q; c.b_k = b_k; c.b_v = b_v; c.b_o = b_o; c.slot_pe = slot_pe;
-    c.out_feats = out_feats; c.C = C; c.heads = heads; c.nslots = (int32_t)nslots; c.mask_empty = mask_empty ? 1 : 0;
+  if (tc) {
+    c.cell_map = ctx->cell_map; c.region_key = ctx->region_key;
     return dsvt_launch_pool_tc(ctx, c);
   }
   // bfloat16 weights, C in {64, 128, 192}, head dim <= 32: other slot counts: the mma.sync kernel

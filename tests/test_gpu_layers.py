@@ -102,6 +102,27 @@ def test_chain_on_extreme_tile_plans(gpu, oracle, window, tau, n):
     check_close(y.cpu().numpy(), _oracle_chain(oracle, cfg, cfg["blocks"]), "bf16", "chain, window %s" % (window,))
 
 
+@pytest.mark.parametrize("C,heads", [(192, 8), (128, 8), (128, 4), (64, 4)])
+@pytest.mark.parametrize("window,tau,n", [
+    ((2, 2, 1), 36, 1024),   # full sets of four rows: eight per 32 rows, all that the codes of head dim 24 tell apart
+    ((3, 1, 1), 36, 1000),   # up to three rows: more than eight sets per 32 rows, sixteen at most
+    ((2, 1, 1), 36, 1024),   # full sets of two rows: sixteen per 32 rows
+    ((2, 1, 1), 36, 700),    # one or two rows: on both sides of sixteen
+    ((6, 6, 1), 36, 600),    # sets that lie across a warp's 32 rows
+    ((16, 16, 1), 96, 384),  # sets of up to 96 rows
+    ((12, 12, 1), 36, 1),    # a tile of one row
+])
+def test_attention_on_both_sides_of_the_set_codes(gpu, oracle, C, heads, window, tau, n):
+    """Warps whose keys span few enough sets leave them to the codes in the product, the others mask by comparing."""
+    cfg = di.random_case(n + C, n, (32, 32, 1), window, tau, C, heads, hidden=2 * C, layernorm=True, bf16=True)
+    ctx, tabs, ws = _setup(gpu, cfg, cfg["blocks"])
+    x = dev(cfg["feats"])
+    y = torch.empty_like(x)
+    ctx.layers(x, tabs, ws, y)
+    assert ctx.status_sync() == 0
+    check_close(y.cpu().numpy(), _oracle_chain(oracle, cfg, cfg["blocks"]), "bf16", "C=%d window=%s" % (C, window))
+
+
 def test_chain_with_other_tables_per_block(gpu, oracle):
     """Hybrid windows: the second block runs on the tables of another window cut, so a tile of its first layer
     reads rows that tiles anywhere in the previous layer wrote (the stamps are per voxel, not per window)."""

@@ -535,6 +535,64 @@ def test_pool_matches_oracle(gpu, oracle, grid, pool, batch, n, C, heads, with_p
     check_close(of[:m].cpu().numpy(), ref.feats, "bf16" if bf16 else "fp32", "pool")
 
 
+@pytest.mark.parametrize("grid", [
+    (32, 2, 1),       # 32 regions: one full word of the bitmap of non-empty regions
+    (33, 2, 1),       # one region in a second word
+    (512, 1026, 1),   # one word beyond what one block of the rank scan takes
+    (4104, 4096, 1),  # more regions than the scan takes in one launch
+])
+def test_pool_ranks_regions_across_words_and_blocks(gpu, oracle, grid):
+    rng = np.random.default_rng(grid[1])
+    n, C = 60, 16
+    coords = rng.integers(0, (1,) + grid, size=(n, 4))
+    coords[0, 1:], coords[1, 1:] = (0, 0, 0), (grid[0] - 1, grid[1] - 1, 0)  # the first and the last region
+    coords = np.unique(coords, axis=0).astype(np.int32)
+    feats = rng.standard_normal((len(coords), C), dtype=np.float32)
+    Wt = di.make_pool_weights(rng, C, 4, False, 2, False)
+    ctx = gpu.Context(len(coords), grid[0] * grid[1] // 2, C)
+    w = gpu.device_weights(Wt, gpu.FP32, ctx.device)
+    oc, of, num, reg, slot = ctx.pool(dev(coords), dev(feats), 1, grid, (1, 2, 1), w, extras=True)
+    assert ctx.status_sync() == 0
+    ref = oracle.pool(coords, feats, 1, grid, (1, 2, 1), Wt["W_q"], Wt["W_k"], Wt["W_v"], Wt["W_o"], Wt["b_q"],
+                      Wt["b_k"], Wt["b_v"], Wt["b_o"], 4, slot_pe=Wt["slot_pe"])
+    m = int(num.item())
+    assert m == ref.coords.shape[0] and np.array_equal(oc[:m].cpu().numpy(), ref.coords)
+    assert np.array_equal(reg.cpu().numpy(), ref.region_of)
+    check_close(of[:m].cpu().numpy(), ref.feats, "fp32", "pool")
+
+
+@pytest.mark.parametrize("mask_empty,with_pe", [(0, False), (1, True), (0, True)])
+@pytest.mark.parametrize("pool,grid,n,C,heads", [
+    ((1, 1, 1), (12, 12, 1), 129, 64, 4),        # regions of one voxel, one more than a tile's rows
+    ((4, 4, 1), (16, 16, 1), 256, 128, 8),       # full regions of 16: eight per 128 rows, seven per window
+    ((4, 4, 2), (32, 16, 4), 2048, 192, 8),      # full regions of 32 rows
+    ((4, 4, 2), (40, 40, 2), 1100, 128, 4),      # regions of up to 32 rows that lie across every 32-row boundary
+    ((1, 1, 4), (64, 64, 4), 1, 192, 8),         # one voxel
+    ((2, 2, 1), (64, 64, 1), 125, 192, 8),       # as many voxels as regions may start in one tile (125 of 128 rows)
+    ((2, 2, 1), (20, 20, 1), 400, 192, 8),       # full regions of 4: a window of 125 rows ends inside a region
+])
+def test_pool_tiles_of_voxels_in_region_order(gpu, oracle, pool, grid, n, C, heads, mask_empty, with_pe):
+    rng = np.random.default_rng(n + C)
+    coords = di.unique_cells(rng, n, grid, 1)
+    feats = rng.standard_normal((n, C), dtype=np.float32)
+    Wt = di.make_pool_weights(rng, C, heads, True, int(np.prod(pool)), with_pe)
+    ctx = gpu.Context(n, int(np.prod([-(-g // p) for g, p in zip(grid, pool)])), C)
+    w = gpu.device_weights(Wt, gpu.BF16_FP32ACC, ctx.device)
+    oc, of, num, reg, slot = ctx.pool(dev(coords), dev(feats), 1, grid, pool, w, mask_empty=mask_empty, extras=True)
+    assert ctx.status_sync() == 0
+    ref = oracle.pool(coords, feats, 1, grid, pool, Wt["W_q"], Wt["W_k"], Wt["W_v"], Wt["W_o"], Wt["b_q"], Wt["b_k"],
+                      Wt["b_v"], Wt["b_o"], heads, slot_pe=Wt["slot_pe"], mask_empty=mask_empty)
+    m = int(num.item())
+    assert m == ref.coords.shape[0] and np.array_equal(oc[:m].cpu().numpy(), ref.coords)
+    assert np.array_equal(reg.cpu().numpy(), ref.region_of) and np.array_equal(slot.cpu().numpy(), ref.slot_of)
+    check_close(of[:m].cpu().numpy(), ref.feats, "bf16", "pool")
+    # an output with room for the first half of the regions: those rows alone, bitwise
+    half = (m + 1) // 2
+    oc2, of2, num2, _, _ = ctx.pool(dev(coords), dev(feats), 1, grid, pool, w, mask_empty=mask_empty, cap_m=half)
+    assert ctx.status_sync() == (gpu.STATUS_TABLE_OVERFLOW if m > half else 0) and int(num2.item()) == half
+    assert torch.equal(oc2, oc[:half]) and torch.equal(of2, of[:half])
+
+
 def test_pool_flags_duplicate_cells_and_overflow(gpu):
     rng = np.random.default_rng(3)
     C = 16
