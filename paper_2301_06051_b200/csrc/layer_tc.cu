@@ -874,34 +874,35 @@ __device__ __noinline__ void stamp_role(int32_t* __restrict__ row_stamp) {
 // may use depend on what the widest phase leaves to the caller).
 
 // Gather (Eq. 4): the fp32 rows listed in buffer b -> bf16 A operand; all 128 rows are written (rows past the tile as
-// zeros).  A unit of one or two rows is a whole number of coalesced 16-byte warp loads; all of a warp's eight rows are
-// in flight at once (C = 192: 12 loads per lane; with two rounds of four rows and a quarter of the lanes idle the gather
-// cost one L2 round trip more).  ADD_PE: the current tile's rows once more, with the positional term added (the operand
-// of the key and query projections).
+// zeros).  16 lanes to a row (256 bytes), all of a thread's rows in flight at once (C = 192: 12 loads; in two rounds the
+// gather cost one L2 round trip more).  A thread's rows are 32 apart and its chunks 16, so that every address is one base
+// plus constants (in lane-linear units, with a division, a row lookup and a swizzled address per 16 bytes, gather, x staging
+// and row stores took 1 % more of a 25,000-pillar frame and 4 % more of two layers on 2000 rows).  ADD_PE: the current tile's rows once more, with the positional
+// term added (the operand of the key and query projections).
+constexpr int kUnitRows = kComputeThreads / 16;
 template <int C, int D, bool RPB, bool ADD_PE>
 __device__ __forceinline__ void phase_gather(int b, int rows) {
-  constexpr int C4 = C / 4, RU = C4 % 32 == 0 ? 1 : 2, IU = RU * C4 / 32;  // chunks per row; rows, loads per unit
-  constexpr int kFly = ADD_PE ? (RU == 2 ? 2 : 4) : 8 / RU;                // units in flight
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int P = kTM / kUnitRows, J = C / 64, kFly = ADD_PE ? P / 2 : P;  // a thread's rows, chunks, rows in flight
+  const int r0 = threadIdx.x / 16, c0 = threadIdx.x % 16;
   const float* x = ADD_PE ? s_mi.x : s_mi.next_x[b];
-  const uint32_t a_tile = s_mi.sbase + s_mi.off_a;
+  const uint32_t to = s_mi.sbase + s_mi.off_a + swz(r0, c0 >> 1) + 8 * (c0 & 1);
   const int* rowvox = s_mi.rowvox[b];
   if (!ADD_PE) write_codes<D>(b, rows);  // (the previous tile's attention is over)
-  for (int r0 = RU * warp; r0 < kTM; r0 += kFly * RU * kComputeWarps) {
-    float4 f[kFly][IU];
+#pragma unroll
+  for (int p0 = 0; p0 < P; p0 += kFly) {
+    float4 f[kFly][J];
 #pragma unroll
     for (int u = 0; u < kFly; ++u) {
+      const int r = r0 + kUnitRows * (p0 + u), v = r < rows ? rowvox[r] : -1;
 #pragma unroll
-      for (int i = 0; i < IU; ++i) {
-        const int e = lane + 32 * i, r = r0 + u * RU * kComputeWarps + e / C4, c4 = e % C4;
-        const int v = r < rows ? rowvox[r] : -1;
-        f[u][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int j = 0; j < J; ++j) {
+        f[u][j] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (v >= 0) {
           // (L2: the rows of a later layer were written during this launch, by any SM)
-          f[u][i] = __ldcg(reinterpret_cast<const float4*>(x + (size_t)v * C) + c4);
+          f[u][j] = __ldcg(reinterpret_cast<const float4*>(x + (size_t)v * C) + c0 + 16 * j);
           if (ADD_PE) {
-            const float4 p = __ldg(reinterpret_cast<const float4*>(s_mi.pe + (size_t)v * C) + c4);
-            f[u][i].x += p.x; f[u][i].y += p.y; f[u][i].z += p.z; f[u][i].w += p.w;
+            const float4 p = __ldg(reinterpret_cast<const float4*>(s_mi.pe + (size_t)v * C) + c0 + 16 * j);
+            f[u][j].x += p.x; f[u][j].y += p.y; f[u][j].z += p.z; f[u][j].w += p.w;
           }
         }
       }
@@ -909,11 +910,9 @@ __device__ __forceinline__ void phase_gather(int b, int rows) {
 #pragma unroll
     for (int u = 0; u < kFly; ++u) {
 #pragma unroll
-      for (int i = 0; i < IU; ++i) {
-        const int e = lane + 32 * i, r = r0 + u * RU * kComputeWarps + e / C4, c4 = e % C4;
-        sts2(a_tile + swz(r, c4 >> 1) + 8 * (c4 & 1),
-             make_uint2(pack_bf16(f[u][i].x, f[u][i].y), pack_bf16(f[u][i].z, f[u][i].w)));
-      }
+      for (int j = 0; j < J; ++j)
+        sts2(to + (p0 + u) * (kUnitRows * 128) + j * (kTM * 128),
+             make_uint2(pack_bf16(f[u][j].x, f[u][j].y), pack_bf16(f[u][j].z, f[u][j].w)));
     }
   }
   if (RPB && !ADD_PE) {
@@ -1022,23 +1021,23 @@ __device__ __forceinline__ void stage_late_vectors() {
 // x rows (fp32) for the first residual: asynchronous 16-byte copies global -> shared staging.
 template <int C>
 __device__ __forceinline__ void phase_stage_x() {
-  constexpr int C4 = C / 4, RU = C4 % 32 == 0 ? 1 : 2, IU = RU * C4 / 32;  // as in phase_gather
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int P = kTM / kUnitRows, J = C / 64;  // as in phase_gather
+  const int r0 = threadIdx.x / 16, c0 = threadIdx.x % 16;
   const float* __restrict__ x = s_mi.x;
-  const uint32_t stage = s_mi.sbase + s_mi.off_kv;
+  const uint32_t to = s_mi.sbase + s_mi.off_kv + stage_off<C>(r0, c0);
   const int rows = s_mi.rows;
   const int* rowvox = s_mi.rowvox[s_mi.buf];
 #pragma unroll
-  for (int u = 0; u < kTM / (RU * kComputeWarps); ++u) {
+  for (int p = 0; p < P; ++p) {
+    const int r = r0 + kUnitRows * p;
+    if (r < rows) {
+      const int v = rowvox[r];
 #pragma unroll
-    for (int i = 0; i < IU; ++i) {
-      const int e = lane + 32 * i, r = RU * (warp + u * kComputeWarps) + e / C4, c4 = e % C4;
-      if (r < rows) {
-        const int v = rowvox[r];
-        const uint32_t dst = stage + stage_off<C>(r, c4);
+      for (int j = 0; j < J; ++j) {
+        const uint32_t dst = to + p * (kUnitRows * C * 4) + j * 256;
         if (v >= 0)
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
-                       "l"(reinterpret_cast<const float4*>(x + (size_t)v * C) + c4) : "memory");
+                       "l"(reinterpret_cast<const float4*>(x + (size_t)v * C) + c0 + 16 * j) : "memory");
         else
           sts4(dst, make_float4(0.f, 0.f, 0.f, 0.f));
       }
@@ -1051,26 +1050,21 @@ __device__ __forceinline__ void phase_stage_x() {
 // fp32 rows staged in shared memory -> coalesced global rows.
 template <int C>
 __device__ __forceinline__ void phase_store_rows() {
-  constexpr int C4 = C / 4, RU = C4 % 32 == 0 ? 1 : 2, IU = RU * C4 / 32;  // as in phase_gather
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int P = kTM / kUnitRows, J = C / 64;  // as in phase_gather
+  const int r0 = threadIdx.x / 16, c0 = threadIdx.x % 16;
   float* __restrict__ y = s_mi.y;
-  const uint32_t stage = s_mi.sbase + s_mi.off_kv;
+  const uint32_t from = s_mi.sbase + s_mi.off_kv + stage_off<C>(r0, c0);
   const int rows = s_mi.rows;
   const int* rowvox = s_mi.rowvox[s_mi.buf];
 #pragma unroll
-  for (int u = 0; u < kTM / (RU * kComputeWarps); ++u) {
-    float4 f[IU];
+  for (int p = 0; p < P; ++p) {
+    const int r = r0 + kUnitRows * p, v = r < rows ? rowvox[r] : -1;
+    float4 f[J];
 #pragma unroll
-    for (int i = 0; i < IU; ++i) {
-      const int e = lane + 32 * i, r = RU * (warp + u * kComputeWarps) + e / C4, c4 = e % C4;
-      f[i] = lds4(stage + stage_off<C>(r, c4));
-    }
+    for (int j = 0; j < J; ++j) f[j] = lds4(from + p * (kUnitRows * C * 4) + j * 256);
 #pragma unroll
-    for (int i = 0; i < IU; ++i) {
-      const int e = lane + 32 * i, r = RU * (warp + u * kComputeWarps) + e / C4, c4 = e % C4;
-      const int v = r < rows ? rowvox[r] : -1;
-      if (v >= 0) reinterpret_cast<float4*>(y + (size_t)v * C)[c4] = f[i];
-    }
+    for (int j = 0; j < J; ++j)
+      if (v >= 0) reinterpret_cast<float4*>(y + (size_t)v * C)[c0 + 16 * j] = f[j];
   }
 }
 
