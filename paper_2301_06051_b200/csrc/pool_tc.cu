@@ -534,10 +534,14 @@ __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const __grid_const
           }
         }
         compute_sync();
-        const int n = min(n_out - r0, kTM / 2);
-        for (int i = tid; i < n * (C / 4); i += kComputeThreads) {
-          const int r = i / (C / 4), c4 = i - r * (C / 4);
-          reinterpret_cast<float4*>(a.out_feats + (size_t)(rank0 + r0 + r) * C)[c4] = lds4(ps_s + out_off<C>(r, c4));
+        const int n = min(n_out - r0, kTM / 2), r1 = tid / 16, c1 = tid % 16;
+#pragma unroll
+        for (int p = 0; p < kTM / 2; p += kComputeThreads / 16) {  // (addresses as in the gather)
+#pragma unroll
+          for (int j = 0; j < C / 64; ++j)
+            if (r1 + p < n)
+              reinterpret_cast<float4*>(a.out_feats + (size_t)(rank0 + r0 + r1 + p) * C)[c1 + 16 * j] =
+                  lds4(ps_s + out_off<C>(r1, c1) + p * (C * 4) + j * 256);
         }
       }
     }
