@@ -1081,9 +1081,13 @@ template <int C, int QC, class Slot>
 __device__ __forceinline__ void layer_norm_rows(float (&t)[QC], float sum, uint32_t gain, uint32_t shift, float eps,
                                                 int hq, Slot slot) {
   const float mq = sum * (1.0f / (float)QC);
-  float m2 = 0.f;
+  float2 sq = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int i = 0; i < QC; ++i) { const float d = t[i] - mq; m2 = fmaf(d, d, m2); }
+  for (int i = 0; i < QC; i += 2) {
+    const float2 d = __fadd2_rn(make_float2(t[i], t[i + 1]), make_float2(-mq, -mq));
+    sq = __ffma2_rn(d, d, sq);
+  }
+  const float m2 = sq.x + sq.y;
   sts2(slot(hq), make_float2(mq, m2));
   quarter_sync();
   const float2 s0 = lds2(slot(0)), s1 = lds2(slot(1)), s2 = lds2(slot(2)), s3 = lds2(slot(3));
@@ -1094,10 +1098,11 @@ __device__ __forceinline__ void layer_norm_rows(float (&t)[QC], float sum, uint3
 #pragma unroll
   for (int i4 = 0; i4 < QC / 4; ++i4) {
     const float4 g4 = lds4(gain + 4u * (uint32_t)(hq * QC + 4 * i4)), b4 = lds4(shift + 4u * (uint32_t)(hq * QC + 4 * i4));
-    t[4 * i4] = (t[4 * i4] - mean) * inv * g4.x + b4.x;
-    t[4 * i4 + 1] = (t[4 * i4 + 1] - mean) * inv * g4.y + b4.y;
-    t[4 * i4 + 2] = (t[4 * i4 + 2] - mean) * inv * g4.z + b4.z;
-    t[4 * i4 + 3] = (t[4 * i4 + 3] - mean) * inv * g4.w + b4.w;
+    const float2 u = __fmul2_rn(__fadd2_rn(make_float2(t[4 * i4], t[4 * i4 + 1]), make_float2(-mean, -mean)), make_float2(inv, inv));
+    const float2 w = __fmul2_rn(__fadd2_rn(make_float2(t[4 * i4 + 2], t[4 * i4 + 3]), make_float2(-mean, -mean)), make_float2(inv, inv));
+    const float2 y0 = __ffma2_rn(u, make_float2(g4.x, g4.y), make_float2(b4.x, b4.y));
+    const float2 y1 = __ffma2_rn(w, make_float2(g4.z, g4.w), make_float2(b4.z, b4.w));
+    t[4 * i4] = y0.x; t[4 * i4 + 1] = y0.y; t[4 * i4 + 2] = y1.x; t[4 * i4 + 3] = y1.y;
   }
 }
 
@@ -1177,11 +1182,11 @@ __device__ __forceinline__ void phase_epi_f2() {
   mbar_arrive(&s_mi.acc_free[2]);
   const bool ln = s_mi.ln2 != 0;
   if (ln) {
-    float sum = 0.f;
+    float2 sums = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int q = 0; q < QC / 4; ++q) sum += (t[4 * q] + t[4 * q + 1]) + (t[4 * q + 2] + t[4 * q + 3]);
+    for (int q = 0; q < QC / 2; ++q) sums = __fadd2_rn(sums, make_float2(t[2 * q], t[2 * q + 1]));
     auto slot = [&](int quarter) { return stage + stage_off<C>(row, quarter * (QC / 4)); };
-    layer_norm_rows<C, QC>(t, sum, par + 4 * ParOff<C>::ln2_g, par + 4 * ParOff<C>::ln2_b, s_mi.eps, hq, slot);
+    layer_norm_rows<C, QC>(t, sums.x + sums.y, par + 4 * ParOff<C>::ln2_g, par + 4 * ParOff<C>::ln2_b, s_mi.eps, hq, slot);
   }
 #pragma unroll
   for (int i4 = 1; i4 < QC / 4; ++i4)
