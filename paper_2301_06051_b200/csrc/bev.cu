@@ -10,12 +10,23 @@
 
 namespace {
 
+__global__ void fill_kernel(uint32_t* __restrict__ p, uint32_t v, int64_t words) {
+  pdl_enter();
+  const int64_t stride = 4 * (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); i < words; i += stride) {
+    if (i + 4 <= words) *reinterpret_cast<uint4*>(p + i) = make_uint4(v, v, v, v);
+    else
+      for (int64_t j = i; j < words; ++j) p[j] = v;
+  }
+}
+
 struct BevGeom {
   int32_t B, X, Y, Z, C;
 };
 
 __global__ void bev_mark_kernel(const int4* __restrict__ coords, int32_t n, BevGeom g, int32_t* __restrict__ cell_map,
                                 int32_t* __restrict__ status) {
+  pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int4 c = coords[i];
@@ -39,6 +50,7 @@ constexpr int kUnroll = 4;
 __global__ void __launch_bounds__(kThreads)
 bev_planes_kernel(const float* __restrict__ feats, const int32_t* __restrict__ cell_map, BevGeom g, int32_t groups,
                   int32_t lines_per_block, int64_t lines, float* __restrict__ out) {
+  pdl_enter();
   const int cg = blockIdx.x % groups;
   const int64_t line0 = (int64_t)(blockIdx.x / groups) * lines_per_block;
   const int c0 = cg * kGroup;
@@ -94,6 +106,7 @@ bev_planes_kernel(const float* __restrict__ feats, const int32_t* __restrict__ c
 __global__ void __launch_bounds__(kThreads)
 bev_planes4_kernel(const float* __restrict__ feats, const int32_t* __restrict__ cell_map, BevGeom g, int32_t groups,
                    int32_t lines_per_block, int64_t lines, float* __restrict__ out) {
+  pdl_enter();
   const int cg = blockIdx.x % groups;
   const int64_t line0 = (int64_t)(blockIdx.x / groups) * lines_per_block;
   const int c0 = cg * kGroup;
@@ -137,6 +150,7 @@ bev_planes4_kernel(const float* __restrict__ feats, const int32_t* __restrict__ 
 __global__ void __launch_bounds__(kThreads)
 bev_cells_kernel(const float4* __restrict__ feats, const int32_t* __restrict__ cell_map, int32_t C4, int64_t total4,
                  float4* __restrict__ out) {
+  pdl_enter();
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   for (int64_t e0 = (int64_t)blockIdx.x * kThreads + threadIdx.x; e0 < total4; e0 += stride * kUnroll) {
     int v[kUnroll];
@@ -170,6 +184,7 @@ bev_cells_kernel(const float4* __restrict__ feats, const int32_t* __restrict__ c
 __global__ void __launch_bounds__(kThreads)
 bev_columns_kernel(const float* __restrict__ feats, const int32_t* __restrict__ cell_map, BevGeom g, int64_t total,
                    float* __restrict__ out) {
+  pdl_enter();
   const int CH = g.C * g.Z;
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   for (int64_t e = (int64_t)blockIdx.x * kThreads + threadIdx.x; e < total; e += stride) {
@@ -186,6 +201,17 @@ bev_columns_kernel(const float* __restrict__ feats, const int32_t* __restrict__ 
 }
 
 }  // namespace
+
+// (A memset between kernels waits for the one before it to drain and holds up the one behind it; a kernel's launch
+// overlaps its neighbours': the BEV map of a 468 x 468 grid with it and the
+// writer launched the same way: 44.9 -> 38.9 us.)
+int dsvt_launch_fill(dsvt_ctx* ctx, void* p, uint32_t v, int64_t words) {
+  int64_t blocks = dsvt_ceil_div(words, 4 * 512);
+  if (blocks > 4 * (int64_t)ctx->sm_count) blocks = 4 * (int64_t)ctx->sm_count;
+  DSVT_CUDA_TRY(ctx, launch_pdl(fill_kernel, dim3((unsigned)blocks), dim3(512), 0, ctx->stream, (uint32_t*)p, v, words));
+  DSVT_LAUNCHED(ctx);
+  return DSVT_OK;
+}
 
 extern "C" int dsvt_bev_scatter(dsvt_ctx* ctx, const int32_t* coords, const float* feats, int32_t n, int32_t C,
                                 int32_t batch, const int32_t grid[3], int32_t channels_last, float* out) {
@@ -208,10 +234,11 @@ extern "C" int dsvt_bev_scatter(dsvt_ctx* ctx, const int32_t* coords, const floa
     DSVT_CUDA_TRY(ctx, cudaMalloc((void**)&ctx->cell_map, (size_t)cells * sizeof(int32_t)));
     ctx->cell_map_entries = (size_t)cells;
   }
-  DSVT_CUDA_TRY(ctx, cudaMemsetAsync(ctx->cell_map, 0xFF, (size_t)cells * sizeof(int32_t), st));
+  const int rc = dsvt_launch_fill(ctx, ctx->cell_map, 0xFFFFFFFFu, cells);
+  if (rc != DSVT_OK) return rc;
   if (n > 0) {
-    bev_mark_kernel<<<(unsigned)dsvt_ceil_div(n, 256), 256, 0, st>>>((const int4*)coords, n, g, ctx->cell_map,
-                                                                      ctx->status);
+    DSVT_CUDA_TRY(ctx, launch_pdl(bev_mark_kernel, dim3((unsigned)dsvt_ceil_div(n, 256)), dim3(256), 0, st, (const int4*)coords, n, g,
+                                  ctx->cell_map, ctx->status));
     DSVT_LAUNCHED(ctx);
   }
   const int64_t grid_cap = (int64_t)ctx->sm_count * 8 * 4;  // grid-stride kernels: a few waves of resident blocks
@@ -221,12 +248,13 @@ extern "C" int dsvt_bev_scatter(dsvt_ctx* ctx, const int32_t* coords, const floa
       const int64_t total4 = total / 4;
       int64_t blocks = dsvt_ceil_div(total4, (int64_t)kThreads * kUnroll);
       if (blocks > grid_cap) blocks = grid_cap;
-      bev_cells_kernel<<<(unsigned)blocks, kThreads, 0, st>>>((const float4*)feats, ctx->cell_map, C / 4, total4,
-                                                             (float4*)out);
+      DSVT_CUDA_TRY(ctx, launch_pdl(bev_cells_kernel, dim3((unsigned)blocks), dim3(kThreads), 0, st, (const float4*)feats,
+                                    (const int32_t*)ctx->cell_map, C / 4, total4, (float4*)out));
     } else {
       int64_t blocks = dsvt_ceil_div(total, kThreads);
       if (blocks > grid_cap) blocks = grid_cap;
-      bev_columns_kernel<<<(unsigned)blocks, kThreads, 0, st>>>(feats, ctx->cell_map, g, total, out);
+      DSVT_CUDA_TRY(ctx, launch_pdl(bev_columns_kernel, dim3((unsigned)blocks), dim3(kThreads), 0, st, feats,
+                                    (const int32_t*)ctx->cell_map, g, total, out));
     }
     DSVT_LAUNCHED(ctx);
     return DSVT_OK;
@@ -237,10 +265,8 @@ extern "C" int dsvt_bev_scatter(dsvt_ctx* ctx, const int32_t* coords, const floa
   const int32_t lines_per_block = g.X >= kThreads * kUnroll ? 1 : (kThreads * kUnroll) / g.X;
   const int64_t blocks = dsvt_ceil_div(lines, lines_per_block) * groups;
   if (blocks >= (1ll << 31)) return DSVT_ERR_UNSUPPORTED;
-  if (g.X % 4 == 0)
-    bev_planes4_kernel<<<(unsigned)blocks, kThreads, 0, st>>>(feats, ctx->cell_map, g, groups, lines_per_block, lines, out);
-  else
-    bev_planes_kernel<<<(unsigned)blocks, kThreads, 0, st>>>(feats, ctx->cell_map, g, groups, lines_per_block, lines, out);
+  DSVT_CUDA_TRY(ctx, launch_pdl(g.X % 4 == 0 ? bev_planes4_kernel : bev_planes_kernel, dim3((unsigned)blocks), dim3(kThreads), 0, st,
+                                feats, (const int32_t*)ctx->cell_map, g, groups, lines_per_block, lines, out));
   DSVT_LAUNCHED(ctx);
   return DSVT_OK;
 }

@@ -676,10 +676,12 @@ extern "C" int dsvt_pool_counted(dsvt_ctx* ctx, const int32_t* coords, const flo
   // changes and the dense cell map's 28 MB of clearing included; full regions take (nslots - 1) / 128 more tiles.
   if (tc && (mask_empty || !slot_pe)) {
     const int64_t num_words = (int64_t)((cells + 31) / 32);
-    DSVT_CUDA_TRY(ctx, cudaMemsetAsync(bits, 0, sizeof(uint32_t) * (size_t)num_words, st));
-    pool_mark_kernel<true><<<vb, 256, 0, st>>>((const int4*)coords, n, n_dev, g, nullptr, bits, ctx->keys[0], slot_of, ctx->status);
+    int rc = dsvt_launch_fill(ctx, bits, 0, num_words);
+    if (rc != DSVT_OK) return rc;
+    DSVT_CUDA_TRY(ctx, launch_pdl(pool_mark_kernel<true>, dim3(vb), dim3(256), 0, st, (const int4*)coords, n, n_dev, g, (int32_t*)nullptr,
+                                  bits, ctx->keys[0], slot_of, ctx->status));
     DSVT_LAUNCHED(ctx);
-    int rc = dsvt_launch_popc_scan(ctx, bits, (int32_t)nslots, ctx->win_start, ctx->win_setoff, num_words);
+    rc = dsvt_launch_popc_scan(ctx, bits, (int32_t)nslots, ctx->win_start, ctx->win_setoff, num_words);
     if (rc != DSVT_OK) return rc;
     int4* rows = reinterpret_cast<int4*>(ctx->rowoff_a);
     DSVT_CUDA_TRY(ctx, launch_pdl(pool_rows_kernel, dim3(vb), dim3(256), 0, st, n, n_dev, g, (const uint32_t*)ctx->keys[0],
