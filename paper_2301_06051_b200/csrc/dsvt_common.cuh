@@ -97,8 +97,8 @@ static inline int64_t dsvt_ceil_div(int64_t a, int64_t b) { return (a + b - 1) /
 // ---- launchers implemented in the .cu files (all enqueue on ctx->stream) ----
 // Exclusive scan; out has count + 1 entries (out[count] = total).  in == out is allowed.
 int dsvt_launch_scan_i32(dsvt_ctx* ctx, const int32_t* in, int32_t* out, int64_t count, int32_t* total_out);
-// Sets `words` 32-bit words from p (16-byte aligned) to v.
-int dsvt_launch_fill(dsvt_ctx* ctx, void* p, uint32_t v, int64_t words);
+// Sets `words` 32-bit words from p (16-byte aligned) to v; overlap: the launch may overlap its predecessor's tail.
+int dsvt_launch_fill(dsvt_ctx* ctx, void* p, uint32_t v, int64_t words, bool overlap);
 constexpr int DSVT_POPC_TILE = 1024;  // words per block of the bitmap scan
 // Exclusive scans over a bitmap's words (16-byte aligned): of their popcounts, and (out_fields != NULL) of how many of their fields of
 // `field` bits (a power of two) are not empty.  Outputs have count + 1 entries, count <= max_windows + 1.

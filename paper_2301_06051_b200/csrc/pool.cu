@@ -676,7 +676,7 @@ extern "C" int dsvt_pool_counted(dsvt_ctx* ctx, const int32_t* coords, const flo
   // changes and the dense cell map's 28 MB of clearing included; full regions take (nslots - 1) / 128 more tiles.
   if (tc && (mask_empty || !slot_pe)) {
     const int64_t num_words = (int64_t)((cells + 31) / 32);
-    int rc = dsvt_launch_fill(ctx, bits, 0, num_words);
+    int rc = dsvt_launch_fill(ctx, bits, 0, num_words, true);
     if (rc != DSVT_OK) return rc;
     DSVT_CUDA_TRY(ctx, launch_pdl(pool_mark_kernel<true>, dim3(vb), dim3(256), 0, st, (const int4*)coords, n, n_dev, g, (int32_t*)nullptr,
                                   bits, ctx->keys[0], slot_of, ctx->status));
