@@ -876,9 +876,9 @@ __device__ __noinline__ void stamp_role(int32_t* __restrict__ row_stamp) {
 // Gather (Eq. 4): the fp32 rows listed in buffer b -> bf16 A operand; all 128 rows are written (rows past the tile as
 // zeros).  16 lanes to a row (256 bytes), all of a thread's rows in flight at once (C = 192: 12 loads; in two rounds the
 // gather cost one L2 round trip more).  A thread's rows are 32 apart and its chunks 16, so that every address is one base
-// plus constants (in lane-linear units, with a division, a row lookup and a swizzled address per 16 bytes, gather, x staging
-// and row stores took 1 % more of a 25,000-pillar frame and 4 % more of two layers on 2000 rows).  ADD_PE: the current tile's rows once more, with the positional
-// term added (the operand of the key and query projections).
+// plus constants (in lane-linear units, with a division, a row lookup and a swizzled address per 16 bytes, gather, x
+// staging and row stores took 1 % more of a 32,000-pillar frame and 4 % more of two layers on 2531 rows).  ADD_PE: the
+// current tile's rows once more, with the positional term added (the operand of the key and query projections).
 constexpr int kUnitRows = kComputeThreads / 16;
 template <int C, int D, bool RPB, bool ADD_PE>
 __device__ __forceinline__ void phase_gather(int b, int rows) {

@@ -82,15 +82,7 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
-      : "memory");
-}
-// The same with descriptors given as low and high words, and with the A operand in TMEM (two bf16 K elements per 32-bit
+// One MMA with descriptors given as low and high words, and the same with the A operand in TMEM (two bf16 K elements per 32-bit
 // column, row i of the tile in lane i).
 __device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
                                         uint32_t idesc, uint32_t acc) {
@@ -185,27 +177,6 @@ __device__ __forceinline__ void tmem_st_row(uint32_t taddr, const float (&v)[N])
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x2_trans(uint32_t addr, uint32_t (&r)[2]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
-}
-__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-      "{%0, %1, %2, %3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void mma_1688(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%0, %1, %2, %3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a0), "r"(a1), "r"(b0));
-}
-
 // Accesses to the big regions by shared-space address (through a generic pointer they would be generic accesses).
 // Volatile, so that they stay in program order and none is hoisted into registers ahead of its use.
 __device__ __forceinline__ float4 lds4(uint32_t a) {
@@ -246,12 +217,9 @@ __device__ __forceinline__ uint32_t swz(int row, int c8) {
   return (uint32_t)((c8 >> 3) * (kTM * 128) + (row >> 3) * 1024 + (row & 7) * 128 + (((c8 & 7) ^ (row & 7)) << 4));
 }
 
-// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr) {
-  return (uint64_t)((saddr >> 4) & 0x3FFF) | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
-}
-// Words of such a descriptor (low: address and leading offset; high: stride and layout), and of one for an unswizzled
-// operand made of 8-row x 16-byte core matrices of 128 bytes.  K-major: lbo = bytes to the next core matrix along K,
+// Words of a shared-memory matrix descriptor (low: address and leading offset; high: stride and layout): K-major, 128-byte
+// swizzle, 8-row groups 1024 bytes apart; and of one for an unswizzled operand made of
+// 8-row x 16-byte core matrices of 128 bytes.  K-major: lbo = bytes to the next core matrix along K,
 // sbo = bytes to the next 8 rows.  N-major: lbo = bytes to the next 8 K, sbo = to the next 8 N.
 constexpr uint32_t kDescHiSwizzled = 64u | 1u << 14 | 2u << 29;
 __device__ __forceinline__ uint32_t desc_lo_swizzled(uint32_t saddr) { return saddr >> 4 | 1u << 16; }
