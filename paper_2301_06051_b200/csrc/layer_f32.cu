@@ -258,7 +258,8 @@ __global__ void __launch_bounds__(kT, 1) layer_f32_kernel(const __grid_constant_
       const int e = warp_lower_bound(a.rowoff, s_lo + 1, s_end + 1, base + want + 1) - 1;  // last boundary within `want` rows
       if (lane == 0) bounds[0] = max(e, s_lo + 1);
     }
-    for (int r = tid; r < TM; r += kT) { rowvox[r] = -1; rowlin[r] = 0; }
+    // (rows that no set fills, where the offsets claim more than a set has, are keys and queries of their own)
+    for (int r = tid; r < TM; r += kT) { rowvox[r] = -1; rowlin[r] = 0; row_lo[r] = (unsigned char)r; row_n[r] = 1; }
     __syncthreads();
     nsets = bounds[0] - s_lo;
     const int rows = __ldg(a.rowoff + s_lo + nsets) - base;

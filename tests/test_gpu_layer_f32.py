@@ -4,7 +4,7 @@ import pytest
 import torch
 
 import dsvt_inputs as di
-from gpu_helpers import check_close, dev
+from gpu_helpers import check_close, dev, upload_table
 
 pytestmark = pytest.mark.gpu
 
@@ -41,3 +41,26 @@ def test_layer_fp32_matches_oracle(oracle, n, grid, window, tau, C, heads, hidde
     z = x.clone()  # in place: a tile's rows are its own
     ctx.layer(z, table, w, z, pe=None if pe is None else dev(pe), coords=coords)
     assert ctx.status_sync() == 0 and torch.equal(y, z)
+
+
+@pytest.mark.parametrize("C,heads,hidden", [(128, 8, 0), (192, 8, 384)])
+def test_row_offsets_that_claim_more_rows_than_a_set_has(oracle, C, heads, hidden):
+    """Caller-made row offsets with room for seven members that their set does not have: DSVT_STATUS_BAD_INDEX, and the
+    voxels of all other sets come out right."""
+    from paper_2301_06051_b200 import api
+
+    n, tau = 700, 36
+    case = di.random_case(C, n, (48, 48, 1), (12, 12, 1), tau, C, heads, hidden, layernorm=hidden > 0)
+    layer = case["blocks"][0][0]
+    p = oracle.partition(case["coords"], 1, case["grid"], case["window"], tau, 0)
+    table = upload_table(p.set_table)
+    long = len(p.set_table) // 2
+    table.set_rowoff[long + 1 : len(p.set_table) + 1] += 7
+    ctx = api.Context(n, 16, C)
+    x = dev(case["feats"])
+    y = torch.empty_like(x)
+    ctx.layer(x, table, api.device_weights(layer, api.FP32, ctx.device), y)
+    assert ctx.status_sync() == api.STATUS_BAD_INDEX
+    others = np.setdiff1d(np.arange(n), p.set_table[long])
+    want = oracle.layer(case["feats"], p.set_table, layer)
+    check_close(y.cpu().numpy()[others], want[others], "fp32", "the other sets")
