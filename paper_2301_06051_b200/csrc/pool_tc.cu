@@ -348,23 +348,23 @@ __global__ void __launch_bounds__(kThreads, 1) pool_tc_kernel(const __grid_const
                  "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // everything above touched this CTA's own state; what follows reads what the kernels before it in the stream wrote
+  // (the row list, the number of regions; the weights and biases too: every launch of the call may start early, the first
+  // of them under the tail of a kernel that writes them): wait for them if this launch was allowed to start early
+  pdl_enter();
+  const int m = min(*a.num_out, a.cap_m);
+  PoolRows pr;
+  pr.padded = a.rows == nullptr;
+  pr.n_rows = pr.padded ? m * ns : *a.num_rows;
   for (int i = tid; i < 4 * C; i += kThreads) {
     const int which = i / C;
     const float* v = which == 0 ? a.b_q : which == 1 ? a.b_k : which == 2 ? a.b_v : a.b_o;
     par[i] = v ? __ldg(v + i % C) : 0.f;
   }
-  // everything above touched this CTA's own state and the call's weights; what follows reads what the kernels before
-  // it in the stream wrote (the region list, the cell map, the number of regions): wait for them if this launch was
-  // allowed to start early
-  pdl_enter();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_pm.tmem_base;
-  const int m = min(*a.num_out, a.cap_m);
-  PoolRows pr;
-  pr.padded = a.rows == nullptr;
-  pr.n_rows = pr.padded ? m * ns : *a.num_rows;
   pr.step = pr.padded ? kTM : kTM + 1 - ns;
   if (!pr.padded) {  // as many rounds of tiles as steps of that length take, evenly filled
     const int rounds = max(1, (pr.n_rows + pr.step * (int)gridDim.x - 1) / (pr.step * (int)gridDim.x));

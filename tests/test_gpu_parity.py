@@ -593,6 +593,34 @@ def test_pool_tiles_of_voxels_in_region_order(gpu, oracle, pool, grid, n, C, hea
     assert torch.equal(oc2, oc[:half]) and torch.equal(of2, of[:half])
 
 
+@pytest.mark.parametrize("mask_empty,with_pe", [(1, False), (0, True)])
+def test_pool_right_behind_the_kernels_that_write_its_parameters(gpu, mask_empty, with_pe):
+    """Calls back to back on one stream, each behind copies that change weights and biases in place: every call takes
+    the values that were there when its turn came."""
+    rng = np.random.default_rng(9)
+    n, C, heads, grid, pool = 1500, 192, 8, (40, 40, 4), (2, 2, 2)
+    coords, feats = dev(di.unique_cells(rng, n, grid, 1)), dev(rng.standard_normal((n, C), dtype=np.float32))
+    ctx = gpu.Context(n, 20 * 20 * 2, C)
+    sets = [gpu.device_weights(di.make_pool_weights(rng, C, heads, True, 8, with_pe), gpu.BF16_FP32ACC, ctx.device) for _ in range(3)]
+    call = lambda w: ctx.pool(coords, feats, 1, grid, pool, w, mask_empty=mask_empty)
+    want, m = [], 0
+    for w in sets:
+        r = call(w)
+        assert ctx.status_sync() == 0
+        m = int(r[2].item())
+        want.append(r[1][:m].clone())
+    live = {k: v.clone() if torch.is_tensor(v) else v for k, v in sets[0].items()}
+    got = []
+    for i in range(12):
+        for k, v in sets[i % 3].items():
+            if torch.is_tensor(v):
+                live[k].copy_(v)
+        got.append(call(live)[1])
+    assert ctx.status_sync() == 0
+    for i, g in enumerate(got):
+        assert torch.equal(g[:m], want[i % 3]), i
+
+
 def test_pool_flags_duplicate_cells_and_overflow(gpu):
     rng = np.random.default_rng(3)
     C = 16
