@@ -383,8 +383,8 @@ __global__ void __launch_bounds__(kT, 1) layer_f32_kernel(const __grid_constant_
             }
           }
           if (!two) lg[1] = -INFINITY;
-          const float nm = fmaxf(mx, fmaxf(lg[0], lg[1]));
-          const float al = expf(mx - nm), e0 = expf(lg[0] - nm), e1 = expf(lg[1] - nm);  // (exp(-inf) = 0)
+          const float nm = fmaxf(mx, fmaxf(lg[0], lg[1])), from = nm == -INFINITY ? 0.f : nm;  // (a bias may rule out all keys so far)
+          const float al = expf(mx - from), e0 = expf(lg[0] - from), e1 = expf(lg[1] - from);  // (exp(-inf) = 0)
           mx = nm;
           den = den * al + (e0 + e1);
 #pragma unroll

@@ -204,6 +204,36 @@ def test_bias_table_narrower_than_a_set_is_flagged_on_the_tensor_core_path(gpu, 
     assert torch.isfinite(out).all()
 
 
+@pytest.mark.parametrize("n,grid,window,tau,C,heads,bf16", [
+    (1500, 48, 12, 36, 128, 8, False),  # fp32 kernel: running softmax over pairs of keys
+    (1500, 48, 12, 36, 192, 8, False),
+    (700, 40, 10, 36, 32, 4, False),    # general-shape kernel
+])
+@pytest.mark.parametrize("mask", [-np.inf, np.finfo(np.float32).min, -1e31])
+def test_bias_that_masks_offsets(gpu, oracle, n, grid, window, tau, C, heads, bf16, mask):
+    """Table entries that rule offsets out.  Heads 1 and 2 keep the voxel itself and every fourth offset; with a finite
+    mask head 0 masks every offset alike, which leaves equal weights inside the set and nothing outside it.  (The lowest
+    float overflows when it is scaled to the unscaled logits: a row of it alone has no defined result.)"""
+    cfg = di.random_case(n, n, (grid, grid, 1), (window, window, 1), tau, C, heads, bf16=bf16)
+    rng = np.random.default_rng(n + C)
+    L = _with_bias(rng, cfg["blocks"][0][0], heads, (window, window, 1), oracle)
+    keep = rng.random(L["rpb"].shape[1]) < 0.25
+    keep[L["rpb"].shape[1] // 2] = True  # offset zero
+    L["rpb"][1:3, ~keep] = mask
+    if mask == -1e31:
+        L["rpb"][0] = mask
+    ctx = gpu.Context(n, _nwin(1, cfg["grid"], cfg["window"]), C)
+    x, coords = dev(cfg["feats"]), dev(cfg["coords"])
+    t = ctx.partition(coords, 1, cfg["grid"], cfg["window"], tau, 0)
+    out = torch.empty_like(x)
+    ctx.set_attention(x, t, gpu.device_weights(L, precision_of(cfg), ctx.device), out, coords=coords)
+    assert ctx.status_sync() == 0
+    ref_t = oracle.partition(cfg["coords"], 1, cfg["grid"], cfg["window"], tau, 0).set_table
+    want, _ = oracle.set_attention(cfg["feats"], ref_t, L["W_qkv"], L["b_qkv"], L["W_o"], L["b_o"], heads, rpb=L["rpb"],
+                                   coords=cfg["coords"], rpb_extent=cfg["window"])
+    check_close(out.cpu().numpy(), want, cfg["precision"], "masking bias")
+
+
 # ------------------------------------------------------------------------------------------------ BEV projection
 @pytest.mark.parametrize("grid,batch,n,C", [
     ((33, 7, 1), 1, 60, 8),       # one full 32-cell segment and a ragged tail of one cell
