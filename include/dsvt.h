@@ -232,6 +232,8 @@ int dsvt_partition_noalloc(void* cuda_stream, const int32_t* coords, int32_t n, 
  *   heads       head h owns channels [h*d, (h+1)*d), d = C / heads; logits are scaled by 1/sqrt(d).
  *   pe          optional float [n][C] positional term, added to the input of the query and key maps only.
  *
+ * A voxel with features that are not finite spoils the rows of its own set and no others.
+ *
  * Needs C % 8 == 0, (C/heads) % 4 == 0, set_size <= 128 (else DSVT_ERR_UNSUPPORTED).
  */
 int dsvt_set_attention(dsvt_ctx* ctx, const float* feats, int32_t n, int32_t C, const int32_t* set_table,

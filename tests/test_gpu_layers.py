@@ -123,6 +123,52 @@ def test_attention_on_both_sides_of_the_set_codes(gpu, oracle, C, heads, window,
     check_close(y.cpu().numpy(), _oracle_chain(oracle, cfg, cfg["blocks"]), "bf16", "C=%d window=%s" % (C, window))
 
 
+@pytest.mark.parametrize("C,heads,window,tau,hidden,option", [
+    (192, 8, 12, 36, 384, ""),
+    (192, 8, 12, 36, 192, "pe"),
+    (192, 8, 2, 36, 0, ""),       # dozens of sets in a tile
+    (128, 8, 30, 90, 256, ""),    # sets of most of a tile
+    (128, 4, 12, 36, 0, "rpb"),
+    (64, 4, 12, 36, 128, ""),
+])
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), 3.4e38, 1e35])
+def test_a_wild_row_stays_in_its_set(gpu, C, heads, window, tau, hidden, option, value):
+    """Voxels of features that are not finite, or so large that scores with them leave the range of the codes that keep
+    a tile's sets apart, change no row outside their own sets (bitwise), although sets share 128-row tiles."""
+    n, grid = 2500, (60, 60, 1)
+    cfg = di.random_case(n + C, n, grid, (window, window, 1), tau, C, heads, hidden, layernorm=hidden > 0, bf16=True)
+    layer, rng = cfg["blocks"][0][0], np.random.default_rng(C)
+    if option == "rpb":
+        layer["rpb"] = rng.standard_normal((heads, (2 * window - 1) ** 2)).astype(np.float32)
+        layer["rpb_extent"] = (window, window, 1)
+    ctx = gpu.Context(n, (-(-grid[0] // window)) ** 2, C)
+    coords, x = dev(cfg["coords"]), dev(cfg["feats"])
+    pe = dev(rng.standard_normal((n, C)).astype(np.float32)) if option == "pe" else None
+    t = ctx.partition(coords, 1, grid, (window, window, 1), tau, 0)
+    w = gpu.device_weights(layer, gpu.BF16_FP32ACC, ctx.device)
+    clean = torch.empty_like(x)
+    ctx.layer(x, t, w, clean, pe=pe, coords=coords)
+    S = int(t.num_sets.item())
+    table = t.set_table[:S]
+    wild = torch.as_tensor(rng.choice(n, 6, replace=False), device="cuda")
+    sets = torch.isin(table, wild.to(torch.int32)).any(dim=1)
+    inside = torch.zeros(n, dtype=torch.bool, device="cuda")
+    inside[table[sets].reshape(-1).long()] = True
+    for spoilt in ("x", "pe") if option == "pe" else ("x",):
+        y, src = torch.empty_like(x), {"x": x.clone(), "pe": pe}
+        if spoilt == "pe":
+            src["pe"] = pe.clone()
+        src[spoilt][wild, ::5] = value
+        src[spoilt][wild[0]] = value  # (and one whole row)
+        ctx.layer(src["x"], t, w, y, pe=src["pe"], coords=coords)
+        assert ctx.status_sync() == 0
+        assert torch.equal(y[~inside], clean[~inside])
+        if value != value:  # NaN reaches every row of its sets
+            assert torch.isnan(y[inside]).any(dim=1).all()
+    ctx.layer(x, t, w, y, pe=pe, coords=coords)
+    assert torch.equal(y, clean)
+
+
 def test_chain_with_other_tables_per_block(gpu, oracle):
     """Hybrid windows: the second block runs on the tables of another window cut, so a tile of its first layer
     reads rows that tiles anywhere in the previous layer wrote (the stamps are per voxel, not per window)."""
