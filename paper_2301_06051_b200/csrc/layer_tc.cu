@@ -163,7 +163,7 @@ struct alignas(1024) Misc {
   int rows, buf;
   int next_rows[2];        // rows of the tile listed in buffer b (< 0: there is no such tile), valid after rl_ready[b]
   const float* next_x[2];  // where that tile's input rows are read from
-  int wild[2];             // a row of buffer b holds a value of 2^60 or more, or none (see phase_gather)
+  int wild[2];             // kTM if a row of buffer b holds a value of 2^60 or more or NaN, else 0 (see phase_gather)
   int st_rows[2], st_stamp[2];  // for the stamp warp: rows of the stored tile in buffer b, the stamp they get (0: none)
   // row lists, double buffered: the loader warp fills buffer (k + 1) & 1 while the compute warps work on tile k;
   // the compute warps gather tile k + 1 as soon as tile k's MMAs no longer read the A operand
@@ -273,7 +273,7 @@ __device__ __forceinline__ KeyRange key_range(int r0, int rows) {
     const int lo = min(max(from - 32 * j, 0), 32), hi = min(max(to - 32 * j, 0), 32);
     if (hi > lo) sets += __popc(s_mi.starts[s_mi.buf][j] & (0xffffffffu >> (32 - hi)) & (0xffffffffu << lo));
   }
-  k.coded = sets <= kCodes<D>;
+  k.coded = sets + s_mi.wild[s_mi.buf] <= kCodes<D>;
   return k;
 }
 
@@ -336,10 +336,10 @@ __device__ __forceinline__ float softmax_rows(uint32_t t_s, const KeyRange& k, i
 }
 
 // A flagged tile (see phase_gather): what is not finite in the value operand becomes zero, for the other sets' zero weights
-// to meet.  Returns whether this thread's row belongs to a set of which a value was not finite.
+// to meet; the rows of a set of which a value was not finite get no keys, so that 0 x 1 / 0 makes them NaN.
 //   at      this thread's quarter row of the operand (chunks * 8 columns)
 //   row     its tile row, if the warp has rows (on)
-__device__ __noinline__ bool spoilt_set(uint32_t at, int chunks, int row, bool on) {
+__device__ __noinline__ void contain_wild(uint32_t at, int chunks, int row, bool on) {
   unsigned char* row_n = s_mi.row_n[s_mi.buf];
   const int lo = s_mi.row_lo[s_mi.buf][row], n = row_n[row];
   compute_sync();
@@ -360,9 +360,8 @@ __device__ __noinline__ bool spoilt_set(uint32_t at, int chunks, int row, bool o
   bool spoilt = false;
   for (int j = 0; j < n; ++j) spoilt |= row_n[lo + j] == 255;
   compute_sync();
-  row_n[row] = (unsigned char)n;
+  row_n[row] = (unsigned char)(spoilt ? 0 : n);  // (key_range: the sets before a warp's last one end at its first row)
   compute_sync();
-  return spoilt;
 }
 
 // Attention of tile k: warps 4 q + (0..3) take heads q, q + 4, ... ; their S, then P, then O live in TMEM columns
@@ -376,15 +375,11 @@ __device__ __forceinline__ void attend(int k) {
   const bool on = 32 * (warp & 3) < rows;  // (the whole warp)
   const uint32_t t_s = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + 128 * q;
   if (PE) compute_sync();  // (the flag says nothing until every thread has written its rows with the positional term)
-  const bool wild = s_mi.wild[s_mi.buf] != 0;
-  bool spoilt = false;
-  if (wild)
-    spoilt = spoilt_set(s_mi.sbase + s_mi.off_kv + (uint32_t)(C / 8 + q * (C / 32)) * kChunkBytes + row * 16, C / 32, row, on);
+  if (s_mi.wild[s_mi.buf])
+    contain_wild(s_mi.sbase + s_mi.off_kv + (uint32_t)(C / 8 + q * (C / 32)) * kChunkBytes + row * 16, C / 32, row, on);
   KeyRange kr = {0, 0, true};
   if (on) kr = key_range<D>(32 * (warp & 3), rows);
-  if (wild) kr.coded = false;
-  const int lo = s_mi.row_lo[s_mi.buf][row];
-  const int n = spoilt ? 0 : s_mi.row_n[s_mi.buf][row];  // (no keys: 0 x 1 / 0 makes the row NaN)
+  const int lo = s_mi.row_lo[s_mi.buf][row], n = s_mi.row_n[s_mi.buf][row];
 #pragma unroll 1
   for (int h = q; h < s_mi.heads; h += 4) {
     const uint32_t par = (uint32_t)(k * (s_mi.heads >> 2) + (h >> 2)) & 1u;  // (heads so far of this group)
@@ -925,8 +920,9 @@ __device__ __noinline__ void stamp_role(int32_t* __restrict__ row_stamp) {
 // The products of the attention run over the whole tile, and zero weights or codes do not stop what is not finite: such a
 // row would reach the other sets of its tile.  A tile with a value of 2^60 or more (scores with rows of ordinary size then
 // come near the codes' 2^100), infinity or NaN is flagged; its scores are masked by comparing and its values are made
-// finite (spoilt_set).  The look costs 24 three-way maxima per thread: 32,000-pillar frame 399.8 -> 402.2 us, 120,000 voxels
-// 1406.6 -> 1416.2, windows of 30 x 30 387.9 -> 385.9 (with the repair in the value epilogue the first two 0.3 % more).
+// finite (contain_wild).  The look is hidden under the loads; the branch in the attention costs 0.4 %: 32,000-pillar frame
+// 399.5 -> 401.1 us, 120,000 voxels 1401.6 -> 1407.5 (0.6 % with the repair's results in the attention's registers, 1 %
+// with the repair in the value epilogue).
 __device__ __forceinline__ float max_abs3(float a, float b, float c) {  // (NaN if one of them is)
   float m;
   asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
@@ -972,7 +968,7 @@ __device__ __forceinline__ void phase_gather(int b, int rows) {
       }
     }
   }
-  if (!(max_abs3(m0, m1, 0.f) < 0x1p60f)) s_mi.wild[b] = 1;
+  if (!(max_abs3(m0, m1, 0.f) < 0x1p60f)) s_mi.wild[b] = kTM;
   if (RPB && !ADD_PE) {
     for (int r = threadIdx.x; r < kTM; r += kComputeThreads) {
       const int v = r < rows ? rowvox[r] : -1;
