@@ -143,6 +143,8 @@ int dsvt_launch_layer_tc(dsvt_ctx* ctx, const dsvt_fused_args& a);
 // DSVT_MAX_CHAIN_LAYERS layers; every voxel a later layer reads must be written by the layer before it.
 bool dsvt_layer_tc_chainable(const dsvt_fused_args& a, const dsvt_fused_args& b);
 int dsvt_launch_layers_tc(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_layers);
+// Whether the driver offers the entry point that encodes tensor maps.
+bool dsvt_tensor_maps_available();
 // CUtensorMap (128 bytes, 64-byte aligned) of a row-major bf16 (fp32) matrix [rows][cols]: boxes of 64 (32) columns x
 // box_rows rows, 128-byte swizzle; encoded once per matrix and context.  Returns false if the driver cannot encode it.
 bool dsvt_cached_weight_map(dsvt_ctx* ctx, void* tensor_map, const void* w, int rows, int cols, int box_rows,

@@ -11,7 +11,8 @@
 // as they were loaded.  A first version staged weights by cp.async from all threads, 16 k at a time with a block-wide
 // barrier per stage: a third of its instructions were copies and their addresses.
 //
-// Every wait is bounded; one that gives up raises DSVT_STATUS_TIMEOUT and the block leaves.
+// Every wait is bounded; one that gives up raises DSVT_STATUS_TIMEOUT, and the block leaves at the end of its tile
+// without having stored any of its rows.
 //
 // Measured (B200): two full layers, 12,345 pillars, C = 192: 0.78 ms, 19 TFLOP/s = 27 % of the FMA peak (layer_fma.cu:
 // 1.79 ms); two attention-only layers, 2,000 pillars, C = 128: 0.11 ms (0.38 ms).  A C x C product of a 41-row tile takes
@@ -219,6 +220,7 @@ __global__ void __launch_bounds__(kT, 1) layer_f32_kernel(const __grid_constant_
   const dsvt_fused_args& a = f.a;
   const F32Geom& g = f.g;
   int32_t* status = f.status;
+  volatile int* abort_flag = &s_ring.abort_flag;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   float* bufA = reinterpret_cast<float*>(ring + kSt * Shape<C>::stage_bytes);
@@ -251,7 +253,7 @@ __global__ void __launch_bounds__(kT, 1) layer_f32_kernel(const __grid_constant_
   __syncthreads();
   const int s_end = bounds[1];
   for (int s_lo = bounds[0], nsets; s_lo < s_end; s_lo += nsets) {
-    __syncthreads();  // the previous tile's last reads
+    if (__syncthreads_or(*abort_flag)) break;  // (also orders the previous tile's last reads)
     const int base = __ldg(a.rowoff + s_lo), left = __ldg(a.rowoff + s_end) - base;
     if (warp == 0) {
       const int cuts = (left + TM - 1) / TM, want = cuts > 1 ? min(TM, (left + cuts - 1) / cuts + tau / 2) : TM;
@@ -424,7 +426,7 @@ __global__ void __launch_bounds__(kT, 1) layer_f32_kernel(const __grid_constant_
     __syncthreads();
     const bool mlp = hidden > 0;
     // ---- x1 = LN1(x + Z): to the operand buffer, or to y where the layer ends here ----
-    for (int r = warp; r < rows; r += kW) {
+    for (int r = *abort_flag ? rows : warp; r < rows; r += kW) {  // (a wait that gave up did so before the barrier)
       const int v = rowvox[r];
       float tr[C / 32];
 #pragma unroll
@@ -444,7 +446,7 @@ __global__ void __launch_bounds__(kT, 1) layer_f32_kernel(const __grid_constant_
     run_product<C>(rm, f, ring, Job{bufK, bufA, p.b_2, stage0 + (4 + hidden / C) * per, hidden / kKS, stage0, total, false, true, false});
     __syncthreads();
     // ---- y = LN2(x1 + M) ----
-    for (int r = warp; r < rows; r += kW) {
+    for (int r = *abort_flag ? rows : warp; r < rows; r += kW) {
       const int v = rowvox[r];
       float tr[C / 32];
 #pragma unroll
@@ -458,7 +460,7 @@ __global__ void __launch_bounds__(kT, 1) layer_f32_kernel(const __grid_constant_
     stage0 += total;
   }
   __syncthreads();
-  if (tid == 0 && s_ring.abort_flag) {
+  if (tid == 0 && *abort_flag) {
     atomicOr(status, DSVT_STATUS_TIMEOUT);
     // no load may still be writing into this block's shared memory when it retires
     for (int g0 = max(stage0 - kSt, 0); g0 < stage0; ++g0)
@@ -481,7 +483,7 @@ int launch_f32(dsvt_ctx* ctx, const F32Args& f, int grid, unsigned flag) {
 
 bool dsvt_layer_f32_supported(const dsvt_fused_args& a) {
   const dsvt_layer_params& p = a.p;
-  if (p.precision != DSVT_FP32) return false;
+  if (p.precision != DSVT_FP32 || !dsvt_tensor_maps_available()) return false;
   const int d = p.C / p.heads, hidden = a.attention_only ? 0 : p.hidden;
   if (hidden != 0 && hidden != p.C && hidden != 2 * p.C) return false;
   if (p.C == 192) return d == 24 && p.set_size <= 64;

@@ -1744,6 +1744,8 @@ int dsvt_launch_layers_tc(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_la
 
 int dsvt_launch_layer_tc(dsvt_ctx* ctx, const dsvt_fused_args& a) { return dsvt_launch_layers_tc(ctx, &a, 1); }
 
+bool dsvt_tensor_maps_available() { return encode_fn() != nullptr; }
+
 // Tensor map of a row-major bf16 (fp32) matrix [rows][cols] for boxes of 64 (32) columns x box_rows rows with the 128-byte
 // swizzle (the layout every operand tile here uses), from the context's cache; false if the driver entry point is
 // missing or refuses.
