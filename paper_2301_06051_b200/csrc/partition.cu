@@ -275,6 +275,13 @@ __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(const uint3
 // ---- per-window scans (Eq. 2) ------------------------------------------------------------------
 // Where the sort keys of the tile plan lie in a row-offset buffer (one per set, until the plan's order takes their place).
 __device__ __forceinline__ int32_t* plan_keys(int32_t* rowoff, int32_t cap_sets) { return rowoff + 2 * (size_t)cap_sets + 3; }
+// Whether they are written: not for more sets than a plan takes, and not where windows hold many sets, whose keys one block
+// writes at a line per key (250,000 voxels, 12 x 12 windows, sets of 4: tables for both axes 146.6 us with, 112.8 without;
+// 90,000 voxels 118.3 and 107.6; four frames with sets of 36, one or two to a window: 53.3 with, 59.0 without).
+constexpr int kPlanMaxSets = 24576;
+__device__ __forceinline__ bool writes_plan_keys(int sets, int32_t num_windows) {
+  return sets <= kPlanMaxSets && sets <= 24 * (int64_t)num_windows;
+}
 
 // Single block.  win_start = exclusive scan of N_w; win_setoff = exclusive scan of S_w = ceil(N_w / tau).
 // ITEMS: windows per thread and round (two while that covers all windows in one round, so that the block's threads share
@@ -397,8 +404,7 @@ __global__ void table_unique_count_kernel(const int32_t* __restrict__ table, int
 // plan[0] = number of tiles, plan[1 + t] = first set of tile t, plan[1 + tiles] = number of sets;
 // plan[0] = -1 if there are more sets than this kernel handles (the layer kernel then schedules by
 // row segments).  The greedy chain 0 -> next(0) -> next(next(0)) ... is found by pointer doubling, all
-// sets in parallel: single block, arrays in shared memory.
-constexpr int kPlanMaxSets = 24576;
+// sets in parallel: single block, arrays in shared memory; at most kPlanMaxSets sets.
 // Scratch of the packed plan behind the three per-set arrays: per-warp bin counts / cursors of the counting sort,
 // bin starts, the histogram (later the flags of the tile counts on trial).
 constexpr int kPackBins = 132;  // set sizes 1 .. 128, rounded up
@@ -419,7 +425,7 @@ __host__ __device__ constexpr size_t plan_smem_bytes(int smax) {
 // Written behind the plan header: the sets in tile order (order[p]) and the rows before each position (prow[p]);
 // tile t covers positions [plan[1 + t], plan[2 + t]).  Returns the number of tiles, or 0 (nothing written) if some set
 // has no row or more than max_rows, or no candidate below `limit` tiles fits.
-struct PlanWindows {  // optional: the windows behind the sets (sets of a window are consecutive), or all NULL
+struct PlanWindows {  // optional: the windows behind the sets (sets of a window are consecutive), or NULL
   const int32_t* keys;  // the rows of the largest set of each set's window; or, in the window arrays, what gives them
   const int32_t* win_setoff;
   const int32_t* win_count;
@@ -781,6 +787,7 @@ __global__ void __launch_bounds__(kScanThreads) bm_scan_kernel(const int32_t* __
     // on a cold cache (2,000 voxels 29.7 us against 21.5 now, 30,000 pillars in 30 x 30 windows 49.0 and 34.7, 32,000
     // in 12 x 12 windows 36.0 and 28.6, 200,000 skewed 79.1 and 72.8).
     int32_t* first = rowoff0 ? rowoff0 : rowoff1;
+    const bool keys = writes_plan_keys(min(win_setoff[num_windows], cap_sets), num_windows);
 #pragma unroll 1
     for (int w = threadIdx.x; w < num_windows; w += kScanThreads) {
       const int N = win_count[w];
@@ -793,7 +800,7 @@ __global__ void __launch_bounds__(kScanThreads) bm_scan_kernel(const int32_t* __
         const int v = start + (small ? (int)((unsigned)(j * N) / (unsigned)S) : (int)(((int64_t)j * N) / S));
         if (rowoff0) rowoff0[so + j] = v;
         if (rowoff1) rowoff1[so + j] = v;
-        plan_keys(first, cap_sets)[so + j] = key;
+        if (keys) plan_keys(first, cap_sets)[so + j] = key;
       }
     }
     if (threadIdx.x == 0) {
@@ -855,8 +862,9 @@ __global__ void __launch_bounds__(kScanThreads) bm_place_fill_kernel(int32_t n_m
   if (blockIdx.x == 0) {  // the plan (one for both axes: their row offsets are the same)
     int32_t* r0 = out.rowoff[0] ? out.rowoff[0] : out.rowoff[1];
     int32_t* r1 = out.rowoff[0] ? out.rowoff[1] : nullptr;
-    const PlanWindows pw{r0 ? plan_keys(r0, cap_sets) : nullptr, nullptr, nullptr, 0};
-    if (r0) tile_plan_body(r0, r1, min(*num_sets, cap_sets), cap_sets, smax, 128, pw, plan_smem, warp_tot);
+    const int S = min(*num_sets, cap_sets);
+    const PlanWindows pw{r0 && writes_plan_keys(S, num_windows) ? plan_keys(r0, cap_sets) : nullptr, win_setoff, win_count, num_windows};
+    if (r0) tile_plan_body(r0, r1, S, cap_sets, smax, 128, pw, plan_smem, warp_tot);
     return;
   }
   const int i = (blockIdx.x - 1) * blockDim.x + threadIdx.x;

@@ -169,6 +169,26 @@ def test_a_wild_row_stays_in_its_set(gpu, C, heads, window, tau, hidden, option,
     assert torch.equal(y, clean)
 
 
+@pytest.mark.parametrize("tau", [5, 6])  # 27 and 23 sets in a window: the tile plan's sort keys from the windows, from the scan
+def test_tile_plan_where_windows_hold_many_sets(gpu, oracle, tau):
+    n, grid, C = 1200, (36, 36, 1), 64
+    cfg = di.random_case(tau, n, grid, (12, 12, 1), tau, C, 4, 128, layernorm=True, bf16=True)
+    ctx = gpu.Context(n, 9, C)
+    x = dev(cfg["feats"])
+    y = torch.empty_like(x)
+    ws = [gpu.device_weights(l, gpu.BF16_FP32ACC, ctx.device) for l in cfg["blocks"][0]]
+    t0, t1 = ctx.partition_rotated(dev(cfg["coords"]), 1, grid, (12, 12, 1), tau)
+    tiles = int(t0.set_rowoff[t0.cap_sets + 1].item())
+    assert tiles & 0x40000000 and tiles & 0xffff == 10  # packed, as few as 1200 rows take
+    ctx.layers(x, [t0, t1], ws, y)
+    assert ctx.status_sync() == 0
+    want = cfg["feats"]
+    for axis in (0, 1):
+        p = oracle.partition(cfg["coords"], 1, grid, (12, 12, 1), tau, axis)
+        want = oracle.layer(want, p.set_table, cfg["blocks"][0][axis])
+    check_close(y.cpu().numpy(), want, "bf16", "sets of %d" % tau)
+
+
 def test_chain_with_other_tables_per_block(gpu, oracle):
     """Hybrid windows: the second block runs on the tables of another window cut, so a tile of its first layer
     reads rows that tiles anywhere in the previous layer wrote (the stamps are per voxel, not per window)."""
