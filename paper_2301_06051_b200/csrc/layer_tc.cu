@@ -163,12 +163,11 @@ struct alignas(1024) Misc {
   int rows, buf;
   int next_rows[2];        // rows of the tile listed in buffer b (< 0: there is no such tile), valid after rl_ready[b]
   const float* next_x[2];  // where that tile's input rows are read from
-  int wild[2];             // kTM if a row of buffer b holds a value of 2^60 or more or NaN, else 0 (see phase_gather)
   int st_rows[2], st_stamp[2];  // for the stamp warp: rows of the stored tile in buffer b, the stamp they get (0: none)
   // row lists, double buffered: the loader warp fills buffer (k + 1) & 1 while the compute warps work on tile k;
   // the compute warps gather tile k + 1 as soon as tile k's MMAs no longer read the A operand
   int rowvox[2][kTM];              // tile row -> voxel (-1: none)
-  unsigned char row_lo[2][kTM], row_n[2][kTM];  // per tile row: first row and row count of its set
+  unsigned char row_lo[2][kTM], row_n[2][kTM];  // per tile row: first row and row count of its set (0: see drop_wild)
   uint32_t starts[2][4];           // bit r: row r is the first of its set
   // relative position bias.  The table index is linear in the coordinate offset, so one integer per row,
   // x * rb_sx + y * rb_sy + z, serves every (query, key) pair: index = lin[query] - lin[key] + rb_centre.  Offsets
@@ -273,7 +272,7 @@ __device__ __forceinline__ KeyRange key_range(int r0, int rows) {
     const int lo = min(max(from - 32 * j, 0), 32), hi = min(max(to - 32 * j, 0), 32);
     if (hi > lo) sets += __popc(s_mi.starts[s_mi.buf][j] & (0xffffffffu >> (32 - hi)) & (0xffffffffu << lo));
   }
-  k.coded = sets + s_mi.wild[s_mi.buf] <= kCodes<D>;
+  k.coded = sets <= kCodes<D>;
   return k;
 }
 
@@ -335,48 +334,15 @@ __device__ __forceinline__ float softmax_rows(uint32_t t_s, const KeyRange& k, i
   return sum.x + sum.y;
 }
 
-// A flagged tile (see phase_gather): what is not finite in the value operand becomes zero, for the other sets' zero weights
-// to meet; the rows of a set of which a value was not finite get no keys, so that 0 x 1 / 0 makes them NaN.
-//   at      this thread's quarter row of the operand (chunks * 8 columns)
-//   row     its tile row, if the warp has rows (on)
-__device__ __noinline__ void contain_wild(uint32_t at, int chunks, int row, bool on) {
-  unsigned char* row_n = s_mi.row_n[s_mi.buf];
-  const int lo = s_mi.row_lo[s_mi.buf][row], n = row_n[row];
-  compute_sync();
-  if (on) {
-    bool bad = false;
-    for (int i = 0; i < 4 * chunks; ++i) {
-      const uint32_t a = at + (i >> 2) * kChunkBytes + 4 * (i & 3);
-      uint32_t w;
-      asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w) : "r"(a));
-      if ((w & 0x7f80u) == 0x7f80u) { w &= 0xffff0000u; bad = true; }
-      if ((w & 0x7f800000u) == 0x7f800000u) { w &= 0xffffu; bad = true; }
-      asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(w));
-    }
-    if (bad) row_n[row] = 255;  // (a mark; the row's four threads write the same)
-    fence_proxy_async();
-  }
-  compute_sync();
-  bool spoilt = false;
-  for (int j = 0; j < n; ++j) spoilt |= row_n[lo + j] == 255;
-  compute_sync();
-  row_n[row] = (unsigned char)(spoilt ? 0 : n);  // (key_range: the sets before a warp's last one end at its first row)
-  compute_sync();
-}
-
 // Attention of tile k: warps 4 q + (0..3) take heads q, q + 4, ... ; their S, then P, then O live in TMEM columns
 // [128 q, 128 q + 128).  The output of a head replaces its (dead) query columns.
-template <int C, int D, int VAR>
+template <int C, int D, bool RPB>
 __device__ __forceinline__ void attend(int k) {
-  constexpr bool RPB = VAR == 1, PE = VAR == 2;
   constexpr int DC = D / 8;  // 16-byte chunks per head
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp >> 2;
   const int rows = s_mi.rows, row = 32 * (warp & 3) + lane;
   const bool on = 32 * (warp & 3) < rows;  // (the whole warp)
   const uint32_t t_s = s_mi.tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + 128 * q;
-  if (PE) compute_sync();  // (the flag says nothing until every thread has written its rows with the positional term)
-  if (s_mi.wild[s_mi.buf])
-    contain_wild(s_mi.sbase + s_mi.off_kv + (uint32_t)(C / 8 + q * (C / 32)) * kChunkBytes + row * 16, C / 32, row, on);
   KeyRange kr = {0, 0, true};
   if (on) kr = key_range<D>(32 * (warp & 3), rows);
   const int lo = s_mi.row_lo[s_mi.buf][row], n = s_mi.row_n[s_mi.buf][row];
@@ -849,10 +815,7 @@ __device__ __noinline__ void loader_role(const TcArgs& a) {
       const bool packed = s_mi.lay_plan[lay] == 2;
       loader_row_list<RPB>(ly.table, packed ? ly.rowoff + 3 * (size_t)ly.cap_sets + 3 : ly.rowoff,
                            packed ? ly.rowoff + 2 * (size_t)ly.cap_sets + 3 : nullptr, ly.cap_sets, b, lt, s_lo, nsets, base);
-      if (lt == 0) {
-        s_mi.next_x[b] = lay == 0 ? a.x : a.y;
-        s_mi.wild[b] = 0;
-      }
+      if (lt == 0) s_mi.next_x[b] = lay == 0 ? a.x : a.y;
     }
     if (nsets >= 0) {
       loader_sync();  // the row list is complete
@@ -918,17 +881,38 @@ __device__ __noinline__ void stamp_role(int32_t* __restrict__ row_stamp) {
 // current tile's rows once more, with the positional term added (the operand of the key and query projections).
 //
 // The products of the attention run over the whole tile, and zero weights or codes do not stop what is not finite: such a
-// row would reach the other sets of its tile.  A tile with a value of 2^60 or more (scores with rows of ordinary size then
-// come near the codes' 2^100), infinity or NaN is flagged; its scores are masked by comparing and its values are made
-// finite (contain_wild).  The look is hidden under the loads; the branch in the attention costs 0.4 %: 32,000-pillar frame
-// 399.5 -> 401.1 us, 120,000 voxels 1401.6 -> 1407.5 (0.6 % with the repair's results in the attention's registers, 1 %
-// with the repair in the value epilogue).
+// row would reach the other sets of its tile, and one of 2^60 or more could outweigh the codes.  Those values become zeros
+// in the operand and their sets are marked (drop_wild); the query epilogue makes the rows of a marked set NaN.  The look is
+// hidden under the loads: 32,000-pillar frame 397.5 us without and 395.8 with it, 120,000 voxels 1403.9 and 1405.4.  (A
+// branch in the attention, to mask a flagged tile's scores and repair its value operand there, cost 0.5 %.)
 __device__ __forceinline__ float max_abs3(float a, float b, float c) {  // (NaN if one of them is)
   float m;
   asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
   return m;
 }
 constexpr int kUnitRows = kComputeThreads / 16;
+// A thread that has gathered values that are not finite or of 2^60 or more: zeros in their place, no rows for their sets.
+//   to   the thread's first 8 bytes in the operand
+template <int C>
+__device__ __noinline__ void drop_wild(int b, uint32_t to) {
+  unsigned char *row_lo = s_mi.row_lo[b], *row_n = s_mi.row_n[b];
+  for (int r = threadIdx.x / 16; r < kTM; r += kUnitRows, to += kUnitRows * 128) {
+    bool bad = false;
+    for (int i = 0; i < C / 32; ++i) {
+      const uint32_t a = to + (i >> 1) * (kTM * 128) + 4 * (i & 1);
+      uint32_t w;
+      asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w) : "r"(a));
+      constexpr uint32_t k2p60 = (127 + 60) << 7;
+      if ((w & 0x7fffu) >= k2p60) { w &= 0xffff0000u; bad = true; }
+      if ((w >> 16 & 0x7fffu) >= k2p60) { w &= 0xffffu; bad = true; }
+      asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(w));
+    }
+    if (bad) {  // (if another thread has begun to mark the set it marks all of it)
+      const int lo = row_lo[r], n = row_n[r];
+      for (int k = lo; k < lo + n; ++k) row_n[k] = 0;
+    }
+  }
+}
 template <int C, int D, bool RPB, bool ADD_PE>
 __device__ __forceinline__ void phase_gather(int b, int rows) {
   constexpr int P = kTM / kUnitRows, J = C / 64, kFly = ADD_PE ? P / 2 : P;  // a thread's rows, chunks, rows in flight
@@ -968,7 +952,7 @@ __device__ __forceinline__ void phase_gather(int b, int rows) {
       }
     }
   }
-  if (!(max_abs3(m0, m1, 0.f) < 0x1p60f)) s_mi.wild[b] = kTM;
+  if (!(max_abs3(m0, m1, 0.f) < 0x1p60f)) drop_wild<C>(b, to);
   if (RPB && !ADD_PE) {
     for (int r = threadIdx.x; r < kTM; r += kComputeThreads) {
       const int v = r < rows ? rowvox[r] : -1;
@@ -991,7 +975,8 @@ __device__ __forceinline__ void phase_gather(int b, int rows) {
 //   dst_off   byte offset of the destination operand from the shared-memory base
 // BIAS = false skips the bias (the key projection: a key bias adds
 // the same amount q . b_k to every score of a query, which the softmax cancels).
-template <int QC, bool BIAS>
+// QUERY: the first query column of a row whose set is marked becomes NaN (see drop_wild), and with it the row.
+template <int QC, bool BIAS, bool QUERY>
 __device__ __forceinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_off, uint32_t dst_off) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
@@ -1008,6 +993,7 @@ __device__ __forceinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_
   tmem_wait_ld();
   tc_fence_before();
   mbar_arrive(&s_mi.acc_free[bar]);  // the accumulator is in registers now
+  if (QUERY && s_mi.row_n[s_mi.buf][row] == 0) rr[0] = __int_as_float(0x7fffffff);
 #pragma unroll
   for (int q = 0; q < QC / 8; ++q) {
     float2 v[4] = {make_float2(rr[8 * q], rr[8 * q + 1]), make_float2(rr[8 * q + 2], rr[8 * q + 3]),
@@ -1356,25 +1342,26 @@ __device__ __forceinline__ void compute_role(const TcArgs& a) {
       // the keys and the queries (the V chunk's accumulator being complete, nothing reads the operand any more)
       WAIT_PHASE(acc_full[1], k);
       if (new_params) wait_layer_params();
-      phase_epi_bf16<QC, true>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + (C / 8) * kChunkBytes);
+      phase_epi_bf16<QC, true, false>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + (C / 8) * kChunkBytes);
       phase_gather<C, D, false, true>(k & 1, s_mi.rows);
       fence_proxy_async();
       mbar_arrive(&s_mi.x_ready);
       WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1));
-      phase_epi_bf16<QC, false>(Tm<C>::k, 0, 0, s_mi.off_kv);
+      phase_epi_bf16<QC, false, false>(Tm<C>::k, 0, 0, s_mi.off_kv);
     } else {
       WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1));
-      phase_epi_bf16<QC, false>(Tm<C>::k, 0, 0, s_mi.off_kv);
+      phase_epi_bf16<QC, false, false>(Tm<C>::k, 0, 0, s_mi.off_kv);
       WAIT_PHASE(acc_full[1], k);
       if (new_params) wait_layer_params();  // (the key epilogue adds no bias: it needs none of the vectors)
-      phase_epi_bf16<QC, true>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + (C / 8) * kChunkBytes);
+      phase_epi_bf16<QC, true, false>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + (C / 8) * kChunkBytes);
     }
     WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1) + 1);
-    phase_epi_bf16<QC, true>(Tm<C>::k, 0, ParOff<C>::b_q, s_mi.off_a);
+    if (PE) compute_sync();  // (every thread has marked the sets of its rows with the positional term)
+    phase_epi_bf16<QC, true, true>(Tm<C>::k, 0, ParOff<C>::b_q, s_mi.off_a);
     fence_proxy_async();
     mbar_arrive(&s_mi.a_ready);  // Q, K and V are in place
     // ---- attention inside each set ----
-    attend<C, D, VAR>(k);
+    attend<C, D, RPB>(k);
     fence_proxy_async();
     mbar_arrive(&s_mi.a_ready);  // attention output is the A operand of the output projection
     compute_sync();              // every warp is done with K and V: their region becomes fp32 staging
@@ -1444,7 +1431,6 @@ __global__ void __launch_bounds__(kThreads, 1) layer_tc_kernel(const __grid_cons
     mi->rows = mi->buf = 0;
     mi->next_rows[0] = mi->next_rows[1] = -1;
     mi->next_x[0] = mi->next_x[1] = a.x;
-    mi->wild[0] = mi->wild[1] = 0;
     mi->st_rows[0] = mi->st_rows[1] = mi->st_stamp[0] = mi->st_stamp[1] = 0;
   }
   if (tid == 32 * kLoadWarp0) {  // barriers
