@@ -548,7 +548,7 @@ def run_ours(args):
     rooflines.append({"kernel": "rotated partition (both axes; memset + 3 launches)", "config": args.config,
                       "bound": "hbm", "bytes": pb, "ms": t_p, "achieved": pb / (t_p * 1e-3) / 1e9,
                       "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": pb / (t_p * 1e-3) / 1e9 / peaks["hbm_gbs"],
-                      "note": "a few MB of traffic: bound by the latency of three dependent launches, not by HBM"})
+                      "note": "a few MB of traffic: bound by the latency of four dependent launches, not by HBM"})
     if world == 1 and args.per_config:
         t_b, bev_bytes = time_bev(cfg, ctx, dev, 10, flush)
         rooflines.append({"kernel": "BEV projection (cell-map clear + mark + dense writer)", "config": args.config,

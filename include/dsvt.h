@@ -64,8 +64,9 @@ typedef struct dsvt_ctx dsvt_ctx; /* opaque: device workspace, stream, device st
  * Creates a context on CUDA device `device` whose kernels run on `cuda_stream` (a cudaStream_t;
  * NULL = the legacy default stream).  Reserves all workspace up front for calls with at most
  * `max_voxels` voxels, `max_windows` windows (or pooling regions) per call and `max_channels`
- * feature channels; later calls allocate nothing, except dsvt_pool, which grows its dense cell
- * map once if a call's grid has more cells than any earlier call.
+ * feature channels; later calls allocate nothing, except dsvt_bev_scatter and dsvt_pool, which grow
+ * a dense cell map (which poolings of bfloat16 weights in tensor-core shapes without a counting slot
+ * term do not need) once if a call's grid has more cells than any earlier call.
  * The context must be used by one host thread at a time.
  */
 int dsvt_create(dsvt_ctx** out, int device, void* cuda_stream, int64_t max_voxels, int64_t max_windows,

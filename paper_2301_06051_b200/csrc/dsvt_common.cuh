@@ -27,11 +27,11 @@ struct dsvt_ctx {
   int32_t* vals[2];     // radix sort ping-pong voxel ids   [max_voxels]
   int32_t* hist;        // per-tile digit histograms        [256 * sort tiles + 1]
   int32_t* scan_tmp;    // block sums of the generic scan
-  uint64_t* popc_sums;
-  int32_t* win_count;   // [max_windows + 1]  (pooling: region occupancy flags)
-  int32_t* win_start;   // [max_windows + 1]  (pooling: region rank)
-  int32_t* win_setoff;  // [max_windows + 1]
-  int32_t* rowoff_a;    // [4 max_voxels + 4] row offsets + tile plan derived from a caller table
+  uint64_t* popc_sums;  // block sums of the bitmap scan       [max_windows / DSVT_POPC_TILE + 2]
+  int32_t* win_count;   // [max_windows + 1]  (pooling: bitmap of occupied cells or of non-empty regions)
+  int32_t* win_start;   // [max_windows + 1]  (pooling: cells, or regions, before each word of the bitmap)
+  int32_t* win_setoff;  // [max_windows + 1]  (pooling: regions before each word)
+  int32_t* rowoff_a;    // [4 max_voxels + 4] row offsets + tile plan derived from a caller table (pooling: row list)
   int32_t* rowoff_b;    // [4 max_voxels + 4]
   int32_t* region_key;  // [max_voxels] pooling: dense region id of each output row
   // partition, bitmap route (bm_words == 0: route not available)

@@ -1,5 +1,5 @@
 // PTX wrappers and operand-layout helpers shared by the tensor-core kernels (tcgen05 + TMEM + TMA): mbarriers with
-// bounded waits, single-CTA TMA loads, UMMA descriptors and issue, TMEM loads / stores, ldmatrix / mma.sync, and the
+// bounded waits, single-CTA TMA loads, UMMA descriptors and issue, TMEM loads / stores, shared-memory accesses, and the
 // K-major 128-byte-swizzled operand layout.
 #pragma once
 #include <cuda.h>
@@ -115,7 +115,6 @@ __device__ __forceinline__ void umma_commit(unsigned long long* bar) {
                : "memory");
 }
 
-// 32 consecutive fp32 columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // 16 fp32 columns of this thread's TMEM lane into / from elements [OFF, OFF + 16) of a register array
 // (compile-time offsets keep the array in registers).
