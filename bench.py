@@ -545,7 +545,7 @@ def run_ours(args):
     rooflines.append(layer_roof)
     t_p = float(np.median(t_part))
     pb = partition_bytes(n, S, cfg["set_size"])
-    rooflines.append({"kernel": "rotated partition (both axes; memset + 3 launches)", "config": args.config,
+    rooflines.append({"kernel": "rotated partition (both axes; four launches)", "config": args.config,
                       "bound": "hbm", "bytes": pb, "ms": t_p, "achieved": pb / (t_p * 1e-3) / 1e9,
                       "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": pb / (t_p * 1e-3) / 1e9 / peaks["hbm_gbs"],
                       "note": "a few MB of traffic: bound by the latency of four dependent launches, not by HBM"})
@@ -577,7 +577,7 @@ def run_ours(args):
                                   "frac": a_t / fma_peak, "flops": extra["flops_stage1"],
                                   "ms": extra["t_stage1_blocks_ms"],
                                   "peak_source": "measured in this run with the library's FMA probe kernel",
-                                  "note": "2,000 voxels: 56 thread blocks of work, bound by launch and memory "
+                                  "note": "2,000 voxels: 71 sets, one share of them per SM, bound by launch and memory "
                                           "latency rather than by the FMA pipes"})
             if "pool" in extra:
                 pl = extra["pool"]

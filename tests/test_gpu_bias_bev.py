@@ -208,19 +208,22 @@ def test_bias_table_narrower_than_a_set_is_flagged_on_the_tensor_core_path(gpu, 
     (1500, 48, 12, 36, 128, 8, False),  # fp32 kernel: running softmax over pairs of keys
     (1500, 48, 12, 36, 192, 8, False),
     (700, 40, 10, 36, 32, 4, False),    # general-shape kernel
+    (2500, 60, 12, 36, 192, 8, True),   # set codes keep the sets of a tile apart
+    (1500, 48, 3, 9, 64, 4, True),      # more sets in a warp's key range than there are codes
 ])
 @pytest.mark.parametrize("mask", [-np.inf, np.finfo(np.float32).min, -1e31])
 def test_bias_that_masks_offsets(gpu, oracle, n, grid, window, tau, C, heads, bf16, mask):
-    """Table entries that rule offsets out.  Heads 1 and 2 keep the voxel itself and every fourth offset; with a finite
-    mask head 0 masks every offset alike, which leaves equal weights inside the set and nothing outside it.  (The lowest
-    float overflows when it is scaled to the unscaled logits: a row of it alone has no defined result.)"""
+    """Table entries that rule offsets out.  Heads 1 and 2 keep the voxel itself and every fourth offset; in fp32 with
+    -1e31 head 0 masks every offset alike, which leaves equal weights inside the set and nothing outside it.  (The lowest
+    float overflows when it is scaled to the unscaled logits, and the tensor-core kernel's exponent of -1e31 less itself is
+    its rounding error: rows of them alone have no defined result.)"""
     cfg = di.random_case(n, n, (grid, grid, 1), (window, window, 1), tau, C, heads, bf16=bf16)
     rng = np.random.default_rng(n + C)
     L = _with_bias(rng, cfg["blocks"][0][0], heads, (window, window, 1), oracle)
     keep = rng.random(L["rpb"].shape[1]) < 0.25
     keep[L["rpb"].shape[1] // 2] = True  # offset zero
     L["rpb"][1:3, ~keep] = mask
-    if mask == -1e31:
+    if mask == -1e31 and not bf16:
         L["rpb"][0] = mask
     ctx = gpu.Context(n, _nwin(1, cfg["grid"], cfg["window"]), C)
     x, coords = dev(cfg["feats"]), dev(cfg["coords"])
