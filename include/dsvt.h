@@ -233,7 +233,8 @@ int dsvt_partition_noalloc(void* cuda_stream, const int32_t* coords, int32_t n, 
  *   heads       head h owns channels [h*d, (h+1)*d), d = C / heads; logits are scaled by 1/sqrt(d).
  *   pe          optional float [n][C] positional term, added to the input of the query and key maps only.
  *
- * A voxel with features that are not finite spoils the rows of its own set and no others.
+ * A voxel with features that are not finite spoils the rows of its own set and no others.  (With bfloat16 weights in
+ * tensor-core shapes, see dsvt_layer, features of 2^60 or more in magnitude count as not finite.)
  *
  * Needs C % 8 == 0, (C/heads) % 4 == 0, set_size <= 128 (else DSVT_ERR_UNSUPPORTED).
  */
