@@ -22,7 +22,8 @@
  *     dsvt_status_sync reports it.
  *   - No call throws, aborts, or frees caller memory.
  *   - Matrices are row-major; a linear map is y = W x + b with W stored [out][in].
- *   - precision = DSVT_FP32: weights are float, arithmetic is fp32 throughout.
+ *   - precision = DSVT_FP32: weights are float, arithmetic is fp32 throughout; in the shapes that the tensor cores take (C of
+ *     64, 128, 192) a product's operands go in as three bfloat16 parts each, which hold all of their 24 bits.
  *     precision = DSVT_BF16_FP32ACC: weights are bfloat16 (16-bit storage); products
  *     accumulate in fp32; residual stream, LayerNorm, softmax and GELU are fp32.
  *     Features (x, y, feats, out) and biases / LayerNorm parameters are always float.

@@ -28,10 +28,9 @@ void carve(dsvt_ctx* c, unsigned char* base, size_t* total) {
   if (nw + 1 > longest_scan) longest_scan = nw + 1;
   if (nv + 1 > longest_scan) longest_scan = nv + 1;
   c->status = k.take<int32_t>(64);
-  c->keys[0] = k.take<uint32_t>(nv);
-  c->keys[1] = k.take<uint32_t>(nv);
-  c->vals[0] = k.take<int32_t>(nv);
-  c->vals[1] = k.take<int32_t>(nv);
+  const size_t ns = nv > 1024 ? nv : 1024;
+  for (int i = 0; i < 2; ++i) c->keys[i] = k.take<uint32_t>(ns);
+  for (int i = 0; i < 2; ++i) c->vals[i] = k.take<int32_t>(ns);
   c->hist = k.take<int32_t>(hist);
   c->scan_tmp = k.take<int32_t>(longest_scan / 8192 + 2);
   c->popc_sums = k.take<uint64_t>(nw / DSVT_POPC_TILE + 2);
@@ -95,7 +94,7 @@ int run_layer(dsvt_ctx* ctx, const float* x, int32_t n, const int32_t* table, in
     a.rowoff = rowoff_scratch;
   }
   if (tc) return dsvt_launch_layer_tc(ctx, a);
-  if (dsvt_layer_f32_supported(a)) return dsvt_launch_layer_f32(ctx, a);
+  if (dsvt_layer_f32_supported(a)) return dsvt_launch_layers_f32(ctx, &a, 1);
   return dsvt_launch_layer_fma(ctx, a);
 }
 
@@ -110,14 +109,16 @@ int check_common(const dsvt_ctx* ctx, const float* x, const float* y, int32_t n,
 
 
 // A chain of layers, layer i on tables[i]: layer 0 reads x and writes y, the later ones run in place on y.
-// Consecutive layers of one shape that the tensor-core kernel covers share a launch; the rest run one by one.
+// Consecutive layers of one shape that the tensor-core kernel covers share a launch, consecutive fp32 layers their row
+// lists; the rest run one by one.
 int run_layers(dsvt_ctx* ctx, const float* x, int32_t n, int32_t num_layers, const dsvt_table_ref* tables,
                const dsvt_layer_params* params, float* y) {
   dsvt_fused_args chain[DSVT_MAX_CHAIN_LAYERS];
   int len = 0;
+  bool tc_chain = false;
   auto flush = [&]() -> int {
     if (len == 0) return DSVT_OK;
-    const int rc = dsvt_launch_layers_tc(ctx, chain, len);
+    const int rc = tc_chain ? dsvt_launch_layers_tc(ctx, chain, len) : dsvt_launch_layers_f32(ctx, chain, len);
     len = 0;
     return rc;
   };
@@ -130,11 +131,13 @@ int run_layers(dsvt_ctx* ctx, const float* x, int32_t n, int32_t num_layers, con
     a.p = params[i];
     a.attention_only = 0;
     const bool tc = t.set_rowoff != nullptr && dsvt_layer_tc_supported(a);
-    if (len > 0 && (!tc || len == DSVT_MAX_CHAIN_LAYERS || !dsvt_layer_tc_chainable(chain[0], a))) {
+    const bool f32 = t.set_rowoff != nullptr && !tc && dsvt_layer_f32_supported(a);
+    if (len > 0 && (tc != tc_chain || !(tc || f32) || len == DSVT_MAX_CHAIN_LAYERS || (tc && !dsvt_layer_tc_chainable(chain[0], a)))) {
       const int rc = flush();
       if (rc != DSVT_OK) return rc;
     }
-    if (tc) {
+    if (tc || f32) {
+      tc_chain = tc;
       chain[len++] = a;
       continue;
     }

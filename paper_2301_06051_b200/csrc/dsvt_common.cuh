@@ -19,12 +19,13 @@ struct dsvt_ctx {
   int last_cuda_error;
   unsigned attr_flags;  // kernels whose shared-memory attribute has been raised on this context's device
   int64_t launches;
-  // one device allocation carved into the arrays below
+  // one device allocation carved into the arrays below.  The partition's own (keys and vals, each pair in one piece; bm_zero and
+  // bm_wordrank, in one piece) hold nothing between calls and are the fp32 layers' workspace (layer_f32.cu).
   void* arena;
   size_t arena_bytes;
   int32_t* status;      // device status word
-  uint32_t* keys[2];    // radix sort ping-pong keys        [max_voxels]
-  int32_t* vals[2];     // radix sort ping-pong voxel ids   [max_voxels]
+  uint32_t* keys[2];    // radix sort ping-pong keys        [max(max_voxels, 1024)]
+  int32_t* vals[2];     // radix sort ping-pong voxel ids   [max(max_voxels, 1024)]
   int32_t* hist;        // per-tile digit histograms        [256 * sort tiles + 1]
   int32_t* scan_tmp;    // block sums of the generic scan
   uint64_t* popc_sums;  // block sums of the bitmap scan       [max_windows / DSVT_POPC_TILE + 2]
@@ -41,7 +42,7 @@ struct dsvt_ctx {
   int32_t* bm_dup;       // [max_voxels] -1, or the voxel's ticket among the duplicates of its window
   // tensor-core layer kernel: tile counter of a launch ([0] next tile, [1] CTAs that have left; zero between
   // launches), per-voxel completion stamps of a chain of layers, and the serial number the stamps are built from
-  int32_t* tc_counter;   // [2]
+  int32_t* tc_counter;   // [2], then the fp32 attention's [1]
   int32_t* row_stamp;    // [max_voxels]
   uint32_t stamp_serial;
   dsvt_map_cache* maps;
@@ -74,9 +75,11 @@ struct dsvt_ctx {
 // predecessor in the stream still runs; it lets its own successor start early and then waits for the predecessor
 // (and everything before it) to have completed and flushed.  Both are no-ops in an ordinary launch.
 #ifdef __CUDACC__
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_launch();
+  pdl_wait();
 }
 #endif
 
@@ -131,10 +134,12 @@ struct dsvt_fused_args {
   dsvt_layer_params p;
   int32_t attention_only;  // 1: y = attention output (no residual, LN, MLP)
 };
-int dsvt_launch_layer_fma(dsvt_ctx* ctx, const dsvt_fused_args& a);
-// fp32 weights, C in {64, 128, 192}, hidden in {0, C, 2C} (layer_f32.cu); everything else is layer_fma.cu's.
+// (the sets whose first row, in the order of the table, is from_row or later)
+int dsvt_launch_layer_fma(dsvt_ctx* ctx, const dsvt_fused_args& a, int64_t from_row = 0);
+// fp32 weights, C in {64, 128, 192}, hidden a multiple of 64 (layer_f32.cu); everything else is layer_fma.cu's.  Layers one
+// after the other: a layer reads its own x, whatever wrote it.
 bool dsvt_layer_f32_supported(const dsvt_fused_args& a);
-int dsvt_launch_layer_f32(dsvt_ctx* ctx, const dsvt_fused_args& a);
+int dsvt_launch_layers_f32(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_layers);
 // tcgen05 path: bfloat16 weights, C in {64, 128, 192}, head dim in {16, 24, 32}, set size <= 96.
 bool dsvt_layer_tc_supported(const dsvt_fused_args& a);
 int dsvt_launch_layer_tc(dsvt_ctx* ctx, const dsvt_fused_args& a);
@@ -143,12 +148,9 @@ int dsvt_launch_layer_tc(dsvt_ctx* ctx, const dsvt_fused_args& a);
 // DSVT_MAX_CHAIN_LAYERS layers; every voxel a later layer reads must be written by the layer before it.
 bool dsvt_layer_tc_chainable(const dsvt_fused_args& a, const dsvt_fused_args& b);
 int dsvt_launch_layers_tc(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_layers);
-// Whether the driver offers the entry point that encodes tensor maps.
-bool dsvt_tensor_maps_available();
-// CUtensorMap (128 bytes, 64-byte aligned) of a row-major bf16 (fp32) matrix [rows][cols]: boxes of 64 (32) columns x
-// box_rows rows, 128-byte swizzle; encoded once per matrix and context.  Returns false if the driver cannot encode it.
-bool dsvt_cached_weight_map(dsvt_ctx* ctx, void* tensor_map, const void* w, int rows, int cols, int box_rows,
-                            bool fp32 = false);
+// CUtensorMap (128 bytes, 64-byte aligned) of a row-major bf16 matrix [rows][cols]: boxes of 64 columns x box_rows rows,
+// 128-byte swizzle; encoded once per matrix and context.  Returns false if the driver cannot encode it.
+bool dsvt_cached_weight_map(dsvt_ctx* ctx, void* tensor_map, const void* w, int rows, int cols, int box_rows);
 
 // Attention-style pooling with the projections on tcgen05 (pool_tc.cu): bfloat16 weights, C / head dim as for the
 // layer kernel, a power-of-two number of slots per region (at most 32).  The region bookkeeping (row list or cell map

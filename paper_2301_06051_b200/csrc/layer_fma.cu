@@ -22,6 +22,7 @@ struct FmaGeom {
   int TMn;   // nominal rows per tile: a set belongs to the tile its first row falls in
   int LDQ;   // row stride of the wide buffer (>= 3C, LDQ % 32 == 4)
   int C, hidden, heads, d, tau;
+  int from;  // sets whose first row lies before this one are left out
   // relative position bias: entries per head, strides of the x and y offsets, index of the zero offset
   int rb_len, rb_sx, rb_sy, rb_centre;
 };
@@ -71,16 +72,17 @@ layer_fma_kernel(dsvt_fused_args a, FmaGeom g, int32_t* __restrict__ status) {
   const WT* W1 = reinterpret_cast<const WT*>(p.W_1);
   const WT* W2 = reinterpret_cast<const WT*>(p.W_2);
 
+  pdl_enter();  // everything below may read what earlier kernels of the stream wrote
   const int S = min(*a.num_sets, a.cap_sets);
   if (S <= 0) return;
   const int R = a.rowoff[S];
-  const int num_tiles = (R + g.TMn - 1) / g.TMn;
+  const int num_tiles = (R - g.from + g.TMn - 1) / g.TMn;
 
   for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
     __syncthreads();
     if (tid == 0) {
-      // sets whose first row lies in [t*TMn, (t+1)*TMn)
-      const int lo_row = t * g.TMn, hi_row = lo_row + g.TMn;
+      // sets whose first row lies in [from + t*TMn, from + (t+1)*TMn)
+      const int lo_row = g.from + t * g.TMn, hi_row = lo_row + g.TMn;
       int lo = 0, hi = S;
       while (lo < hi) { const int m = (lo + hi) >> 1; if (a.rowoff[m] < lo_row) lo = m + 1; else hi = m; }
       const int s_lo = lo;
@@ -289,7 +291,7 @@ int launch_one(dsvt_ctx* ctx, const dsvt_fused_args& a, const FmaGeom& g, int gr
   const size_t smem = fma_smem_bytes(g);
   cudaError_t e = cudaFuncSetAttribute(layer_fma_kernel<WT, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) { ctx->last_cuda_error = (int)e; return DSVT_ERR_CUDA; }
-  layer_fma_kernel<WT, RM><<<grid, kThreads, smem, ctx->stream>>>(a, g, ctx->status);
+  DSVT_CUDA_TRY(ctx, launch_pdl(layer_fma_kernel<WT, RM>, dim3((unsigned)grid), dim3(kThreads), smem, ctx->stream, a, g, ctx->status));
   DSVT_LAUNCHED(ctx);
   return DSVT_OK;
 }
@@ -309,7 +311,7 @@ int launch_rm(dsvt_ctx* ctx, const dsvt_fused_args& a, const FmaGeom& g, int gri
 
 }  // namespace
 
-int dsvt_launch_layer_fma(dsvt_ctx* ctx, const dsvt_fused_args& a) {
+int dsvt_launch_layer_fma(dsvt_ctx* ctx, const dsvt_fused_args& a, int64_t from_row) {
   const dsvt_layer_params& p = a.p;
   FmaGeom g;
   g.C = p.C; g.hidden = a.attention_only ? 0 : p.hidden; g.heads = p.heads; g.d = p.C / p.heads; g.tau = p.set_size;
@@ -331,6 +333,7 @@ int dsvt_launch_layer_fma(dsvt_ctx* ctx, const dsvt_fused_args& a) {
   }
   if (g.TM == 0) return DSVT_ERR_UNSUPPORTED;
   g.TMn = g.TM - g.tau + 1;
+  g.from = (int)from_row;
   int64_t rmax = (int64_t)a.cap_sets * g.tau;
   if (rmax > a.n) rmax = a.n;
   int64_t grid = dsvt_ceil_div(rmax, g.TMn);

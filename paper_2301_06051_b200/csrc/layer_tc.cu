@@ -1535,15 +1535,15 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// bf16 (fp32) matrix [rows][cols] row-major; box = 64 (32) columns x box_rows rows, 128-byte swizzle.
-bool make_weight_map(CUtensorMap* m, const void* w, int rows, int cols, int box_rows, bool fp32) {
+// bf16 matrix [rows][cols] row-major; box = 64 columns x box_rows rows, 128-byte swizzle.
+bool make_weight_map(CUtensorMap* m, const void* w, int rows, int cols, int box_rows) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)cols * (fp32 ? 4 : 2)};
-  const cuuint32_t box[2] = {fp32 ? 32u : 64u, (cuuint32_t)box_rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
+  const cuuint32_t box[2] = {64u, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1u, 1u};
-  return fn(m, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(w), dims, strides, box, estr,
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(w), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -1556,7 +1556,6 @@ struct dsvt_map_cache {
   struct Entry {
     const void* w;
     int rows, cols, box_rows;
-    bool fp32;
     CUtensorMap map;
   };
   std::vector<Entry> entries;
@@ -1567,15 +1566,15 @@ void dsvt_map_cache_destroy(dsvt_map_cache* c) { delete c; }
 
 namespace {
 
-bool cached_weight_map(dsvt_ctx* ctx, CUtensorMap* out, const void* w, int rows, int cols, int box_rows, bool fp32 = false) {
+bool cached_weight_map(dsvt_ctx* ctx, CUtensorMap* out, const void* w, int rows, int cols, int box_rows) {
   if (!ctx->maps) ctx->maps = new (std::nothrow) dsvt_map_cache();
   if (!ctx->maps) return false;
   auto& v = ctx->maps->entries;
   for (const auto& e : v)
-    if (e.w == w && e.rows == rows && e.cols == cols && e.box_rows == box_rows && e.fp32 == fp32) { *out = e.map; return true; }
+    if (e.w == w && e.rows == rows && e.cols == cols && e.box_rows == box_rows) { *out = e.map; return true; }
   dsvt_map_cache::Entry e;
-  e.w = w; e.rows = rows; e.cols = cols; e.box_rows = box_rows; e.fp32 = fp32;
-  if (!make_weight_map(&e.map, w, rows, cols, box_rows, fp32)) return false;
+  e.w = w; e.rows = rows; e.cols = cols; e.box_rows = box_rows;
+  if (!make_weight_map(&e.map, w, rows, cols, box_rows)) return false;
   if (v.size() >= 256) v.erase(v.begin(), v.begin() + 128);  // (a caller that keeps changing its weights)
   v.push_back(e);
   *out = e.map;
@@ -1730,11 +1729,8 @@ int dsvt_launch_layers_tc(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_la
 
 int dsvt_launch_layer_tc(dsvt_ctx* ctx, const dsvt_fused_args& a) { return dsvt_launch_layers_tc(ctx, &a, 1); }
 
-bool dsvt_tensor_maps_available() { return encode_fn() != nullptr; }
-
-// Tensor map of a row-major bf16 (fp32) matrix [rows][cols] for boxes of 64 (32) columns x box_rows rows with the 128-byte
-// swizzle (the layout every operand tile here uses), from the context's cache; false if the driver entry point is
-// missing or refuses.
-bool dsvt_cached_weight_map(dsvt_ctx* ctx, void* tensor_map, const void* w, int rows, int cols, int box_rows, bool fp32) {
-  return cached_weight_map(ctx, reinterpret_cast<CUtensorMap*>(tensor_map), w, rows, cols, box_rows, fp32);
+// Tensor map of a row-major bf16 matrix [rows][cols] for boxes of 64 columns x box_rows rows with the 128-byte swizzle (the
+// layout every operand tile here uses), from the context's cache; false if the driver entry point is missing or refuses.
+bool dsvt_cached_weight_map(dsvt_ctx* ctx, void* tensor_map, const void* w, int rows, int cols, int box_rows) {
+  return cached_weight_map(ctx, reinterpret_cast<CUtensorMap*>(tensor_map), w, rows, cols, box_rows);
 }

@@ -17,6 +17,9 @@ pytestmark = pytest.mark.gpu
     (3000, 60, 30, 96, 128, 4, 256, ""),      # tiles of up to 96 rows, head dim 32
     (9000, 100, 12, 36, 64, 4, 128, "pe"),    # several tiles per block
     (20000, 150, 12, 36, 128, 8, 128, "rpb"),
+    (700, 36, 12, 36, 192, 8, 256, ""),       # a deep second product of two equal chunks and a short one
+    (14001, 150, 12, 36, 192, 8, 64, "pe"),   # two passes; the narrowest tile of the first MLP product
+    (45000, 240, 12, 48, 64, 4, 64, ""),      # two passes of many tiles per block
 ])
 def test_layer_fp32_matches_oracle(oracle, n, grid, window, tau, C, heads, hidden, option):
     from paper_2301_06051_b200 import api
@@ -64,3 +67,44 @@ def test_row_offsets_that_claim_more_rows_than_a_set_has(oracle, C, heads, hidde
     others = np.setdiff1d(np.arange(n), p.set_table[long])
     want = oracle.layer(case["feats"], p.set_table, layer)
     check_close(y.cpu().numpy()[others], want[others], "fp32", "the other sets")
+
+
+def test_voxels_in_many_sets_take_the_general_kernel(oracle):
+    """A table with more rows than there are voxels (every set eight times over): the sets past the workspace's passes run on
+    the kernel for general shapes, with the same results."""
+    from paper_2301_06051_b200 import api
+
+    n, tau, C, heads, hidden = 300, 36, 128, 8, 256
+    case = di.random_case(7, n, (36, 36, 1), (12, 12, 1), tau, C, heads, hidden, layernorm=True)
+    layer = case["blocks"][0][0]
+    p = oracle.partition(case["coords"], 1, case["grid"], case["window"], tau, 0)
+    table = np.concatenate([p.set_table] * 8)
+    ctx = api.Context(n, 9, C)
+    x = dev(case["feats"])
+    y = torch.empty_like(x)
+    ctx.layer(x, upload_table(table), api.device_weights(layer, api.FP32, ctx.device), y)
+    assert ctx.status_sync() == 0
+    check_close(y.cpu().numpy(), oracle.layer(case["feats"], p.set_table, layer), "fp32", "voxels in many sets")
+
+
+def test_chain_of_fp32_layers_on_several_tables(oracle):
+    """Layers in one call share row lists and prepared weights, two at a time: five layers on three tables."""
+    from paper_2301_06051_b200 import api
+
+    n, tau, C, heads = 900, 36, 64, 4
+    case = di.random_case(11, n, (48, 48, 1), (12, 12, 1), tau, C, heads, 128, layernorm=True)
+    rng = np.random.default_rng(11)
+    layers = [di.make_layer(rng, C, heads, 128, True, False) for _ in range(5)]
+    ctx = api.Context(n, 16, C)
+    coords, x = dev(case["coords"]), dev(case["feats"])
+    t = [ctx.partition(coords, 1, case["grid"], w, tau, a) for w, a in (((12, 12, 1), 0), ((12, 12, 1), 1), ((16, 16, 1), 0))]
+    r = [oracle.partition(case["coords"], 1, case["grid"], w, tau, a).set_table
+         for w, a in (((12, 12, 1), 0), ((12, 12, 1), 1), ((16, 16, 1), 0))]
+    order = [0, 1, 2, 2, 0]
+    y = torch.empty_like(x)
+    ctx.layers(x, [t[i] for i in order], [api.device_weights(l, api.FP32, ctx.device) for l in layers], y)
+    assert ctx.status_sync() == 0
+    want = case["feats"].astype(np.float64)
+    for i, l in zip(order, layers):
+        want = oracle.layer(want, r[i], l)
+    check_close(y.cpu().numpy(), want, "fp32", "five layers")
