@@ -300,6 +300,29 @@ __device__ __forceinline__ KeyRange key_range(int r0, int rows) {
 // pairs, columns [t_s, t_s + 64), zeros outside the warp's key blocks).  Returns the row's sum.  P overwrites S: block
 // b's 8 columns lie in S blocks up to b, which have been read by then.
 // [lo, lo + n): the rows of this row's set, by which keys are masked where the codes do not do it (!coded).
+// Pairs of a block's 16 exponentials (bits) that the FMA pipe forms: an exponential takes the MUFU as long as four FMA
+// instructions issue, and 80 of them per row are half of the attention.  A quarter is best: 32,000 pillars 384.2 us with none, 383.3 with
+// one pair of eight, 379.4 with two, 384.6 with three, 390.0 with four; 120,000 voxels 1373.6 with none, 1355.2 with two.
+constexpr uint32_t kFmaPairs = 0x88;
+
+// 2^u for u <= 127, by the FMA pipe: 2^round(u) into the exponent of a minimax polynomial of degree 5 (relative error 7.5e-8; 2.1e-7
+// with fp32's roundings).  Below -125, masked scores among them, it is 2^-125.
+__device__ __forceinline__ float2 ex2_fma2(float2 u) {
+  constexpr float kMagic = 12582912.0f;  // 1.5 2^23: the sum's low bits are the rounded integer
+  auto two = [](float v) { return make_float2(v, v); };
+  u = make_float2(fmaxf(u.x, -125.0f), fmaxf(u.y, -125.0f));
+  const float2 t = __fadd2_rn(u, two(kMagic));
+  const float2 n = __fadd2_rn(t, two(-kMagic));
+  const float2 f = __ffma2_rn(n, two(-1.0f), u);
+  float2 p = __ffma2_rn(two(1.327647205e-03f), f, two(9.675541385e-03f));
+  p = __ffma2_rn(p, f, two(5.550713274e-02f));
+  p = __ffma2_rn(p, f, two(2.402211972e-01f));
+  p = __ffma2_rn(p, f, two(6.931469671e-01f));
+  p = __ffma2_rn(p, f, two(1.000000072e+00f));
+  return make_float2(__uint_as_float(__float_as_uint(p.x) + (__float_as_uint(t.x) << 23)),
+                     __uint_as_float(__float_as_uint(p.y) + (__float_as_uint(t.y) << 23)));
+}
+
 struct Softmax {
   uint32_t t_s;
   float sc, off;  // exponents are s sc + off
@@ -317,7 +340,7 @@ struct Softmax {
     for (int i = 0; i < 8; ++i) {
       float2 u = make_float2(s[2 * i], s[2 * i + 1]);
       if (!SCALED) u = __ffma2_rn(u, make_float2(sc, sc), make_float2(off, off));
-      const float2 e = make_float2(ex2_approx(u.x), ex2_approx(u.y));
+      const float2 e = SCALED && (kFmaPairs >> i & 1) ? ex2_fma2(u) : make_float2(ex2_approx(u.x), ex2_approx(u.y));
       sum = __fadd2_rn(sum, e);
       p[i] = pack_bf16(e.x, e.y);
     }
@@ -362,8 +385,8 @@ __device__ __forceinline__ void softmax_rows(Softmax& sm, const KeyRange& k, int
 }
 
 // Without: every |q| |k| of the warp's rows and the tile's keys is at most kOnceBound, so that the exponentials lie in
-// [2^-32, 2^32] and sums and products are as exact as with a maximum taken off.  The next block is loaded under this one's
-// exponentials.
+// [2^-32, 2^32] (masked ones at 2^-125 or 0) and sums and products are as exact as with a maximum taken off.  The next block is
+// loaded under this one's exponentials.  32,000 pillars 397 -> 388.5 us against the two passes above.
 constexpr float kOnceBound = 32.0f;
 __device__ __forceinline__ void softmax_once(Softmax& sm, const KeyRange& k) {
   const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
@@ -416,7 +439,7 @@ __device__ __forceinline__ void attend(int k, const float (&query_norm)[2]) {
       const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
       for (int b = kr.kb1; b < (rows + 15) >> 4; ++b) tmem_st8_u32(t_s + 8 * b, zero);
       tmem_wait_st();
-      l = sm.sum.x + sm.sum.y;
+      l = n > 0 ? sm.sum.x + sm.sum.y : __int_as_float(0x7fffffff);  // (a marked set: no key at all where its keys are masked)
     }
     tc_fence_before();
     mbar_arrive(&s_mi.p_ready[q]);
