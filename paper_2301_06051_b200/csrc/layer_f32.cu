@@ -17,8 +17,8 @@
 // where the kernel on the FMA pipes was off by 1.2e-7 ... 3.9e-7.
 //
 // Measured (B200): two full layers and their partition, 12,345 pillars, C = 192: 776 us on the FMA pipes (27 % of their peak:
-// shared-memory reads for the products, and the phases between them), 288 us now; two attention-only layers, 2,000 pillars,
-// C = 128: 109 us and 90 us.  A product's tile of 128 rows takes 9 to 11 k cycles, the start of each of its kernels 4 k
+// shared-memory reads for the products, and the phases between them), 282 us now; two attention-only layers, 2,000 pillars,
+// C = 128: 109 us and 91 us.  A product's tile of 128 rows takes 9 to 11 k cycles, the start of each of its kernels 4 k
 // (first instructions, lists, operands) and its epilogue 6 k.
 //
 // Every wait is bounded; one that gives up raises DSVT_STATUS_TIMEOUT, and the block stores nothing more.
@@ -32,12 +32,12 @@ namespace {
 using namespace dsvt_tc;
 
 // Warps: epilogue (two threads to a row of the tile), conversion of the operand rows, weight copies, MMA issue.
-constexpr int kEpiThreads = 2 * kTM, kConvThreads = 128;
+constexpr int kEpiThreads = 2 * kTM, kConvThreads = 256;
 constexpr int kConvWarp = kEpiThreads / 32, kCopyWarp = kConvWarp + kConvThreads / 32, kMmaWarp = kCopyWarp + 1;
 constexpr int kThreads = 32 * (kMmaWarp + 1);
 constexpr int kKS = 16;        // k per operand stage: one MMA step
 constexpr int kSt = 4;         // stages
-constexpr int kFly = 3;        // stages of operand rows in a converting thread's registers
+constexpr int kFly = 3;        // stages of operand rows in a converting thread's registers (4: 281.6 us, 6: 284.7)
 constexpr int kParts = 3;      // bfloat16 parts of an operand
 constexpr int kChunk = 96 / kKS;  // most stages between two readings of the leading accumulator
 constexpr uint32_t kCorr = 256;  // TMEM column of the accumulator of the small products (the leading one is at 0)
