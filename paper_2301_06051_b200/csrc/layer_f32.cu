@@ -32,6 +32,8 @@ namespace {
 using namespace dsvt_tc;
 
 // Warps: epilogue (two threads to a row of the tile), conversion of the operand rows, weight copies, MMA issue.
+// (Eight warps convert: with four a stage's conversion takes longer than its MMAs; two full layers of 12,345 pillars 287.6 us with
+// four, 281.3 with eight.)
 constexpr int kEpiThreads = 2 * kTM, kConvThreads = 256;
 constexpr int kConvWarp = kEpiThreads / 32, kCopyWarp = kConvWarp + kConvThreads / 32, kMmaWarp = kCopyWarp + 1;
 constexpr int kThreads = 32 * (kMmaWarp + 1);
