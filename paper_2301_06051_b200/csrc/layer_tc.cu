@@ -177,10 +177,7 @@ struct alignas(1024) Misc {
   const float* rpb;
   const int4* coords;
   int rb_len, rb_sx, rb_sy, rb_centre, rb_ext[3];
-  union {
-    alignas(16) short rowlin[kTM];
-    uint32_t key_norm[kComputeWarps][2];  // without a bias: squares (float bits) of the largest key norms of a warp's rows, per head
-  };
+  alignas(16) short rowlin[kTM];
   alignas(16) float par[6 * 192];
 };
 static_assert(sizeof(Misc) == 7 * 1024, "shared memory");
@@ -272,10 +269,6 @@ __device__ __forceinline__ void write_codes(int b, int rows) {
   }
 }
 
-// Queries are scaled to give exponents of two, log2(e) / sqrt(d) q k (not with a position bias, which is added to the bare scores).
-template <int D, bool RPB>
-__device__ __forceinline__ float query_scale() { return RPB ? 1.0f : 1.4426950408889634f * rsqrtf((float)D); }
-
 // The keys of a warp's 32 rows: blocks of 16 tile rows [kb0, kb1), and whether the codes keep their sets apart.
 struct KeyRange { int kb0, kb1; bool coded; };
 template <int D>
@@ -300,58 +293,14 @@ __device__ __forceinline__ KeyRange key_range(int r0, int rows) {
 // pairs, columns [t_s, t_s + 64), zeros outside the warp's key blocks).  Returns the row's sum.  P overwrites S: block
 // b's 8 columns lie in S blocks up to b, which have been read by then.
 // [lo, lo + n): the rows of this row's set, by which keys are masked where the codes do not do it (!coded).
-// Pairs of a block's 16 exponentials (bits) that the FMA pipe forms: an exponential takes the MUFU as long as four FMA
-// instructions issue, and 80 of them per row are half of the attention.  A quarter is best: 32,000 pillars 384.2 us with none, 383.3 with
-// one pair of eight, 379.4 with two, 384.6 with three, 390.0 with four; 120,000 voxels 1373.6 with none, 1355.2 with two.
-constexpr uint32_t kFmaPairs = 0x88;
-
-// 2^u for u <= 127, by the FMA pipe: 2^round(u) into the exponent of a minimax polynomial of degree 5 (relative error 7.5e-8; 2.1e-7
-// with fp32's roundings).  Below -125, masked scores among them, it is 2^-125.
-__device__ __forceinline__ float2 ex2_fma2(float2 u) {
-  constexpr float kMagic = 12582912.0f;  // 1.5 2^23: the sum's low bits are the rounded integer
-  auto two = [](float v) { return make_float2(v, v); };
-  u = make_float2(fmaxf(u.x, -125.0f), fmaxf(u.y, -125.0f));
-  const float2 t = __fadd2_rn(u, two(kMagic));
-  const float2 n = __fadd2_rn(t, two(-kMagic));
-  const float2 f = __ffma2_rn(n, two(-1.0f), u);
-  float2 p = __ffma2_rn(two(1.327647205e-03f), f, two(9.675541385e-03f));
-  p = __ffma2_rn(p, f, two(5.550713274e-02f));
-  p = __ffma2_rn(p, f, two(2.402211972e-01f));
-  p = __ffma2_rn(p, f, two(6.931469671e-01f));
-  p = __ffma2_rn(p, f, two(1.000000072e+00f));
-  return make_float2(__uint_as_float(__float_as_uint(p.x) + (__float_as_uint(t.x) << 23)),
-                     __uint_as_float(__float_as_uint(p.y) + (__float_as_uint(t.y) << 23)));
-}
-
-struct Softmax {
-  uint32_t t_s;
-  float sc, off;  // exponents are s sc + off
-  int lo, n;
-  float2 sum;
-  __device__ __forceinline__ void mask(float (&s)[16], int b) const {
+template <int D, bool RPB>
+__device__ __forceinline__ float softmax_rows(uint32_t t_s, const KeyRange& k, int n_blocks, int row, int lo, int n, int h) {
+  const float sc = 1.4426950408889634f * rsqrtf((float)D);  // log2(e) / sqrt(d)
+  auto mask = [&](float (&s)[16], int b) {
 #pragma unroll
     for (int i = 0; i < 16; ++i)
       if ((unsigned)(16 * b + i - lo) >= (unsigned)n) s[i] = -INFINITY;
-  }
-  template <bool SCALED>
-  __device__ __forceinline__ void block(const float (&s)[16], int b) {
-    uint32_t p[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      float2 u = make_float2(s[2 * i], s[2 * i + 1]);
-      if (!SCALED) u = __ffma2_rn(u, make_float2(sc, sc), make_float2(off, off));
-      const float2 e = SCALED && (kFmaPairs >> i & 1) ? ex2_fma2(u) : make_float2(ex2_approx(u.x), ex2_approx(u.y));
-      sum = __fadd2_rn(sum, e);
-      p[i] = pack_bf16(e.x, e.y);
-    }
-    tmem_st8_u32(t_s + 8 * b, p);
-  }
-};
-
-// With a look for the row's maximum first.
-template <int D, bool RPB>
-__device__ __forceinline__ void softmax_rows(Softmax& sm, const KeyRange& k, int row, int h) {
-  const uint32_t t_s = sm.t_s;
+  };
   float mx = -INFINITY;
 #pragma unroll 1
   for (int b = k.kb0; b < k.kb1; ++b) {
@@ -363,55 +312,42 @@ __device__ __forceinline__ void softmax_rows(Softmax& sm, const KeyRange& k, int
       add_rpb(s, s_mi.rpb + (size_t)h * s_mi.rb_len, from, b, sqrtf((float)D));
       tmem_st16_at<0>(t_s + 16 * b, s);
     }
-    if (!k.coded) sm.mask(s, b);
+    if (!k.coded) mask(s, b);
     float m0 = fmaxf(s[0], s[1]), m1 = fmaxf(s[2], s[3]);
 #pragma unroll
     for (int i = 4; i < 16; i += 4) { m0 = fmaxf(m0, fmaxf(s[i], s[i + 1])); m1 = fmaxf(m1, fmaxf(s[i + 2], s[i + 3])); }
     mx = fmaxf(mx, fmaxf(m0, m1));
   }
   if (RPB) tmem_wait_st();
-  sm.sc = RPB ? 1.4426950408889634f * rsqrtf((float)D) : 1.0f;
-  sm.off = mx == -INFINITY ? 0.f : -mx * sm.sc;  // (rows past the tile may have no key)
+  const float off = mx == -INFINITY ? 0.f : -mx * sc;  // (rows past the tile may have no key)
   const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
   for (int b = 0; b < k.kb0; ++b) tmem_st8_u32(t_s + 8 * b, zero);
+  float2 sum = make_float2(0.f, 0.f);
 #pragma unroll 1
   for (int b = k.kb0; b < k.kb1; ++b) {
     float s[16];
     tmem_ld16_at<0>(t_s + 16 * b, s);
     tmem_wait_ld();
-    if (!k.coded) sm.mask(s, b);
-    sm.block<false>(s, b);
+    if (!k.coded) mask(s, b);
+    uint32_t p[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float2 u = __ffma2_rn(make_float2(s[2 * i], s[2 * i + 1]), make_float2(sc, sc), make_float2(off, off));
+      const float2 e = make_float2(ex2_approx(u.x), ex2_approx(u.y));
+      sum = __fadd2_rn(sum, e);
+      p[i] = pack_bf16(e.x, e.y);
+    }
+    tmem_st8_u32(t_s + 8 * b, p);
   }
+  for (int b = k.kb1; b < n_blocks; ++b) tmem_st8_u32(t_s + 8 * b, zero);
+  tmem_wait_st();
+  return sum.x + sum.y;
 }
 
-// Without: every |q| |k| of the warp's rows and the tile's keys is at most kOnceBound, so that the exponentials lie in
-// [2^-32, 2^32] (masked ones at 2^-125 or 0) and sums and products are as exact as with a maximum taken off.  The next block is
-// loaded under this one's exponentials.  32,000 pillars 397 -> 388.5 us against the two passes above.
-constexpr float kOnceBound = 32.0f;
-__device__ __forceinline__ void softmax_once(Softmax& sm, const KeyRange& k) {
-  const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-  float s[16], t[16];
-  tmem_ld16_at<0>(sm.t_s + 16 * k.kb0, s);
-  for (int b = 0; b < k.kb0; ++b) tmem_st8_u32(sm.t_s + 8 * b, zero);  // (columns before those of the first block)
-#pragma unroll 1
-  for (int b = k.kb0; b < k.kb1; b += 2) {
-    tmem_wait_ld();
-    if (b + 1 < k.kb1) tmem_ld16_at<0>(sm.t_s + 16 * (b + 1), t);
-    if (!k.coded) sm.mask(s, b);
-    sm.block<true>(s, b);
-    if (b + 1 >= k.kb1) break;
-    tmem_wait_ld();
-    if (b + 2 < k.kb1) tmem_ld16_at<0>(sm.t_s + 16 * (b + 2), s);
-    if (!k.coded) sm.mask(t, b + 1);
-    sm.block<true>(t, b + 1);
-  }
-}
-
-// Attention of tile k: warps 4 q + (0..3) take heads rounds q, rounds q + 1, ... (rounds = heads / 4; the columns whose K and Q
-// epilogue they have done); their S, then P, then O live in TMEM columns [128 q, 128 q + 128).  query_norm: the squares of the
-// largest query norms of the warp's rows in these heads.  The output of a head replaces its (dead) query columns.
+// Attention of tile k: warps 4 q + (0..3) take heads q, q + 4, ... ; their S, then P, then O live in TMEM columns
+// [128 q, 128 q + 128).  The output of a head replaces its (dead) query columns.
 template <int C, int D, bool RPB>
-__device__ __forceinline__ void attend(int k, const float (&query_norm)[2]) {
+__device__ __forceinline__ void attend(int k) {
   constexpr int DC = D / 8;  // 16-byte chunks per head
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp >> 2;
   const int rows = s_mi.rows, row = 32 * (warp & 3) + lane;
@@ -420,27 +356,12 @@ __device__ __forceinline__ void attend(int k, const float (&query_norm)[2]) {
   KeyRange kr = {0, 0, true};
   if (on) kr = key_range<D>(32 * (warp & 3), rows);
   const int lo = s_mi.row_lo[s_mi.buf][row], n = s_mi.row_n[s_mi.buf][row];
-  const int rounds = s_mi.heads >> 2;
 #pragma unroll 1
-  for (int j = RPB ? q * rounds : 0; j < (RPB ? (q + 1) * rounds : rounds); ++j) {  // (the form that spills less in each variant)
-    const int h = RPB ? j : q * rounds + j;
-    const uint32_t par = (uint32_t)((RPB ? k - q : k) * rounds + j) & 1u;  // (heads so far of this group)
+  for (int h = q; h < s_mi.heads; h += 4) {
+    const uint32_t par = (uint32_t)(k * (s_mi.heads >> 2) + (h >> 2)) & 1u;  // (heads so far of this group)
     wait_phase(smem_u32(&s_mi.s_full[0]) + 8 * q, par);
     float l = 1.f;
-    if (on) {
-      bool once = false;
-      if (!RPB) {
-        const uint32_t kn = max(max(s_mi.key_norm[4 * q][j], s_mi.key_norm[4 * q + 1][j]), max(s_mi.key_norm[4 * q + 2][j], s_mi.key_norm[4 * q + 3][j]));
-        once = (j ? query_norm[1] : query_norm[0]) * __uint_as_float(kn) <= kOnceBound * kOnceBound;  // (not if one is NaN)
-      }
-      Softmax sm = {t_s, 1.0f, 0.f, lo, n, make_float2(0.f, 0.f)};
-      if (once && kr.kb0 < kr.kb1) softmax_once(sm, kr);
-      else softmax_rows<D, RPB>(sm, kr, row, h);
-      const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-      for (int b = kr.kb1; b < (rows + 15) >> 4; ++b) tmem_st8_u32(t_s + 8 * b, zero);
-      tmem_wait_st();
-      l = n > 0 ? sm.sum.x + sm.sum.y : __int_as_float(0x7fffffff);  // (a marked set: no key at all where its keys are masked)
-    }
+    if (on) l = softmax_rows<D, RPB>(t_s, kr, (rows + 15) >> 4, row, lo, n, h);
     tc_fence_before();
     mbar_arrive(&s_mi.p_ready[q]);
     wait_phase(smem_u32(&s_mi.ov_full[0]) + 8 * q, par);
@@ -715,7 +636,7 @@ __device__ __forceinline__ void mma_role(const RoleCtx& rc) {
       const uint32_t id_s = umma_idesc(16 * n_blocks), id_o = umma_idesc(D == 24 ? 32 : D) | (1u << 16);  // V: N-major
       const int rounds = rc.heads >> 2;
       auto scores = [&](int q, int i) {
-        const uint32_t d = tmem + 128 * q, step = (uint32_t)(rounds * q + i) * kHeadStep;
+        const uint32_t d = tmem + 128 * q, step = (uint32_t)(4 * i + q) * kHeadStep;
         umma_ss(d, q_lo + step, KM, k_lo + step, KM, id_s, 0u);
         if (D == 24) {  // the last 8 columns and the code: the leading offset leads from one to the other
           const uint32_t qa = (a_addr >> 4) + 2 * kChunk16 + step, ka = (k_addr >> 4) + 2 * kChunk16 + step;
@@ -747,7 +668,7 @@ __device__ __forceinline__ void mma_role(const RoleCtx& rc) {
             if (st & 1) {
               scores(q, i + 1);
             } else {
-              const uint32_t v = v_lo + (uint32_t)(rounds * q + i) * kHeadStep;
+              const uint32_t v = v_lo + (uint32_t)(4 * i + q) * kHeadStep;
 #pragma unroll
               for (int s = 0; s < 8; ++s)  // (16 keys: 8 columns of P, 256 bytes of each chunk of V)
                 if (s < n_blocks)
@@ -1064,15 +985,11 @@ __device__ __forceinline__ void phase_gather(int b, int rows) {
 //   dst_off   byte offset of the destination operand from the shared-memory base
 // BIAS = false skips the bias (the key projection: a key bias adds
 // the same amount q . b_k to every score of a query, which the softmax cancels).
-// Queries are scaled (query_scale); the first query column of a row whose set is marked becomes NaN (see drop_wild), and with it
-// the row.  For keys and queries `norm` receives the squares of the warp's largest norms, per head of D columns.
-enum Operand { kKey, kValue, kQuery };
-template <int QC, int D, Operand OP, bool RPB>
-__device__ __forceinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_off, uint32_t dst_off, float (&norm)[2]) {
-  constexpr bool BIAS = OP != kKey, QUERY = OP == kQuery;
+// QUERY: the first query column of a row whose set is marked becomes NaN (see drop_wild), and with it the row.
+template <int QC, bool BIAS, bool QUERY>
+__device__ __forceinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_off, uint32_t dst_off) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = 32 * (warp & 3) + lane, hq = warp >> 2;
-  norm[0] = norm[1] = 0.f;
   if (32 * (warp & 3) >= s_mi.rows) {
     tc_fence_before();
     mbar_arrive(&s_mi.acc_free[bar]);
@@ -1086,10 +1003,7 @@ __device__ __forceinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_
   tmem_wait_ld();
   tc_fence_before();
   mbar_arrive(&s_mi.acc_free[bar]);  // the accumulator is in registers now
-  const bool wild = QUERY && s_mi.row_n[s_mi.buf][row] == 0;  // (its norm is that of the operand: the other rows' path stays as it is)
-  float2 sq[QC / D];
-#pragma unroll
-  for (int i = 0; i < QC / D; ++i) sq[i] = make_float2(0.f, 0.f);
+  if (QUERY && s_mi.row_n[s_mi.buf][row] == 0) rr[0] = __int_as_float(0x7fffffff);
 #pragma unroll
   for (int q = 0; q < QC / 8; ++q) {
     float2 v[4] = {make_float2(rr[8 * q], rr[8 * q + 1]), make_float2(rr[8 * q + 2], rr[8 * q + 3]),
@@ -1101,29 +1015,9 @@ __device__ __forceinline__ void phase_epi_bf16(uint32_t tcol, int bar, int bias_
       v[2] = __fadd2_rn(v[2], make_float2(b1.x, b1.y));
       v[3] = __fadd2_rn(v[3], make_float2(b1.z, b1.w));
     }
-    if (QUERY && !RPB) {
-      const float sc = query_scale<D, RPB>();
-#pragma unroll
-      for (int i = 0; i < 4; ++i) v[i] = __fmul2_rn(v[i], make_float2(sc, sc));
-    }
-    if (OP != kValue && !RPB) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) sq[8 * q / D] = __ffma2_rn(v[i], v[i], sq[8 * q / D]);
-    }
-    if (QUERY && q == 0 && wild) v[0].x = __int_as_float(0x7fffffff);
     sts4(dst + q * kChunkBytes,
          make_uint4(pack_bf16(v[0].x, v[0].y), pack_bf16(v[1].x, v[1].y), pack_bf16(v[2].x, v[2].y), pack_bf16(v[3].x, v[3].y)));
   }
-  if (OP != kValue && !RPB) {
-#pragma unroll
-    for (int i = 0; i < QC / D; ++i)  // (not negative: their bits are in order)
-      norm[i] = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(sq[i].x + sq[i].y) & 0x7fffffffu));
-  }
-}
-
-__device__ __forceinline__ void set_key_norm(const float (&norm)[2]) {
-  s_mi.key_norm[threadIdx.x >> 5][0] = __float_as_uint(norm[0]);
-  s_mi.key_norm[threadIdx.x >> 5][1] = __float_as_uint(norm[1]);
 }
 
 // MLP-1 piece: HC = NF / 4 hidden columns per thread, H = gelu(x1 W_1^T + b_1) into TMEM as the A operand of MLP-2.
@@ -1453,34 +1347,31 @@ __device__ __forceinline__ void compute_role(const TcArgs& a) {
 
     // (uses of the accumulators before this tile: V and R one each per tile, the first one K, Q and the MLP-1 pieces)
     // ---- chunks 0..2: K, V, Q epilogues: (+ bias,) to bf16, into the operand layout ----
-    float norm[2];
     if (PE) {
       // the values come from the bare rows; the operand is then rewritten with the positional term added, for
       // the keys and the queries (the V chunk's accumulator being complete, nothing reads the operand any more)
       WAIT_PHASE(acc_full[1], k);
       if (new_params) wait_layer_params();
-      phase_epi_bf16<QC, D, kValue, RPB>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + (C / 8) * kChunkBytes, norm);
+      phase_epi_bf16<QC, true, false>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + (C / 8) * kChunkBytes);
       phase_gather<C, D, false, true>(k & 1, s_mi.rows);
       fence_proxy_async();
       mbar_arrive(&s_mi.x_ready);
       WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1));
-      phase_epi_bf16<QC, D, kKey, RPB>(Tm<C>::k, 0, 0, s_mi.off_kv, norm);
-      if ((threadIdx.x & 31) == 0) set_key_norm(norm);
+      phase_epi_bf16<QC, false, false>(Tm<C>::k, 0, 0, s_mi.off_kv);
     } else {
       WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1));
-      phase_epi_bf16<QC, D, kKey, RPB>(Tm<C>::k, 0, 0, s_mi.off_kv, norm);
-      if (!RPB && (threadIdx.x & 31) == 0) set_key_norm(norm);
+      phase_epi_bf16<QC, false, false>(Tm<C>::k, 0, 0, s_mi.off_kv);
       WAIT_PHASE(acc_full[1], k);
       if (new_params) wait_layer_params();  // (the key epilogue adds no bias: it needs none of the vectors)
-      phase_epi_bf16<QC, D, kValue, RPB>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + (C / 8) * kChunkBytes, norm);
+      phase_epi_bf16<QC, true, false>(Tm<C>::v, 1, ParOff<C>::b_v, s_mi.off_kv + (C / 8) * kChunkBytes);
     }
     WAIT_PHASE(acc_full[0], k * (2 + s_mi.n_f1) + 1);
     if (PE) compute_sync();  // (every thread has marked the sets of its rows with the positional term)
-    phase_epi_bf16<QC, D, kQuery, RPB>(Tm<C>::k, 0, ParOff<C>::b_q, s_mi.off_a, norm);
+    phase_epi_bf16<QC, true, true>(Tm<C>::k, 0, ParOff<C>::b_q, s_mi.off_a);
     fence_proxy_async();
     mbar_arrive(&s_mi.a_ready);  // Q, K and V are in place
     // ---- attention inside each set ----
-    attend<C, D, RPB>(k, norm);
+    attend<C, D, RPB>(k);
     fence_proxy_async();
     mbar_arrive(&s_mi.a_ready);  // attention output is the A operand of the output projection
     compute_sync();              // every warp is done with K and V: their region becomes fp32 staging
