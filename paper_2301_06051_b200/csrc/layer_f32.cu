@@ -468,9 +468,24 @@ __device__ __forceinline__ void prepare_weights(const WeightJob& j) {
   }
 }
 
+// Whether set s claims the positions up to the next set's first and can have as many rows.
+__device__ __forceinline__ bool sound_claim(int off, int end, int tau) { return off >= 0 && end > off && (int64_t)end - off <= tau; }
+
+// Whether position x lies in the claim of a set that writes it.
+__device__ __noinline__ bool claimed(const ListJob& j, int S, int x) {
+  int lo = 0, hi = S;  // the first set that starts behind x
+  while (lo < hi) { const int m = (lo + hi) >> 1; if (__ldg(j.rowoff + m) <= x) lo = m + 1; else hi = m; }
+  if (lo == 0) return false;
+  const int off = __ldg(j.rowoff + lo - 1), end = __ldg(j.rowoff + lo);
+  return off <= x && x < end && sound_claim(off, end, j.tau);
+}
+
 // A set belongs to the pass its first row lies in: pass p takes the sets whose row offset is in [p R, (p + 1) R), R =
 // pass_rows, and a position's place in it is its row offset less p R.  One warp per set writes the set's distinct slots
 // (Eq. 4); the first blocks find the passes' first and last sets.
+// The lists hold what an earlier call left.  A set whose claim is not sound is skipped (its positions become -1), and every set
+// writes its claim in each list that holds it: of the positions between two sets' first rows each lies in the claim of some set
+// between them, whatever the offsets are, so that a pass has no position that nobody wrote.
 __global__ void __launch_bounds__(256) f32_prepare_kernel(const __grid_constant__ PrepArgs a) {
   pdl_enter();
   if ((int)blockIdx.y < a.n_weights) {
@@ -498,17 +513,24 @@ __global__ void __launch_bounds__(256) f32_prepare_kernel(const __grid_constant_
   }
   const int warps = gridDim.x * (blockDim.x >> 5);
   for (int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); s < S; s += warps) {
-    const int off = __ldg(j.rowoff + s), cap = __ldg(j.rowoff + s + 1) - off;
-    const int p = off < 0 ? j.passes : off / R;
-    bool bad = off < 0 || cap <= 0 || cap > kTM;  // row offsets that do not describe this table
-    if (p >= j.passes) {  // (more rows than voxels: some voxels are in several sets; the general kernel takes these sets)
-      if (bad && lane == 0) atomicOr(a.status, DSVT_STATUS_BAD_INDEX);
-      continue;
+    const int off = __ldg(j.rowoff + s), end = __ldg(j.rowoff + s + 1);
+    const bool sound = sound_claim(off, end, j.tau);
+    const int p = sound ? off / R : -1, cap = sound ? end - off : 0;
+    if (!sound && lane == 0) atomicOr(a.status, DSVT_STATUS_BAD_INDEX);
+    // (a sound claim that does not cross into another pass's list does nothing here)
+    const int lo = max(off, 0);
+    const int64_t last = min((int64_t)end, (int64_t)j.passes * R + kTM);
+    for (int q = max(lo - kTM, 0) / R; q < j.passes && (int64_t)q * R < last; ++q) {
+      if (q == p) continue;
+      const int64_t o = (int64_t)q * R, to = min(last, o + a.rows);
+      for (int64_t x = max((int64_t)lo, o) + lane; x < to; x += 32)
+        if (sound || !claimed(j, S, (int)x)) j.list[(size_t)q * a.rows + (x - o)] = -1;
     }
-    const int room = max(0, min(cap, kTM));
+    if (!sound || p >= j.passes) continue;  // (more rows than voxels: some voxels are in several sets; the general kernel takes these)
     int32_t* to = j.list + (size_t)p * a.rows + (off - p * R);
     const int32_t* row = j.table + (size_t)s * j.tau;
     int cnt = 0;
+    bool bad = false;
     for (int k0 = 0; k0 < j.tau; k0 += 32) {
       const int k = k0 + lane;
       int v = -1;
@@ -519,13 +541,13 @@ __global__ void __launch_bounds__(256) f32_prepare_kernel(const __grid_constant_
       }
       const unsigned bal = __ballot_sync(0xffffffffu, uniq);
       const int pos = cnt + __popc(bal & ((1u << lane) - 1u));
-      if (uniq && pos < room) {
+      if (uniq && pos < cap) {
         if (v < 0 || v >= a.n) { bad = true; v = -1; }
         to[pos] = v;
       }
       cnt += __popc(bal);
     }
-    for (int k = cnt + lane; k < room; k += 32) to[k] = -1;
+    for (int k = cnt + lane; k < cap; k += 32) to[k] = -1;
     if (__any_sync(0xffffffffu, bad || cnt != cap) && lane == 0) atomicOr(a.status, DSVT_STATUS_BAD_INDEX);
   }
 }
@@ -678,10 +700,10 @@ __global__ void __launch_bounds__(kAttThreads, D == 16 ? 4 : 3) f32_attend_kerne
     const int s = ps.s_first + u / kHeads;
     if (s >= ps.s_end) return false;
     h = u % kHeads;
-    const int off = __ldg(a.rowoff + s);
+    const int off = __ldg(a.rowoff + s), end = __ldg(a.rowoff + s + 1);
     base = off - a.origin;
-    m = min(__ldg(a.rowoff + s + 1) - off, a.tau);  // (a valid set has no more rows than slots)
-    if (base < 0 || base >= a.pass_rows) m = 0;     // (row offsets that do not ascend)
+    m = sound_claim(off, end, a.tau) ? end - off : 0;
+    if (base < 0 || base >= a.pass_rows) m = 0;  // (row offsets that do not ascend)
     return true;
   };
   bool more = draw();

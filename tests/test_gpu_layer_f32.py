@@ -69,6 +69,43 @@ def test_row_offsets_that_claim_more_rows_than_a_set_has(oracle, C, heads, hidde
     check_close(y.cpu().numpy()[others], want[others], "fp32", "the other sets")
 
 
+@pytest.mark.parametrize("C,heads,hidden,passes", [(128, 8, 0, 1), (192, 8, 384, 1), (192, 8, 64, 2)])
+@pytest.mark.parametrize("kind", ["two hundred rows too many", "one offset far too large"])
+def test_rows_that_no_set_fills_reach_no_voxel(oracle, C, heads, hidden, passes, kind):
+    """Caller-made row offsets with more room than any set can fill, in a context whose buffers hold an earlier call's voxel
+    ids: the sets that the offsets spoil are skipped, all other voxels come out right."""
+    from paper_2301_06051_b200 import api
+
+    tau, n = 36, 700 if passes == 1 else 14001
+    grid = 48 if passes == 1 else 144
+    case = di.random_case(C, n, (grid, grid, 1), (12, 12, 1), tau, C, heads, hidden, layernorm=hidden > 0)
+    layer = case["blocks"][0][0]
+    p = oracle.partition(case["coords"], 1, case["grid"], case["window"], tau, 0)
+    want = oracle.layer(case["feats"], p.set_table, layer)
+    S = len(p.set_table)
+    ctx = api.Context(n + (300 if passes == 2 else 0), (grid // 12) ** 2, C)
+    x, w = dev(case["feats"]), api.device_weights(layer, api.FP32, ctx.device)
+    table = upload_table(p.set_table)
+    y = torch.full_like(x, 77.0)
+    ctx.layer(x, table, w, y)  # (leaves its lists in the context)
+    assert ctx.status_sync() == 0
+    check_close(y.cpu().numpy(), want, "fp32", "sound offsets")
+    at = S // 2 if passes == 1 else S // 4
+    if kind == "one offset far too large":
+        table.set_rowoff[at + 1] = 1 << 30
+        spoiled = [at, at + 1]
+    else:
+        table.set_rowoff[at + 1 : S + 1] += 200
+        spoiled = [at]
+    y.fill_(77.0)
+    ctx.layer(x, table, w, y)
+    assert ctx.status_sync() == api.STATUS_BAD_INDEX
+    got, members = y.cpu().numpy(), np.unique(p.set_table[spoiled])
+    others = np.setdiff1d(np.arange(n), members)
+    check_close(got[others], want[others], "fp32", "the other sets")
+    assert np.all(got[members] == 77.0)
+
+
 def test_voxels_in_many_sets_take_the_general_kernel(oracle):
     """A table with more rows than there are voxels (every set eight times over): the sets past the workspace's passes run on
     the kernel for general shapes, with the same results."""
