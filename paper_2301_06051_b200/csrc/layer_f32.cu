@@ -571,7 +571,8 @@ constexpr int kAttThreads = 128;
 __host__ __device__ constexpr int warp_floats(int d, int tau) { return tau * (2 * d) + (tau + 3) / 4 * 4; }  // keys | values, linear coordinates
 
 // The attention of Q query rows per lane of a half warp (rows r0 + lane, r0 + 16 + lane); the two halves take every other
-// key, K at a time with a running softmax, and meet at the end.
+// key, K at a time with a running softmax, and meet at the end.  Scores stay in natural units up to the difference from the
+// maximum: times log2(e), a bias of the lowest float would be -inf, and a row of such biases 0 / 0.
 template <int D, int Q, bool RPB>
 __device__ __forceinline__ void attend_rows(float* qkv, int ld, const float* kv, const int* lin, int rows, int r0, float scale,
                                             const float* rpb, int rb_len, int rb_centre) {
@@ -622,7 +623,7 @@ __device__ __forceinline__ void attend_rows(float* qkv, int ld, const float* kv,
         lg[w][u] = (s[w].x + s[w].y) * scale;
         if (RPB) {
           const int idx = lin[r[w]] - lin[k] + rb_centre;
-          lg[w][u] = fmaf(__ldg(rpb + min(max(idx, 0), rb_len - 1)), 1.4426950408889634f, lg[w][u]);
+          lg[w][u] += __ldg(rpb + min(max(idx, 0), rb_len - 1));
         }
         if (k0 + 2 * u >= rows) lg[w][u] = -INFINITY;
       }
@@ -633,12 +634,12 @@ __device__ __forceinline__ void attend_rows(float* qkv, int ld, const float* kv,
 #pragma unroll
       for (int u = 0; u < K; u += 2) nm = fmaxf(nm, fmaxf(lg[w][u], lg[w][u + 1]));
       const float from = nm == -INFINITY ? 0.f : nm;  // (a bias may rule out all keys so far)
-      const float al = ex2_approx(mx[w] - from);      // (2^-inf = 0)
+      const float al = expf(mx[w] - from);            // (exp(-inf) = 0)
       mx[w] = nm;
       float sum = 0.f;
 #pragma unroll
       for (int u = 0; u < K; ++u) {
-        lg[w][u] = ex2_approx(lg[w][u] - from);
+        lg[w][u] = expf(lg[w][u] - from);
         sum += lg[w][u];
       }
       den[w] = fmaf(den[w], al, sum);
@@ -662,7 +663,7 @@ __device__ __forceinline__ void attend_rows(float* qkv, int ld, const float* kv,
 #pragma unroll
   for (int w = 0; w < Q; ++w) {  // (the second half has no keys if the set holds one row)
     const float nm = fmaxf(mx[w], __shfl_xor_sync(0xffffffffu, mx[w], 16));
-    const float al = nm == -INFINITY ? 0.f : ex2_approx(mx[w] - nm);
+    const float al = nm == -INFINITY ? 0.f : expf(mx[w] - nm);
     den[w] *= al;
     const float inv = al / (den[w] + __shfl_xor_sync(0xffffffffu, den[w], 16));
     const bool on = r0 + 16 * w + l16 < rows;
@@ -691,7 +692,7 @@ __global__ void __launch_bounds__(kAttThreads, D == 16 ? 4 : 3) f32_attend_kerne
   float* kv = smem + (size_t)(threadIdx.x >> 5) * warp_floats(D, a.tau);  // [row][K | V]
   int* lin = reinterpret_cast<int*>(kv + a.tau * 2 * D);
   const Pass ps = *a.pass;
-  const float scale = 1.4426950408889634f * rsqrtf((float)D);  // log2(e) / sqrt(d)
+  const float scale = rsqrtf((float)D);
   int h, base, m;
   auto draw = [&]() -> bool {  // the next unit: head, first position, rows
     int u = 0;

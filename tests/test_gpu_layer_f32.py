@@ -4,7 +4,7 @@ import pytest
 import torch
 
 import dsvt_inputs as di
-from gpu_helpers import check_close, dev, upload_table
+from gpu_helpers import check_close, dev, rowoff_of, upload_table
 
 pytestmark = pytest.mark.gpu
 
@@ -104,6 +104,38 @@ def test_rows_that_no_set_fills_reach_no_voxel(oracle, C, heads, hidden, passes,
     others = np.setdiff1d(np.arange(n), members)
     check_close(got[others], want[others], "fp32", "the other sets")
     assert np.all(got[members] == 77.0)
+
+
+@pytest.mark.parametrize("tau,C,heads", [(36, 192, 8), (64, 192, 8), (96, 128, 4), (36, 64, 4)])
+def test_bias_of_the_lowest_and_the_largest_float(oracle, tau, C, heads):
+    """A position bias that is the lowest float for every pair of a head leaves its keys with equal weights, and so does one
+    of the largest; sets of a single voxel, whose only pair is the zero offset, are among them."""
+    from paper_2301_06051_b200 import api
+
+    n = 400
+    case = di.random_case(tau + C, n, (120, 36, 1), (12, 12, 1), tau, C, heads, 0)
+    case["coords"][:, 1] = np.where(np.arange(n) < n - 4, case["coords"][:, 1] % 60, 60 + 12 * (np.arange(n) % 5))
+    case["coords"] = case["coords"][np.sort(np.unique(case["coords"], axis=0, return_index=True)[1])]
+    n = len(case["coords"])
+    layer = case["blocks"][0][0]
+    rng = np.random.default_rng(C)
+    fmax = np.finfo(np.float32).max
+    rpb = rng.standard_normal((heads, 23 * 23)).astype(np.float32)
+    rpb[0], rpb[1] = -fmax, fmax
+    rpb[2, (23 * 23) // 2] = -fmax  # the voxel itself is masked: a set of one voxel has no other key
+    rpb[3, ::2] = -fmax
+    layer["rpb"], layer["rpb_extent"] = rpb, (12, 12, 1)
+    ctx = api.Context(n, 30, C)
+    coords, x = dev(case["coords"]), dev(case["feats"][:n])
+    table = ctx.partition(coords, 1, case["grid"], case["window"], tau, 0)
+    y = torch.empty_like(x)
+    ctx.set_attention(x, table, api.device_weights(layer, api.FP32, ctx.device), y, coords=coords)
+    assert ctx.status_sync() == 0
+    p = oracle.partition(case["coords"], 1, case["grid"], case["window"], tau, 0)
+    assert np.min(np.diff(rowoff_of(p.set_table))) == 1
+    want, _ = oracle.set_attention(case["feats"][:n], p.set_table, layer["W_qkv"], layer["b_qkv"], layer["W_o"], layer["b_o"],
+                                   heads, rpb=rpb, coords=case["coords"], rpb_extent=(12, 12, 1))
+    check_close(y.cpu().numpy(), want, "fp32", "bias")
 
 
 def test_voxels_in_many_sets_take_the_general_kernel(oracle):
