@@ -8,13 +8,23 @@
 // [position][Q, attention output or x1 | K, then MLP hidden | V].  One fused kernel cannot hold a tile: its operands take 144 KB
 // in three parts (below) and Q, K and V 295 KB.  The workspace is bounded, so a layer of many rows runs in passes of whole sets.
 //
-// An fp32 product on tcgen05: each operand is the sum of three bfloat16 parts (8 + 8 + 8 bits: the first truncated, the
-// others rounded, exact together), and of the nine partial products the six largest are formed, each exact in fp32.  The
-// tensor cores' additions truncate: with all six in one accumulator the error is 1.2e-6 of the result's 2-norm at K = 192,
-// seven times that of fp32 multiply-adds with two running sums (1.8e-7).  So the leading product has an accumulator of
-// its own, which is read out and cleared every kChunk stages, and the five small ones share another, where truncation is
-// 2^-8 as large: 0.8e-7 with chunks of 64 k, 1.6e-7 with one of 192.  Against float64, two layers are off by 1.2e-7 ... 2.4e-7
-// where the kernel on the FMA pipes was off by 1.2e-7 ... 3.9e-7.
+// An fp32 product on tcgen05 (Henry, Tang, Heinecke, "Leveraging the bfloat16 artificial intelligence datatype for
+// higher-precision computations", ARITH 2019): each operand is the sum of three bfloat16 parts, exact together, and of the nine
+// partial products the six largest are formed, each exact in fp32.  With all parts rounded the three that are left out are at most
+// 0.9 x 2^-24 of a product (with the first part truncated: 3.5 x 2^-24).  The tensor cores' additions truncate (for which reason
+// Ootomo and Yokota, "Recovering single precision accuracy from tensor cores while surpassing the FP32 theoretical peak
+// performance", 2022, add partial sums outside of them): with all six in one accumulator the error is 1.2e-6 of the result's
+// 2-norm at K = 192, seven times that of fp32 multiply-adds with two running sums (1.8e-7).  So the leading product has an
+// accumulator of its own, which is read out and cleared every kChunk stages, and the five small ones share another, where truncation
+// is 2^-8 as large.
+// Error against float64 of two layers, kernel on the FMA pipes -> now (12 seeds; 2-norm, and largest error in units of the
+// result's root mean square):
+//   C = 192, hidden 384       3.1e-7 -> 1.9e-7    2.1e-6 -> 1.5e-6
+//   C = 192, hidden 256       4.0e-7 -> 1.9e-7    2.6e-6 -> 1.4e-6
+//   C = 192, attention alone  1.4e-7 -> 1.1e-7    8.9e-7 -> 7.9e-7
+//   C = 128, attention alone  1.23e-7 -> 0.98e-7  7.2e-7 -> 6.5e-7
+//   C = 64, hidden 128        1.9e-7 -> 1.6e-7    1.2e-6 -> 1.1e-6
+// One attention with positive weights and features, where truncations add up: 0.8e-7 -> 1.2e-7.
 //
 // Measured (B200): two full layers and their partition, 12,345 pillars, C = 192: 776 us on the FMA pipes (27 % of their peak:
 // shared-memory reads for the products, and the phases between them), 282 us now; two attention-only layers, 2,000 pillars,
@@ -41,7 +51,12 @@ constexpr int kKS = 16;        // k per operand stage: one MMA step
 constexpr int kSt = 4;         // stages
 constexpr int kFly = 3;        // stages of operand rows in a converting thread's registers (4: 281.6 us, 6: 284.7)
 constexpr int kParts = 3;      // bfloat16 parts of an operand
-constexpr int kChunk = 96 / kKS;  // most stages between two readings of the leading accumulator
+// Most stages between two readings of the leading accumulator, as few as keep every error of the table above below the FMA
+// kernel's: with 96 k the largest error of attention alone is 9.0e-7 (C = 192) and 7.9e-7 (128), and 12,345 pillars take 244 us instead
+// of 255; with 32 for N = 192 284 us.
+template <int N>
+constexpr int kChunk = (N == 192 ? 64 : 48) / kKS;
+constexpr int kSpare = 64;         // columns of a half's sum of chunks in TMEM: at N and at kCorr + N
 constexpr uint32_t kCorr = 256;  // TMEM column of the accumulator of the small products (the leading one is at 0)
 
 // Operand parts in shared memory: unswizzled, [8-column chunk][row][16 bytes].
@@ -56,7 +71,8 @@ struct Sm {
 struct Pass { int s_first, s_end, row0, row_end; };  // sets and (local) positions of a pass
 
 // Stages of a chunk of the leading product: as few chunks as kChunk allows, of about the same size.
-__device__ __forceinline__ int chunk_stages(int ns) { const int n = (ns + kChunk - 1) / kChunk; return (ns + n - 1) / n; }
+template <int N>
+__device__ __forceinline__ int chunk_stages(int ns) { const int n = (ns + kChunk<N> - 1) / kChunk<N>; return (ns + n - 1) / n; }
 
 enum Epilogue { kBias = 0, kNorm = 1, kGelu = 2 };
 
@@ -92,11 +108,10 @@ __device__ __forceinline__ void split4(const float4 f, uint2& h, uint2& m, uint2
   uint32_t p[3][2];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
-    const uint32_t a = __float_as_uint(v[2 * i]), b = __float_as_uint(v[2 * i + 1]);
-    p[0][i] = __byte_perm(a, b, 0x7632);
-    // (truncated, so that the first part of a large finite value is finite)
+    // (saturating, so that the first part of a large finite value is finite)
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(p[0][i]) : "f"(v[2 * i + 1]), "f"(v[2 * i]));
     const float2 r = __fadd2_rn(make_float2(v[2 * i], v[2 * i + 1]),
-                                make_float2(-__uint_as_float(a & 0xffff0000u), -__uint_as_float(b & 0xffff0000u)));
+                                make_float2(-__uint_as_float(p[0][i] << 16), -__uint_as_float(p[0][i] & 0xffff0000u)));
     p[1][i] = pack_bf16(r.x, r.y);
     const float2 q = __fadd2_rn(r, make_float2(-__uint_as_float(p[1][i] << 16), -__uint_as_float(p[1][i] & 0xffff0000u)));
     p[2][i] = pack_bf16(q.x, q.y);
@@ -153,7 +168,7 @@ __device__ __forceinline__ void mma_role(uint32_t sbase, int tiles, int ns) {
   constexpr uint32_t hi = desc_hi_plain(128), idesc = umma_idesc(N);
   volatile int* abort_flag = &s_gm.abort_flag;
   const uint32_t tmem = __shfl_sync(0xffffffffu, s_gm.tmem, 0);
-  const int chunk = chunk_stages(ns);
+  const int chunk = chunk_stages<N>(ns);
   uint32_t g = 0, it = 0, chunks = 0;
   bool ok = true;
   for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x, ++it) {
@@ -259,8 +274,9 @@ __device__ __forceinline__ void epilogue_role(const GemmArgs& a, const Pass& ps,
   const int tid = threadIdx.x, row = tid & (kTM - 1), half = tid / kTM, c0 = half * H;
   const int r16 = tid >> 4, c16 = tid & 15;  // in and out: 16 lanes to a row, a thread's rows 16 apart
   const bool add = EPI == kNorm && (a.res || a.add_x);
-  const int ns = a.k / kKS, chunk = chunk_stages(ns);
-  const uint32_t taddr = s_gm.tmem + ((uint32_t)(row & ~31) << 16) + c0, par = smem_u32(s_gm.par) + 4 * c0;
+  const int ns = a.k / kKS, chunk = chunk_stages<N>(ns);
+  const uint32_t lane0 = s_gm.tmem + ((uint32_t)(row & ~31) << 16), taddr = lane0 + c0, tsum = lane0 + (half ? kCorr : 0u) + N;
+  const uint32_t par = smem_u32(s_gm.par) + 4 * c0;
   uint32_t it = 0, chunks = 0;
   for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {
     const int rt = t / a.tiles_n, nt = t - rt * a.tiles_n, p0 = rt * kTM;
@@ -285,7 +301,8 @@ __device__ __forceinline__ void epilogue_role(const GemmArgs& a, const Pass& ps,
       asm volatile("cp.async.wait_all;" ::: "memory");
     }
     bar_or(1, kEpiThreads, false);  // bias and residual are in place
-    // the leading accumulator's chunks meet in the staging area (on top of the residual)
+    // The leading accumulator's chunks meet in the TMEM columns that are left, kSpare for each half, apart from the residual: a
+    // sum with it would be rounded once more, at the residual's size.  (N = 192: the last third in the staging area, on top of it.)
     for (int s = chunk; s < ns; s += chunk) {
       mbar_wait(&s_gm.chunk_full, chunks++ & 1u, abort_flag);
       tc_fence_after();
@@ -293,6 +310,16 @@ __device__ __forceinline__ void epilogue_role(const GemmArgs& a, const Pass& ps,
       for (int q = 0; q < H; q += 32) {
         float m[32];
         tmem_ld_row(taddr + q, m);
+        if (q < kSpare) {
+          float p[32];
+          if (s > chunk) tmem_ld_row(tsum + q, p);
+          tmem_wait_ld();
+          if (s > chunk)
+#pragma unroll
+            for (int i = 0; i < 32; ++i) m[i] += p[i];
+          tmem_st_row(tsum + q, m);
+          continue;
+        }
         tmem_wait_ld();
 #pragma unroll
         for (int i = 0; i < 32; i += 4) {
@@ -302,6 +329,7 @@ __device__ __forceinline__ void epilogue_role(const GemmArgs& a, const Pass& ps,
           sts4(at, make_float4(v.x + m[i], v.y + m[i + 1], v.z + m[i + 2], v.w + m[i + 3]));
         }
       }
+      tmem_wait_st();
       tc_fence_before();
       mbar_arrive(&s_gm.chunk_free);
     }
@@ -310,16 +338,21 @@ __device__ __forceinline__ void epilogue_role(const GemmArgs& a, const Pass& ps,
     float2 sum = make_float2(0.f, 0.f);
 #pragma unroll 1
     for (int q = 0; q < H; q += 16) {
-      float m[16], k[16];
+      float m[16], k[16], p[16];
+      const bool spare = ns > chunk && q < kSpare;
       tmem_ld16_at<0>(taddr + q, m);
       tmem_ld16_at<0>(taddr + kCorr + q, k);
+      if (spare) tmem_ld16_at<0>(tsum + q, p);
       tmem_wait_ld();
+      if (spare)
+#pragma unroll
+        for (int i = 0; i < 16; ++i) m[i] += p[i];
 #pragma unroll
       for (int i = 0; i < 16; i += 4) {
         const uint32_t at = staging + stage_off<N>(row, (c0 + q + i) / 4);
         const float4 b4 = lds4(par + 4 * (q + i));
         float4 v = make_float4(m[i] + k[i] + b4.x, m[i + 1] + k[i + 1] + b4.y, m[i + 2] + k[i + 2] + b4.z, m[i + 3] + k[i + 3] + b4.w);
-        if (EPI == kNorm || ns > chunk) {
+        if (EPI == kNorm || (ns > chunk && q >= kSpare)) {
           const float4 x4 = lds4(at);
           v.x += x4.x; v.y += x4.y; v.z += x4.z; v.w += x4.w;
         }
@@ -568,11 +601,14 @@ struct AttendArgs {
 };
 
 constexpr int kAttThreads = 128;
+constexpr float kLog2e = 1.4426950408889634f;
 __host__ __device__ constexpr int warp_floats(int d, int tau) { return tau * (2 * d) + (tau + 3) / 4 * 4; }  // keys | values, linear coordinates
 
 // The attention of Q query rows per lane of a half warp (rows r0 + lane, r0 + 16 + lane); the two halves take every other
 // key, K at a time with a running softmax, and meet at the end.  Scores stay in natural units up to the difference from the
-// maximum: times log2(e), a bias of the lowest float would be -inf, and a row of such biases 0 / 0.
+// maximum: times log2(e), a bias of the lowest float would be -inf, and a row of such biases 0 / 0.  Rounding the scaled difference
+// costs a weight e^-a at most a e^-a 2^-24 <= 0.4 x 2^-24 of the largest one.  Two layers with expf instead (12 seeds, 2-norm): attention
+// alone 1.20e-7 for 1.14e-7 (C = 128) and 1.40e-7 for 1.33e-7 (192), full layers 2.24e-7 for 2.21e-7, and 254 us for 249 (12,345 pillars).
 template <int D, int Q, bool RPB>
 __device__ __forceinline__ void attend_rows(float* qkv, int ld, const float* kv, const int* lin, int rows, int r0, float scale,
                                             const float* rpb, int rb_len, int rb_centre) {
@@ -634,12 +670,12 @@ __device__ __forceinline__ void attend_rows(float* qkv, int ld, const float* kv,
 #pragma unroll
       for (int u = 0; u < K; u += 2) nm = fmaxf(nm, fmaxf(lg[w][u], lg[w][u + 1]));
       const float from = nm == -INFINITY ? 0.f : nm;  // (a bias may rule out all keys so far)
-      const float al = expf(mx[w] - from);            // (exp(-inf) = 0)
+      const float al = ex2_approx((mx[w] - from) * kLog2e);  // (2^-inf = 0)
       mx[w] = nm;
       float sum = 0.f;
 #pragma unroll
       for (int u = 0; u < K; ++u) {
-        lg[w][u] = expf(lg[w][u] - from);
+        lg[w][u] = ex2_approx((lg[w][u] - from) * kLog2e);
         sum += lg[w][u];
       }
       den[w] = fmaf(den[w], al, sum);
@@ -663,7 +699,7 @@ __device__ __forceinline__ void attend_rows(float* qkv, int ld, const float* kv,
 #pragma unroll
   for (int w = 0; w < Q; ++w) {  // (the second half has no keys if the set holds one row)
     const float nm = fmaxf(mx[w], __shfl_xor_sync(0xffffffffu, mx[w], 16));
-    const float al = nm == -INFINITY ? 0.f : expf(mx[w] - nm);
+    const float al = nm == -INFINITY ? 0.f : ex2_approx((mx[w] - nm) * kLog2e);
     den[w] *= al;
     const float inv = al / (den[w] + __shfl_xor_sync(0xffffffffu, den[w], 16));
     const bool on = r0 + 16 * w + l16 < rows;

@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
     (3000, 60, 30, 96, 128, 4, 256, ""),      # tiles of up to 96 rows, head dim 32
     (9000, 100, 12, 36, 64, 4, 128, "pe"),    # several tiles per block
     (20000, 150, 12, 36, 128, 8, 128, "rpb"),
-    (700, 36, 12, 36, 192, 8, 256, ""),       # a deep second product of two equal chunks and a short one
+    (700, 36, 12, 36, 192, 8, 256, ""),       # a deep second product of four chunks
     (14001, 150, 12, 36, 192, 8, 64, "pe"),   # two passes; the narrowest tile of the first MLP product
     (45000, 240, 12, 48, 64, 4, 64, ""),      # two passes of many tiles per block
 ])
@@ -67,6 +67,58 @@ def test_row_offsets_that_claim_more_rows_than_a_set_has(oracle, C, heads, hidde
     others = np.setdiff1d(np.arange(n), p.set_table[long])
     want = oracle.layer(case["feats"], p.set_table, layer)
     check_close(y.cpu().numpy()[others], want[others], "fp32", "the other sets")
+
+
+@pytest.mark.parametrize("tau,C,heads,hidden", [(36, 192, 8, 384), (36, 192, 8, 256), (36, 192, 8, 0), (36, 128, 8, 256), (90, 128, 4, 0),
+                                                (36, 64, 4, 128)])
+def test_layer_fp32_is_as_precise_as_fp32(oracle, tau, C, heads, hidden):
+    """One layer against float64.  Sums of 64 to 384 products with a rounding of 2^-24 each, two to four of them in a chain, come
+    to 1e-7 ... 3e-7 of the result (2-norm); the bounds are 4e-7 and 12 times that for the largest error, where operands of
+    two bfloat16 parts (2^-17) show 5e-6."""
+    from paper_2301_06051_b200 import api
+
+    n = 1500
+    case = di.random_case(C + hidden, n, (72, 72, 1), (12, 12, 1), tau, C, heads, hidden, layernorm=hidden > 0)
+    layer = case["blocks"][0][0]
+    ctx = api.Context(n, 36, C)
+    x = dev(case["feats"])
+    table = ctx.partition(dev(case["coords"]), 1, case["grid"], case["window"], tau, 0)
+    y = torch.empty_like(x)
+    ctx.layer(x, table, api.device_weights(layer, api.FP32, ctx.device), y)
+    assert ctx.status_sync() == 0
+    want = oracle.layer(case["feats"], oracle.partition(case["coords"], 1, case["grid"], case["window"], tau, 0).set_table, layer)
+    err = y.cpu().numpy().astype(np.float64) - want
+    assert np.linalg.norm(err) <= 4e-7 * np.linalg.norm(want)
+    assert np.abs(err).max() <= 5e-6 * np.sqrt((want ** 2).mean())
+
+
+@pytest.mark.parametrize("C,heads", [(192, 8), (128, 8), (64, 4)])
+def test_single_products_are_exact_to_a_rounding(C, heads):
+    """Sets of one voxel and one weight per row: an output is a product of a product.  Each is off by 0.9 x 2^-24 (partial
+    products that are not formed) and one rounding of 2^-24, and 0.1 x 2^-24 of truncations: 4 x 2^-24 for both."""
+    from paper_2301_06051_b200 import api
+
+    n = 2000
+    rng = np.random.default_rng(C)
+    case = di.random_case(C, n, (60, 60, 1), (1, 1, 1), 36, C, heads, 0)
+    layer = case["blocks"][0][0]
+    col, val = {}, {}
+    for k in ("W_qkv", "W_o"):
+        rows = layer[k].shape[0]
+        col[k], val[k] = rng.integers(0, C, rows), rng.standard_normal(rows).astype(np.float32)
+        layer[k] = np.zeros((rows, C), np.float32)
+        layer[k][np.arange(rows), col[k]] = val[k]
+        layer["b" + k[1:]] = np.zeros(rows, np.float32)
+    ctx = api.Context(n, 3600, C)
+    x = dev(case["feats"])
+    table = ctx.partition(dev(case["coords"]), 1, case["grid"], case["window"], 36, 0)
+    y = torch.empty_like(x)
+    ctx.set_attention(x, table, api.device_weights(layer, api.FP32, ctx.device), y)
+    assert ctx.status_sync() == 0
+    v = case["feats"].astype(np.float64)[:, col["W_qkv"][2 * C :]] * val["W_qkv"][2 * C :]
+    want = v[:, col["W_o"]] * val["W_o"]
+    rel = np.abs(y.cpu().numpy() - want) / np.abs(want)
+    assert rel.max() <= 4 * 2.0 ** -24, rel.max() * 2 ** 24
 
 
 @pytest.mark.parametrize("C,heads,hidden,passes", [(128, 8, 0, 1), (192, 8, 384, 1), (192, 8, 64, 2)])
