@@ -208,6 +208,29 @@ def test_voxels_in_many_sets_take_the_general_kernel(oracle):
     check_close(y.cpu().numpy(), oracle.layer(case["feats"], p.set_table, layer), "fp32", "voxels in many sets")
 
 
+def test_passes_follow_the_call_and_not_the_context(oracle):
+    """7,000 voxels (a pass of 192 channels holds 12,800) in contexts made for more: as many kernels and the same results as
+    in a context of their size; 14,001 voxels take two passes in either."""
+    from paper_2301_06051_b200 import api
+
+    tau, C, heads = 36, 192, 8
+    for n, sizes in ((7000, (7000, 12801, 40000)), (14001, (14001, 60000))):
+        case = di.random_case(n, n, (144, 144, 1), (12, 12, 1), tau, C, heads, 64, layernorm=True)
+        seen = []
+        for size in sizes:
+            ctx = api.Context(size, 144, C)
+            x = dev(case["feats"])
+            table = ctx.partition(dev(case["coords"]), 1, case["grid"], case["window"], tau, 0)
+            w = api.device_weights(case["blocks"][0][0], api.FP32, ctx.device)
+            y, before = torch.empty_like(x), ctx.launch_count()
+            ctx.layer(x, table, w, y)
+            assert ctx.status_sync() == 0
+            seen.append((ctx.launch_count() - before, y))
+        assert all(k == seen[0][0] and torch.equal(y, seen[0][1]) for k, y in seen)
+        p = oracle.partition(case["coords"], 1, case["grid"], case["window"], tau, 0)
+        check_close(seen[0][1].cpu().numpy(), oracle.layer(case["feats"], p.set_table, case["blocks"][0][0]), "fp32", "n=%d" % n)
+
+
 def test_chain_of_fp32_layers_on_several_tables(oracle):
     """Layers in one call share row lists and prepared weights, two at a time: five layers on three tables."""
     from paper_2301_06051_b200 import api
