@@ -77,7 +77,7 @@ int check_layer_shape(const dsvt_ctx* ctx, const dsvt_layer_params& p, bool atte
 // Runs one fused layer; derives the row offsets from the table when the caller has none.
 int run_layer(dsvt_ctx* ctx, const float* x, int32_t n, const int32_t* table, int32_t cap_sets,
               const int32_t* num_sets, const int32_t* rowoff, const dsvt_layer_params& p, float* y,
-              bool attention_only, int32_t* rowoff_scratch) {
+              bool attention_only, int32_t* rowoff_scratch, bool new_call = true) {
   if (n == 0 || cap_sets == 0) return DSVT_OK;
   dsvt_fused_args a;
   a.x = x; a.y = y; a.n = n; a.table = table; a.num_sets = num_sets; a.rowoff = rowoff; a.cap_sets = cap_sets;
@@ -94,7 +94,7 @@ int run_layer(dsvt_ctx* ctx, const float* x, int32_t n, const int32_t* table, in
     a.rowoff = rowoff_scratch;
   }
   if (tc) return dsvt_launch_layer_tc(ctx, a);
-  if (dsvt_layer_f32_supported(a)) return dsvt_launch_layers_f32(ctx, &a, 1);
+  if (dsvt_layer_f32_supported(a)) return dsvt_launch_layers_f32(ctx, &a, 1, new_call);
   return dsvt_launch_layer_fma(ctx, a);
 }
 
@@ -115,10 +115,11 @@ int run_layers(dsvt_ctx* ctx, const float* x, int32_t n, int32_t num_layers, con
                const dsvt_layer_params* params, float* y) {
   dsvt_fused_args chain[DSVT_MAX_CHAIN_LAYERS];
   int len = 0;
-  bool tc_chain = false;
+  bool tc_chain = false, new_call = true;  // (of the fp32 layers)
   auto flush = [&]() -> int {
     if (len == 0) return DSVT_OK;
-    const int rc = tc_chain ? dsvt_launch_layers_tc(ctx, chain, len) : dsvt_launch_layers_f32(ctx, chain, len);
+    const int rc = tc_chain ? dsvt_launch_layers_tc(ctx, chain, len) : dsvt_launch_layers_f32(ctx, chain, len, new_call);
+    if (!tc_chain) new_call = false;
     len = 0;
     return rc;
   };
@@ -142,8 +143,9 @@ int run_layers(dsvt_ctx* ctx, const float* x, int32_t n, int32_t num_layers, con
       continue;
     }
     const int rc = run_layer(ctx, a.x, n, t.set_table, t.cap_sets, t.num_sets, t.set_rowoff, params[i], y, false,
-                             (i & 1) ? ctx->rowoff_b : ctx->rowoff_a);
+                             (i & 1) ? ctx->rowoff_b : ctx->rowoff_a, new_call);
     if (rc != DSVT_OK) return rc;
+    if (dsvt_layer_f32_supported(a)) new_call = false;
   }
   return flush();
 }

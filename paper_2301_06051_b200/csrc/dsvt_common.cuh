@@ -23,7 +23,7 @@ struct dsvt_ctx {
   // bm_wordrank, in one piece) hold nothing between calls and are the fp32 layers' workspace (layer_f32.cu).
   void* arena;
   size_t arena_bytes;
-  int32_t* status;      // device status word
+  int32_t* status;      // [0] device status word; fp32 layers: [1] number of the call, [2] the last one in which a wait gave up
   uint32_t* keys[2];    // radix sort ping-pong keys        [max(max_voxels, 1024)]
   int32_t* vals[2];     // radix sort ping-pong voxel ids   [max(max_voxels, 1024)]
   int32_t* hist;        // per-tile digit histograms        [256 * sort tiles + 1]
@@ -134,12 +134,13 @@ struct dsvt_fused_args {
   dsvt_layer_params p;
   int32_t attention_only;  // 1: y = attention output (no residual, LN, MLP)
 };
-// (the sets whose first row, in the order of the table, is from_row or later)
-int dsvt_launch_layer_fma(dsvt_ctx* ctx, const dsvt_fused_args& a, int64_t from_row = 0);
+// (the sets whose first row, in the order of the table, is from_row or later; none if calls[0] == calls[1]: an earlier kernel of
+// the call has given up)
+int dsvt_launch_layer_fma(dsvt_ctx* ctx, const dsvt_fused_args& a, int64_t from_row = 0, const int32_t* calls = nullptr);
 // fp32 weights, C in {64, 128, 192}, hidden a multiple of 64 (layer_f32.cu); everything else is layer_fma.cu's.  Layers one
 // after the other: a layer reads its own x, whatever wrote it.
 bool dsvt_layer_f32_supported(const dsvt_fused_args& a);
-int dsvt_launch_layers_f32(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_layers);
+int dsvt_launch_layers_f32(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_layers, bool new_call);  // (false: a call's later layers)
 // tcgen05 path: bfloat16 weights, C in {64, 128, 192}, head dim in {16, 24, 32}, set size <= 96.
 bool dsvt_layer_tc_supported(const dsvt_fused_args& a);
 int dsvt_launch_layer_tc(dsvt_ctx* ctx, const dsvt_fused_args& a);

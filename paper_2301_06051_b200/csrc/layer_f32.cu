@@ -31,7 +31,8 @@
 // C = 128: 109 us and 91 us.  A product's tile of 128 rows takes 9 to 11 k cycles, the start of each of its kernels 4 k
 // (first instructions, lists, operands) and its epilogue 6 k.
 //
-// Every wait is bounded; one that gives up raises DSVT_STATUS_TIMEOUT, and the block stores nothing more.
+// Every wait is bounded; one that gives up raises DSVT_STATUS_TIMEOUT, its block stores nothing more, and no later kernel of the call
+// stores to y (what lies in the workspace for its rows is another call's).
 #include <limits.h>
 
 #include "dsvt_common.cuh"
@@ -87,7 +88,7 @@ struct GemmArgs {
   float* y;
   const float* res;      // kNorm: residual rows [position][ldr], or NULL: rows of x if add_x
   const float *ln_g, *ln_b;
-  int32_t* status;
+  int32_t* status;       // [0] status bits, [1] this call's number, [2] the last call in which a wait gave up
   int32_t* counter;      // kBias: set to zero, for the kernel behind
   int32_t n, lda, ldr, k, tiles_n, pe_tiles, ldo, add_x;
   float eps;
@@ -96,7 +97,7 @@ struct GemmArgs {
 struct GemmShared {
   unsigned long long full[kSt], empty[kSt], acc_full, acc_free, chunk_full, chunk_free, drain;
   uint32_t tmem;
-  int abort_flag;
+  int abort_flag, leave_y;
   alignas(16) float par[3 * 192];  // bias, gain, shift
   float2 stat[2][kTM];             // (sum, sum of squared deviations) of a row's halves
 };
@@ -138,7 +139,8 @@ template <int N>
 __device__ __forceinline__ void copy_role(const GemmArgs& a, uint32_t sbase, int ns) {
   volatile int* abort_flag = &s_gm.abort_flag;
   pdl_wait();
-  const int tiles = num_tiles(a);
+  const int tiles = num_tiles(a), leave = !a.out && __ldcg(a.status + 1) == __ldcg(a.status + 2);
+  s_gm.leave_y = leave;  // (before the first stage, without which no tile is finished; an epilogue thread that reads the words costs 3 %)
   uint32_t g = 0;
   for (int t = blockIdx.x; t < tiles && !*abort_flag; t += gridDim.x)
     for (int s = 0; s < ns; ++s, ++g) {
@@ -382,10 +384,11 @@ __device__ __forceinline__ void epilogue_role(const GemmArgs& a, const Pass& ps,
       }
     }
     if (bar_or(1, kEpiThreads, *abort_flag != 0)) break;
+    const Pass to = {ps.s_first, ps.s_end, ps.row0, EPI == kNorm && s_gm.leave_y ? 0 : ps.row_end};
 #pragma unroll 4
     for (int p = 0; p < P; ++p) {
       const int rr = r16 + kRows * p, pos = p0 + rr;
-      const int v = a.out ? (pos >= ps.row0 && pos < ps.row_end ? pos : -1) : voxel_at(a, ps, pos);
+      const int v = a.out ? (pos >= to.row0 && pos < to.row_end ? pos : -1) : voxel_at(a, to, pos);
       float4* dst = reinterpret_cast<float4*>(a.out ? a.out + (size_t)v * a.ldo + nt * N : a.y + (size_t)v * N) + c16;
       float4 f[J];
 #pragma unroll
@@ -395,7 +398,10 @@ __device__ __forceinline__ void epilogue_role(const GemmArgs& a, const Pass& ps,
         if (v >= 0) dst[16 * j] = f[j];
     }
   }
-  if (threadIdx.x == 0 && *abort_flag) atomicOr(a.status, DSVT_STATUS_TIMEOUT);
+  if (threadIdx.x == 0 && *abort_flag) {
+    atomicOr(a.status, DSVT_STATUS_TIMEOUT);
+    atomicExch(a.status + 2, __ldcg(a.status + 1));
+  }
 }
 
 // out = epilogue(rows W^T + bias): tiles of 128 positions x N outputs, persistent blocks; a tile's epilogue runs under the
@@ -472,7 +478,7 @@ struct PrepArgs {
   WeightJob weight[4 * kPrepLayers];
   ListJob job[2];
   int32_t n, pass_rows, rows;  // positions whose sets a pass takes; entries of a pass (a set may reach past the former)
-  int32_t n_weights;
+  int32_t n_weights, new_call;
   int32_t* status;
 };
 
@@ -513,6 +519,7 @@ __device__ __noinline__ bool claimed(const ListJob& j, int S, int x) {
 // between them, whatever the offsets are, so that a pass has no position that nobody wrote.
 __global__ void __launch_bounds__(256) f32_prepare_kernel(const __grid_constant__ PrepArgs a) {
   pdl_enter();
+  if (a.new_call && (blockIdx.x | blockIdx.y | threadIdx.x) == 0) atomicAdd(a.status + 1, 1);
   if ((int)blockIdx.y < a.n_weights) {
     prepare_weights(a.weight[blockIdx.y]);
     return;
@@ -875,10 +882,10 @@ bool dsvt_layer_f32_supported(const dsvt_fused_args& a) {
 
 // Preparation for layers[0 .. kPrepLayers): the parts of their weights, and the row lists of the (at most kPrepLayers) tables
 // they run on.  `list` receives which of the two lists each layer uses; returns how many layers have been prepared.
-static int prepare(dsvt_ctx* ctx, const Work& ws, const dsvt_fused_args* layers, int n_layers, int (&list)[kPrepLayers], int* prepared) {
+static int prepare(dsvt_ctx* ctx, const Work& ws, const dsvt_fused_args* layers, int n_layers, bool new_call, int (&list)[kPrepLayers], int* prepared) {
   const int64_t R = ws.pass_rows;
   PrepArgs a = {};
-  a.n = layers[0].n; a.pass_rows = (int32_t)R; a.rows = (int32_t)ws.entries; a.status = ctx->status;
+  a.n = layers[0].n; a.pass_rows = (int32_t)R; a.rows = (int32_t)ws.entries; a.status = ctx->status; a.new_call = new_call;
   const int count = n_layers < kPrepLayers ? n_layers : kPrepLayers;
   int n_lists = 0;
   int64_t units = 0;
@@ -916,7 +923,7 @@ static int prepare(dsvt_ctx* ctx, const Work& ws, const dsvt_fused_args* layers,
   return DSVT_OK;
 }
 
-int dsvt_launch_layers_f32(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_layers) {
+int dsvt_launch_layers_f32(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_layers, bool new_call) {
   const Work ws = workspace(ctx, layers[0].p.C, layers[0].n);
   const int64_t R = ws.pass_rows, E = ws.entries;
   int lists[kPrepLayers], first = 0, prepared = 0;  // layers [first, first + prepared) are prepared
@@ -924,7 +931,7 @@ int dsvt_launch_layers_f32(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_l
   for (int i = 0; i < n_layers; ++i) {
     if (i == first + prepared) {
       first = i;
-      const int rc = prepare(ctx, ws, layers + i, n_layers - i, lists, &prepared);
+      const int rc = prepare(ctx, ws, layers + i, n_layers - i, new_call && i == 0, lists, &prepared);
       if (rc != DSVT_OK) return rc;
       parts = ws.parts;
     }
@@ -985,7 +992,7 @@ int dsvt_launch_layers_f32(dsvt_ctx* ctx, const dsvt_fused_args* layers, int n_l
     parts += layer_weights(C, hidden);
     // a table may hold more rows than there are voxels (voxels in several sets): the sets past the passes
     if (slots > passes * R) {
-      const int rc = dsvt_launch_layer_fma(ctx, a, (int64_t)passes * R);
+      const int rc = dsvt_launch_layer_fma(ctx, a, (int64_t)passes * R, ctx->status + 1);
       if (rc != DSVT_OK) return rc;
     }
   }

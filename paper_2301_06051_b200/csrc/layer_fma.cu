@@ -23,6 +23,7 @@ struct FmaGeom {
   int LDQ;   // row stride of the wide buffer (>= 3C, LDQ % 32 == 4)
   int C, hidden, heads, d, tau;
   int from;  // sets whose first row lies before this one are left out
+  const int32_t* calls;  // or NULL (see dsvt_launch_layer_fma)
   // relative position bias: entries per head, strides of the x and y offsets, index of the zero offset
   int rb_len, rb_sx, rb_sy, rb_centre;
 };
@@ -73,8 +74,9 @@ layer_fma_kernel(dsvt_fused_args a, FmaGeom g, int32_t* __restrict__ status) {
   const WT* W2 = reinterpret_cast<const WT*>(p.W_2);
 
   pdl_enter();  // everything below may read what earlier kernels of the stream wrote
+  const bool leave = g.calls && __ldcg(g.calls) == __ldcg(g.calls + 1);
   const int S = min(*a.num_sets, a.cap_sets);
-  if (S <= 0) return;
+  if (S <= 0 || leave) return;
   const int R = a.rowoff[S];
   const int num_tiles = (R - g.from + g.TMn - 1) / g.TMn;
 
@@ -311,7 +313,7 @@ int launch_rm(dsvt_ctx* ctx, const dsvt_fused_args& a, const FmaGeom& g, int gri
 
 }  // namespace
 
-int dsvt_launch_layer_fma(dsvt_ctx* ctx, const dsvt_fused_args& a, int64_t from_row) {
+int dsvt_launch_layer_fma(dsvt_ctx* ctx, const dsvt_fused_args& a, int64_t from_row, const int32_t* calls) {
   const dsvt_layer_params& p = a.p;
   FmaGeom g;
   g.C = p.C; g.hidden = a.attention_only ? 0 : p.hidden; g.heads = p.heads; g.d = p.C / p.heads; g.tau = p.set_size;
@@ -334,6 +336,7 @@ int dsvt_launch_layer_fma(dsvt_ctx* ctx, const dsvt_fused_args& a, int64_t from_
   if (g.TM == 0) return DSVT_ERR_UNSUPPORTED;
   g.TMn = g.TM - g.tau + 1;
   g.from = (int)from_row;
+  g.calls = calls;
   int64_t rmax = (int64_t)a.cap_sets * g.tau;
   if (rmax > a.n) rmax = a.n;
   int64_t grid = dsvt_ceil_div(rmax, g.TMn);

@@ -1,4 +1,6 @@
 """The fp32 layer kernel through the C ABI against the CPU oracle, at the sizes where its tiling changes.  Needs a B200."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -229,6 +231,56 @@ def test_passes_follow_the_call_and_not_the_context(oracle):
         assert all(k == seen[0][0] and torch.equal(y, seen[0][1]) for k, y in seen)
         p = oracle.partition(case["coords"], 1, case["grid"], case["window"], tau, 0)
         check_close(seen[0][1].cpu().numpy(), oracle.layer(case["feats"], p.set_table, case["blocks"][0][0]), "fp32", "n=%d" % n)
+
+
+class _ContextHead(ctypes.Structure):
+    """The beginning of the library's context, up to the address of its device status words."""
+    _fields_ = [("device", ctypes.c_int), ("stream", ctypes.c_void_p), ("max_voxels", ctypes.c_int64), ("max_windows", ctypes.c_int64),
+                ("max_channels", ctypes.c_int32), ("sm_count", ctypes.c_int), ("layer_ctas", ctypes.c_int), ("last_cuda_error", ctypes.c_int),
+                ("attr_flags", ctypes.c_uint), ("launches", ctypes.c_int64), ("arena", ctypes.c_void_p), ("arena_bytes", ctypes.c_size_t),
+                ("status", ctypes.c_void_p)]
+
+
+def _status_words(ctx):
+    head = _ContextHead.from_address(ctx._h.value)
+    assert head.max_voxels == ctx.limits[0] and head.status == head.arena  # (the layout is still this one)
+
+    class Words:
+        __cuda_array_interface__ = {"shape": (3,), "typestr": "<i4", "data": (head.status, False), "version": 3}
+
+    return torch.as_tensor(Words(), device="cuda")
+
+
+@pytest.mark.parametrize("C,heads,hidden,copies", [(192, 8, 384, 1), (128, 8, 0, 1), (64, 4, 128, 6)])
+def test_after_a_wait_has_given_up_the_call_leaves_y_alone(oracle, C, heads, hidden, copies):
+    """The call's number is put down as that of a call one of whose waits has given up, as the kernel that gives up does: the
+    kernels behind it store nothing to y, those for sets past the passes (voxels in several sets) included, and the next call is as ever."""
+    from paper_2301_06051_b200 import api
+
+    n, tau = 900, 36
+    case = di.random_case(n + C, n, (48, 48, 1), (12, 12, 1), tau, C, heads, hidden, layernorm=hidden > 0)
+    ctx = api.Context(n, 16, C)
+    x = dev(case["feats"])
+    p = [oracle.partition(case["coords"], 1, case["grid"], case["window"], tau, a).set_table for a in (0, 1)]
+    tables = [upload_table(np.concatenate([q] * copies)) for q in p]
+    layers = (case["blocks"][0] * 2)[: 1 if copies > 1 else 3]
+    w = [api.device_weights(l, api.FP32, ctx.device) for l in layers]
+    t = [tables[i & 1] for i in range(len(layers))]
+    want = case["feats"]
+    for i, l in enumerate(layers):
+        want = oracle.layer(want, p[i & 1], l)
+    y = torch.empty_like(x)
+    words = _status_words(ctx)
+    for given_up in (False, True, False):
+        y.fill_(77.0)
+        if given_up:
+            words[2] = words[1] + 1
+        ctx.layers(x, t, w, y)
+        if given_up:
+            assert torch.all(y == 77.0)
+        else:
+            check_close(y.cpu().numpy(), want, "fp32", "a call in which no wait gave up")
+        assert ctx.status_sync() == 0
 
 
 def test_chain_of_fp32_layers_on_several_tables(oracle):
