@@ -233,6 +233,48 @@ def test_passes_follow_the_call_and_not_the_context(oracle):
         check_close(seen[0][1].cpu().numpy(), oracle.layer(case["feats"], p.set_table, case["blocks"][0][0]), "fp32", "n=%d" % n)
 
 
+@pytest.mark.parametrize("C,heads,window,tau,hidden,option", [
+    (192, 8, 12, 36, 384, "pe"),
+    (192, 8, 2, 36, 0, ""),       # dozens of sets in a tile of 128 rows
+    (128, 4, 30, 90, 256, "rpb"),
+    (64, 4, 12, 36, 128, ""),
+])
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), 3.4e38])
+def test_a_wild_row_stays_in_its_set_in_fp32(C, heads, window, tau, hidden, option, value):
+    """Voxels of features that are not finite, or whose products overflow, change no row outside their own sets (bitwise),
+    although sets share tiles and the workspace keeps what they left."""
+    from paper_2301_06051_b200 import api
+
+    n, grid = 2500, (60, 60, 1)
+    case = di.random_case(n + C, n, grid, (window, window, 1), tau, C, heads, hidden, layernorm=hidden > 0)
+    layer, rng = case["blocks"][0][0], np.random.default_rng(C)
+    if option == "rpb":
+        layer["rpb"] = rng.standard_normal((heads, (2 * window - 1) ** 2)).astype(np.float32)
+        layer["rpb_extent"] = (window, window, 1)
+    ctx = api.Context(n, (60 // window) ** 2, C)
+    coords, x = dev(case["coords"]), dev(case["feats"])
+    pe = dev(rng.standard_normal((n, C)).astype(np.float32)) if option == "pe" else None
+    t = ctx.partition(coords, 1, grid, (window, window, 1), tau, 0)
+    w = api.device_weights(layer, api.FP32, ctx.device)
+    clean, y = torch.empty_like(x), torch.empty_like(x)
+    ctx.layer(x, t, w, clean, pe=pe, coords=coords)
+    table = t.set_table[: int(t.num_sets.item())]
+    wild = torch.as_tensor(rng.choice(n, 6, replace=False), device="cuda")
+    sets = torch.isin(table, wild.to(torch.int32)).any(dim=1)
+    inside = torch.zeros(n, dtype=torch.bool, device="cuda")
+    inside[table[sets].reshape(-1).long()] = True
+    spoilt = x.clone()
+    spoilt[wild, ::5] = value
+    spoilt[wild[0]] = value  # (and one whole row)
+    ctx.layer(spoilt, t, w, y, pe=pe, coords=coords)
+    assert ctx.status_sync() == 0
+    assert torch.equal(y[~inside], clean[~inside])
+    if value != value:
+        assert torch.isnan(y[inside]).any(dim=1).all()
+    ctx.layer(x, t, w, y, pe=pe, coords=coords)
+    assert torch.equal(y, clean)
+
+
 class _ContextHead(ctypes.Structure):
     """The beginning of the library's context, up to the address of its device status words."""
     _fields_ = [("device", ctypes.c_int), ("stream", ctypes.c_void_p), ("max_voxels", ctypes.c_int64), ("max_windows", ctypes.c_int64),
