@@ -22,8 +22,13 @@
  *     dsvt_status_sync reports it.
  *   - No call throws, aborts, or frees caller memory.
  *   - Matrices are row-major; a linear map is y = W x + b with W stored [out][in].
- *   - precision = DSVT_FP32: weights are float, arithmetic is fp32 throughout; in the shapes that the tensor cores take (C of
- *     64, 128, 192) a product's operands go in as three bfloat16 parts each, which hold all of their 24 bits.
+ *   - precision = DSVT_FP32: weights are float, arithmetic is fp32 throughout.  In the shapes that the tensor cores take (C of
+ *     64, 128 or 192, hidden a multiple of 64) a product's operands go in as three bfloat16 parts each, which hold all of
+ *     their 24 bits; of the nine products of parts the three smallest are left out (at most 0.9 x 2^-24 of a product), the
+ *     tensor cores' additions truncate and are read out every 48 or 64 terms into sums that round, and the softmax takes the
+ *     hardware's approximate exponential of base two.  Two layers are off by 1.0e-7 ... 2.4e-7 of the result (2-norm, against
+ *     float64); sums whose terms all have one sign are off by more than fp32 multiply-adds (attention with positive weights
+ *     and features: 1.2e-7 where these are off by 0.8e-7).
  *     precision = DSVT_BF16_FP32ACC: weights are bfloat16 (16-bit storage); products
  *     accumulate in fp32; residual stream, LayerNorm, softmax and GELU are fp32.
  *     Features (x, y, feats, out) and biases / LayerNorm parameters are always float.
@@ -273,7 +278,8 @@ typedef struct dsvt_layer_params {
    * coords[query] - coords[key].  coords: int32 [n][4] = (b, x, y, z), required with rpb.
    * rpb_extent = (L, W, H): the window extent the table covers, at least the window the set
    * table was cut with.  A set whose members are spread wider raises DSVT_STATUS_BAD_INDEX and
-   * its out-of-table pairs read a clamped entry. */
+   * its out-of-table pairs read a clamped entry.  An entry of -inf or of the lowest float masks its pairs.  A row
+   * with masked pairs only gets equal weights with DSVT_FP32 and the lowest float; otherwise it is not defined. */
   const float* rpb;
   const int32_t* coords;
   int32_t rpb_extent[3];
@@ -282,8 +288,9 @@ typedef struct dsvt_layer_params {
 /*
  * One DSVT layer (Eq. 5 with Appendix B.1.1): x1 = LN1(x + MHSA_sets(x));
  * y = LN2(x1 + W_2 gelu(W_1 x1 + b_1) + b_2), gelu(t) = t/2 (1 + erf(t/sqrt 2)); LayerNorm over the
- * C channels with biased variance.  y may alias x (each voxel belongs to one set, and a set is
- * processed by one thread block).  Rows of voxels in no set are left untouched in y.
+ * C channels with biased variance.  y may alias x (each voxel belongs to one set, and a set's rows of y are
+ * written after everything that reads its rows of x).  Rows of voxels in no set are left untouched in y.
+ * If a bounded wait expires (DSVT_STATUS_TIMEOUT), rows that were not written by then may stay as they were.
  */
 int dsvt_layer(dsvt_ctx* ctx, const float* x, int32_t n, const int32_t* set_table, int32_t cap_sets,
                const int32_t* num_sets, const int32_t* set_rowoff, const dsvt_layer_params* params, float* y);
@@ -377,8 +384,8 @@ int dsvt_bev_scatter(dsvt_ctx* ctx, const int32_t* coords, const float* feats, i
 /*
  * A measurement aid (the paper has no counterpart): launches a kernel of `blocks` x `threads` threads that
  * each run `iters` rounds of eight independent fp32 fused multiply-adds and nothing else, on the context's stream.
- * A benchmark times it to learn the FP32 FMA rate of the device, which bounds the fp32 layer path (that path's
- * arithmetic runs on the FMA pipes, not on the tensor cores).  *flops (HOST, optional) receives the number of
+ * A benchmark times it to learn the FP32 FMA rate of the device, which bounds the layer kernel for general shapes (its
+ * products run on the FMA pipes, not on the tensor cores).  *flops (HOST, optional) receives the number of
  * floating-point operations of the launch (2 per multiply-add); sink is a device float the kernel may write.
  * threads: a multiple of 32, at most 1024.
  */

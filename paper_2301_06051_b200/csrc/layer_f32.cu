@@ -26,9 +26,10 @@
 //   C = 64, hidden 128        1.9e-7 -> 1.6e-7    1.2e-6 -> 1.1e-6
 // One attention with positive weights and features, where truncations add up: 0.8e-7 -> 1.2e-7.
 //
-// Measured (B200): two full layers and their partition, 12,345 pillars, C = 192: 776 us on the FMA pipes (27 % of their peak:
-// shared-memory reads for the products, and the phases between them), 282 us now; two attention-only layers, 2,000 pillars,
-// C = 128: 109 us and 91 us.  A product's tile of 128 rows takes 9 to 11 k cycles, the start of each of its kernels 4 k
+// Measured (B200): two full layers and their partition, 12,345 pillars, C = 192: 775.8 us on the FMA pipes (27 % of their peak:
+// shared-memory reads for the products, and the phases between them), 290.5 us now; two attention-only layers, 2,000 pillars,
+// C = 128: 110.3 us and 90.9.  A single voxel, which then was one launch of a tile of eight rows, has got slower: a full layer
+// 50.4 us -> 65.0 (60 voxels 84.9 -> 73.2).  A product's tile of 128 rows takes 9 to 11 k cycles, the start of each of its kernels 4 k
 // (first instructions, lists, operands) and its epilogue 6 k.
 //
 // Every wait is bounded; one that gives up raises DSVT_STATUS_TIMEOUT, its block stores nothing more, and no later kernel of the call

@@ -3,8 +3,8 @@
 // LayerNorm -> scatter (Appendix B.1.1).  One thread block owns a tile of whole sets; because the sets
 // partition the voxels (Theorems A.2, A.3), no two blocks touch the same voxel row.
 //
-// This kernel is the fp32 path (DSVT_FP32) and the general-shape path of DSVT_BF16_FP32ACC: weights
-// may be float or bfloat16, all arithmetic is fp32.
+// This kernel takes the shapes that the tensor-core kernels (layer_tc.cu, layer_f32.cu) do not, and the sets of fp32 layers past
+// layer_f32.cu's passes: weights may be float or bfloat16, all arithmetic is fp32.
 //
 // Only the distinct members of a set are brought into the tile (a duplicated slot is masked as a key
 // and never written back, so it contributes nothing); a set's distinct members occupy consecutive

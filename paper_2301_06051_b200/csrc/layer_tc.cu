@@ -206,8 +206,8 @@ __device__ __forceinline__ float2 gelu_fast2(float2 t) {
 // A block of 16 keys' relative position biases onto a row's scores, from the rows' linear coordinates; `tab` is the head's table,
 // `root` the square root of the head dimension (the scores are still unscaled dot products when the bias is added).  An index is
 // formed in the upper half of a word (`from`: (the row's coordinate + centre) 2^16 + 65535, so that the lower half never borrows),
-// two keys to a word of shared memory (hybrid windows, 20,011 pillars: 309.2 us with a 16-bit read and a sign extension per key,
-// 300.8 now).  A negative index is large there and takes the last entry like one past the table.
+// two keys to a word of shared memory (hybrid windows, 20,011 pillars: 309.4 us with a 16-bit read and a sign extension per key,
+// 304.2 now).  A negative index is large there and takes the last entry like one past the table.
 __device__ __forceinline__ void add_rpb(float (&s)[16], const float* __restrict__ tab, uint32_t from, int b, float root) {
   const uint32_t last = (uint32_t)(s_mi.rb_len - 1) << 16 | 0xffffu;
   const uint4* lin = reinterpret_cast<const uint4*>(&s_mi.rowlin[16 * b]);

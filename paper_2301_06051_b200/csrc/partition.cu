@@ -1129,7 +1129,8 @@ int partition_bitmap(dsvt_ctx* ctx, const PartCall& pc, int32_t wpw, int naxes, 
   uint32_t* bitmap0 = reinterpret_cast<uint32_t*>(dup_count + (nw + 1));
   // (not overlapped: frames run one after the other are partitioned under the tail of the last chain of layers, which
   // blocks that wait there slow down: 32,000-pillar frame 398.6 us, overlapped 400.0, with a memset 399.2; the tables of
-  // a batch alone 59.0, 57.9 and 59.4 us)
+  // a batch alone 59.0, 57.9 and 59.4 us.  One that overlaps must not write before its wait: these arrays are the workspace
+  // of the context's fp32 layers, whose last kernel may still be reading them)
   int rc = dsvt_launch_fill(ctx, counts, 0, 2 * (int64_t)(nw + 1) + (int64_t)naxes * words, false);
   if (rc != DSVT_OK) return rc;
   BmJob job;

@@ -1,6 +1,6 @@
 // A measurement aid, not a step of the method: a kernel that does nothing but dependent-free fp32 fused
-// multiply-adds, so that a benchmark can time the FP32 FMA rate of the device it runs on (the bound of the fp32
-// layer path, whose arithmetic runs on the FMA pipes and not on the tensor cores).
+// multiply-adds, so that a benchmark can time the FP32 FMA rate of the device it runs on (the bound of the layer kernel
+// for general shapes, whose products run on the FMA pipes and not on the tensor cores).
 #include "dsvt_common.cuh"
 
 namespace {
