@@ -32,8 +32,8 @@
 // 50.4 us -> 65.0 (60 voxels 84.9 -> 73.2).  A product's tile of 128 rows takes 9 to 11 k cycles, the start of each of its kernels 4 k
 // (first instructions, lists, operands) and its epilogue 6 k.
 //
-// Every wait is bounded; one that gives up raises DSVT_STATUS_TIMEOUT, its block stores nothing more, and no later kernel of the call
-// stores to y (what lies in the workspace for its rows is another call's).
+// Every wait is bounded; one that gives up raises DSVT_STATUS_TIMEOUT, its block stores nothing more, and no later kernel of
+// the call's fp32 layers stores to y (what lies in the workspace for its rows is another call's).
 #include <limits.h>
 
 #include "dsvt_common.cuh"
